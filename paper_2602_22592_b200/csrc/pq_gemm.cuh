@@ -49,7 +49,7 @@ struct Segment {
   int acc;                  // accumulator of the tile this segment adds into
   int nkb;                  // k-blocks (128 bytes of K each: 128 int8 / 64 bf16)
   int bn;                   // UMMA N for this segment (multiple of 16, <= 256; MN-major B: multiple of 64)
-  int ksteps;               // UMMA k-steps issued per k-block (1..4)
+  int ksteps;               // UMMA k-steps issued per k-block: 4, or fewer (MODE_BF_KM only)
   const CUtensorMap* ta;
   const CUtensorMap* tb;
   int a_x, a_y, a_z;        // K operand: (k0, row0, z);  MN operand: (mn0, k0, z)
@@ -263,43 +263,70 @@ __device__ __forceinline__ void gemm_body(const typename P::Params& p) {
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      PipeState st, ac;
-      bool ok = true;
-      for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
-        typename P::Tile t;
-        P::tile_init(p, tile, t);
-        const int nseg = P::num_segments(p, t);
-        if (!pipe_wait(tempty_bar(ac.stage), ac.phase ^ 1, WHERE_MMA, abort_flag)) { ok = false; break; }
-        tc_fence_after();
-        uint32_t started[2] = {0u, 0u};
-        for (int s = 0; ok && s < nseg; ++s) {
-          Segment sg;
-          sg.b2_y = -1;
-          P::segment(p, t, s, sg);
-          const uint32_t d_tmem = tmem_base + Acc::col(ac.stage, sg.acc);
-          const bool amn = a_is_mn(sg.mode), bmn = b_is_mn(sg.mode);
-          const uint32_t idesc = (sg.mode == MODE_I8_KK) ? umma_idesc(2, 1, 0, 0, sg.bn)
-                                                          : umma_idesc(1, 1, amn ? 1 : 0, bmn ? 1 : 0, sg.bn);
+    // The whole warp walks the loops, one elected thread issues.  What a tcgen05.mma costs to issue decides the rate: with
+    // the descriptors put together per instruction in 64-bit arithmetic, the operand form tested inside the loop and a loop
+    // over the k-steps the kernels ran at 190-230 cycles per MMA whatever the operands did (8192^3 int8: 2.7 POP/s with the
+    // loads taken out); with the loop below, unrolled and specialised on the operand form, at the 128 cycles of the tensor
+    // pipe (4.5 POP/s int8, 2.2 PFLOP/s bf16, loads taken out).
+    PipeState st, ac;
+    bool ok = true;
+    auto all_wait = [&](uint32_t bar, uint32_t parity) {
+      const bool got = __all_sync(0xffffffffu, pipe_wait(bar, parity, WHERE_MMA, abort_flag));
+      tc_fence_after();
+      return got;
+    };
+    for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
+      typename P::Tile t;
+      P::tile_init(p, tile, t);
+      const int nseg = P::num_segments(p, t);
+      if (!all_wait(tempty_bar(ac.stage), ac.phase ^ 1)) { ok = false; break; }
+      uint32_t opened = 0u;              // bit a: accumulator a has been written to
+      for (int s = 0; ok && s < nseg; ++s) {
+        Segment sg;
+        sg.b2_y = -1;
+        P::segment(p, t, s, sg);
+        const uint32_t d_tmem = tmem_base + Acc::col(ac.stage, sg.acc);
+        uint32_t started = (opened >> sg.acc) & 1u;
+        opened |= 1u << sg.acc;
+        // OP: operand form, STEPS: k-steps per k-block (0: as the segment says)
+        auto contract = [&](auto op, auto steps) {
+          constexpr int OP = decltype(op)::value, STEPS = decltype(steps)::value;
+          constexpr bool amn = OP == MODE_BF_MM, bmn = OP >= MODE_BF_KM;
+          constexpr uint32_t astep = amn ? 2048 >> 4 : 32 >> 4, bstep = bmn ? 2048 >> 4 : 32 >> 4;
+          const uint32_t idesc = OP == MODE_I8_KK ? umma_idesc(2, 1, 0, 0, sg.bn) : umma_idesc(1, 1, amn ? 1 : 0, bmn ? 1 : 0, sg.bn);
+          const uint64_t a0 = umma_smem_desc(smem_base, amn ? kMnBoxBytes : 16, 1024);
+          const uint64_t b0 = umma_smem_desc(smem_base + kStageABytes, bmn ? kMnBoxBytes : 16, 1024);
+          const uint32_t ahi = (uint32_t)(a0 >> 32), bhi = (uint32_t)(b0 >> 32);
           for (int kb = 0; kb < sg.nkb; ++kb) {
-            if (!pipe_wait(full_bar(st.stage), st.phase, WHERE_MMA, abort_flag)) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t sa = smem_base + st.stage * kStageBytes;
-            const uint32_t sb = sa + kStageABytes;
-            for (int k = 0; k < sg.ksteps; ++k) {
-              const uint64_t ad = amn ? umma_smem_desc(sa + k * 2048, kMnBoxBytes, 1024) : umma_smem_desc(sa + k * 32, 16, 1024);
-              const uint64_t bd = bmn ? umma_smem_desc(sb + k * 2048, kMnBoxBytes, 1024) : umma_smem_desc(sb + k * 32, 16, 1024);
-              if (sg.mode == MODE_I8_KK) umma_i8(d_tmem, ad, bd, idesc, started[sg.acc]);
-              else umma_f16(d_tmem, ad, bd, idesc, started[sg.acc]);
-              started[sg.acc] = 1u;
+            if (!all_wait(full_bar(st.stage), st.phase)) { ok = false; break; }
+            const uint32_t off = (st.stage * kStageBytes) >> 4;   // addresses stay below 2^18: no carry out of the field
+            const uint32_t alo = (uint32_t)a0 + off, blo = (uint32_t)b0 + off;
+            auto step = [&](int k) {
+              const uint64_t ad = ((uint64_t)ahi << 32) | (alo + k * astep), bd = ((uint64_t)bhi << 32) | (blo + k * bstep);
+              if (OP == MODE_I8_KK) umma_i8(d_tmem, ad, bd, idesc, k ? 1u : started);
+              else umma_f16(d_tmem, ad, bd, idesc, k ? 1u : started);
+            };
+            if (elect_one()) {
+              if (STEPS > 0) {
+#pragma unroll
+                for (int k = 0; k < STEPS; ++k) step(k);
+              } else {
+                for (int k = 0; k < sg.ksteps; ++k) step(k);
+              }
+              umma_commit(empty_bar(st.stage));  // frees the smem stage once these MMAs retire
             }
-            umma_commit(empty_bar(st.stage));  // frees the smem stage once these MMAs retire
+            started = 1u;
             st.advance(kStages);
           }
-        }
-        if (ok) umma_commit(tfull_bar(ac.stage));
-        ac.advance(kAccStages);
+        };
+        if (sg.ksteps != 4) contract(std::integral_constant<int, MODE_BF_KM>{}, std::integral_constant<int, 0>{});   // the router's one step
+        else if (sg.mode == MODE_I8_KK) contract(std::integral_constant<int, MODE_I8_KK>{}, std::integral_constant<int, 4>{});
+        else if (sg.mode == MODE_BF_KK) contract(std::integral_constant<int, MODE_BF_KK>{}, std::integral_constant<int, 4>{});
+        else if (sg.mode == MODE_BF_KM) contract(std::integral_constant<int, MODE_BF_KM>{}, std::integral_constant<int, 4>{});
+        else contract(std::integral_constant<int, MODE_BF_MM>{}, std::integral_constant<int, 4>{});
       }
+      if (ok && elect_one()) umma_commit(tfull_bar(ac.stage));
+      ac.advance(kAccStages);
     }
   } else {
     // ------------------------------------------------------------ epilogue warps
