@@ -77,6 +77,9 @@ static size_t carve_saved(const pq_desc* d, void* base, SavedPtrs* out) {
   s.rt.items = c.take<int4>(s.max_items);
   s.rt.tile_item_begin = c.take<int>(mtiles_of(d) + 1);
   s.rt.expert_item_begin = c.take<int>(E + 1);
+  const int mpairs = (mtiles_of(d) + 1) / 2;
+  s.rt.pair_begin = c.take<int>(mpairs + 1);
+  s.rt.pair_items = c.take<int4>(mpairs + E - 1);
   if (out) *out = s;
   return c.off;
 }

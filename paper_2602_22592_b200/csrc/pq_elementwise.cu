@@ -346,28 +346,31 @@ __global__ void __launch_bounds__(512) k_route_scan(int T, int E, int nblocks, c
 
   // items: one thread per tile counts its items, a block-wide scan places them
   const int mtiles = (T + kTileRows - 1) / kTileRows;
-  for (int base = 0; base < mtiles; base += blockDim.x) {
-    const int tile = base + threadIdx.x;
-    const int r0 = tile * kTileRows, r1 = min(T, r0 + kTileRows);
-    const int cnt = tile < mtiles ? tile_items(off, Ee, r0, r1, [](int, int, int, int) {}) : 0;
-    int inc = cnt;
-    for (int d = 1; d < 32; d <<= 1) {
-      const int u = __shfl_up_sync(0xffffffffu, inc, d);
-      if (lane >= d) inc += u;
+  auto scan_tiles = [&](int ntiles, int rows, auto place) {
+    for (int base = 0; base < ntiles; base += blockDim.x) {
+      const int tile = base + threadIdx.x;
+      const int r0 = tile * rows, r1 = min(T, r0 + rows);
+      const int cnt = tile < ntiles ? tile_items(off, Ee, r0, r1, [](int, int, int, int) {}) : 0;
+      int inc = cnt;
+      for (int d = 1; d < 32; d <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= d) inc += u;
+      }
+      if (lane == 31) warp_sums[warp] = inc;
+      __syncthreads();
+      int before = carry_sh;
+      for (int w = 0; w < warp; ++w) before += warp_sums[w];
+      const int first = before + inc - cnt;
+      if (tile < ntiles) place(tile, r0, r1, first);
+      __syncthreads();
+      if (threadIdx.x == blockDim.x - 1) carry_sh = first + cnt;
+      __syncthreads();
     }
-    if (lane == 31) warp_sums[warp] = inc;
-    __syncthreads();
-    int before = carry_sh;
-    for (int w = 0; w < warp; ++w) before += warp_sums[w];
-    const int first = before + inc - cnt;
-    if (tile < mtiles) {
-      rt.tile_item_begin[tile] = first;
-      tile_items(off, Ee, r0, r1, [&](int k, int e, int lo, int hi) { rt.items[first + k] = make_int4(tile, e, lo - r0, hi - r0); });
-    }
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry_sh = first + cnt;
-    __syncthreads();
-  }
+  };
+  scan_tiles(mtiles, kTileRows, [&](int tile, int r0, int r1, int first) {
+    rt.tile_item_begin[tile] = first;
+    tile_items(off, Ee, r0, r1, [&](int k, int e, int lo, int hi) { rt.items[first + k] = make_int4(tile, e, lo - r0, hi - r0); });
+  });
   const int n_items = carry_sh;
   if (threadIdx.x == 0) { rt.tile_item_begin[mtiles] = n_items; rt.n_items[0] = n_items; }
   // first item of each expert: the first item of the tile holding its first row, plus the items of the
@@ -384,6 +387,20 @@ __global__ void __launch_bounds__(512) k_route_scan(int T, int E, int nblocks, c
     }
     rt.expert_item_begin[threadIdx.x] = idx;
   }
+  // the same for pairs of tiles; the items of a tile are in expert order, so each expert of the pair takes the next one
+  __syncthreads();
+  if (threadIdx.x == 0) carry_sh = 0;
+  __syncthreads();
+  const int mpairs = (mtiles + 1) / 2;
+  scan_tiles(mpairs, 2 * kTileRows, [&](int pair, int r0, int r1, int first) {
+    const int mid = r0 + kTileRows;
+    int i0 = rt.tile_item_begin[2 * pair], i1 = mid < r1 ? rt.tile_item_begin[2 * pair + 1] : 0;
+    rt.pair_begin[pair] = first;
+    tile_items(off, Ee, r0, r1, [&](int k, int e, int lo, int hi) {
+      rt.pair_items[first + k] = make_int4(e, lo < mid ? i0++ : -1, hi > mid ? i1++ : -1, pair);
+    });
+  });
+  if (threadIdx.x == 0) rt.pair_begin[mpairs] = carry_sh;
 }
 
 // ---------------------------------------------------------------------------

@@ -1,10 +1,18 @@
 // Persistent, warp-specialised tcgen05 GEMM engine for sm_100a.
 //
-// One CTA per SM, 320 threads: warp 0 = TMA producer, warp 1 = MMA issuer
-// (also owns the TMEM allocation), warps 2-9 = epilogue (two per TMEM lane
-// quadrant, which take alternate column chunks of the tile).  Operands travel global -> shared by TMA into a ring (4 stages of 48 KB; more, smaller ones for narrow tiles) of
-// 128-byte-swizzled tiles; tcgen05.mma accumulates 128 x (<=256) tiles in
-// TMEM; the epilogue reads them back with tcgen05.ld.
+// Warp 0 = TMA producer, warp 1 = MMA issuer (also owns the TMEM allocation), the others = epilogue (kEpiWarps / 4 per
+// TMEM lane quadrant, which share the column chunks of the tile).  Operands travel global -> shared by TMA into a ring
+// of 128-byte-swizzled stages; tcgen05.mma accumulates in TMEM; the epilogue reads the accumulators with tcgen05.ld.
+//
+// Two forms, chosen by the problem (P::CG):
+//   CG = 2  a pair of CTAs (cluster of two, one CTA per SM) works on a tile of 256 rows x (<= 256) columns: each CTA
+//           loads its 128 rows of A and its half of B's columns, one thread of the first CTA issues the MMAs for both,
+//           and each CTA's TMEM receives its own 128 rows of the result.  This is the form of the large products: a step
+//           of 64 (bf16) or 128 (int8) contraction values of a 128 x 256 tile is 512 MMA cycles, but 48 KB of operands for
+//           one CTA alone -- 768 cycles of the 64 bytes per clock that an SM takes in from L2 -- and 32 KB, 512 cycles,
+//           for a CTA of a pair.
+//   CG = 1  one CTA, tiles of 128 rows: the small grouped products of the HP branch, whose rows belong to one expert
+//           per 128-row item.
 //
 // A tile's contraction is a list of SEGMENTS.  Each segment names its operand
 // form (int8 or bf16; each operand either contraction-contiguous "K" or
@@ -23,18 +31,15 @@
 
 namespace pq {
 
-constexpr int kEpiWarps = 8;
-constexpr int kGemmThreads = 64 + 32 * kEpiWarps;
-constexpr int kMaxStages = 8;             // barrier pairs reserved for the operand ring
+constexpr int kMaxStages = 12;            // barrier pairs reserved for the operand ring
 constexpr int kTileM = 128;
-constexpr int kStageABytes = 128 * 128;  // 128 rows x 128 B, or two 64x64 bf16 MN boxes
-constexpr int kStageBBytes = 256 * 128;  // up to 256 rows x 128 B, or four MN boxes
-constexpr int kRingBytes = 4 * (kStageABytes + kStageBBytes);   // operand ring: four stages of a 256-column tile
+constexpr int kOperandBytes = 128 * 128;  // 128 rows x 128 B, or two 64x64 bf16 MN boxes: one stage of one operand of a CTA
+constexpr int kRingBytes = 12 * kOperandBytes;
 constexpr int kMnBoxBytes = 64 * 128;    // one MN-major box: 64 k-rows of 64 bf16
 constexpr int kTmemCols = 512;
-constexpr int kAccCols = 256;            // TMEM columns of one accumulator stage in the default layout
-constexpr int kEpiWarpBytes = 32 * 128;                // per epilogue warp: 32 rows of one 128-byte chunk (xor-swizzled)
-constexpr int kGemmSmemBytes = kRingBytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kEpiWarps * kEpiWarpBytes;
+constexpr int kAccCols = 256;            // TMEM columns of one accumulator
+constexpr int kStagingBytes = 32 * 1024; // epilogue warps: transposing buffers (kStagingBytes / kEpiWarps each)
+constexpr int kGemmSmemBytes = kRingBytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kStagingBytes;
 static_assert(kGemmSmemBytes <= 227 * 1024, "shared memory of one CTA");
 
 enum OpMode : int {
@@ -44,47 +49,57 @@ enum OpMode : int {
   MODE_BF_MM = 3   // bf16, A M-contiguous, B N-contiguous
 };
 
+// What one CTA contributes to a step of 128 contraction bytes (64 rows of an MN-major operand) of a tile: 128 rows of A
+// and its share of B -- all of it (CG = 1) or one half of its columns (CG = 2).  Coordinates are this CTA's own.  Both CTAs
+// of a pair describe the same number of steps and bytes; a CTA without rows of its own in a segment gives coordinates
+// outside the tensor (TMA then fills with zeros).
 struct Segment {
   int mode;                 // OpMode
   int acc;                  // accumulator of the tile this segment adds into
   int nkb;                  // k-blocks (128 bytes of K each: 128 int8 / 64 bf16)
-  int bn;                   // UMMA N for this segment (multiple of 16, <= 256; MN-major B: multiple of 64)
+  int bn;                   // UMMA N for this segment (multiple of 16 (CG = 1) or 32 (CG = 2), <= 256)
   int ksteps;               // UMMA k-steps issued per k-block: 4, or fewer (MODE_BF_KM only)
   const CUtensorMap* ta;
   const CUtensorMap* tb;
   int a_x, a_y, a_z;        // K operand: (k0, row0, z);  MN operand: (mn0, k0, z)
   int b_x, b_y, b_z;
   int a_rank, b_rank;       // tensor-map rank (2 or 3)
-  int b_box;                // K-major B: rows one TMA load delivers (box height of tb); bn is covered by
-                            // ceil(bn / b_box) loads.  Per k-block B always occupies bn * 128 bytes.
-  int b2_y;                 // MN-major B only, -1 = unused: the columns [bn/2, bn) of B come from a second row range of
-                            // tb starting at k row b2_y (same columns b_x), e.g. the second bf16 plane of an operand
-  int a_blk, b_blk;         // MN-major operand read through a "blocked" tensor map (64-wide column blocks as an
-                            // extra dimension): number of blocks one load delivers; 0 = one 64 x 64 box per load
+  int a_blk;                // MN-major A: > 0 = read through a "blocked" tensor map (64-wide column blocks as an extra
+                            // dimension, both blocks in one load), else one 64 x 64 box per load
+  int b_blk;                // MN-major B: > 0 = blocked map delivering that many blocks in one load; < 0 = -b_blk plain boxes
+  int b_bytes;              // bytes of B this CTA loads per k-block (K-major: the box of tb)
 };
 
-// Output tiles are 128 rows x `bn` columns, the cells of an (mt x nt) grid walked row by row.
+// Output tiles are P::CG * 128 rows x `bn` columns, the cells of an (mt x nt) grid walked row by row.
 struct TileGrid {
   int mt, nt, bn, total;
 };
 __host__ inline TileGrid make_tile_grid(int mt, int nt, int bn) { return TileGrid{mt, nt, bn, mt * nt}; }
-struct TileCoord { int m, n0, bn; };
-__device__ __forceinline__ TileCoord tile_coord(const TileGrid& g, int i) {
-  return TileCoord{i / g.nt, (i % g.nt) * g.bn, g.bn};
+struct TileCoord { int m, n0, bn; };   // m: this CTA's 128-row tile
+template <int CG>
+__device__ __forceinline__ TileCoord tile_coord(const TileGrid& g, int i, int rank) {
+  return TileCoord{(i / g.nt) * CG + rank, (i % g.nt) * g.bn, g.bn};
 }
 
 __device__ __forceinline__ bool a_is_mn(int mode) { return mode == MODE_BF_MM; }
 __device__ __forceinline__ bool b_is_mn(int mode) { return mode >= MODE_BF_KM; }
 
-
+template <int CG>
 __device__ __forceinline__ void tma_fetch(uint32_t dst, const CUtensorMap* t, uint32_t bar, int rank, int x, int y, int z) {
-  if (rank == 3) tma_load_3d(dst, t, bar, x, y, z);
-  else tma_load_2d(dst, t, bar, x, y);
+  if (rank == 3) {
+    if (CG == 2) tma_pair_load_3d(dst, t, bar, x, y, z); else tma_load_3d(dst, t, bar, x, y, z);
+  } else {
+    if (CG == 2) tma_pair_load_2d(dst, t, bar, x, y); else tma_load_2d(dst, t, bar, x, y);
+  }
 }
 // Blocked view of an MN-major operand: dimensions (64 columns of a block, k row, block index[, batch]).
+template <int CG>
 __device__ __forceinline__ void tma_fetch_blocked(uint32_t dst, const CUtensorMap* t, uint32_t bar, int base_rank, int k, int blk, int z) {
-  if (base_rank == 3) tma_load_4d(dst, t, bar, 0, k, blk, z);
-  else tma_load_3d(dst, t, bar, 0, k, blk);
+  if (base_rank == 3) {
+    if (CG == 2) tma_pair_load_4d(dst, t, bar, 0, k, blk, z); else tma_load_4d(dst, t, bar, 0, k, blk, z);
+  } else {
+    if (CG == 2) tma_pair_load_3d(dst, t, bar, 0, k, blk); else tma_load_3d(dst, t, bar, 0, k, blk);
+  }
 }
 
 struct PipeState {
@@ -110,23 +125,26 @@ __device__ __forceinline__ bool pipe_wait(uint32_t bar, uint32_t parity, int whe
   return true;
 }
 
-// Coalescing store for epilogues.  Each lane holds 128 contiguous bytes (8 x 16 B) of ITS OWN output
-// row, and rows may live anywhere in global memory (row_ptr = 0 skips the row).  The warp transposes
-// through its staging buffer so that every store instruction writes 4 rows x 128 contiguous bytes
-// instead of 32 rows x 16 bytes.  Only the first valid_bytes of each row are written.  The 16-byte
-// piece j of row r sits at position j ^ (r & 7) of the row, which keeps both passes free of bank conflicts.
-__device__ __forceinline__ void warp_store_rows(uint8_t* stage, const uint4 (&v)[8], void* row_ptr, int valid_bytes, int lane) {
-  uint4* mine = reinterpret_cast<uint4*>(stage + lane * 128);
+// Coalescing store for epilogues.  Each lane holds PIECES * 16 contiguous bytes of ITS OWN output row, and rows may live
+// anywhere in global memory (row_ptr = 0 skips the row).  The warp transposes through its staging buffer (32 rows x
+// PIECES * 16 bytes) so that a store instruction writes whole runs of PIECES * 16 contiguous bytes instead of 32 rows x 16
+// bytes.  Only the first valid_bytes of each row are written.  The 16-byte piece j of row r sits at position
+// j ^ (r & 7) (eight pieces) or j ^ ((r >> 1) & 3) (four), which keeps both passes free of bank conflicts.
+template <int PIECES>
+__device__ __forceinline__ void warp_store_rows(uint8_t* stage, const uint4 (&v)[PIECES], void* row_ptr, int valid_bytes, int lane) {
+  static_assert(PIECES == 8 || PIECES == 4, "row pieces");
+  auto spot = [](int r, int j) { return PIECES == 8 ? (j ^ (r & 7)) : (j ^ ((r >> 1) & 3)); };
+  uint4* mine = reinterpret_cast<uint4*>(stage + lane * (PIECES * 16));
 #pragma unroll
-  for (int j = 0; j < 8; ++j) mine[j ^ (lane & 7)] = v[j];
+  for (int j = 0; j < PIECES; ++j) mine[spot(lane, j)] = v[j];
   __syncwarp();
   const unsigned long long my = reinterpret_cast<unsigned long long>(row_ptr);
-  const int c = lane & 7;
+  const int c = lane % PIECES;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int row = 4 * i + (lane >> 3);
+  for (int i = 0; i < PIECES; ++i) {
+    const int row = (32 / PIECES) * i + lane / PIECES;
     const unsigned long long dst = __shfl_sync(0xffffffffu, my, row);
-    const uint4 val = *reinterpret_cast<const uint4*>(stage + row * 128 + ((c ^ (row & 7)) << 4));
+    const uint4 val = *reinterpret_cast<const uint4*>(stage + row * (PIECES * 16) + (spot(row, c) << 4));
     if (dst != 0ull && c * 16 < valid_bytes) *reinterpret_cast<uint4*>(dst + c * 16) = val;
   }
   __syncwarp();
@@ -135,67 +153,71 @@ __device__ __forceinline__ void warp_store_rows(uint8_t* stage, const uint4 (&v)
 // Problems whose epilogue needs nothing fetched ahead of the accumulator
 struct NoPre {};
 
-// Widest B operand of a launch, in tile columns (B takes that many x 128 bytes of a stage): the ring holds as many
-// stages as fit, so a launch of narrow tiles keeps more k-blocks in flight.  Problems without `stage_cols` use 256.
+// Widest B operand of a CTA, in rows of 128 bytes (columns of the tile, or half of them for a pair): the ring holds as
+// many stages as fit, so a launch of narrow tiles keeps more k-blocks in flight.  Problems without `stage_rows` use
+// 256 (CG = 1) or 128 (CG = 2).
 template <class P, class = void>
-struct stage_cols_of {
-  __device__ static int get(const typename P::Params&) { return 256; }
+struct stage_rows_of {
+  __device__ static int get(const typename P::Params&) { return 256 / P::CG; }
 };
 template <class P>
-struct stage_cols_of<P, std::void_t<decltype(&P::stage_cols)>> {
-  __device__ static int get(const typename P::Params& p) { return P::stage_cols(p); }
+struct stage_rows_of<P, std::void_t<decltype(&P::stage_rows)>> {
+  __device__ static int get(const typename P::Params& p) { return P::stage_rows(p); }
 };
 
-// Accumulator layouts in TMEM (column of accumulator `acc` of pipeline stage `stage`).
-//   AccDouble     : one accumulator per tile, two stages of 256 columns.
-//   AccPair       : two accumulators of 256 columns per tile (all of TMEM), one stage: the epilogue of
-//                   a tile does not overlap the next tile's contraction.
-struct AccDouble {
-  static constexpr int kStages = 2;
-  __device__ static uint32_t col(int stage, int /*acc*/) { return stage * kAccCols; }
-};
-struct AccPair {
-  static constexpr int kStages = 1;
-  __device__ static uint32_t col(int /*stage*/, int acc) { return acc * kAccCols; }
-};
+// Accumulators in TMEM.
+//   AccDouble : one accumulator per tile, two stages of 256 columns: the epilogue of a tile overlaps the next tile's
+//               contraction.
+//   AccSplit  : two accumulators of 256 columns per tile (all of TMEM), each with barriers of its own.  The segments of
+//               accumulator 1 come first and are short; the epilogue takes accumulator 1 into registers while
+//               accumulator 0 is still being computed, so that the next tile's accumulator-1 segments run while the
+//               epilogue empties accumulator 0.
+struct AccDouble { static constexpr bool kSplit = false; };
+struct AccSplit { static constexpr bool kSplit = true; };
 
 template <class P>
 __device__ __forceinline__ void gemm_body(const typename P::Params& p) {
   extern __shared__ uint8_t smem_raw[];
-  using Acc = typename P::Acc;
+  constexpr int CG = P::CG;
+  constexpr int kEpiWarps = P::kEpiWarps;
+  constexpr bool kSplit = P::Acc::kSplit;
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t kStageBytes = kStageABytes + (uint32_t)stage_cols_of<P>::get(p) * 128u;   // a multiple of 1024
+  const uint32_t kStageBytes = kOperandBytes + (uint32_t)stage_rows_of<P>::get(p) * 128u;   // a multiple of 1024
   const int kStages = min(kMaxStages, (int)(kRingBytes / kStageBytes));
   const uint32_t bar_base = smem_base + kRingBytes;
-  // barrier block: full[8] empty[8] tfull[2] tempty[2] (8 B each), then tmem ptr, abort flag
+  // barrier block: full[12] empty[12] tfull[2] tempty[2] (8 B each), then tmem ptr, abort flag
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (kMaxStages + s); };
   auto tfull_bar = [&](int s) { return bar_base + 8u * (2 * kMaxStages + s); };
   auto tempty_bar = [&](int s) { return bar_base + 8u * (2 * kMaxStages + 2 + s); };
   uint8_t* bar_generic = smem_raw + (bar_base - smem_u32(smem_raw));
-  volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(bar_generic + 8 * (2 * kMaxStages + 5));
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_generic + 8 * (2 * kMaxStages + 5) + 8);
-  uint8_t* epi_stage = bar_generic + 256;  // kEpiWarps x kEpiWarpBytes
+  volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(bar_generic + 8 * (2 * kMaxStages + 4));
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_generic + 8 * (2 * kMaxStages + 4) + 8);
+  uint8_t* epi_stage = bar_generic + 256;
 
-  constexpr int kAccStages = Acc::kStages;
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
+  const int rank = CG == 2 ? (int)cluster_rank() : 0;   // which CTA of the pair
+  const int group = blockIdx.x / CG, ngroups = gridDim.x / CG;
 
   if (threadIdx.x == 0) {
+    // the operand barriers complete when every CTA's bytes have arrived at the issuing CTA; an accumulator is empty
+    // when the epilogue warps of every CTA have read it
     for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    for (int s = 0; s < 2; ++s) { mbar_init(tfull_bar(s), 1); mbar_init(tempty_bar(s), kEpiWarps); }
+    for (int s = 0; s < 2; ++s) { mbar_init(tfull_bar(s), 1); mbar_init(tempty_bar(s), CG * kEpiWarps); }
     *abort_flag = 0;
     mbar_fence_init();
   }
   if (warp == 1) {
-    tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_holder)), kTmemCols);
-    tmem_relinquish();
+    tmem_alloc<CG>(smem_u32(const_cast<uint32_t*>(tmem_holder)), kTmemCols);
+    tmem_relinquish<CG>();
   }
   // Launched with programmatic stream serialisation: the next kernel's CTAs may start (and do their own set-up)
   // while this one's last tiles run; nothing of global memory is touched before the previous kernel has finished.
   pdl_launch_dependents();
   tc_fence_before();
   __syncthreads();
+  if (CG == 2) cluster_sync_all();
   tc_fence_after();
   pdl_wait();
   const uint32_t tmem_base = *tmem_holder;
@@ -206,150 +228,167 @@ __device__ __forceinline__ void gemm_body(const typename P::Params& p) {
     if (lane == 0) {
       PipeState st;
       bool ok = true;
-      for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
+      for (int tile = group; ok && tile < ntiles; tile += ngroups) {
         typename P::Tile t;
-        P::tile_init(p, tile, t);
+        P::tile_init(p, tile, rank, t);
         const int nseg = P::num_segments(p, t);
         for (int s = 0; ok && s < nseg; ++s) {
           Segment sg;
-          sg.b2_y = -1;
           P::segment(p, t, s, sg);
           const int a_step = (sg.mode == MODE_I8_KK) ? 128 : 64;
-          // both operands of k-block kb into the stage at sa
-          auto fetch = [&](int kb, uint32_t sa, uint32_t bar) {
-            const uint32_t sb = sa + kStageABytes;
-            if (a_is_mn(sg.mode)) {
-              if (sg.a_blk) {
-                tma_fetch_blocked(sa, sg.ta, bar, sg.a_rank, sg.a_y + kb * 64, sg.a_x >> 6, sg.a_z);
-              } else {
-                tma_fetch(sa, sg.ta, bar, sg.a_rank, sg.a_x, sg.a_y + kb * 64, sg.a_z);
-                tma_fetch(sa + kMnBoxBytes, sg.ta, bar, sg.a_rank, sg.a_x + 64, sg.a_y + kb * 64, sg.a_z);
-              }
-            } else {
-              tma_fetch(sa, sg.ta, bar, sg.a_rank, sg.a_x + kb * a_step, sg.a_y, sg.a_z);
-            }
-            if (b_is_mn(sg.mode)) {
-              const int parts = sg.b2_y >= 0 ? 2 : 1;
-              for (int part = 0; part < parts; ++part) {
-                const int krow = (part ? sg.b2_y : sg.b_y) + kb * 64;
-                if (sg.b_blk) {
-                  tma_fetch_blocked(sb + part * sg.b_blk * kMnBoxBytes, sg.tb, bar, sg.b_rank, krow, sg.b_x >> 6, sg.b_z);
-                } else {
-                  const int nbox = sg.bn / (64 * parts);
-                  for (int b = 0; b < nbox; ++b)
-                    tma_fetch(sb + (part * nbox + b) * kMnBoxBytes, sg.tb, bar, sg.b_rank, sg.b_x + 64 * b, krow, sg.b_z);
-                }
-              }
-            } else {
-              for (int row = 0; row < sg.bn; row += sg.b_box)
-                tma_fetch(sb + row * 128, sg.tb, bar, sg.b_rank, sg.b_x + kb * a_step, sg.b_y + row, sg.b_z);
-            }
-          };
           for (int kb = 0; kb < sg.nkb; ++kb) {
             if (!pipe_wait(empty_bar(st.stage), st.phase ^ 1, WHERE_PRODUCER, abort_flag)) { ok = false; break; }
-            const uint32_t bar = full_bar(st.stage);
-            const uint32_t sa = smem_base + st.stage * kStageBytes;
-            if (b_is_mn(sg.mode)) {
-              mbar_expect_tx(bar, kStageABytes + (sg.b_blk ? (sg.b2_y >= 0 ? 2 : 1) * sg.b_blk * kMnBoxBytes : sg.bn * 128));
+            // the barrier of the issuing CTA counts the bytes of both
+            uint32_t bar = full_bar(st.stage);
+            if (rank == 0) mbar_expect_tx(bar, CG * (kOperandBytes + sg.b_bytes));
+            if (CG == 2) bar = cluster_map(bar, 0);
+            const uint32_t sa = smem_base + st.stage * kStageBytes, sb = sa + kOperandBytes;
+            if (a_is_mn(sg.mode)) {
+              if (sg.a_blk > 0) {
+                tma_fetch_blocked<CG>(sa, sg.ta, bar, sg.a_rank, sg.a_y + kb * 64, sg.a_x >> 6, sg.a_z);
+              } else {
+                tma_fetch<CG>(sa, sg.ta, bar, sg.a_rank, sg.a_x, sg.a_y + kb * 64, sg.a_z);
+                tma_fetch<CG>(sa + kMnBoxBytes, sg.ta, bar, sg.a_rank, sg.a_x + 64, sg.a_y + kb * 64, sg.a_z);
+              }
             } else {
-              const int nload = (sg.bn + sg.b_box - 1) / sg.b_box;
-              mbar_expect_tx(bar, kStageABytes + nload * sg.b_box * 128);
+              tma_fetch<CG>(sa, sg.ta, bar, sg.a_rank, sg.a_x + kb * a_step, sg.a_y, sg.a_z);
             }
-            fetch(kb, sa, bar);
+            if (b_is_mn(sg.mode)) {
+              if (sg.b_blk > 0) {
+                tma_fetch_blocked<CG>(sb, sg.tb, bar, sg.b_rank, sg.b_y + kb * 64, sg.b_x >> 6, sg.b_z);
+              } else {
+                for (int b = 0; b < -sg.b_blk; ++b)
+                  tma_fetch<CG>(sb + b * kMnBoxBytes, sg.tb, bar, sg.b_rank, sg.b_x + 64 * b, sg.b_y + kb * 64, sg.b_z);
+              }
+            } else {
+              tma_fetch<CG>(sb, sg.tb, bar, sg.b_rank, sg.b_x + kb * a_step, sg.b_y, sg.b_z);
+            }
             st.advance(kStages);
           }
         }
       }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer
+    // ------------------------------------------------------------ MMA issuer (first CTA of the pair)
     // The whole warp walks the loops, one elected thread issues.  What a tcgen05.mma costs to issue decides the rate: with
     // the descriptors put together per instruction in 64-bit arithmetic, the operand form tested inside the loop and a loop
     // over the k-steps the kernels ran at 190-230 cycles per MMA whatever the operands did (8192^3 int8: 2.7 POP/s with the
     // loads taken out); with the loop below, unrolled and specialised on the operand form, at the 128 cycles of the tensor
     // pipe (4.5 POP/s int8, 2.2 PFLOP/s bf16, loads taken out).
-    PipeState st, ac;
-    bool ok = true;
-    auto all_wait = [&](uint32_t bar, uint32_t parity) {
-      const bool got = __all_sync(0xffffffffu, pipe_wait(bar, parity, WHERE_MMA, abort_flag));
-      tc_fence_after();
-      return got;
-    };
-    for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
-      typename P::Tile t;
-      P::tile_init(p, tile, t);
-      const int nseg = P::num_segments(p, t);
-      if (!all_wait(tempty_bar(ac.stage), ac.phase ^ 1)) { ok = false; break; }
-      uint32_t opened = 0u;              // bit a: accumulator a has been written to
-      for (int s = 0; ok && s < nseg; ++s) {
-        Segment sg;
-        sg.b2_y = -1;
-        P::segment(p, t, s, sg);
-        const uint32_t d_tmem = tmem_base + Acc::col(ac.stage, sg.acc);
-        uint32_t started = (opened >> sg.acc) & 1u;
-        opened |= 1u << sg.acc;
-        // OP: operand form, STEPS: k-steps per k-block (0: as the segment says)
-        auto contract = [&](auto op, auto steps) {
-          constexpr int OP = decltype(op)::value, STEPS = decltype(steps)::value;
-          constexpr bool amn = OP == MODE_BF_MM, bmn = OP >= MODE_BF_KM;
-          constexpr uint32_t astep = amn ? 2048 >> 4 : 32 >> 4, bstep = bmn ? 2048 >> 4 : 32 >> 4;
-          const uint32_t idesc = OP == MODE_I8_KK ? umma_idesc(2, 1, 0, 0, sg.bn) : umma_idesc(1, 1, amn ? 1 : 0, bmn ? 1 : 0, sg.bn);
-          const uint64_t a0 = umma_smem_desc(smem_base, amn ? kMnBoxBytes : 16, 1024);
-          const uint64_t b0 = umma_smem_desc(smem_base + kStageABytes, bmn ? kMnBoxBytes : 16, 1024);
-          const uint32_t ahi = (uint32_t)(a0 >> 32), bhi = (uint32_t)(b0 >> 32);
-          for (int kb = 0; kb < sg.nkb; ++kb) {
-            if (!all_wait(full_bar(st.stage), st.phase)) { ok = false; break; }
-            const uint32_t off = (st.stage * kStageBytes) >> 4;   // addresses stay below 2^18: no carry out of the field
-            const uint32_t alo = (uint32_t)a0 + off, blo = (uint32_t)b0 + off;
-            auto step = [&](int k) {
-              const uint64_t ad = ((uint64_t)ahi << 32) | (alo + k * astep), bd = ((uint64_t)bhi << 32) | (blo + k * bstep);
-              if (OP == MODE_I8_KK) umma_i8(d_tmem, ad, bd, idesc, k ? 1u : started);
-              else umma_f16(d_tmem, ad, bd, idesc, k ? 1u : started);
-            };
-            if (elect_one()) {
-              if (STEPS > 0) {
-#pragma unroll
-                for (int k = 0; k < STEPS; ++k) step(k);
-              } else {
-                for (int k = 0; k < sg.ksteps; ++k) step(k);
-              }
-              umma_commit(empty_bar(st.stage));  // frees the smem stage once these MMAs retire
+    if (rank == 0) {
+      PipeState st, ac;
+      bool ok = true;
+      auto all_wait = [&](uint32_t bar, uint32_t parity) {
+        const bool got = __all_sync(0xffffffffu, pipe_wait(bar, parity, WHERE_MMA, abort_flag));
+        tc_fence_after();
+        return got;
+      };
+      auto commit = [&](uint32_t bar) { if (elect_one()) umma_commit<CG>(bar); };
+      for (int tile = group; ok && tile < ntiles; tile += ngroups) {
+        typename P::Tile t;
+        P::tile_init(p, tile, rank, t);
+        const int nseg = P::num_segments(p, t);
+        if (!kSplit && !all_wait(tempty_bar(ac.stage), ac.phase ^ 1)) { ok = false; break; }
+        int open = -1;                   // accumulator whose segments are being issued
+        for (int s = 0; ok && s < nseg; ++s) {
+          Segment sg;
+          P::segment(p, t, s, sg);
+          uint32_t started = open == sg.acc;
+          if (!started) {
+            if (kSplit) {
+              if (open >= 0) commit(tfull_bar(open));
+              if (!all_wait(tempty_bar(sg.acc), ac.phase ^ 1)) { ok = false; break; }
             }
-            started = 1u;
-            st.advance(kStages);
+            open = sg.acc;
           }
-        };
-        if (sg.ksteps != 4) contract(std::integral_constant<int, MODE_BF_KM>{}, std::integral_constant<int, 0>{});   // the router's one step
-        else if (sg.mode == MODE_I8_KK) contract(std::integral_constant<int, MODE_I8_KK>{}, std::integral_constant<int, 4>{});
-        else if (sg.mode == MODE_BF_KK) contract(std::integral_constant<int, MODE_BF_KK>{}, std::integral_constant<int, 4>{});
-        else if (sg.mode == MODE_BF_KM) contract(std::integral_constant<int, MODE_BF_KM>{}, std::integral_constant<int, 4>{});
-        else contract(std::integral_constant<int, MODE_BF_MM>{}, std::integral_constant<int, 4>{});
+          const uint32_t d_tmem = tmem_base + (kSplit ? sg.acc : ac.stage) * kAccCols;
+          // OP: operand form, STEPS: k-steps per k-block (0: as the segment says)
+          auto contract = [&](auto op, auto steps) {
+            constexpr int OP = decltype(op)::value, STEPS = decltype(steps)::value;
+            constexpr bool amn = OP == MODE_BF_MM, bmn = OP >= MODE_BF_KM;
+            constexpr uint32_t astep = amn ? 2048 >> 4 : 32 >> 4, bstep = bmn ? 2048 >> 4 : 32 >> 4;
+            const uint32_t idesc = OP == MODE_I8_KK ? umma_idesc(2, 1, 0, 0, sg.bn, CG * 128)
+                                                    : umma_idesc(1, 1, amn ? 1 : 0, bmn ? 1 : 0, sg.bn, CG * 128);
+            const uint64_t a0 = umma_smem_desc(smem_base, amn ? kMnBoxBytes : 16, 1024);
+            const uint64_t b0 = umma_smem_desc(smem_base + kOperandBytes, bmn ? kMnBoxBytes : 16, 1024);
+            const uint32_t ahi = (uint32_t)(a0 >> 32), bhi = (uint32_t)(b0 >> 32);
+            for (int kb = 0; kb < sg.nkb; ++kb) {
+              if (!all_wait(full_bar(st.stage), st.phase)) { ok = false; break; }
+              const uint32_t off = (st.stage * kStageBytes) >> 4;   // addresses stay below 2^18: no carry out of the field
+              const uint32_t alo = (uint32_t)a0 + off, blo = (uint32_t)b0 + off;
+              auto step = [&](int k) {
+                const uint64_t ad = ((uint64_t)ahi << 32) | (alo + k * astep), bd = ((uint64_t)bhi << 32) | (blo + k * bstep);
+                if (OP == MODE_I8_KK) umma_i8<CG>(d_tmem, ad, bd, idesc, k ? 1u : started);
+                else umma_f16<CG>(d_tmem, ad, bd, idesc, k ? 1u : started);
+              };
+              if (elect_one()) {
+                if (STEPS > 0) {
+#pragma unroll
+                  for (int k = 0; k < STEPS; ++k) step(k);
+                } else {
+                  for (int k = 0; k < sg.ksteps; ++k) step(k);
+                }
+                umma_commit<CG>(empty_bar(st.stage));  // frees the smem stage (of both CTAs) once these MMAs retire
+              }
+              started = 1u;
+              st.advance(kStages);
+            }
+          };
+          if (sg.ksteps != 4) contract(std::integral_constant<int, MODE_BF_KM>{}, std::integral_constant<int, 0>{});   // the router's one step
+          else if (sg.mode == MODE_I8_KK) contract(std::integral_constant<int, MODE_I8_KK>{}, std::integral_constant<int, 4>{});
+          else if (sg.mode == MODE_BF_KK) contract(std::integral_constant<int, MODE_BF_KK>{}, std::integral_constant<int, 4>{});
+          else if (sg.mode == MODE_BF_KM) contract(std::integral_constant<int, MODE_BF_KM>{}, std::integral_constant<int, 4>{});
+          else contract(std::integral_constant<int, MODE_BF_MM>{}, std::integral_constant<int, 4>{});
+        }
+        if (ok) commit(tfull_bar(kSplit ? 0 : ac.stage));
+        if (kSplit) ac.phase ^= 1;
+        else ac.advance(2);
       }
-      if (ok && elect_one()) umma_commit(tfull_bar(ac.stage));
-      ac.advance(kAccStages);
     }
   } else {
     // ------------------------------------------------------------ epilogue warps
     PipeState ac;
     const int quad = warp & 3;          // TMEM lanes [32*quad, 32*quad+32) are this warp's
-    const int half = (warp - 2) >> 2;   // which of the two warps of the quadrant: it takes column chunks half, half+2, ...
-    bool ok = true;
-    for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
-      typename P::Tile t;
-      P::tile_init(p, tile, t);
-      // per-row factors and addresses are fetched while the contraction is still running
-      const typename P::Pre pre = P::prepare(p, t, quad, lane);
-      // Every lane watches the barrier itself, but the warp takes ONE decision: what follows is full of
-      // warp-collective instructions (tcgen05.ld, shuffles), so a lane that gave up must take the others along.
-      ok = __all_sync(0xffffffffu, pipe_wait(tfull_bar(ac.stage), ac.phase, WHERE_EPILOGUE, abort_flag));
-      if (!ok) break;
-      tc_fence_after();
-      const uint32_t tlane = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
-      P::epilogue(p, t, pre, tlane + Acc::col(ac.stage, 0), tlane + Acc::col(ac.stage, 1), quad, half, lane, epi_stage + (warp - 2) * kEpiWarpBytes);
+    const int part = (warp - 2) >> 2;   // which of the quadrant's warps: it takes column chunks part, part + kEpiWarps / 4, ...
+    uint8_t* stage = epi_stage + (warp - 2) * (kStagingBytes / kEpiWarps);
+    const uint32_t tlane = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
+    const uint32_t tempty0 = CG == 2 ? cluster_map(tempty_bar(0), 0) : tempty_bar(0);   // at the issuing CTA
+    auto release = [&](int a) {
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(tempty_bar(ac.stage));
-      ac.advance(kAccStages);
+      if (lane == 0) {
+        if (CG == 2) mbar_arrive_cluster(tempty0 + 8u * a);
+        else mbar_arrive(tempty0 + 8u * a);
+      }
+    };
+    // Every lane watches the barrier itself, but the warp takes ONE decision: what follows is full of
+    // warp-collective instructions (tcgen05.ld, shuffles), so a lane that gave up must take the others along.
+    auto await = [&](int a, uint32_t phase) {
+      const bool got = __all_sync(0xffffffffu, pipe_wait(tfull_bar(a), phase, WHERE_EPILOGUE, abort_flag));
+      tc_fence_after();
+      return got;
+    };
+    for (int tile = group; tile < ntiles; tile += ngroups) {
+      typename P::Tile t;
+      P::tile_init(p, tile, rank, t);
+      // per-row factors and addresses are fetched while the contraction is still running
+      const typename P::Pre pre = P::prepare(p, t, quad, lane);
+      if constexpr (kSplit) {
+        typename P::Regs regs;
+        if (!await(1, ac.phase)) break;
+        P::take_first(p, t, pre, tlane + kAccCols, part, regs);
+        release(1);
+        if (!await(0, ac.phase)) break;
+        P::combine(p, t, pre, tlane, part, regs);
+        release(0);
+        P::store(p, t, pre, part, lane, stage, regs);
+        ac.phase ^= 1;
+      } else {
+        if (!await(ac.stage, ac.phase)) break;
+        P::epilogue(p, t, pre, tlane + ac.stage * kAccCols, quad, part, lane, stage);
+        release(ac.stage);
+        ac.advance(2);
+      }
     }
   }
 
@@ -360,17 +399,21 @@ __device__ __forceinline__ void gemm_body(const typename P::Params& p) {
     for (int i = 0; i < 200; ++i) __nanosleep(1000);
   }
   __syncthreads();
+  if (CG == 2) cluster_sync_all();   // neither CTA leaves while the other may still signal its barriers or read its operands
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem_base, kTmemCols);
+    tmem_dealloc<CG>(tmem_base, kTmemCols);
   }
 }
 
 // One named kernel per problem, so that profiler listings show which product ran.
-#define PQ_DEFINE_GEMM_KERNEL(name, Problem)                                                      \
-  __global__ void __launch_bounds__(kGemmThreads, 1) name(const __grid_constant__ typename Problem::Params p) { \
-    gemm_body<Problem>(p);                                                                        \
+template <class P>
+constexpr int gemm_threads = 64 + 32 * P::kEpiWarps;
+#define PQ_DEFINE_GEMM_KERNEL(name, Problem)                                                                           \
+  __global__ void __cluster_dims__(Problem::CG, 1, 1) __launch_bounds__(gemm_threads<Problem>, 1)                       \
+      name(const __grid_constant__ typename Problem::Params p) {                                                       \
+    gemm_body<Problem>(p);                                                                                             \
   }
 
 }  // namespace pq

@@ -3,6 +3,7 @@
 //              Y = alpha g (H B_e^T) + beta (lam/gamma) (q S^T)      (Eq. 10, 11)
 //   backward : dH, dX, dW, dB, dA of the straight-through estimator  (App. B.1)
 //   debug    : raw accumulators of one contraction, for bit-exact tests
+#include <algorithm>
 #include <type_traits>
 
 #include "pq_gemm.cuh"
@@ -81,7 +82,7 @@ static bool map3d_i8(CUtensorMap* m, const void* base, uint64_t inner, uint64_t 
 // MN-major operand: matrix [batch][k_total][mn_total] with mn contiguous, read in 64 (mn) x 64 (k) boxes.
 // When mn_total is a multiple of 64 the map views the 64-wide column blocks as a dimension of their own,
 // (64, k_total, mn_total / 64[, batch]) -- base_rank 2 or 3 says whether the operand has the batch dimension --, so that ONE load delivers `nblk` boxes back to back; *blk = nblk.
-// Otherwise (a narrower last block would alias the next row) a plain map with one box per load; *blk = 0.
+// Otherwise (a narrower last block would alias the next row) a plain map with one box per load; *blk = -nblk.
 static bool map_mn(CUtensorMap* m, int* blk, const void* base, uint64_t mn_total, uint64_t k_total, int base_rank, uint64_t batch, int nblk) {
   if (mn_total % 64 == 0) {
     *blk = nblk;
@@ -90,7 +91,7 @@ static bool map_mn(CUtensorMap* m, int* blk, const void* base, uint64_t mn_total
     const uint32_t box[4] = {64, 64, (uint32_t)nblk, 1};
     return make_map(m, false, base, base_rank + 1, dims, strides, box);
   }
-  *blk = 0;
+  *blk = -nblk;
   return base_rank == 3 ? map3d(m, base, mn_total, k_total, batch, 64, 64) : map2d(m, false, base, mn_total, k_total, 64, 64);
 }
 
@@ -105,22 +106,18 @@ static int sm_count() {
   return g_sm_count;
 }
 
-static int grid_for_tiles(int max_tiles) {
-  int grid = max_tiles < sm_count() ? max_tiles : sm_count();
-  return grid < 1 ? 1 : grid;
-}
-
-template <class Params>
-static int launch_gemm(int kernel_id, void (*kernel)(Params), const Params& p, int max_tiles, cudaStream_t st) {
+// max_tiles: tiles of the launch, at most; one CTA (or CTA pair) each, as many as the SMs hold
+template <class P>
+static int launch_gemm(int kernel_id, void (*kernel)(typename P::Params), const typename P::Params& p, int max_tiles, cudaStream_t st) {
   // (cudaFuncSetAttribute is cheap and idempotent; calling it per launch keeps this free of static state per kernel)
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemBytes) != cudaSuccess) return PQ_ERR_CUDA;
-  const int grid = grid_for_tiles(max_tiles);
+  const int grid = P::CG * std::max(1, std::min(max_tiles, sm_count() / P::CG));
   LaunchScope ls(kernel_id, st);
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid, 1, 1); cfg.blockDim = dim3(kGemmThreads, 1, 1); cfg.dynamicSmemBytes = kGemmSmemBytes;
+  cfg.gridDim = dim3(grid, 1, 1); cfg.blockDim = dim3(gemm_threads<P>, 1, 1); cfg.dynamicSmemBytes = kGemmSmemBytes;
   cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, p) == cudaSuccess ? PQ_OK : PQ_ERR_CUDA;
 }
@@ -146,33 +143,36 @@ static inline int h_round_up(int x, int m) { return (x + m - 1) / m * m; }
 // ---------------------------------------------------------------------------
 // debug: D[M,N] = contraction of A and B in one of the four operand forms
 // ---------------------------------------------------------------------------
+template <int CG_>
 struct DebugProblem {
+  static constexpr int CG = CG_, kEpiWarps = 8;
   using Acc = AccDouble;
   struct Params {
     CUtensorMap ta, tb;
     TileGrid g;
-    int mode, M, N, K, a_blk, b_blk;
+    int mode, M, N, K, a_blk, b_blk, b_bytes;
     void* D;
   };
-  struct Tile { TileCoord c; };
+  struct Tile { TileCoord c; int rank; };
   __device__ static int num_tiles(const Params& p) { return p.g.total; }
-  __device__ static void tile_init(const Params& p, int i, Tile& t) { t.c = tile_coord(p.g, i); }
+  __device__ static void tile_init(const Params& p, int i, int rank, Tile& t) { t.c = tile_coord<CG>(p.g, i, rank); t.rank = rank; }
   __device__ static int num_segments(const Params&, const Tile&) { return 1; }
   __device__ static void segment(const Params& p, const Tile& t, int, Segment& s) {
-    s.mode = p.mode; s.acc = 0; s.ksteps = 4; s.b_box = p.g.bn; s.a_blk = p.a_blk; s.b_blk = p.b_blk;
-    s.bn = clip_bn(t.c.bn, t.c.n0, p.N, p.mode >= MODE_BF_KM ? 64 : 32);
+    s.mode = p.mode; s.acc = 0; s.ksteps = 4; s.a_blk = p.a_blk; s.b_blk = p.b_blk; s.b_bytes = p.b_bytes;
+    s.bn = clip_bn(t.c.bn, t.c.n0, p.N, p.mode >= MODE_BF_KM ? 64 * CG : 32);
     const int bk = p.mode == MODE_I8_KK ? 128 : 64;
     s.nkb = (p.K + bk - 1) / bk;
     s.ta = &p.ta; s.tb = &p.tb; s.a_rank = 2; s.b_rank = 2; s.a_z = 0; s.b_z = 0;
+    const int n0 = t.c.n0 + t.rank * (s.bn / CG);
     if (p.mode == MODE_BF_MM) { s.a_x = t.c.m * 128; s.a_y = 0; } else { s.a_x = 0; s.a_y = t.c.m * 128; }
-    if (p.mode >= MODE_BF_KM) { s.b_x = t.c.n0; s.b_y = 0; } else { s.b_x = 0; s.b_y = t.c.n0; }
+    if (p.mode >= MODE_BF_KM) { s.b_x = n0; s.b_y = 0; } else { s.b_x = 0; s.b_y = n0; }
   }
   using Pre = NoPre;
   __device__ static Pre prepare(const Params&, const Tile&, int, int) { return Pre{}; }
-  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t tacc, uint32_t, int quad, int half, int lane, uint8_t* stage) {
+  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t tacc, int quad, int part, int lane, uint8_t* stage) {
     const int row = t.c.m * 128 + quad * 32 + lane;
     uint32_t* D = reinterpret_cast<uint32_t*>(p.D);
-    for (int c = half; c * 32 < t.c.bn; c += 2) {
+    for (int c = part; c * 32 < t.c.bn; c += kEpiWarps / 4) {
       const int n0 = t.c.n0 + c * 32;
       if (n0 >= p.N) break;
       uint32_t v[32];
@@ -182,45 +182,55 @@ struct DebugProblem {
 #pragma unroll
       for (int j = 0; j < 8; ++j) o[j] = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
       const int valid = min(32, p.N - n0) * 4;   // N is a multiple of 8 -> whole 16-byte pieces
-      warp_store_rows(stage, o, row < p.M ? D + (long long)row * p.N + n0 : nullptr, valid, lane);
+      warp_store_rows<8>(stage, o, row < p.M ? D + (long long)row * p.N + n0 : nullptr, valid, lane);
     }
   }
 };
-PQ_DEFINE_GEMM_KERNEL(k_gemm_debug, DebugProblem)
+PQ_DEFINE_GEMM_KERNEL(k_gemm_debug, DebugProblem<2>)
+PQ_DEFINE_GEMM_KERNEL(k_gemm_debug_single, DebugProblem<1>)
 
-int gemm_debug(int mode, int M, int N, int K, const void* A, const void* B, void* D, int tile_n, cudaStream_t st) {
-  DebugProblem::Params p;
+template <class P>
+static int run_debug(void (*kernel)(typename P::Params), int mode, int M, int N, int K, const void* A, const void* B, void* D, int tile_n, cudaStream_t st) {
+  typename P::Params p;
   p.mode = mode; p.M = M; p.N = N; p.K = K; p.D = D; p.a_blk = 0; p.b_blk = 0;
-  const int granule = mode >= MODE_BF_KM ? 64 : 32;
-  if (tile_n <= 0) tile_n = 256;
-  if (tile_n > 256 || tile_n % granule) return PQ_ERR_SHAPE;
-  const int mt = (M + 127) / 128, nt = (N + tile_n - 1) / tile_n;
-  p.g = make_tile_grid(mt, nt, tile_n);
+  const int share = tile_n / P::CG;                  // columns of a tile that one CTA loads
+  p.b_bytes = share * 128;
+  p.g = make_tile_grid((M + 128 * P::CG - 1) / (128 * P::CG), (N + tile_n - 1) / tile_n, tile_n);
   bool ok = true;
   switch (mode) {
     case MODE_I8_KK:
-      ok = map2d(&p.ta, true, A, K, M, 128, 128) && map2d(&p.tb, true, B, K, N, 128, tile_n);
+      ok = map2d(&p.ta, true, A, K, M, 128, 128) && map2d(&p.tb, true, B, K, N, 128, share);
       break;
     case MODE_BF_KK:
-      ok = map2d(&p.ta, false, A, K, M, 64, 128) && map2d(&p.tb, false, B, K, N, 64, tile_n);
+      ok = map2d(&p.ta, false, A, K, M, 64, 128) && map2d(&p.tb, false, B, K, N, 64, share);
       break;
     case MODE_BF_KM:
-      ok = map2d(&p.ta, false, A, K, M, 64, 128) && map_mn(&p.tb, &p.b_blk, B, N, K, 2, 1, tile_n / 64);
+      ok = map2d(&p.ta, false, A, K, M, 64, 128) && map_mn(&p.tb, &p.b_blk, B, N, K, 2, 1, share / 64);
       break;
     case MODE_BF_MM:
-      ok = map_mn(&p.ta, &p.a_blk, A, M, K, 2, 1, 2) && map_mn(&p.tb, &p.b_blk, B, N, K, 2, 1, tile_n / 64);
+      ok = map_mn(&p.ta, &p.a_blk, A, M, K, 2, 1, 2) && map_mn(&p.tb, &p.b_blk, B, N, K, 2, 1, share / 64);
       break;
     default:
       return PQ_ERR_UNSUPPORTED;
   }
   if (!ok) return PQ_ERR_CUDA;
-  return launch_gemm(KID_DEBUG, k_gemm_debug, p, p.g.total, st);
+  return launch_gemm<P>(KID_DEBUG, kernel, p, p.g.total, st);
+}
+
+int gemm_debug(int mode, int M, int N, int K, const void* A, const void* B, void* D, int tile_n, cudaStream_t st) {
+  const int granule = mode >= MODE_BF_KM ? 64 : 32;
+  if (tile_n <= 0) tile_n = 256;
+  if (tile_n > 256 || tile_n % granule) return PQ_ERR_SHAPE;
+  // a pair's CTA loads whole 64-column boxes of an MN-major operand; widths that do not split that way run on one CTA
+  if (granule == 64 && tile_n % 128) return run_debug<DebugProblem<1>>(k_gemm_debug_single, mode, M, N, K, A, B, D, tile_n, st);
+  return run_debug<DebugProblem<2>>(k_gemm_debug, mode, M, N, K, A, B, D, tile_n, st);
 }
 
 // ---------------------------------------------------------------------------
 // F1: hidden activations of the HP branch, H = X_sorted A_e^T, one tile per item
 // ---------------------------------------------------------------------------
 struct HpUpProblem {
+  static constexpr int CG = 1, kEpiWarps = 8;
   using Acc = AccDouble;
   struct Params {
     CUtensorMap tx, ta;  // X sorted [T,K]; A [E,r,K]
@@ -229,19 +239,19 @@ struct HpUpProblem {
     int K, r, bn, item_rows;
   };
   struct Tile { int item; int4 it; };
-  __device__ static int stage_cols(const Params& p) { return p.bn <= 128 ? 128 : 256; }
+  __device__ static int stage_rows(const Params& p) { return p.bn <= 128 ? 128 : 256; }
   __device__ static int num_tiles(const Params& p) { return p.rt.n_items[0]; }
-  __device__ static void tile_init(const Params& p, int i, Tile& t) { t.item = i; t.it = p.rt.items[i]; }
+  __device__ static void tile_init(const Params& p, int i, int, Tile& t) { t.item = i; t.it = p.rt.items[i]; }
   __device__ static int num_segments(const Params&, const Tile&) { return 1; }
   __device__ static void segment(const Params& p, const Tile& t, int, Segment& s) {
     s.mode = MODE_BF_KK; s.acc = 0; s.bn = p.bn; s.ksteps = 4; s.nkb = (p.K + 63) / 64;
     s.ta = &p.tx; s.a_rank = 2; s.a_x = 0; s.a_y = t.it.x * 128; s.a_z = 0;
     s.tb = &p.ta; s.b_rank = 3; s.b_x = 0; s.b_y = 0; s.b_z = t.it.y;
-    s.b_box = p.bn; s.a_blk = 0; s.b_blk = 0;
+    s.b_bytes = p.bn * 128; s.a_blk = 0; s.b_blk = 0;
   }
   using Pre = NoPre;
   __device__ static Pre prepare(const Params&, const Tile&, int, int) { return Pre{}; }
-  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t taddr, uint32_t, int quad, int half, int lane, uint8_t* stage) {
+  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t taddr, int quad, int half, int lane, uint8_t* stage) {
     const int row = quad * 32 + lane;
     const bool live = row >= t.it.z && row < t.it.w;
     uint4* out_hi = reinterpret_cast<uint4*>(p.H + ((long long)t.item * 128 + row) * p.r);
@@ -274,6 +284,7 @@ PQ_DEFINE_GEMM_KERNEL(k_gemm_hp_up, HpUpProblem)
 // writes the codes qh [items*128, rp] (row pitch rp = r rounded up to 16, padding zero) and gamma_h [items*128].
 // ---------------------------------------------------------------------------
 struct HpUp8Problem {
+  static constexpr int CG = 1, kEpiWarps = 8;
   using Acc = AccDouble;
   struct Params {
     CUtensorMap tq, ta;  // q sorted [T,K] s8; A8 [E,r,K] s8
@@ -284,19 +295,19 @@ struct HpUp8Problem {
     int K, r, rp, bn;
   };
   struct Tile { int item; int4 it; };
-  __device__ static int stage_cols(const Params& p) { return p.bn <= 128 ? 128 : 256; }
+  __device__ static int stage_rows(const Params& p) { return p.bn <= 128 ? 128 : 256; }
   __device__ static int num_tiles(const Params& p) { return p.rt.n_items[0]; }
-  __device__ static void tile_init(const Params& p, int i, Tile& t) { t.item = i; t.it = p.rt.items[i]; }
+  __device__ static void tile_init(const Params& p, int i, int, Tile& t) { t.item = i; t.it = p.rt.items[i]; }
   __device__ static int num_segments(const Params&, const Tile&) { return 1; }
   __device__ static void segment(const Params& p, const Tile& t, int, Segment& s) {
     s.mode = MODE_I8_KK; s.acc = 0; s.bn = p.bn; s.ksteps = 4; s.nkb = (p.K + 127) / 128;
     s.ta = &p.tq; s.a_rank = 2; s.a_x = 0; s.a_y = t.it.x * 128; s.a_z = 0;
     s.tb = &p.ta; s.b_rank = 3; s.b_x = 0; s.b_y = 0; s.b_z = t.it.y;
-    s.b_box = p.bn; s.a_blk = 0; s.b_blk = 0;
+    s.b_bytes = p.bn * 128; s.a_blk = 0; s.b_blk = 0;
   }
   using Pre = NoPre;
   __device__ static Pre prepare(const Params&, const Tile&, int, int) { return Pre{}; }
-  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t taddr, uint32_t, int quad, int half, int lane, uint8_t* stage) {
+  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t taddr, int quad, int half, int lane, uint8_t* stage) {
     if (p.raw) {
       int* out = p.raw + ((long long)t.item * 128 + quad * 32 + lane) * p.r;
       for (int c = half; c * 32 < p.r; c += 2) {
@@ -356,8 +367,12 @@ PQ_DEFINE_GEMM_KERNEL(k_gemm_hp_up8, HpUp8Problem)
 // ---------------------------------------------------------------------------
 template <bool HP>
 struct FwdProblem {
-  // with the HP branch a tile holds an int32 and an fp32 accumulator of 256 columns each: all of TMEM
-  using Acc = typename std::conditional<HP, AccPair, AccDouble>::type;
+  // With the HP branch a tile holds an int32 and an fp32 accumulator of 256 columns each, all of TMEM.  Sixteen epilogue
+  // warps, 64 columns of a row per thread: the fp32 accumulator waits in 64 registers while the int8 contraction runs, and
+  // what the next tile's int8 contraction has to wait for is only the read of the int32 accumulator, which the next tile's
+  // HP segments cover.
+  static constexpr int CG = 2, kEpiWarps = HP ? 16 : 8;
+  using Acc = typename std::conditional<HP, AccSplit, AccDouble>::type;
   struct Params {
     CUtensorMap tq, ts, th, tb;  // q [T,K] s8; S [N,K] s8; H [items*128,r]; B [E,N,r]
     RoutingTables rt;
@@ -376,38 +391,41 @@ struct FwdProblem {
     int hp_ext;              // the codes of h and gamma_h were written by the caller
     int T, N, K, r, sstride, item_rows;
   };
-  struct Tile { TileCoord c; int bn, ib, ie; };
+  struct Tile { TileCoord c; int bn, pb, pe, rank; };
   __device__ static int num_tiles(const Params& p) { return p.g.total; }
-  __device__ static void tile_init(const Params& p, int i, Tile& t) {
-    t.c = tile_coord(p.g, i);
+  __device__ static void tile_init(const Params& p, int i, int rank, Tile& t) {
+    t.c = tile_coord<CG>(p.g, i, rank);
+    t.rank = rank;
     t.bn = clip_bn(t.c.bn, t.c.n0, p.N, 32);
-    if (HP) { t.ib = p.rt.tile_item_begin[t.c.m]; t.ie = p.rt.tile_item_begin[t.c.m + 1]; } else { t.ib = t.ie = 0; }
+    if (HP) { t.pb = p.rt.pair_begin[t.c.m >> 1]; t.pe = p.rt.pair_begin[(t.c.m >> 1) + 1]; } else { t.pb = t.pe = 0; }
   }
   // The HP product uses the leading bf16 plane of H only: its 2^-9 relative rounding is of the size of the
   // output's own rounding to bf16; the second plane serves the backward pass, whose sums are longer.
-  __device__ static int num_segments(const Params&, const Tile& t) { return 1 + (t.ie - t.ib); }
+  __device__ static int num_segments(const Params&, const Tile& t) { return (t.pe - t.pb) + 1; }
   __device__ static void segment(const Params& p, const Tile& t, int i, Segment& s) {
-    s.bn = t.bn; s.ksteps = 4; s.a_z = 0; s.b_z = 0; s.b_box = 256; s.a_blk = 0; s.b_blk = 0;
-    if (i == 0) {
+    s.bn = t.bn; s.ksteps = 4; s.a_z = 0; s.b_z = 0; s.a_blk = 0; s.b_blk = 0; s.b_bytes = kOperandBytes;
+    s.b_x = 0; s.b_y = t.c.n0 + t.rank * (t.bn >> 1);
+    if (i == t.pe - t.pb) {
       s.mode = MODE_I8_KK; s.acc = 0; s.nkb = (p.K + 127) / 128;
       s.ta = &p.tq; s.a_rank = 2; s.a_x = 0; s.a_y = t.c.m * 128;
-      s.tb = &p.ts; s.b_rank = 2; s.b_x = 0; s.b_y = t.c.n0;
+      s.tb = &p.ts; s.b_rank = 2;
     } else {
-      const int item = t.ib + (i - 1);
-      const int e = p.rt.items[item].y;
-      if (p.gamma_h) { s.mode = MODE_I8_KK; s.acc = 1; s.nkb = (p.r + 127) / 128; }
-      else { s.mode = MODE_BF_KK; s.acc = 1; s.nkb = (p.r + 63) / 64; }
-      s.ta = &p.th; s.a_rank = p.gamma_h ? 3 : 2; s.a_x = 0; s.a_y = item * 128;
-      s.tb = &p.tb; s.b_rank = 3; s.b_x = 0; s.b_y = t.c.n0; s.b_z = e;
+      const int4 pi = p.rt.pair_items[t.pb + i];
+      const int item = t.rank ? pi.z : pi.y;
+      if (p.gamma_h) { s.mode = MODE_I8_KK; s.nkb = (p.r + 127) / 128; }
+      else { s.mode = MODE_BF_KK; s.nkb = (p.r + 63) / 64; }
+      s.acc = 1;
+      s.ta = &p.th; s.a_rank = p.gamma_h ? 3 : 2; s.a_x = 0;
+      s.a_y = item >= 0 ? item * 128 : 2 * p.item_rows;    // no rows of this expert here: beyond both planes of H, read as zeros
+      s.tb = &p.tb; s.b_rank = 3; s.b_z = pi.x;
     }
   }
-  // y = cb_n * acc + ca_n * z for 32 consecutive columns starting at n, packed to 16 bf16 pairs
+  // y = cb_n * acc + ca_n * z for 16 consecutive columns starting at n, packed to 8 bf16 pairs
   template <bool VEC>
-  __device__ static __forceinline__ void combine32(const Params& p, int n, float cb, float ca, const uint32_t (&a)[32], const uint32_t (&z)[32],
-                                                  uint4* out, bool z_is_int) {
-    uint32_t w[16];
+  __device__ static __forceinline__ void combine16(const Params& p, int n, float cb, float ca, const uint32_t (&a)[16], const uint32_t* z,
+                                                  uint32_t* w, bool z_is_int) {
 #pragma unroll
-    for (int q4 = 0; q4 < 8; ++q4) {
+    for (int q4 = 0; q4 < 4; ++q4) {
       float b4[4] = {cb, cb, cb, cb}, a4[4] = {ca, ca, ca, ca};
       if (VEC) {
         const float4 bv = __ldg(reinterpret_cast<const float4*>(p.beta + n) + q4);
@@ -426,8 +444,6 @@ struct FwdProblem {
       w[2 * q4] = pack_bf16x2(y[0], y[1]);
       w[2 * q4 + 1] = pack_bf16x2(y[2], y[3]);
     }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) out[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
   }
   // per-row factors: 1-bit branch lam / gamma_t (Eq. 10), HP branch g_t; scalar feature scales folded in
   struct Pre { uint16_t* yrow; float cb, ca; };
@@ -443,7 +459,7 @@ struct FwdProblem {
         // the item of this row: its expert's weight scales and the row's own hidden scale
         const int rel = quad * 32 + lane;
         float deq = 0.f;
-        for (int it = t.ib; it < t.ie; ++it) {
+        for (int it = p.rt.tile_item_begin[t.c.m]; it < p.rt.tile_item_begin[t.c.m + 1]; ++it) {
           const int4 d = p.rt.items[it];
           if (rel >= d.z && rel < d.w) {
             const float gh = p.gamma_h[(long long)it * 128 + rel];
@@ -458,25 +474,65 @@ struct FwdProblem {
     }
     return r;
   }
-  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t tacc, uint32_t tz, int quad, int half, int lane, uint8_t* stage) {
+  // pure 1-bit tile
+  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t tacc, int quad, int part, int lane, uint8_t* stage) {
     const bool vec = p.sstride != 0;
-    for (int c = half; c * 64 < t.bn; c += 2) {     // 64 output columns = 128 bytes of the row per pass
+    for (int c = part; c * 64 < t.bn; c += kEpiWarps / 4) {     // 64 output columns = 128 bytes of the row per pass
       const int n0 = t.c.n0 + c * 64;
       if (n0 >= p.N) break;
-      uint4 o[8];
+      uint32_t w[32];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int nb = n0 + h * 32;
-        if (c * 64 + h * 32 < t.bn && nb < p.N) {
-          uint32_t a[32], z[32];
-          tmem_ld32(tacc + c * 64 + h * 32, a);
-          if (HP) tmem_ld32(tz + c * 64 + h * 32, z);
+      for (int h = 0; h < 4; ++h) {
+        const int nb = n0 + h * 16;
+        if (c * 64 + h * 16 < t.bn && nb < p.N) {
+          uint32_t a[16];
+          tmem_ld16(tacc + c * 64 + h * 16, a);
           tmem_ld_wait();
-          if (vec) combine32<true>(p, nb, pre.cb, pre.ca, a, z, o + 4 * h, p.gamma_h != nullptr);
-          else combine32<false>(p, nb, pre.cb, pre.ca, a, z, o + 4 * h, p.gamma_h != nullptr);
+          if (vec) combine16<true>(p, nb, pre.cb, 0.f, a, a, w + 8 * h, false);
+          else combine16<false>(p, nb, pre.cb, 0.f, a, a, w + 8 * h, false);
         }
       }
-      warp_store_rows(stage, o, pre.yrow ? pre.yrow + n0 : nullptr, min(64, min(t.bn - c * 64, p.N - n0)) * 2, lane);
+      uint4 o[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) o[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+      warp_store_rows<8>(stage, o, pre.yrow ? pre.yrow + n0 : nullptr, min(64, min(t.bn - c * 64, p.N - n0)) * 2, lane);
+    }
+  }
+  // tile with an HP branch: thread = row, columns [64 part, 64 part + 64)
+  struct Regs { uint32_t z[64]; };
+  __device__ static __forceinline__ void take_first(const Params&, const Tile& t, const Pre&, uint32_t tz, int part, Regs& r) {
+    if (part * 64 < t.bn) {
+      tmem_ld32(tz + part * 64, *reinterpret_cast<uint32_t(*)[32]>(r.z));
+      tmem_ld32(tz + part * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(r.z + 32));
+      tmem_ld_wait();
+    }
+  }
+  // the results take the place of the z values they are made from: pair j of the row's 64 columns ends up in z[j]
+  __device__ static __forceinline__ void combine(const Params& p, const Tile& t, const Pre& pre, uint32_t tacc, int part, Regs& r) {
+    const bool vec = p.sstride != 0;
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int n0 = t.c.n0 + part * 64 + h * 16;
+      if (part * 64 + h * 16 < t.bn && n0 < p.N) {
+        uint32_t a[16], w[8];
+        tmem_ld16(tacc + part * 64 + h * 16, a);
+        tmem_ld_wait();
+        if (vec) combine16<true>(p, n0, pre.cb, pre.ca, a, r.z + 16 * h, w, p.gamma_h != nullptr);
+        else combine16<false>(p, n0, pre.cb, pre.ca, a, r.z + 16 * h, w, p.gamma_h != nullptr);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) r.z[8 * h + j] = w[j];
+      }
+    }
+  }
+  __device__ static __forceinline__ void store(const Params& p, const Tile& t, const Pre& pre, int part, int lane, uint8_t* stage, const Regs& r) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int n0 = t.c.n0 + part * 64 + h * 32;
+      if (part * 64 + h * 32 >= t.bn || n0 >= p.N) break;
+      uint4 o[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) o[j] = make_uint4(r.z[16 * h + 4 * j], r.z[16 * h + 4 * j + 1], r.z[16 * h + 4 * j + 2], r.z[16 * h + 4 * j + 3]);
+      warp_store_rows<4>(stage, o, pre.yrow ? pre.yrow + n0 : nullptr, min(32, p.N - n0) * 2, lane);
     }
   }
 };
@@ -492,25 +548,24 @@ static inline float* hp8_gamma_h(const SavedPtrs& sv, int r) {
 template <bool HP>
 static int fill_forward_params(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, uint16_t* Y, typename FwdProblem<HP>::Params& f) {
   using P = FwdProblem<HP>;
-  const int mtiles = (a.T + 127) / 128;
   if (!map2d(&f.tq, true, sv.q, a.K, a.T, 128, 128)) return PQ_ERR_CUDA;
-  if (!map2d(&f.ts, true, w_s8, a.K, a.N, 128, 256)) return PQ_ERR_CUDA;
+  if (!map2d(&f.ts, true, w_s8, a.K, a.N, 128, 128)) return PQ_ERR_CUDA;
   f.th = f.tq; f.tb = f.tq;
   f.gamma_h = nullptr; f.hp_scales = a.hp_scales; f.hp_ext = a.hp_ext ? 1 : 0;
   if (HP && a.hp_scales) {
     // INT8 branch: codes of h [items*128, r] and of B_e [E, N, r], one byte per value
     const uint64_t rows = (uint64_t)sv.max_items * 128;
     if (!map3d_i8(&f.th, sv.h, a.r, a.r, rows, 1, 128)) return PQ_ERR_CUDA;
-    if (!map3d_i8(&f.tb, a.B, a.r, a.r, a.N, a.E, 256)) return PQ_ERR_CUDA;
+    if (!map3d_i8(&f.tb, a.B, a.r, a.r, a.N, a.E, 128)) return PQ_ERR_CUDA;
     f.gamma_h = hp8_gamma_h(sv, a.r);
   } else if (HP) {
     if (!map2d(&f.th, false, sv.h, a.r, (uint64_t)sv.max_items * 256, 64, 128)) return PQ_ERR_CUDA;
-    if (!map3d(&f.tb, a.B, a.r, a.N, a.E, 64, 256)) return PQ_ERR_CUDA;
+    if (!map3d(&f.tb, a.B, a.r, a.N, a.E, 64, 128)) return PQ_ERR_CUDA;
   }
   f.rt = sv.rt; f.perm = (HP && a.E > 1) ? sv.perm : nullptr; f.gamma = sv.gamma; f.gate = sv.gate; f.w_scales = a.w_scales;
   f.alpha = a.alpha; f.beta = a.beta; f.Y = Y; f.T = a.T; f.N = a.N; f.K = a.K; f.r = a.r; f.sstride = a.scale_stride;
   f.item_rows = sv.max_items * 128;
-  f.g = make_tile_grid(mtiles, (a.N + 255) / 256, 256);
+  f.g = make_tile_grid((a.T + 255) / 256, (a.N + 255) / 256, 256);
   return PQ_OK;
 }
 
@@ -522,7 +577,7 @@ int gemm_hp_up8(const LayerArgs& a, const SavedPtrs& sv, const void* A8, int* ra
   p.K = a.K; p.r = a.r; p.rp = a.r; p.bn = h_round_up(a.r, 16);
   if (!map2d(&p.tq, true, sv.q, a.K, a.T, 128, 128)) return PQ_ERR_CUDA;
   if (!map3d_i8(&p.ta, A8, a.K, a.K, a.r, a.E, p.bn)) return PQ_ERR_CUDA;
-  return launch_gemm(KID_HP_UP, k_gemm_hp_up8, p, sv.max_items, st);
+  return launch_gemm<HpUp8Problem>(KID_HP_UP, k_gemm_hp_up8, p, sv.max_items, st);
 }
 
 int gemm_forward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, const uint16_t* xs, uint16_t* Y, cudaStream_t st,
@@ -537,26 +592,26 @@ int gemm_forward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, co
     rc = fill_forward_params<true>(a, w_s8, sv, Y, f);
     if (rc) return rc;
     if (before_main && cudaStreamWaitEvent(st, before_main, 0) != cudaSuccess) return PQ_ERR_CUDA;
-    return launch_gemm(KID_FWD, k_gemm_fwd_hp, f, f.g.total, st);
+    return launch_gemm<FwdProblem<true>>(KID_FWD, k_gemm_fwd_hp, f, f.g.total, st);
   }
   if (a.r > 0) {
     HpUpProblem::Params p;
     p.rt = sv.rt; p.H = sv.h; p.K = a.K; p.r = a.r; p.bn = h_round_up(a.r, 16); p.item_rows = sv.max_items * 128;
     if (!map2d(&p.tx, false, xs, a.K, a.T, 64, 128)) return PQ_ERR_CUDA;
     if (!map3d(&p.ta, a.A, a.K, a.r, a.E, 64, p.bn)) return PQ_ERR_CUDA;
-    int rc = launch_gemm(KID_HP_UP, k_gemm_hp_up, p, sv.max_items, st);
+    int rc = launch_gemm<HpUpProblem>(KID_HP_UP, k_gemm_hp_up, p, sv.max_items, st);
     if (rc) return rc;
     FwdProblem<true>::Params f;
     rc = fill_forward_params<true>(a, w_s8, sv, Y, f);
     if (rc) return rc;
     if (before_main && cudaStreamWaitEvent(st, before_main, 0) != cudaSuccess) return PQ_ERR_CUDA;
-    return launch_gemm(KID_FWD, k_gemm_fwd_hp, f, f.g.total, st);
+    return launch_gemm<FwdProblem<true>>(KID_FWD, k_gemm_fwd_hp, f, f.g.total, st);
   }
   FwdProblem<false>::Params f;
   int rc = fill_forward_params<false>(a, w_s8, sv, Y, f);
   if (rc) return rc;
   if (before_main && cudaStreamWaitEvent(st, before_main, 0) != cudaSuccess) return PQ_ERR_CUDA;
-  return launch_gemm(KID_FWD, k_gemm_fwd_1bit, f, f.g.total, st);
+  return launch_gemm<FwdProblem<false>>(KID_FWD, k_gemm_fwd_1bit, f, f.g.total, st);
 }
 
 
@@ -579,6 +634,7 @@ __device__ __forceinline__ float dx_scale(const float* w_scales, const float* be
 //   gh = g H (bf16, masked),  dl[t,j] = dg g (delta_je - p_tj),  dlc = dl / c
 // ---------------------------------------------------------------------------
 struct HpDhProblem {
+  static constexpr int CG = 1, kEpiWarps = 8;
   using Acc = AccDouble;
   struct Params {
     CUtensorMap tdy, tba;  // dYs [T,N]; (alpha) B [E,N,r]
@@ -596,20 +652,19 @@ struct HpDhProblem {
     int T, N, r, E, bn, sstride, item_rows, ba_blk;
   };
   struct Tile { int item; int4 it; };
-  __device__ static int stage_cols(const Params& p) { return p.bn <= 128 ? 128 : 256; }
+  __device__ static int stage_rows(const Params& p) { return p.bn <= 128 ? 128 : 256; }
   __device__ static int num_tiles(const Params& p) { return p.rt.n_items[0]; }
-  __device__ static void tile_init(const Params& p, int i, Tile& t) { t.item = i; t.it = p.rt.items[i]; }
+  __device__ static void tile_init(const Params& p, int i, int, Tile& t) { t.item = i; t.it = p.rt.items[i]; }
   __device__ static int num_segments(const Params&, const Tile&) { return 1; }
   __device__ static void segment(const Params& p, const Tile& t, int, Segment& s) {
-    s.a_blk = 0; s.b_blk = p.ba_blk;
+    s.a_blk = 0; s.b_blk = p.ba_blk; s.b_bytes = p.bn * 128;
     s.mode = MODE_BF_KM; s.acc = 0; s.bn = p.bn; s.ksteps = 4; s.nkb = (p.N + 63) / 64;
     s.ta = &p.tdy; s.a_rank = 2; s.a_x = 0; s.a_y = t.it.x * 128; s.a_z = 0;
     s.tb = &p.tba; s.b_rank = 3; s.b_x = 0; s.b_y = 0; s.b_z = t.it.y;
-    s.b_box = 0;
   }
   using Pre = NoPre;
   __device__ static Pre prepare(const Params&, const Tile&, int, int) { return Pre{}; }
-  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t taddr, uint32_t, int quad, int half, int lane, uint8_t* stage) {
+  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t taddr, int quad, int half, int lane, uint8_t* stage) {
     if (half) return;   // each row's sum over all r columns stays in one thread
     const int row = quad * 32 + lane;
     const bool live = row >= t.it.z && row < t.it.w;
@@ -684,6 +739,7 @@ PQ_DEFINE_GEMM_KERNEL(k_gemm_hp_dh, HpDhProblem)
 // scattered back to token order.
 // ---------------------------------------------------------------------------
 struct BwdDxProblem {
+  static constexpr int CG = 2, kEpiWarps = 8;
   using Acc = AccDouble;
   struct Params {
     CUtensorMap tdy, tsb, tdh, ta3, tdl, twr;
@@ -695,19 +751,20 @@ struct BwdDxProblem {
     TileGrid g;
     int T, N, K, r, E, sstride, item_rows, sb_blk, a3_blk, wr_blk;
   };
-  struct Tile { TileCoord c; int m, bn, ib, ie, skip1; };
+  struct Tile { TileCoord c; int m, rank, bn, pb, pe, skip1; };
   __device__ static int num_tiles(const Params& p) { return p.g.total; }
-  __device__ static void tile_init(const Params& p, int i, Tile& t) {
-    t.c = tile_coord(p.g, i);
+  __device__ static void tile_init(const Params& p, int i, int rank, Tile& t) {
+    t.c = tile_coord<CG>(p.g, i, rank);
     t.m = t.c.m;
-    t.bn = clip_bn(t.c.bn, t.c.n0, p.K, 64);
-    if (p.r > 0) { t.ib = p.rt.tile_item_begin[t.m]; t.ie = p.rt.tile_item_begin[t.m + 1]; } else { t.ib = t.ie = 0; }
+    t.rank = rank;
+    t.bn = clip_bn(t.c.bn, t.c.n0, p.K, 128);
+    if (p.r > 0) { t.pb = p.rt.pair_begin[t.m >> 1]; t.pe = p.rt.pair_begin[(t.m >> 1) + 1]; } else { t.pb = t.pe = 0; }
     t.skip1 = dx_scale(p.w_scales, p.beta, p.sstride) == 0.f;
   }
-  __device__ static int num_segments(const Params& p, const Tile& t) { return (t.skip1 ? 0 : 1) + 2 * (t.ie - t.ib) + (p.E > 1 ? 1 : 0); }
+  __device__ static int num_segments(const Params& p, const Tile& t) { return (t.skip1 ? 0 : 1) + 2 * (t.pe - t.pb) + (p.E > 1 ? 1 : 0); }
   __device__ static void segment(const Params& p, const Tile& t, int i, Segment& s) {
     s.mode = MODE_BF_KM; s.acc = 0; s.bn = t.bn; s.ksteps = 4; s.a_rank = 2; s.a_x = 0; s.a_z = 0;
-    s.b_x = t.c.n0; s.b_y = 0; s.b_z = 0; s.b_box = 0; s.a_blk = 0;
+    s.b_x = t.c.n0 + t.rank * (t.bn >> 1); s.b_y = 0; s.b_z = 0; s.b_bytes = kOperandBytes; s.a_blk = 0;
     if (!t.skip1) {
       if (i == 0) {
         s.nkb = (p.N + 63) / 64;
@@ -717,11 +774,12 @@ struct BwdDxProblem {
       }
       --i;
     }
-    if (i < 2 * (t.ie - t.ib)) {
-      const int item = t.ib + (i >> 1), plane = i & 1;
+    if (i < 2 * (t.pe - t.pb)) {
+      const int4 pi = p.rt.pair_items[t.pb + (i >> 1)];
+      const int item = t.rank ? pi.z : pi.y, plane = i & 1;
       s.nkb = (p.r + 63) / 64;
-      s.ta = &p.tdh; s.a_y = plane * p.item_rows + item * 128;
-      s.tb = &p.ta3; s.b_rank = 3; s.b_z = p.rt.items[item].y; s.b_blk = p.a3_blk;
+      s.ta = &p.tdh; s.a_y = item >= 0 ? plane * p.item_rows + item * 128 : 2 * p.item_rows;   // beyond both planes: zeros
+      s.tb = &p.ta3; s.b_rank = 3; s.b_z = pi.x; s.b_blk = p.a3_blk;
       return;
     }
     s.nkb = 1; s.ksteps = 1;
@@ -736,10 +794,10 @@ struct BwdDxProblem {
     if (pos < p.T) r.xrow = p.dX + (long long)(p.perm ? p.perm[pos] : pos) * p.K;
     return r;
   }
-  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t taddr, uint32_t, int quad, int half, int lane, uint8_t* stage) {
+  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t taddr, int quad, int part, int lane, uint8_t* stage) {
     const float cc = pre.cc;
     const bool has = num_segments(p, t) > 0;
-    for (int c64 = half; c64 * 64 < t.bn; c64 += 2) {
+    for (int c64 = part; c64 * 64 < t.bn; c64 += kEpiWarps / 4) {
       const int k0 = t.c.n0 + c64 * 64;
       if (k0 >= p.K) break;
       uint32_t v0[32], v1[32];
@@ -755,24 +813,28 @@ struct BwdDxProblem {
       }
 #pragma unroll
       for (int j = 0; j < 8; ++j) o[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
-      warp_store_rows(stage, o, pre.xrow ? pre.xrow + k0 : nullptr, min(64, p.K - k0) * 2, lane);
+      warp_store_rows<8>(stage, o, pre.xrow ? pre.xrow + k0 : nullptr, min(64, p.K - k0) * 2, lane);
     }
   }
 };
 PQ_DEFINE_GEMM_KERNEL(k_gemm_bwd_dx, BwdDxProblem)
 
 // ---------------------------------------------------------------------------
-// B3: the two products that contract dYs^T over tokens, in one launch.
-//   dW tiles: G = dYs^T . xt; dW = beta_n G; per-tile partial of dbeta_n = lam * sum_k S[n,k] G[n,k].
-//   dB tiles (one per expert and 128 output features, after the dW tiles): dBraw_e = dYs^T . (g H) over
-//     the expert's items, the hi and lo planes of g H side by side as the two halves of the tile's
-//     columns; dB = alpha_n dBraw, and the partial of dalpha_n = sum_j B[e,n,j] dBraw[n,j].
-//   router tiles (one per 256 columns of K): dWr = c * (dl / c)^T . Xs, the logit gradient in the
-//     bf16 form the dX tile also uses, rows >= E of the tile unused (Sec. 3.3, "trained end-to-end").
-//   dA tiles (one per expert and 256 columns of K): dA_e = c * (dH / c)^T . Xs over the expert's items, with the
+// B3: the products that contract over tokens.
+//   dW tiles (256 output features x 256 columns of K): G = dYs^T . xt; dW = beta_n G; per-tile partial of
+//     dbeta_n = lam * sum_k S[n,k] G[n,k].
+//   dB tiles (one per expert and 256 output features): dBraw_e = dYs^T . (g H) over the expert's items, the hi and lo
+//     planes of g H side by side as the two halves of the tile's columns (one half per CTA of the pair);
+//     dB = alpha_n dBraw, and the partial of dalpha_n = sum_j B[e,n,j] dBraw[n,j].
+//   router tiles (one per 256 columns of K): dWr^T = c * Xs^T . (dl / c), the logit gradient in the bf16 form the dX tile
+//     also uses (Sec. 3.3, "trained end-to-end").
+//   dA tiles (one per expert and 256 columns of K): dA_e^T = c * Xs^T . (dH / c) over the expert's items, with the
 //     leading bf16 plane of dH / c (its 2^-9 rounding averages out over the tokens of the sum).
+// The last two have K as the rows of the tile, 256 of them for the pair, and the r (or E) short dimension as columns: the
+// other way round half of a pair's rows would be empty.
 // ---------------------------------------------------------------------------
 struct BwdDwProblem {
+  static constexpr int CG = 2, kEpiWarps = 8;
   using Acc = AccDouble;
   enum Kind : int { KIND_DW = 0, KIND_DB = 1, KIND_DWR = 2, KIND_DA = 3 };
   struct Params {
@@ -792,15 +854,13 @@ struct BwdDwProblem {
     TileGrid g;
     int T, N, K, r, r64, E, sstride, dy_blk, xt_blk, gh_blk, xs_blk, dh_blk, item_rows, ntn, ntk, db_tiles, wr_tiles, da_tiles;
   };
-  struct Tile { TileCoord c; int kind, nt, bn, e, ib, ie; };
+  struct Tile { int kind, rank, nt, n0, bn, e, ib, ie; };   // nt: this CTA's block of 128 rows (features, or columns of K)
   __device__ static int num_tiles(const Params& p) { return p.wr_tiles + p.da_tiles + p.g.total + p.db_tiles; }
   // order: the tiles whose contraction runs over all tokens first (router, dA with one expert, dW), the short ones last
-  __device__ static void tile_init(const Params& p, int i, Tile& t) {
-    t.ib = t.ie = 0; t.e = 0; t.nt = 0;
+  __device__ static void tile_init(const Params& p, int i, int rank, Tile& t) {
+    t.ib = t.ie = 0; t.e = 0; t.n0 = 0; t.rank = rank;
     if (i < p.wr_tiles) {
-      t.kind = KIND_DWR;
-      t.c.m = 0; t.c.n0 = i * 256; t.c.bn = 256;
-      t.bn = clip_bn(256, t.c.n0, p.K, 64);
+      t.kind = KIND_DWR; t.nt = 2 * i + rank; t.bn = 128;
       return;
     }
     i -= p.wr_tiles;
@@ -808,71 +868,67 @@ struct BwdDwProblem {
       t.kind = KIND_DA;
       t.e = i / p.ntk;
       t.ib = p.rt.expert_item_begin[t.e]; t.ie = p.rt.expert_item_begin[t.e + 1];
-      t.c.m = 0; t.c.n0 = (i % p.ntk) * 256; t.c.bn = 256;
-      t.bn = clip_bn(256, t.c.n0, p.K, 64);
+      t.nt = 2 * (i % p.ntk) + rank; t.bn = 128;
       return;
     }
     i -= p.da_tiles;
     if (i < p.g.total) {
       t.kind = KIND_DW;
-      t.c = tile_coord(p.g, i);
-      t.nt = t.c.m;
-      t.bn = clip_bn(t.c.bn, t.c.n0, p.K, 64);
+      const TileCoord c = tile_coord<CG>(p.g, i, rank);
+      t.nt = c.m; t.n0 = c.n0;
+      t.bn = clip_bn(c.bn, c.n0, p.K, 128);
       return;
     }
     i -= p.g.total;
     t.kind = KIND_DB;
-    t.e = i / p.ntn; t.nt = i % p.ntn;
+    t.e = i / p.ntn; t.nt = 2 * (i % p.ntn) + rank;
     t.ib = p.rt.expert_item_begin[t.e]; t.ie = p.rt.expert_item_begin[t.e + 1];
     t.bn = 2 * p.r64;
-    t.c.m = t.nt; t.c.n0 = 0; t.c.bn = t.bn;
   }
   __device__ static int num_segments(const Params&, const Tile& t) { return (t.kind == KIND_DW || t.kind == KIND_DWR) ? 1 : t.ie - t.ib; }
   __device__ static void segment(const Params& p, const Tile& t, int i, Segment& s) {
-    s.mode = MODE_BF_MM; s.acc = 0; s.bn = t.bn; s.ksteps = 4; s.b_box = 0;
+    s.mode = MODE_BF_MM; s.acc = 0; s.bn = t.bn; s.ksteps = 4; s.b_bytes = kOperandBytes;
     s.a_rank = 2; s.a_z = 0; s.b_rank = 2; s.b_z = 0;
+    s.a_x = t.nt * 128;
     switch (t.kind) {
       case KIND_DW:
         s.nkb = (p.T + 63) / 64;
-        s.ta = &p.tdyT; s.a_x = t.nt * 128; s.a_y = 0; s.a_blk = p.dy_blk;
-        s.tb = &p.txt; s.b_x = t.c.n0; s.b_y = 0; s.b_blk = p.xt_blk;
-        break;
-      case KIND_DWR:
-        s.nkb = (p.T + 63) / 64;
-        s.ta = &p.tdlT; s.a_x = 0; s.a_y = 0; s.a_blk = 0;          // 16 columns: plain boxes, zero beyond
-        s.tb = &p.txs; s.b_x = t.c.n0; s.b_y = 0; s.b_blk = p.xs_blk;
+        s.ta = &p.tdyT; s.a_y = 0; s.a_blk = p.dy_blk;
+        s.tb = &p.txt; s.b_x = t.n0 + t.rank * (t.bn >> 1); s.b_y = 0; s.b_blk = p.xt_blk;
         break;
       case KIND_DB: {
         const int item = t.ib + i;
         s.nkb = 2;                                        // the 128 tokens of the item's tile (rows outside the item are zero in g H)
-        s.ta = &p.tdyT; s.a_x = t.nt * 128; s.a_y = p.rt.items[item].x * 128; s.a_blk = p.dy_blk;
-        s.tb = &p.tgh; s.b_x = 0; s.b_y = item * 128; s.b2_y = p.item_rows + item * 128; s.b_blk = p.gh_blk;
+        s.ta = &p.tdyT; s.a_y = p.rt.items[item].x * 128; s.a_blk = p.dy_blk;
+        s.tb = &p.tgh; s.b_x = 0; s.b_y = t.rank * p.item_rows + item * 128; s.b_blk = p.gh_blk; s.b_bytes = p.r64 * 128;
         break;
       }
-      default: {                                          // KIND_DA: (dH / c)^T . Xs over the expert's items, leading plane of dH / c
+      case KIND_DWR:
+        s.nkb = (p.T + 63) / 64;
+        s.ta = &p.txs; s.a_y = 0; s.a_blk = p.xs_blk;
+        s.tb = &p.tdlT; s.b_x = t.rank * 64; s.b_y = 0; s.b_blk = -1; s.b_bytes = kMnBoxBytes;   // 16 columns, zeros beyond
+        break;
+      default: {                                          // KIND_DA
         const int item = t.ib + i;
         s.nkb = 2;
-        s.ta = &p.tdhT; s.a_x = 0; s.a_y = item * 128; s.a_blk = p.dh_blk;
-        s.tb = &p.txs; s.b_x = t.c.n0; s.b_y = p.rt.items[item].x * 128; s.b_blk = p.xs_blk;
+        s.ta = &p.txs; s.a_y = p.rt.items[item].x * 128; s.a_blk = p.xs_blk;
+        s.tb = &p.tdhT; s.b_x = t.rank * 64; s.b_y = item * 128; s.b_blk = p.dh_blk; s.b_bytes = kMnBoxBytes;
         break;
       }
     }
   }
   using Pre = NoPre;
   __device__ static Pre prepare(const Params&, const Tile&, int, int) { return Pre{}; }
-  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t taddr, uint32_t, int quad, int half, int lane, uint8_t* stage) {
+  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t taddr, int quad, int part, int lane, uint8_t* stage) {
     if (t.kind == KIND_DWR || t.kind == KIND_DA) {
-      // ---- router tile: row j < E of the accumulator is dWr[j, :] / c;  dA tile: row j < r is dA[e, j, :] / c
-      const int j = quad * 32 + lane;
+      // ---- row k of the tile, column j: dWr[j, k] / c, or dA[e, j, k] / c.  A warp holds 32 consecutive k of one j: whole lines
+      const int k = t.nt * 128 + quad * 32 + lane;
       const float c = dx_scale(p.w_scales, p.beta, p.sstride);
       const float cc = c != 0.f ? c : 1.0f;
       const bool any = t.kind == KIND_DWR || t.ie > t.ib;    // an expert without tokens: exact zeros
-      float* out = nullptr;
-      if (t.kind == KIND_DWR) { if (j < p.E) out = p.dWr + (long long)j * p.K; }
-      else if (j < p.r) out = p.dA + ((long long)t.e * p.r + j) * p.K;
-      for (int c32 = half; c32 * 32 < t.bn; c32 += 2) {
-        const int k0 = t.c.n0 + c32 * 32;
-        if (k0 >= p.K) break;
+      const int cols = t.kind == KIND_DWR ? p.E : p.r;
+      float* out = t.kind == KIND_DWR ? p.dWr + k : p.dA + (long long)t.e * p.r * p.K + k;
+      for (int c32 = part; c32 * 32 < cols; c32 += kEpiWarps / 4) {
         uint32_t v[32];
         if (any) {
           tmem_ld32(taddr + c32 * 32, v);
@@ -881,12 +937,11 @@ struct BwdDwProblem {
 #pragma unroll
           for (int u = 0; u < 32; ++u) v[u] = 0u;
         }
-        uint4 o[8];
+        if (k < p.K) {
 #pragma unroll
-        for (int q4 = 0; q4 < 8; ++q4)
-          o[q4] = make_uint4(__float_as_uint(cc * __uint_as_float(v[4 * q4])), __float_as_uint(cc * __uint_as_float(v[4 * q4 + 1])),
-                             __float_as_uint(cc * __uint_as_float(v[4 * q4 + 2])), __float_as_uint(cc * __uint_as_float(v[4 * q4 + 3])));
-        warp_store_rows(stage, o, out ? out + k0 : nullptr, min(32, p.K - k0) * 4, lane);
+          for (int u = 0; u < 32; ++u)
+            if (c32 * 32 + u < cols) out[(long long)(c32 * 32 + u) * p.K] = cc * __uint_as_float(v[u]);
+        }
       }
       return;
     }
@@ -897,8 +952,8 @@ struct BwdDwProblem {
       const bool any = t.ie > t.ib;                     // an expert without tokens: exact zeros
       const float al = live ? p.alpha[n * p.sstride] : 0.f;
       const long long row = ((long long)t.e * p.N + (live ? n : 0)) * p.r;
-      float part = 0.f;
-      for (int c32 = half; c32 * 32 < p.r; c32 += 2) {
+      float psum = 0.f;
+      for (int c32 = part; c32 * 32 < p.r; c32 += kEpiWarps / 4) {
         uint32_t vh[32], vl[32];
         if (any) {
           tmem_ld32(taddr + c32 * 32, vh);
@@ -914,23 +969,23 @@ struct BwdDwProblem {
           const int j = c32 * 32 + q4 * 4;
           if (live && j < p.r) {
             const uint2 bv = *reinterpret_cast<const uint2*>(p.B + row + j);
-            part = fmaf(bf16lo(bv.x), gsum[0], part); part = fmaf(bf16hi(bv.x), gsum[1], part);
-            part = fmaf(bf16lo(bv.y), gsum[2], part); part = fmaf(bf16hi(bv.y), gsum[3], part);
+            psum = fmaf(bf16lo(bv.x), gsum[0], psum); psum = fmaf(bf16hi(bv.x), gsum[1], psum);
+            psum = fmaf(bf16lo(bv.y), gsum[2], psum); psum = fmaf(bf16hi(bv.y), gsum[3], psum);
           }
           o[q4] = make_uint4(__float_as_uint(al * gsum[0]), __float_as_uint(al * gsum[1]), __float_as_uint(al * gsum[2]),
                              __float_as_uint(al * gsum[3]));
         }
-        warp_store_rows(stage, o, live ? p.dB + row + c32 * 32 : nullptr, min(32, p.r - c32 * 32) * 4, lane);
+        warp_store_rows<8>(stage, o, live ? p.dB + row + c32 * 32 : nullptr, min(32, p.r - c32 * 32) * 4, lane);
       }
-      if (live) p.dalpha_partial[(long long)(2 * t.e + half) * p.N + n] = part;
+      if (live) p.dalpha_partial[(long long)(2 * t.e + part) * p.N + n] = psum;
       return;
     }
     const float be = live ? p.beta[n * p.sstride] : 0.f;
     float* wrow = live ? p.dW + (long long)n * p.K : nullptr;
     const uint4* srow = reinterpret_cast<const uint4*>(p.s8 + (long long)(live ? n : 0) * p.K);
-    float part = 0.f;
-    for (int c32 = half; c32 * 32 < t.bn; c32 += 2) {
-      const int k0 = t.c.n0 + c32 * 32;
+    float psum = 0.f;
+    for (int c32 = part; c32 * 32 < t.bn; c32 += kEpiWarps / 4) {
+      const int k0 = t.n0 + c32 * 32;
       if (k0 >= p.K) break;
       uint32_t v[32];
       tmem_ld32(taddr + c32 * 32, v);
@@ -946,24 +1001,23 @@ struct BwdDwProblem {
         const float g0 = __uint_as_float(v[q4 * 4]), g1 = __uint_as_float(v[q4 * 4 + 1]);
         const float g2 = __uint_as_float(v[q4 * 4 + 2]), g3 = __uint_as_float(v[q4 * 4 + 3]);
         const uint32_t sb = sw[q4];  // four +-1 bytes: bit 7 set <-> -1
-        part += (sb & 0x80u) ? -g0 : g0;
-        part += (sb & 0x8000u) ? -g1 : g1;
-        part += (sb & 0x800000u) ? -g2 : g2;
-        part += (sb & 0x80000000u) ? -g3 : g3;
+        psum += (sb & 0x80u) ? -g0 : g0;
+        psum += (sb & 0x8000u) ? -g1 : g1;
+        psum += (sb & 0x800000u) ? -g2 : g2;
+        psum += (sb & 0x80000000u) ? -g3 : g3;
         o[q4] = make_uint4(__float_as_uint(be * g0), __float_as_uint(be * g1), __float_as_uint(be * g2), __float_as_uint(be * g3));
       }
-      warp_store_rows(stage, o, wrow ? wrow + k0 : nullptr, 128, lane);
+      warp_store_rows<8>(stage, o, wrow ? wrow + k0 : nullptr, 128, lane);
     }
     // one slot per (column tile, warp of the row pair)
-    if (live) p.dbeta_partial[(long long)(2 * (t.c.n0 / 256) + half) * p.N + n] = part;
+    if (live) p.dbeta_partial[(long long)(2 * (t.n0 / 256) + part) * p.N + n] = psum;
   }
 };
 PQ_DEFINE_GEMM_KERNEL(k_gemm_bwd_dw, BwdDwProblem)
 
 int gemm_backward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, const BwdBuffers& b, uint16_t* dX, float* dW, float* dA,
                   float* dB, float* dWr, cudaStream_t st, const BwdStreams& bs) {
-  const int mtiles = (a.T + 127) / 128;
-  const int ntk = (a.K + 255) / 256, ntn128 = (a.N + 127) / 128;
+  const int ntk = (a.K + 255) / 256, ntn = (a.N + 255) / 256;
   const bool hp = a.r > 0;
   const int r64 = h_round_up(a.r, 64);
   const uint64_t item_rows = (uint64_t)sv.max_items * 128;  // rows of one plane; buffers hold two
@@ -973,32 +1027,32 @@ int gemm_backward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, c
   BwdDwProblem::Params w;
   {
     if (!map_mn(&w.tdyT, &w.dy_blk, b.dys, a.N, a.T, 2, 1, 2)) return PQ_ERR_CUDA;
-    if (!map_mn(&w.txt, &w.xt_blk, sv.xt, a.K, a.T, 2, 1, 4)) return PQ_ERR_CUDA;
+    if (!map_mn(&w.txt, &w.xt_blk, sv.xt, a.K, a.T, 2, 1, 2)) return PQ_ERR_CUDA;
     w.tgh = w.txt; w.gh_blk = 0;
     if (hp && !map_mn(&w.tgh, &w.gh_blk, b.gh, a.r, 2 * item_rows, 2, 1, r64 / 64)) return PQ_ERR_CUDA;
     w.rt = sv.rt; w.s8 = w_s8; w.beta = a.beta; w.alpha = a.alpha; w.B = a.B; w.dW = dW; w.dB = dB;
     w.dbeta_partial = b.dbeta_partial; w.dalpha_partial = b.dalpha_partial;
     w.T = a.T; w.N = a.N; w.K = a.K; w.r = a.r; w.r64 = r64; w.E = a.E; w.sstride = a.scale_stride; w.item_rows = (int)item_rows;
-    w.ntn = ntn128; w.ntk = ntk; w.db_tiles = hp ? a.E * ntn128 : 0; w.da_tiles = hp ? a.E * ntk : 0;
+    w.ntn = ntn; w.ntk = ntk; w.db_tiles = hp ? a.E * ntn : 0; w.da_tiles = hp ? a.E * ntk : 0;
     w.tdlT = w.txt; w.txs = w.txt; w.tdhT = w.txt; w.xs_blk = 0; w.dh_blk = 0; w.wr_tiles = 0;
     w.w_scales = a.w_scales; w.dWr = dWr; w.dA = dA;
     if (hp) {
-      if (!map_mn(&w.txs, &w.xs_blk, b.xs, a.K, a.T, 2, 1, 4)) return PQ_ERR_CUDA;
-      if (!map_mn(&w.tdhT, &w.dh_blk, b.dhc, a.r, 2 * item_rows, 2, 1, 2)) return PQ_ERR_CUDA;
+      if (!map_mn(&w.txs, &w.xs_blk, b.xs, a.K, a.T, 2, 1, 2)) return PQ_ERR_CUDA;
+      if (!map_mn(&w.tdhT, &w.dh_blk, b.dhc, a.r, 2 * item_rows, 2, 1, 1)) return PQ_ERR_CUDA;
     }
     if (hp && a.E > 1) {
-      int unused = 0;
-      if (!map_mn(&w.tdlT, &unused, b.dlc, 16, a.T, 2, 1, 2)) return PQ_ERR_CUDA;
+      int one_box = 0;
+      if (!map_mn(&w.tdlT, &one_box, b.dlc, 16, a.T, 2, 1, 1)) return PQ_ERR_CUDA;
       w.wr_tiles = ntk;
     }
-    w.g = make_tile_grid(ntn128, ntk, 256);
+    w.g = make_tile_grid(ntn, ntk, 256);
   }
   if (bs.side) {
     // the dW tiles proper need dY and q / gamma only: they start at once and take every SM; what follows on the
     // other stream moves into their last wave
     BwdDwProblem::Params m = w;
     m.wr_tiles = 0; m.da_tiles = 0; m.db_tiles = 0;
-    rc = launch_gemm(KID_BWD_DW, k_gemm_bwd_dw, m, m.g.total, st);
+    rc = launch_gemm<BwdDwProblem>(KID_BWD_DW, k_gemm_bwd_dw, m, m.g.total, st);
     if (rc) return rc;
   }
   if (hp) {
@@ -1008,32 +1062,32 @@ int gemm_backward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, c
     p.rt = sv.rt; p.H = sv.h; p.gate = sv.gate; p.probs = sv.probs; p.w_scales = a.w_scales; p.alpha = a.alpha; p.beta = a.beta;
     p.dhc = b.dhc; p.gh = b.gh; p.dl = b.dl; p.dlc = b.dlc;
     p.T = a.T; p.N = a.N; p.r = a.r; p.E = a.E; p.bn = r64; p.sstride = a.scale_stride; p.item_rows = (int)item_rows;
-    rc = launch_gemm(KID_HP_DH, k_gemm_hp_dh, p, sv.max_items, sx);
+    rc = launch_gemm<HpDhProblem>(KID_HP_DH, k_gemm_hp_dh, p, sv.max_items, sx);
     if (rc) return rc;
     if (bs.side && cudaEventRecord(bs.dh_done, sx) != cudaSuccess) return PQ_ERR_CUDA;
   }
   {
     BwdDxProblem::Params p;
     if (!map2d(&p.tdy, false, b.dys, a.N, a.T, 64, 128)) return PQ_ERR_CUDA;
-    if (!map_mn(&p.tsb, &p.sb_blk, b.sb, a.K, a.N, 2, 1, 4)) return PQ_ERR_CUDA;
+    if (!map_mn(&p.tsb, &p.sb_blk, b.sb, a.K, a.N, 2, 1, 2)) return PQ_ERR_CUDA;
     p.tdh = p.tdy; p.ta3 = p.tdy; p.tdl = p.tdy; p.twr = p.tdy; p.a3_blk = 0; p.wr_blk = 0;
     if (hp) {
       if (!map2d(&p.tdh, false, b.dhc, a.r, 2 * item_rows, 64, 128)) return PQ_ERR_CUDA;
-      if (!map_mn(&p.ta3, &p.a3_blk, a.A, a.K, a.r, 3, a.E, 4)) return PQ_ERR_CUDA;
+      if (!map_mn(&p.ta3, &p.a3_blk, a.A, a.K, a.r, 3, a.E, 2)) return PQ_ERR_CUDA;
     }
     if (hp && a.E > 1) {
       if (!map2d(&p.tdl, false, b.dlc, 16, a.T, 64, 128)) return PQ_ERR_CUDA;
-      if (!map_mn(&p.twr, &p.wr_blk, a.Wr, a.K, a.E, 2, 1, 4)) return PQ_ERR_CUDA;
+      if (!map_mn(&p.twr, &p.wr_blk, a.Wr, a.K, a.E, 2, 1, 2)) return PQ_ERR_CUDA;
     }
     p.rt = sv.rt; p.perm = (hp && a.E > 1) ? sv.perm : nullptr; p.w_scales = a.w_scales; p.beta = a.beta; p.dX = dX;
     p.T = a.T; p.N = a.N; p.K = a.K; p.r = a.r; p.E = hp ? a.E : 1; p.sstride = a.scale_stride; p.item_rows = (int)item_rows;
-    p.g = make_tile_grid(mtiles, ntk, 256);
-    rc = launch_gemm(KID_BWD_DX, k_gemm_bwd_dx, p, p.g.total, sx);
+    p.g = make_tile_grid((a.T + 255) / 256, ntk, 256);
+    rc = launch_gemm<BwdDxProblem>(KID_BWD_DX, k_gemm_bwd_dx, p, p.g.total, sx);
     if (rc) return rc;
     if (bs.side && cudaEventRecord(bs.side_done, sx) != cudaSuccess) return PQ_ERR_CUDA;
   }
   if (!bs.side) {
-    rc = launch_gemm(KID_BWD_DW, k_gemm_bwd_dw, w, w.wr_tiles + w.da_tiles + w.g.total + w.db_tiles, st);
+    rc = launch_gemm<BwdDwProblem>(KID_BWD_DW, k_gemm_bwd_dw, w, w.wr_tiles + w.da_tiles + w.g.total + w.db_tiles, st);
     if (rc) return rc;
   } else {
     if (hp) {
@@ -1041,7 +1095,7 @@ int gemm_backward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, c
       BwdDwProblem::Params x = w;
       x.g.total = 0;
       if (cudaStreamWaitEvent(st, bs.dh_done, 0) != cudaSuccess) return PQ_ERR_CUDA;
-      rc = launch_gemm(KID_HP_DB, k_gemm_bwd_dw, x, x.wr_tiles + x.da_tiles + x.db_tiles, st);
+      rc = launch_gemm<BwdDwProblem>(KID_HP_DB, k_gemm_bwd_dw, x, x.wr_tiles + x.da_tiles + x.db_tiles, st);
       if (rc) return rc;
     }
     if (cudaStreamWaitEvent(st, bs.side_done, 0) != cudaSuccess) return PQ_ERR_CUDA;

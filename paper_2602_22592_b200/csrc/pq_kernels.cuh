@@ -38,6 +38,10 @@ struct RoutingTables {
   int4* items;             // [max_items] {tile, expert, first row, end row}
   int* tile_item_begin;    // [mtiles + 1]
   int* expert_item_begin;  // [E + 1]
+  // The same cut for pairs of tiles (256 rows), the unit of the large GEMMs: one entry per (pair of tiles, expert with
+  // rows there) = {expert, item in the first tile or -1, item in the second or -1, pair}
+  int* pair_begin;         // [ceil(mtiles / 2) + 1] first entry of each pair of tiles
+  int4* pair_items;        // [ceil(mtiles / 2) + E - 1]
 };
 
 // Device pointers into the caller's `saved` buffer.
