@@ -378,6 +378,7 @@ __device__ __forceinline__ void gemm_body(const typename P::Params& p) {
         if (!await(1, ac.phase)) break;
         P::take_first(p, t, pre, tlane + kAccCols, part, regs);
         release(1);
+        P::scale_first(p, t, pre, part, regs);
         if (!await(0, ac.phase)) break;
         P::combine(p, t, pre, tlane, part, regs);
         release(0);

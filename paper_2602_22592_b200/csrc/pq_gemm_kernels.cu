@@ -365,7 +365,9 @@ PQ_DEFINE_GEMM_KERNEL(k_gemm_hp_up8, HpUp8Problem)
 // (fp32): H B_e^T over r, once per item of the tile (masked H rows are zero).
 // Epilogue: Y[token, n] = alpha_n g z + beta_n (lam / gamma) acc, rounded once.
 // ---------------------------------------------------------------------------
-template <bool HP>
+// GEN = false: scalar feature scales and K < 32768; GEN = true: anything (the extra addresses and branches cost registers the
+// common form does not have to spare).
+template <bool HP, bool GEN>
 struct FwdProblem {
   // With the HP branch a tile holds an int32 and an fp32 accumulator of 256 columns each, all of TMEM.  Sixteen epilogue
   // warps, 64 columns of a row per thread: the fp32 accumulator waits in 64 registers while the int8 contraction runs, and
@@ -420,26 +422,25 @@ struct FwdProblem {
       s.tb = &p.tb; s.b_rank = 3; s.b_z = pi.x;
     }
   }
-  // y = cb_n * acc + ca_n * z for 16 consecutive columns starting at n, packed to 8 bf16 pairs
-  template <bool VEC>
-  __device__ static __forceinline__ void combine16(const Params& p, int n, float cb, float ca, const uint32_t (&a)[16], const uint32_t* z,
-                                                  uint32_t* w, bool z_is_int) {
+  // float of an accumulator of the 1-bit product, exactly.  |acc| <= 128 K: below K = 32768 the integer fits the mantissa of
+  // 1.5 * 2^23, so that an integer add and a float subtract do what the slower conversion instruction does.
+  __device__ static __forceinline__ float acc_float(uint32_t a) {
+    return GEN ? (float)(int)a : __int_as_float((int)a + 0x4B400000) - 12582912.0f;
+  }
+  // y = beta_n cb * acc + z for 16 consecutive columns starting at n (z: the HP term, factors applied), as 8 bf16 pairs
+  __device__ static __forceinline__ void combine16(const Params& p, int n, float cb, const uint32_t (&a)[16], const uint32_t* z, uint32_t* w) {
 #pragma unroll
     for (int q4 = 0; q4 < 4; ++q4) {
-      float b4[4] = {cb, cb, cb, cb}, a4[4] = {ca, ca, ca, ca};
-      if (VEC) {
+      float b4[4] = {cb, cb, cb, cb};
+      if (GEN && p.sstride) {
         const float4 bv = __ldg(reinterpret_cast<const float4*>(p.beta + n) + q4);
         b4[0] *= bv.x; b4[1] *= bv.y; b4[2] *= bv.z; b4[3] *= bv.w;
-        if (HP) {
-          const float4 av = __ldg(reinterpret_cast<const float4*>(p.alpha + n) + q4);
-          a4[0] *= av.x; a4[1] *= av.y; a4[2] *= av.z; a4[3] *= av.w;
-        }
       }
       float y[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        y[u] = b4[u] * (float)(int)a[4 * q4 + u];
-        if (HP) y[u] = fmaf(a4[u], z_is_int ? (float)(int)z[4 * q4 + u] : __uint_as_float(z[4 * q4 + u]), y[u]);
+        const float f = acc_float(a[4 * q4 + u]);
+        y[u] = HP ? fmaf(b4[u], f, __uint_as_float(z[4 * q4 + u])) : b4[u] * f;
       }
       w[2 * q4] = pack_bf16x2(y[0], y[1]);
       w[2 * q4 + 1] = pack_bf16x2(y[2], y[3]);
@@ -476,7 +477,6 @@ struct FwdProblem {
   }
   // pure 1-bit tile
   __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t tacc, int quad, int part, int lane, uint8_t* stage) {
-    const bool vec = p.sstride != 0;
     for (int c = part; c * 64 < t.bn; c += kEpiWarps / 4) {     // 64 output columns = 128 bytes of the row per pass
       const int n0 = t.c.n0 + c * 64;
       if (n0 >= p.N) break;
@@ -488,8 +488,7 @@ struct FwdProblem {
           uint32_t a[16];
           tmem_ld16(tacc + c * 64 + h * 16, a);
           tmem_ld_wait();
-          if (vec) combine16<true>(p, nb, pre.cb, 0.f, a, a, w + 8 * h, false);
-          else combine16<false>(p, nb, pre.cb, 0.f, a, a, w + 8 * h, false);
+          combine16(p, nb, pre.cb, a, a, w + 8 * h);
         }
       }
       uint4 o[8];
@@ -498,18 +497,36 @@ struct FwdProblem {
       warp_store_rows<8>(stage, o, pre.yrow ? pre.yrow + n0 : nullptr, min(64, min(t.bn - c * 64, p.N - n0)) * 2, lane);
     }
   }
-  // tile with an HP branch: thread = row, columns [64 part, 64 part + 64)
+  // Tile with an HP branch: thread = row, columns [64 part, 64 part + 64).  The HP term is finished (alpha, gate, INT8 scales)
+  // while the int8 contraction runs; between that contraction and the next one stand only the read of the int32
+  // accumulator, one multiply-add per value and the rounding.
   struct Regs { uint32_t z[64]; };
-  __device__ static __forceinline__ void take_first(const Params&, const Tile& t, const Pre&, uint32_t tz, int part, Regs& r) {
+  __device__ static __forceinline__ void take_first(const Params& p, const Tile& t, const Pre& pre, uint32_t tz, int part, Regs& r) {
     if (part * 64 < t.bn) {
       tmem_ld32(tz + part * 64, *reinterpret_cast<uint32_t(*)[32]>(r.z));
       tmem_ld32(tz + part * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(r.z + 32));
       tmem_ld_wait();
     }
   }
+  __device__ static __forceinline__ void scale_first(const Params& p, const Tile& t, const Pre& pre, int part, Regs& r) {
+    const bool is_int = p.gamma_h != nullptr;
+#pragma unroll
+    for (int q4 = 0; q4 < 16; ++q4) {
+      const int n = t.c.n0 + part * 64 + q4 * 4;
+      float a4[4] = {pre.ca, pre.ca, pre.ca, pre.ca};
+      if (GEN && p.sstride && n < p.N) {             // N is a multiple of 32: whole groups of four
+        const float4 av = __ldg(reinterpret_cast<const float4*>(p.alpha + n));
+        a4[0] *= av.x; a4[1] *= av.y; a4[2] *= av.z; a4[3] *= av.w;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t v = r.z[4 * q4 + u];
+        r.z[4 * q4 + u] = __float_as_uint(a4[u] * (is_int ? (float)(int)v : __uint_as_float(v)));
+      }
+    }
+  }
   // the results take the place of the z values they are made from: pair j of the row's 64 columns ends up in z[j]
   __device__ static __forceinline__ void combine(const Params& p, const Tile& t, const Pre& pre, uint32_t tacc, int part, Regs& r) {
-    const bool vec = p.sstride != 0;
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
       const int n0 = t.c.n0 + part * 64 + h * 16;
@@ -517,8 +534,7 @@ struct FwdProblem {
         uint32_t a[16], w[8];
         tmem_ld16(tacc + part * 64 + h * 16, a);
         tmem_ld_wait();
-        if (vec) combine16<true>(p, n0, pre.cb, pre.ca, a, r.z + 16 * h, w, p.gamma_h != nullptr);
-        else combine16<false>(p, n0, pre.cb, pre.ca, a, r.z + 16 * h, w, p.gamma_h != nullptr);
+        combine16(p, n0, pre.cb, a, r.z + 16 * h, w);
 #pragma unroll
         for (int j = 0; j < 8; ++j) r.z[8 * h + j] = w[j];
       }
@@ -536,8 +552,15 @@ struct FwdProblem {
     }
   }
 };
-PQ_DEFINE_GEMM_KERNEL(k_gemm_fwd_hp, FwdProblem<true>)
-PQ_DEFINE_GEMM_KERNEL(k_gemm_fwd_1bit, FwdProblem<false>)
+// (the macro takes one name per problem)
+using FwdHp = FwdProblem<true, false>;
+using FwdHpGen = FwdProblem<true, true>;
+using Fwd1 = FwdProblem<false, false>;
+using Fwd1Gen = FwdProblem<false, true>;
+PQ_DEFINE_GEMM_KERNEL(k_gemm_fwd_hp, FwdHp)
+PQ_DEFINE_GEMM_KERNEL(k_gemm_fwd_hp_general, FwdHpGen)
+PQ_DEFINE_GEMM_KERNEL(k_gemm_fwd_1bit, Fwd1)
+PQ_DEFINE_GEMM_KERNEL(k_gemm_fwd_1bit_general, Fwd1Gen)
 
 // INT8 branch: the saved h region holds the codes qh [items*128, r] and, behind them, gamma_h [items*128]
 static inline float* hp8_gamma_h(const SavedPtrs& sv, int r) {
@@ -545,9 +568,12 @@ static inline float* hp8_gamma_h(const SavedPtrs& sv, int r) {
   return reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(sv.h) + codes);
 }
 
-template <bool HP>
-static int fill_forward_params(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, uint16_t* Y, typename FwdProblem<HP>::Params& f) {
-  using P = FwdProblem<HP>;
+// the fused output tile of a layer, with or without an HP branch
+template <bool HP, bool GEN>
+static int launch_forward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, uint16_t* Y, void (*kernel)(typename FwdProblem<HP, GEN>::Params),
+                          cudaStream_t st) {
+  using P = FwdProblem<HP, GEN>;
+  typename P::Params f;
   if (!map2d(&f.tq, true, sv.q, a.K, a.T, 128, 128)) return PQ_ERR_CUDA;
   if (!map2d(&f.ts, true, w_s8, a.K, a.N, 128, 128)) return PQ_ERR_CUDA;
   f.th = f.tq; f.tb = f.tq;
@@ -566,7 +592,7 @@ static int fill_forward_params(const LayerArgs& a, const int8_t* w_s8, const Sav
   f.alpha = a.alpha; f.beta = a.beta; f.Y = Y; f.T = a.T; f.N = a.N; f.K = a.K; f.r = a.r; f.sstride = a.scale_stride;
   f.item_rows = sv.max_items * 128;
   f.g = make_tile_grid((a.T + 255) / 256, (a.N + 255) / 256, 256);
-  return PQ_OK;
+  return launch_gemm<P>(KID_FWD, kernel, f, f.g.total, st);
 }
 
 // h_int = q A8_e^T per item.  raw == nullptr: codes and scales of h into the saved h region; otherwise the exact sums
@@ -583,35 +609,23 @@ int gemm_hp_up8(const LayerArgs& a, const SavedPtrs& sv, const void* A8, int* ra
 int gemm_forward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, const uint16_t* xs, uint16_t* Y, cudaStream_t st,
                  cudaEvent_t before_main) {
   if (a.r > 0 && a.hp_scales) {
-    int rc = PQ_OK;
     if (!a.hp_ext) {
-      rc = gemm_hp_up8(a, sv, a.A, nullptr, st);
+      const int rc = gemm_hp_up8(a, sv, a.A, nullptr, st);
       if (rc) return rc;
     }
-    FwdProblem<true>::Params f;
-    rc = fill_forward_params<true>(a, w_s8, sv, Y, f);
-    if (rc) return rc;
-    if (before_main && cudaStreamWaitEvent(st, before_main, 0) != cudaSuccess) return PQ_ERR_CUDA;
-    return launch_gemm<FwdProblem<true>>(KID_FWD, k_gemm_fwd_hp, f, f.g.total, st);
-  }
-  if (a.r > 0) {
+  } else if (a.r > 0) {
     HpUpProblem::Params p;
     p.rt = sv.rt; p.H = sv.h; p.K = a.K; p.r = a.r; p.bn = h_round_up(a.r, 16); p.item_rows = sv.max_items * 128;
     if (!map2d(&p.tx, false, xs, a.K, a.T, 64, 128)) return PQ_ERR_CUDA;
     if (!map3d(&p.ta, a.A, a.K, a.r, a.E, 64, p.bn)) return PQ_ERR_CUDA;
-    int rc = launch_gemm<HpUpProblem>(KID_HP_UP, k_gemm_hp_up, p, sv.max_items, st);
+    const int rc = launch_gemm<HpUpProblem>(KID_HP_UP, k_gemm_hp_up, p, sv.max_items, st);
     if (rc) return rc;
-    FwdProblem<true>::Params f;
-    rc = fill_forward_params<true>(a, w_s8, sv, Y, f);
-    if (rc) return rc;
-    if (before_main && cudaStreamWaitEvent(st, before_main, 0) != cudaSuccess) return PQ_ERR_CUDA;
-    return launch_gemm<FwdProblem<true>>(KID_FWD, k_gemm_fwd_hp, f, f.g.total, st);
   }
-  FwdProblem<false>::Params f;
-  int rc = fill_forward_params<false>(a, w_s8, sv, Y, f);
-  if (rc) return rc;
   if (before_main && cudaStreamWaitEvent(st, before_main, 0) != cudaSuccess) return PQ_ERR_CUDA;
-  return launch_gemm<FwdProblem<false>>(KID_FWD, k_gemm_fwd_1bit, f, f.g.total, st);
+  const bool general = a.scale_stride != 0 || a.K >= 32768;
+  if (a.r > 0)
+    return general ? launch_forward<true, true>(a, w_s8, sv, Y, k_gemm_fwd_hp_general, st) : launch_forward<true, false>(a, w_s8, sv, Y, k_gemm_fwd_hp, st);
+  return general ? launch_forward<false, true>(a, w_s8, sv, Y, k_gemm_fwd_1bit_general, st) : launch_forward<false, false>(a, w_s8, sv, Y, k_gemm_fwd_1bit, st);
 }
 
 
