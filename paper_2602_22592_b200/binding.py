@@ -154,9 +154,11 @@ def _nbytes(t):
     return 0 if t is None else t.numel() * t.element_size()
 
 
+_device, _raw_stream = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream   # torch.cuda.current_stream() costs microseconds
+
+
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    return ctypes.c_void_p(_raw_stream(_device()) if stream is None else stream.cuda_stream)
 
 
 def _check(fn, status):

@@ -1,20 +1,18 @@
-// Decode path of the pQuant layer (App. A): M <= 16 tokens against weights stored as
-// packed sign bits.  The work is bound by the bytes of the weights (N K / 8 bytes of bits,
-// 2 r (K + N) bytes per expert in use), so the kernels are built around streaming them once:
+// Decode path of the pQuant layer (App. A): M <= 16 tokens against weights stored as packed sign bits, three kernels per group
+// of independent linears:
 //
-//   k_decode_prep  one CTA per (linear, token, slice of the r hidden rows): absmax quantisation
-//                  of the token (Eq. 7-9), router (Sec. 3.3), and its slice of h = A_e x.
-//   k_decode_main  one CTA per SM, each owning a contiguous range of output features of every
-//                  linear of the batch.  A producer warp first fetches the routing of all linears,
-//                  then streams, linear after linear, the sign bits, the activations and the expert
-//                  rows B_e of that range into rings of shared-memory buffers by bulk copies
-//                  (mbarrier full/empty pairs), as far ahead as the rings allow.  Each consumer warp
-//                  owns whole (linear, token group, 16-feature tile) items: 1-bit product on mma.sync
-//                  (u8 bit masks x s8 activations, exact in int32) over all of K, expert product on
-//                  bf16 mma.sync, epilogue Y = alpha g (B_e h) + beta (lam / gamma) (q . S)
-//                  (Eq. 10-11) straight from its registers; warps never wait for one another.
-// A batch is a set of INDEPENDENT linears (the gate and up projections of one block, the q/k/v
-// projections, other sequences): their weights then stream back to back.
+//   k_decode_prep    a cluster of eight CTAs per (linear, token): RMSNorm (optional), absmax quantisation (Eq. 7-9), router
+//                    (Sec. 3.3); every CTA takes its share of the experts' logits and of the codes.
+//   k_decode_hidden  a cluster of CTAs per (linear, expert in use, 16 hidden rows): h = A_e x for all tokens of the expert.
+//   k_decode_main    one CTA per SM, a contiguous share of the output features of all linears each, in units of 16:
+//                    1-bit product on mma.sync (u8 bit masks x s8 codes, exact in int32), expert product z = B_e h on bf16
+//                    mma.sync (dp4a for the INT8 branch), epilogue (Eq. 10-11).
+//
+// A call of one or two linears is a chain of dependent steps, not a stream: its weights take 1-2 us at the memory's rate, a
+// dependent trip to memory about 1 us.  So everything off the chain runs beside it.  The kernels are launched with programmatic
+// stream serialisation; each lets its successor start once the kernels before it have finished, so that a kernel may read what
+// its predecessor's predecessors wrote before it waits for the predecessor itself: k_decode_main has its sign bits multiplied
+// with the codes and the experts' rows of B on their way when h arrives.
 //
 // The sum over k of q S is evaluated as 2 * (sum over the set bits of q) - (sum of q): the bit
 // words feed the tensor cores as 0/1 masks without expansion to +-1.
@@ -24,25 +22,35 @@
 
 namespace pq {
 
-constexpr int kDecodeMaxConsumerWarps = 16;                 // 8 are launched unless a CTA owns more than 128 features
-constexpr int kDecodeMainThreads = 32 * kDecodeMaxConsumerWarps + 32;   // + the producer warp
 constexpr int kDecodeMaxTokens = 16;
-constexpr int kDecodeMaxSlots = 4;      // linears whose sign bits are in flight or in use per CTA
-constexpr int kDecodeMaxQ = 4;          // activation buffers
-constexpr int kDecodeMaxRing = 8;       // expert-row buffers
-constexpr int kDecodeMaxBatch = 16;     // linears per launch (their descriptors travel as kernel parameters)
+constexpr int kDecodeMaxBatch = 96;       // linears per launch (their descriptors travel as kernel parameters)
+constexpr int kPrepThreads = 256;
+constexpr int kPrepWarps = kPrepThreads / 32;
+constexpr int kPrepCluster = 8;           // CTAs that share a token's router
+constexpr int kHiddenSplit = 32;          // shares of the contraction of sixteen hidden rows, added up in order
+constexpr int kHiddenThreads = 256;
+constexpr int kHiddenWarps = kHiddenThreads / 32;
+constexpr int kMainThreads = 512;
+constexpr int kMainWarps = kMainThreads / 32;
+constexpr int kUnit = 16;                 // output features of a unit of work (the rows of one mma tile)
+constexpr int kMaxPassUnits = 8;          // units a CTA works on at once (two warps or more each)
+constexpr int kWarpRows = 2;              // tiles of expert rows a warp of k_decode_main has in flight
+constexpr int kMaxRows = kWarpRows * kMainWarps;
 
-struct DecodeTokInfo {  // one per token, written by k_decode_prep
+struct DecodeTokInfo {  // one per token
   int expert;
   float gate;
   float gamma;
   int rowsum;           // sum over k of q[k]
 };
 
-
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(dst), "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(bar) : "memory");
+}
+// ask `bytes` (a multiple of 16) into L2
+__device__ __forceinline__ void bulk_prefetch(const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<uint64_t>(src)), "r"(bytes) : "memory");
 }
 
 __device__ __forceinline__ void mma_u8s8(int (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
@@ -58,53 +66,68 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1
 
 // ---------------------------------------------------------------------------
 // Layout of the quantised activations handed from prep to main ("q fragments").
-// The contraction index k is walked in pairs of 32-bit weight words (64 values of k).  For pair
-// ip, the thread of a warp with quad index c (lane & 3) takes from a weight word w the bits
-// c + 8 j (mask 0x01010101 of w >> c) and c + 4 + 8 j (mask 0x10101010, i.e. the value 16), j = 0..3.
-// Its four 4-byte operand registers for the tokens' side therefore hold, for token g = lane >> 2,
-//   r0: q[64 ip      + c     + 8 j]   r1: q[64 ip + 32 + c     + 8 j]      (weight-1 masks)
-//   r2: q[64 ip      + c + 4 + 8 j]   r3: q[64 ip + 32 + c + 4 + 8 j]      (weight-16 masks)
-// stored as 16 bytes; only the tokens that exist are stored: with Mg = min(8, M - 8 group) tokens in the group,
-// the piece of (pair ip, token g, quad index c) sits at uint4 index group * npairs * 32 + (ip * Mg + g) * 4 + c.
+// A chunk is 128 values of k: four 32-bit weight words per feature, word c for the threads of quad index c (lane & 3).  For
+// b = 0..3 such a thread takes from its word w the bits b + 8 j (mask 0x01010101 of w >> b) and b + 4 + 8 j (mask 0x10101010,
+// i.e. the value 16), j = 0..3: one 4-byte operand register each.  The tokens' side of bit b is the word of codes
+// q[128 chunk + 32 c + b + 8 j].  The eight words of (chunk, token, c) are two 16-byte pieces, half h holding b = 4 h .. 4 h + 3;
+// only the tokens that exist are stored: with Mg = min(8, M - 8 group) tokens in the group, the piece of (chunk, half h, token
+// g, c) sits at uint4 index group * chunks * 64 + ((2 chunk + h) * Mg + g) * 4 + c.
 // ---------------------------------------------------------------------------
 
 // One linear of a batch: device pointers and sizes (the workspace pointers are carved by the host).
-struct DecodeLinear {
+struct alignas(16) DecodeLinear {
   const uint4* X;           // [M, K] bf16
   const uint4* Wr;          // [E, K] bf16 or null
   const uint16_t* A;        // [E, r, K]
   const uint16_t* B;        // [E, N, r]
   const uint32_t* bits;     // [N, K/32]
+  const uint4* bits_il;     // the same bits as laid out by decode_pack, or null
   const float* w_scales;
   const float* alpha;
   const float* beta;
   uint16_t* Y;              // [M, N]
   DecodeTokInfo* info;      // [16]
-  uint4* qfrag;             // [2, npairs, 32] fragments
+  uint4* qfrag;             // [2 groups][chunks][2][8 tokens][4] fragments
   uint4* hfrag;             // [2 groups][2 planes (hi, lo)][ceil(r/32)][32] fragments of h = A_e x
+  uint16_t* xn;             // [M, K] what k_decode_hidden multiplies: normalised tokens (bf16; X itself without a norm), or int8 codes
   int* acc_dump;            // [M, N] exact 1-bit accumulators (test hook) or null
   const uint4* norm_w;      // [K] bf16 RMSNorm gain or null
+  // INT8 high-precision branch (Sec. 3.2), null without it
+  const int8_t* A8;         // [E, r, K]
+  const uint4* B8_il;       // [E][N / 32 groups, padded to whole 128-feature groups][r / 16][32] pieces of 16 codes
+  const float* hp_scales;   // [E][2]
+  int* h_int;               // [M, r]
+  int* zint_dump;           // [M, N] or null
   float norm_eps;
-  int M, K, N, r, E, sstride, slices, rows_per_slice;
-  // partition of the N / 8 feature groups over the CTAs of k_decode_main: the first `grp_rem` CTAs own grp_base + 1 groups
-  int grp_base, grp_rem;
+  int M, K, N, r, E, sstride;
+  int hidden0;              // first cluster of this linear in k_decode_hidden (min(E, M) * ceil(r / 16) of them)
+  int unit0;                // first unit of work of this linear in the launch
 };
+static_assert(sizeof(DecodeLinear) % 16 == 0, "copied in 16-byte pieces");
+template <int CAP>
 struct DecodeBatch {
-  DecodeLinear lin[kDecodeMaxBatch];
-  int n;
-  // shared-memory carve-up of k_decode_main (bytes from the 128-byte aligned base)
-  int nwarps;               // consumer warps per CTA
-  int prep_rows;            // rows of K values k_decode_prep keeps in shared memory beside the token (2..8, two buffers)
-  int nslot, nq, nring;     // depths of the three buffer rings
-  int off_slots, slot_bytes, off_slot_h, off_q, q_bytes, off_ring, ring_stage_bytes;
+  int n, units;             // linears; units of 16 features of all of them
+  int off_wr, off_gain;     // k_decode_prep: router rows of the CTA, the norm's gains
+  int early;                // k_decode_hidden runs in between: k_decode_main may read prep's results before it waits
+  int hidden_groups, hidden_cluster;   // k_decode_hidden: clusters of all linears, CTAs of each
+  // k_decode_main: buffers of sign bits, their size, and the carve-up of shared memory behind them
+  int nbuf, buf_bytes, off_q, off_h, off_red;
+  int q_chunks;             // chunks of 128 values of k whose codes are in shared memory at once
+  int red_tokens;
+  int unit0[CAP + 1];
+  DecodeLinear lin[CAP];
 };
-// position in a ring of buffers with mbarrier full/empty pairs: the producer waits for empty(idx) with
-// parity phase ^ 1, a consumer for full(idx) with parity phase
-struct DecodeCursor {
-  int idx = 0;
-  uint32_t phase = 0;
-  __device__ __forceinline__ void next(int n) { if (++idx == n) { idx = 0; phase ^= 1u; } }
-};
+
+// A record of the batch into shared memory, one 16-byte piece per warp at a time: a piece of the parameters that no thread has
+// touched yet is a trip to memory, so all are touched at once and before anything has to be waited for.
+template <int CAP>
+__device__ __forceinline__ void copy_record(DecodeLinear* dst, const DecodeBatch<CAP>& bp, int l) {
+  const uint4* src = reinterpret_cast<const uint4*>(&bp.lin[l]);
+  for (int i = threadIdx.x >> 5; i < (int)(sizeof(DecodeLinear) / 16); i += blockDim.x >> 5) {
+    const uint4 v = src[i];
+    if ((threadIdx.x & 31) == 0) reinterpret_cast<uint4*>(dst)[i] = v;
+  }
+}
 
 // Wait with a bound.  Once any wait of the CTA has run out, every later wait returns at once, so that
 // all threads keep the same control flow and the kernel ends (with an error status and undefined output).
@@ -121,527 +144,786 @@ __device__ __forceinline__ void decode_wait(uint32_t bar, uint32_t parity, volat
   }
 }
 
-// grid (slices, M, linears), 256 threads.  Dynamic shared memory: the token's K bf16 values, then two buffers of
-// `prep_rows` / 2 rows of K bf16 values each (router rows first, rows of A_e afterwards).  Whole rows arrive by bulk
-// copies, a round of rows at a time, the next round in flight while one is used, and the dot products run out of
-// shared memory: with plain loads every lane went to memory several times in a row for a long row, and that
-// latency was most of the kernel.
-__global__ void __launch_bounds__(256) k_decode_prep(const __grid_constant__ DecodeBatch bp) {
-  extern __shared__ __align__(128) uint4 xs4[];
-  __shared__ __align__(8) uint64_t pbar[3];   // token; the two row buffers
-  __shared__ float red_f[8];
-  __shared__ int red_i[8];
-  __shared__ float logit_sh[kMaxExperts];
+__device__ __forceinline__ int quant_code(float x, float gamma) { return max(-128, min(127, __float2int_rn(__fmul_rn(x, gamma)))); }
+
+// codes of eight consecutive values, in order, as two words
+__device__ __forceinline__ void quant_codes8(const uint4& v, float gamma, uint32_t (&o)[2]) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  o[0] = o[1] = 0u;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int q0 = quant_code(bf16lo(w[u]), gamma), q1 = quant_code(bf16hi(w[u]), gamma);
+    o[u >> 1] |= ((uint32_t)(q0 & 0xFF) | ((uint32_t)(q1 & 0xFF) << 8)) << (16 * (u & 1));
+  }
+}
+__device__ __forceinline__ double sum_squares(const uint4& v) {
+  const double d0 = bf16lo(v.x), d1 = bf16hi(v.x), d2 = bf16lo(v.y), d3 = bf16hi(v.y);
+  const double d4 = bf16lo(v.z), d5 = bf16hi(v.z), d6 = bf16lo(v.w), d7 = bf16hi(v.w);
+  return ((d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3)) + ((d4 * d4 + d5 * d5) + (d6 * d6 + d7 * d7));
+}
+
+// Element (token m, hidden index j) of the expert product's token-side operand: step j / 32, lane 4 (m % 8) + (j % 32) / 8,
+// 16-bit slot j % 8; hi = bf16(a), lo = bf16(a - hi).
+__device__ __forceinline__ void store_h(const DecodeLinear& L, int m, int j, float a) {
+  const int rsteps = (L.r + 31) >> 5;
+  const __nv_bfloat16 hi = __float2bfloat16_rn(a), lo = __float2bfloat16_rn(a - __bfloat162float(hi));
+  uint16_t* base = reinterpret_cast<uint16_t*>(L.hfrag);
+  const int pos = (((m >> 3) * 2 * rsteps + (j >> 5)) * 32 + (m & 7) * 4 + ((j & 31) >> 3)) * 8 + (j & 7);
+  base[pos] = __bfloat16_as_ushort(hi);
+  base[pos + rsteps * 32 * 8] = __bfloat16_as_ushort(lo);
+}
+
+// grid (8, M, linears), one cluster per token.  Dynamic shared memory: the token's K bf16 values, the router rows of this CTA's
+// experts, the norm's gains.
+template <int CAP>
+__global__ void __cluster_dims__(kPrepCluster, 1, 1) __maxnreg__(80) k_decode_prep(const __grid_constant__ DecodeBatch<CAP> bp) {
+  extern __shared__ __align__(128) uint8_t prep_smem[];
+  __shared__ DecodeLinear L;
+  __shared__ __align__(8) uint64_t wr_bar;
+  __shared__ double red_d[kPrepWarps];
+  __shared__ float red_f[kPrepWarps];
+  __shared__ __align__(16) float logit_sh[kMaxExperts];
+  __shared__ int sum_sh[kPrepCluster][kPrepWarps];
   __shared__ int fail_sh;
-  volatile int* fail = &fail_sh;
-  if (threadIdx.x == 0) {
+  const int m = blockIdx.y, rank = blockIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  copy_record(&L, bp, blockIdx.z);
+  const int off_wr = bp.off_wr, off_gain = bp.off_gain;
+  if (tid == 0) {
     fail_sh = 0;
-    for (int i = 0; i < 3; ++i) mbar_init(smem_u32(&pbar[i]), 1);
+    mbar_init(smem_u32(&wr_bar), 1);
     mbar_fence_init();
   }
-  pdl_launch_dependents();
-  pdl_wait();   // X may come from the previous kernel; the buffers written here may still be read by it
   __syncthreads();
-  const DecodeLinear& L = bp.lin[blockIdx.z];
-  const int m = blockIdx.y, slice = blockIdx.x;
-  if (m >= L.M || slice >= L.slices) return;
+  if (m >= L.M) return;                                        // whole clusters
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   const int K = L.K, E = L.E, r = L.r;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int chunks = K >> 3;
   const uint32_t row_bytes = (uint32_t)K * 2u;
-  const int R = bp.prep_rows >> 1;                             // rows of one buffer (<= 4, one per warp)
-  const uint4* rows4 = xs4 + chunks;
-  const uint32_t rows_s = smem_u32(xs4) + row_bytes;
-  // rounds of up to R rows of a [*, K] bf16 matrix alternate between the two buffers; all threads count them
-  int issued = 0, taken = 0;
-  uint32_t phase0 = 0, phase1 = 0;
-  auto issue = [&](const uint16_t* base, long long row0, int n) {
-    const int b = issued & 1;
-    if (threadIdx.x == 0) {
-      mbar_expect_tx(smem_u32(&pbar[1 + b]), (uint32_t)n * row_bytes);
-      for (int i = 0; i < n; ++i) bulk_load(rows_s + (uint32_t)(b * R + i) * row_bytes, base + (row0 + i) * K, row_bytes, smem_u32(&pbar[1 + b]));
-    }
-    ++issued;
-  };
-  auto take = [&]() {   // waits for the oldest round in flight and returns its buffer's first row
-    const int b = taken & 1;
-    decode_wait(smem_u32(&pbar[1 + b]), b ? phase1 : phase0, fail);
-    if (b) phase1 ^= 1u; else phase0 ^= 1u;
-    ++taken;
-    return rows4 + (size_t)(b * R) * chunks;
-  };
-
-  // the token, and with it the first two rounds of router rows
-  if (threadIdx.x == 0) {
-    mbar_expect_tx(smem_u32(&pbar[0]), row_bytes);
-    bulk_load(smem_u32(xs4), reinterpret_cast<const uint16_t*>(L.X) + (long long)m * K, row_bytes, smem_u32(&pbar[0]));
+  uint4* xs4 = reinterpret_cast<uint4*>(prep_smem);
+  uint4* gain4 = reinterpret_cast<uint4*>(prep_smem + off_gain);
+  const int my_experts = E > 1 && rank < E ? (E - rank + kPrepCluster - 1) / kPrepCluster : 0;   // rank, rank + 8
+  // weights start towards L2 while the previous kernel is still running
+  if (m == 0) {
+    if (tid < my_experts) bulk_prefetch(L.Wr + (long long)(rank + tid * kPrepCluster) * chunks, row_bytes);
+    if (L.norm_w && tid == 32 && rank == 0) bulk_prefetch(L.norm_w, row_bytes);
   }
-  const uint16_t* Wr = reinterpret_cast<const uint16_t*>(L.Wr);
-  const int router_rounds = E > 1 ? (E + R - 1) / R : 0;
-  for (int k = 0; k < min(2, router_rounds); ++k) issue(Wr, k * R, min(R, E - k * R));
-  decode_wait(smem_u32(&pbar[0]), 0, fail);
+  pdl_wait();                // X may come from the previous kernel; the buffers written here may still be read by it
+  pdl_launch_dependents();   // from here on the kernels behind this one may start: what they read early is final
+  if (tid == 0 && my_experts > 0) {
+    mbar_expect_tx(smem_u32(&wr_bar), (uint32_t)my_experts * row_bytes);
+    for (int i = 0; i < my_experts; ++i)
+      bulk_load(smem_u32(prep_smem + off_wr) + (uint32_t)i * row_bytes, L.Wr + (long long)(rank + i * kPrepCluster) * chunks, row_bytes, smem_u32(&wr_bar));
+  }
+
+  // the token (and the norm's gains): all loads of a thread in flight together
+  float amax = 0.f;
+  double ss = 0.0;
+  auto fold_amax = [&](const uint4& v) {
+    amax = fmaxf(amax, fmaxf(fmaxf(fabsf(bf16lo(v.x)), fabsf(bf16hi(v.x))), fmaxf(fabsf(bf16lo(v.y)), fabsf(bf16hi(v.y)))));
+    amax = fmaxf(amax, fmaxf(fmaxf(fabsf(bf16lo(v.z)), fabsf(bf16hi(v.z))), fmaxf(fabsf(bf16lo(v.w)), fabsf(bf16hi(v.w)))));
+  };
+  {
+    const uint4* x4 = L.X + (long long)m * chunks;
+    for (int c0 = tid; c0 < chunks; c0 += 4 * kPrepThreads) {
+      uint4 v[4], g[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const bool in = c0 + u * kPrepThreads < chunks;
+        v[u] = in ? __ldcg(x4 + c0 + u * kPrepThreads) : make_uint4(0u, 0u, 0u, 0u);
+        if (L.norm_w && in) g[u] = __ldcg(L.norm_w + c0 + u * kPrepThreads);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (c0 + u * kPrepThreads < chunks) {
+          xs4[c0 + u * kPrepThreads] = v[u];
+          if (L.norm_w) {
+            gain4[c0 + u * kPrepThreads] = g[u];
+            ss += sum_squares(v[u]);
+          } else {
+            fold_amax(v[u]);
+          }
+        }
+      }
+    }
+  }
   if (L.norm_w) {
     // RMSNorm fused in front of the quantiser (App. A): mean of squares and its reciprocal root in fp64 (thread sums
     // in ascending chunk order, then a fixed tree), the factor rounded once to fp32; the token in shared memory is
     // replaced by bf16(fp32(fp32(x s) w)), which every later step reads.
-    __shared__ double red_d[8];
-    double ss = 0.0;
-    for (int c = threadIdx.x; c < chunks; c += 256) {
-      const uint4 v = xs4[c];
-      const double d0 = bf16lo(v.x), d1 = bf16hi(v.x), d2 = bf16lo(v.y), d3 = bf16hi(v.y);
-      const double d4 = bf16lo(v.z), d5 = bf16hi(v.z), d6 = bf16lo(v.w), d7 = bf16hi(v.w);
-      ss += ((d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3)) + ((d4 * d4 + d5 * d5) + (d6 * d6 + d7 * d7));
-    }
     for (int d = 16; d > 0; d >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, d);
     if (lane == 0) red_d[warp] = ss;
     __syncthreads();
     double tot = 0.0;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) tot += red_d[w];
+    for (int w = 0; w < kPrepWarps; ++w) tot += red_d[w];
     const float s = (float)(1.0 / sqrt(tot / (double)K + (double)L.norm_eps));
-    for (int c = threadIdx.x; c < chunks; c += 256) {
-      const uint4 v = xs4[c], g = __ldg(L.norm_w + c);
-      uint4 o;
-      o.x = pack_bf16x2(__fmul_rn(__fmul_rn(bf16lo(v.x), s), bf16lo(g.x)), __fmul_rn(__fmul_rn(bf16hi(v.x), s), bf16hi(g.x)));
-      o.y = pack_bf16x2(__fmul_rn(__fmul_rn(bf16lo(v.y), s), bf16lo(g.y)), __fmul_rn(__fmul_rn(bf16hi(v.y), s), bf16hi(g.y)));
-      o.z = pack_bf16x2(__fmul_rn(__fmul_rn(bf16lo(v.z), s), bf16lo(g.z)), __fmul_rn(__fmul_rn(bf16hi(v.z), s), bf16hi(g.z)));
-      o.w = pack_bf16x2(__fmul_rn(__fmul_rn(bf16lo(v.w), s), bf16lo(g.w)), __fmul_rn(__fmul_rn(bf16hi(v.w), s), bf16hi(g.w)));
-      xs4[c] = o;
+    for (int c = tid; c < chunks; c += kPrepThreads) {   // each thread reads back the chunks it wrote itself
+      const uint4 v = rms_apply(xs4[c], s, gain4[c]);
+      xs4[c] = v;
+      fold_amax(v);
     }
-    // each thread reads back only the chunks it wrote itself in the pass below; the barrier after it publishes them
-  }
-  float amax = 0.f;
-  for (int c = threadIdx.x; c < chunks; c += 256) {
-    const uint4 v = xs4[c];
-    amax = fmaxf(amax, fmaxf(fmaxf(fabsf(bf16lo(v.x)), fabsf(bf16hi(v.x))), fmaxf(fabsf(bf16lo(v.y)), fabsf(bf16hi(v.y)))));
-    amax = fmaxf(amax, fmaxf(fmaxf(fabsf(bf16lo(v.z)), fabsf(bf16hi(v.z))), fmaxf(fabsf(bf16lo(v.w)), fabsf(bf16hi(v.w)))));
   }
   for (int d = 16; d > 0; d >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, d));
   if (lane == 0) red_f[warp] = amax;
-  __syncthreads();
+  __syncthreads();                                             // the token and the maxima are visible
   amax = red_f[0];
 #pragma unroll
-  for (int w = 1; w < 8; ++w) amax = fmaxf(amax, red_f[w]);
+  for (int w = 1; w < kPrepWarps; ++w) amax = fmaxf(amax, red_f[w]);
   const float gamma = __fdiv_rn(kActQmax, fmaxf(amax, kActAmaxFloor));
 
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");  // every CTA of the cluster is running
   // router: the same pinned fp32 order as the training path (lane j owns the chunks c = j mod 32, ascending,
-  // fused multiply-add; butterfly 16, 8, 4, 2, 1), one warp per expert of the round
-  int best = 0;
-  float gate = 1.0f;
-  if (E > 1) {
-    for (int k = 0; k < router_rounds; ++k) {
-      const int n = min(R, E - k * R);
-      const uint4* buf = take();
-      if (warp < n) {
-        float acc = 0.f;
-        const uint4* wrow = buf + (size_t)warp * chunks;
-        for (int c = lane; c < chunks; c += 32) {
-          const uint4 xv = xs4[c], wv = wrow[c];
-          acc = fmaf(bf16lo(xv.x), bf16lo(wv.x), acc); acc = fmaf(bf16hi(xv.x), bf16hi(wv.x), acc);
-          acc = fmaf(bf16lo(xv.y), bf16lo(wv.y), acc); acc = fmaf(bf16hi(xv.y), bf16hi(wv.y), acc);
-          acc = fmaf(bf16lo(xv.z), bf16lo(wv.z), acc); acc = fmaf(bf16hi(xv.z), bf16hi(wv.z), acc);
-          acc = fmaf(bf16lo(xv.w), bf16lo(wv.w), acc); acc = fmaf(bf16hi(xv.w), bf16hi(wv.w), acc);
-        }
-        for (int d = 16; d > 0; d >>= 1) acc = acc + __shfl_xor_sync(0xffffffffu, acc, d);
-        if (lane == 0) logit_sh[k * R + warp] = acc;
-      }
-      __syncthreads();                                         // this buffer is free, its logits are visible
-      if (k + 2 < router_rounds) issue(Wr, (k + 2) * R, min(R, E - (k + 2) * R));
+  // fused multiply-add; butterfly 16, 8, 4, 2, 1), one warp per expert of this CTA; the cluster exchanges the logits
+  if (warp < my_experts) {
+    decode_wait(smem_u32(&wr_bar), 0, &fail_sh);
+    const uint4* wrow = reinterpret_cast<const uint4*>(prep_smem + off_wr) + (size_t)warp * chunks;
+    float acc = 0.f;
+    auto fold = [&](const uint4& xv, const uint4& wv) {
+      acc = fmaf(bf16lo(xv.x), bf16lo(wv.x), acc); acc = fmaf(bf16hi(xv.x), bf16hi(wv.x), acc);
+      acc = fmaf(bf16lo(xv.y), bf16lo(wv.y), acc); acc = fmaf(bf16hi(xv.y), bf16hi(wv.y), acc);
+      acc = fmaf(bf16lo(xv.z), bf16lo(wv.z), acc); acc = fmaf(bf16hi(xv.z), bf16hi(wv.z), acc);
+      acc = fmaf(bf16lo(xv.w), bf16lo(wv.w), acc); acc = fmaf(bf16hi(xv.w), bf16hi(wv.w), acc);
+    };
+    int c = lane;
+    for (; c + 96 < chunks; c += 128) {
+      uint4 wv[4], xv[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) { wv[u] = wrow[c + 32 * u]; xv[u] = xs4[c + 32 * u]; }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) fold(xv[u], wv[u]);
     }
-    float lmax = logit_sh[0];
-    for (int e = 1; e < E; ++e)
-      if (logit_sh[e] > lmax) { lmax = logit_sh[e]; best = e; }
-    float den = 0.f, pbest = 0.f;
-    for (int e = 0; e < E; ++e) {
-      const float pe = expf(logit_sh[e] - lmax);
-      den += pe;
-      if (e == best) pbest = pe;
-    }
-    gate = pbest * (1.0f / den);
-  }
-  // the first two rounds of this slice's rows of A_e are on their way while slice 0 quantises the token
-  const int j0 = slice * L.rows_per_slice, j1 = min(r, j0 + L.rows_per_slice);
-  const int h_rounds = (r > 0 && j0 < j1) ? (j1 - j0 + R - 1) / R : 0;
-  const long long arow0 = (long long)best * r + j0;
-  for (int k = 0; k < min(2, h_rounds); ++k) issue(L.A, arow0 + k * R, min(R, j1 - j0 - k * R));
-
-  if (slice == 0) {
-    // Eq. 7-9 for this token; every thread turns pairs of weight words (64 values of k) into fragment order
-    const int npairs = (K + 63) >> 6;
+    for (; c < chunks; c += 32) fold(xs4[c], wrow[c]);
+    for (int d = 16; d > 0; d >>= 1) acc = acc + __shfl_xor_sync(0xffffffffu, acc, d);
+    if (lane == 0)
+      asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_map(smem_u32(&logit_sh[rank + warp * kPrepCluster]), 0)), "f"(acc) : "memory");
+  } else {
+    // meanwhile the other warps: this CTA's eighth of the token's codes (Eq. 7-9), in fragment order -- an item is one 16-byte
+    // piece (chunk and half, quad index) -- and, for the INT8 branch, in natural order
+    const int nhalves = 2 * ((K + 127) >> 7), first = my_experts * 32, nthr = kPrepThreads - first;
     const int group = m >> 3, g = m & 7, mg = min(8, L.M - 8 * group);
+    const int i_lo = nhalves * 4 * rank / kPrepCluster, i_hi = nhalves * 4 * (rank + 1) / kPrepCluster;
+    uint4* dst = L.qfrag + (long long)group * nhalves * 32 + g * 4;
+    const uint16_t* xs = reinterpret_cast<const uint16_t*>(prep_smem);
     int rowsum = 0;
-    for (int ip = threadIdx.x; ip < npairs; ip += 256) {
-      int qv[64];
+    for (int i = i_lo + tid - first; i < i_hi; i += nthr) {
+      const int ip = i >> 2, c = i & 3;
+      uint32_t w[4];
 #pragma unroll
-      for (int ch = 0; ch < 8; ++ch) {
-        const bool in = 8 * ip + ch < chunks;
-        const uint4 v = in ? xs4[8 * ip + ch] : make_uint4(0u, 0u, 0u, 0u);
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+      for (int reg = 0; reg < 4; ++reg) {
+        const int base = 128 * (ip >> 1) + 32 * c + 4 * (ip & 1) + reg;
+        w[reg] = 0u;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int q0 = in ? max(-128, min(127, __float2int_rn(__fmul_rn(bf16lo(w[u]), gamma)))) : 0;
-          const int q1 = in ? max(-128, min(127, __float2int_rn(__fmul_rn(bf16hi(w[u]), gamma)))) : 0;
-          qv[8 * ch + 2 * u] = q0;
-          qv[8 * ch + 2 * u + 1] = q1;
-          rowsum += q0 + q1;
+        for (int j = 0; j < 4; ++j) {
+          const int q = base + 8 * j < K ? quant_code(bf16_bits_to_float(xs[base + 8 * j]), gamma) : 0;
+          w[reg] |= (uint32_t)(q & 0xFF) << (8 * j);
+          rowsum += q;
         }
       }
-      uint4 out[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        uint32_t w[4];
-#pragma unroll
-        for (int reg = 0; reg < 4; ++reg) {
-          const int base = (reg & 1) * 32 + c + (reg >> 1) * 4;
-          w[reg] = (qv[base] & 0xFF) | ((qv[base + 8] & 0xFF) << 8) | ((qv[base + 16] & 0xFF) << 16) | ((qv[base + 24] & 0xFF) << 24);
-        }
-        out[c] = make_uint4(w[0], w[1], w[2], w[3]);
-      }
-      uint4* dst = L.qfrag + ((long long)group * npairs * 32 + (long long)(ip * mg + g) * 4);
-#pragma unroll
-      for (int c = 0; c < 4; ++c) dst[c] = out[c];
+      dst[(long long)ip * mg * 4 + c] = make_uint4(w[0], w[1], w[2], w[3]);
     }
     for (int d = 16; d > 0; d >>= 1) rowsum += __shfl_xor_sync(0xffffffffu, rowsum, d);
-    if (lane == 0) red_i[warp] = rowsum;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int tot = 0;
-      for (int w = 0; w < 8; ++w) tot += red_i[w];
-      L.info[m] = DecodeTokInfo{best, gate, gamma, tot};
+    if (lane == 0)
+      asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cluster_map(smem_u32(&sum_sh[rank][warp]), 0)), "r"(rowsum) : "memory");
+    if (L.A8) {
+      const int c_lo = chunks * rank / kPrepCluster, c_hi = chunks * (rank + 1) / kPrepCluster;
+      for (int c = c_lo + tid - first; c < c_hi; c += nthr) {
+        uint32_t o[2];
+        quant_codes8(xs4[c], gamma, o);
+        reinterpret_cast<uint2*>(L.xn)[(long long)m * chunks + c] = make_uint2(o[0], o[1]);
+      }
+    } else if (L.norm_w && r > 0) {
+      const int c_lo = chunks * rank / kPrepCluster, c_hi = chunks * (rank + 1) / kPrepCluster;
+      for (int c = c_lo + tid - first; c < c_hi; c += nthr) reinterpret_cast<uint4*>(L.xn)[(long long)m * chunks + c] = xs4[c];
     }
   }
-
-  // this slice of h = A_e x (fp32 accumulation over the bf16 operands), one warp per row of the round
-  for (int k = 0; k < h_rounds; ++k) {
-    const int n = min(R, j1 - j0 - k * R);
-    const uint4* buf = take();
-    if (warp < n) {
-      const int j = j0 + k * R + warp;
-      const uint4* arow = buf + (size_t)warp * chunks;
-      float a0 = 0.f, a1 = 0.f;
-      for (int c = lane; c < chunks; c += 32) {
-        const uint4 xv = xs4[c], wv = arow[c];
-        a0 = fmaf(bf16lo(xv.x), bf16lo(wv.x), a0); a1 = fmaf(bf16hi(xv.x), bf16hi(wv.x), a1);
-        a0 = fmaf(bf16lo(xv.y), bf16lo(wv.y), a0); a1 = fmaf(bf16hi(xv.y), bf16hi(wv.y), a1);
-        a0 = fmaf(bf16lo(xv.z), bf16lo(wv.z), a0); a1 = fmaf(bf16hi(xv.z), bf16hi(wv.z), a1);
-        a0 = fmaf(bf16lo(xv.w), bf16lo(wv.w), a0); a1 = fmaf(bf16hi(xv.w), bf16hi(wv.w), a1);
-      }
-      float a = a0 + a1;
-      for (int d = 16; d > 0; d >>= 1) a += __shfl_xor_sync(0xffffffffu, a, d);
-      if (lane == 0) {
-        // element (token m, hidden index j) of the expert product's token-side operand: step j / 32, lane
-        // 4 (m % 8) + (j % 32) / 8, 16-bit slot j % 8; hi = bf16(a), lo = bf16(a - hi)
-        const int rsteps = (r + 31) >> 5;
-        const __nv_bfloat16 hi = __float2bfloat16_rn(a), lo = __float2bfloat16_rn(a - __bfloat162float(hi));
-        uint16_t* base = reinterpret_cast<uint16_t*>(L.hfrag);
-        const long long pos = ((long long)((m >> 3) * 2 * rsteps + (j >> 5)) * 32 + (m & 7) * 4 + ((j & 31) >> 3)) * 8 + (j & 7);
-        base[pos] = __bfloat16_as_ushort(hi);
-        base[pos + (long long)rsteps * 32 * 8] = __bfloat16_as_ushort(lo);
-      }
+  cluster_sync_all();
+  if (rank == 0 && warp == 0) {
+    // lane e: expert e (lowest index on ties); the lanes also add up the code sums of the cluster's warps
+    int best = 0;
+    float gate = 1.0f;
+    if (E > 1) {
+      const float lg = lane < E ? logit_sh[lane] : -INFINITY;
+      float lmax = lg;
+      for (int d = 16; d > 0; d >>= 1) lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, d));
+      best = __ffs(__ballot_sync(0xffffffffu, lane < E && lg == lmax)) - 1;
+      if (best < 0) best = 0;                                  // no logit is a number
+      const float pe = lane < E ? expf(lg - lmax) : 0.f;
+      float den = pe;
+      for (int d = 16; d > 0; d >>= 1) den += __shfl_xor_sync(0xffffffffu, den, d);
+      gate = __shfl_sync(0xffffffffu, pe, best) * (1.0f / den);
     }
-    if (k + 2 < h_rounds) {
-      __syncthreads();                                         // this buffer is free
-      issue(L.A, arow0 + (k + 2) * R, min(R, j1 - j0 - (k + 2) * R));
+    int tot = 0;
+#pragma unroll
+    for (int i = 0; i < kPrepCluster * kPrepWarps / 32; ++i) {
+      const int k = i * 32 + lane, rk = k / kPrepWarps, w = k % kPrepWarps;
+      const int routed = E > 1 && rk < E ? (E - rk + kPrepCluster - 1) / kPrepCluster : 0;
+      if (w >= routed) tot += sum_sh[rk][w];
     }
+    for (int d = 16; d > 0; d >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, d);
+    if (lane == 0) L.info[m] = DecodeTokInfo{best, gate, gamma, tot};
   }
 }
 
-// Range of output features of CTA b: whole groups of 8, spread evenly (no division on the device).
-__device__ __forceinline__ void decode_range(int b, const DecodeLinear& L, int& n_lo, int& n_hi) {
-  n_lo = (b * L.grp_base + min(b, L.grp_rem)) << 3;
-  n_hi = n_lo + ((L.grp_base + (b < L.grp_rem ? 1 : 0)) << 3);
+// ---------------------------------------------------------------------------
+// k_decode_hidden: h = A_e x, expert by expert, so that a row of A_e is read once for all tokens of its expert (eight experts,
+// sixteen tokens: about six experts in use).  A cluster of one, two or four CTAs per (linear, k-th expert in use, 16 hidden
+// rows), as many as make about one CTA per SM: k_decode_main's has to fit beside it.  K is cut into 32 shares whatever the
+// cluster's size; a warp contracts over its shares one after the other on mma.sync (bf16, or s8 for the INT8 branch), rows of A
+// as the 16-row operand straight from global memory (a lane takes 16 consecutive bytes: the order of the contraction index is
+// the same on both sides), the expert's tokens as columns; the sums meet in the first CTA's shared memory and are added in
+// the order of the shares.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void mma_s8s8(int (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-constexpr int kDecodeMetaBytes = 256;   // token info at the start of a slot
-
-// Experts used by the tokens [8 G, 8 G + 8) as a bit mask; producer and consumers walk it in ascending order.
-__device__ __forceinline__ unsigned decode_expert_mask(const DecodeTokInfo* tok, int M, int G) {
-  unsigned mask = 0u;
-  for (int t = 8 * G; t < min(M, 8 * G + 8); ++t) mask |= 1u << (tok[t].expert & 15);
-  return mask;
+// Steps [st_lo, st_hi) of 64 bytes per row.  Rows of `pitch` 16-byte pieces; r0, r1, x0, x1 point at this lane's piece of step 0
+// (x0, x1: its columns' tokens, null for columns without one).
+template <bool INT8>
+__device__ __forceinline__ void hidden_walk(const uint4* r0, const uint4* r1, const uint4* x0, const uint4* x1, bool two, int st_lo, int st_hi, int last, int c,
+                                            uint32_t (&z0)[4], uint32_t (&z1)[4]) {
+  constexpr int U = 4;                                         // steps in flight
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  auto mma = [](uint32_t (&z)[4], const uint4& a, const uint4& b, const uint4& v) {
+    if (INT8) {
+      int (&d)[4] = reinterpret_cast<int(&)[4]>(z);
+      mma_s8s8(d, a.x, b.x, a.y, b.y, v.x, v.y);
+      mma_s8s8(d, a.z, b.z, a.w, b.w, v.z, v.w);
+    } else {
+      float (&d)[4] = reinterpret_cast<float(&)[4]>(z);
+      mma_bf16(d, a.x, b.x, a.y, b.y, v.x, v.y);
+      mma_bf16(d, a.z, b.z, a.w, b.w, v.z, v.w);
+    }
+  };
+  for (int st = st_lo; st < st_hi; st += U) {
+    uint4 w0[U], w1[U], v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const bool in = st + u < st_hi && (st + u) * 4 + c < last;   // a row's last step may be half a step (INT8, K % 64 = 32)
+      w0[u] = in ? __ldg(r0 + (st + u) * 4) : zero;
+      w1[u] = in ? __ldg(r1 + (st + u) * 4) : zero;
+      v[u] = in && x0 ? __ldcg(x0 + (st + u) * 4) : zero;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) mma(z0, w0[u], w1[u], v[u]);
+    if (two) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) v[u] = st + u < st_hi && (st + u) * 4 + c < last && x1 ? __ldcg(x1 + (st + u) * 4) : zero;
+#pragma unroll
+      for (int u = 0; u < U; ++u) mma(z1, w0[u], w1[u], v[u]);
+    }
+  }
 }
 
-__global__ void __launch_bounds__(kDecodeMainThreads) k_decode_main(const __grid_constant__ DecodeBatch bp) {
+template <int CAP>
+__global__ void __maxnreg__(80) k_decode_hidden(const __grid_constant__ DecodeBatch<CAP> bp) {
+  __shared__ DecodeLinear L;
+  __shared__ uint32_t red[kHiddenSplit][16][17];               // used in the cluster's first CTA
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int cs = bp.hidden_cluster, rank = (int)cluster_rank(), group = (int)blockIdx.x / cs;
+  int l = 0;
+  for (int i = 1; i < bp.n; ++i)
+    if (bp.lin[i].r > 0 && group >= bp.lin[i].hidden0) l = i;
+  while (bp.lin[l].r <= 0) ++l;
+  copy_record(&L, bp, l);
+  __syncthreads();
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  const int K = L.K, r = L.r, M = L.M;
+  const bool int8 = L.A8 != nullptr;
+  const int pitch = int8 ? K >> 4 : K >> 3, steps = (pitch + 3) >> 2;
+  const int tiles = (r + 15) >> 4, local = group - L.hidden0;
+  const int slot = local / tiles, tile = local - slot * tiles, j0 = tile * 16;   // the slot-th expert in use
+  const int g = lane >> 2, c = lane & 3;
+  const long long row0 = (long long)j0 * pitch, expert_pitch = (long long)r * pitch;
+  const uint4* base = int8 ? reinterpret_cast<const uint4*>(L.A8) : reinterpret_cast<const uint4*>(L.A);
+  // with as many tokens as experts most experts are in use: the rows start towards L2 before it is known which
+  if (M >= L.E) {
+    const uint32_t bytes = (uint32_t)min(16, r - j0) * (uint32_t)pitch * 16u;
+    for (uint32_t at = (rank * kHiddenThreads + tid) * 4096u; at < bytes; at += cs * kHiddenThreads * 4096u)
+      bulk_prefetch(reinterpret_cast<const uint8_t*>(base + slot * expert_pitch + row0) + at, min(4096u, bytes - at));
+  }
+  pdl_wait();
+  pdl_launch_dependents();   // k_decode_main may read k_decode_prep's results from here on
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");  // every CTA of the cluster is running
+  const int my_e = lane < M ? __ldcg(&L.info[lane].expert) : -1;
+  unsigned used = __reduce_or_sync(0xffffffffu, my_e >= 0 ? 1u << (my_e & 15) : 0u);
+  for (int k = 0; k < slot; ++k) used &= used - 1;
+  if (used == 0u) return;                                      // the whole cluster: fewer experts are in use
+  const int e = __ffs(used) - 1;
+  const unsigned mine = __ballot_sync(0xffffffffu, my_e == e);
+  const int cnt = __popc(mine);
+  // up to sixteen tokens: columns 0-7 and 8-15
+  unsigned left = mine;
+  for (int k = 0; k < g; ++k) left &= left - 1;
+  const int t0 = g < cnt ? __ffs(left) - 1 : -1;
+  for (int k = 0; k < 8; ++k) left &= left - 1;
+  const int t1 = g + 8 < cnt ? __ffs(left) - 1 : -1;
+  const uint4* x = (int8 || L.norm_w ? reinterpret_cast<const uint4*>(L.xn) : L.X) + c;
+  const uint4* x0 = t0 >= 0 ? x + (long long)t0 * pitch : nullptr;
+  const uint4* x1 = t1 >= 0 ? x + (long long)t1 * pitch : nullptr;
+  const uint4* rows = base + e * expert_pitch + row0 + c;
+  const uint4 *r0 = rows + (long long)g * pitch, *r1 = rows + (long long)(j0 + g + 8 < r ? g + 8 : g) * pitch;
+  // the rows of B_e that k_decode_main reads next start towards L2 (512-byte pieces)
+  if (!int8) {
+    const int total = (L.N >> 5) * (r >> 3), per = (total + tiles - 1) / tiles, lo = per * tile, hi = min(total, lo + per);
+    const uint8_t* b = reinterpret_cast<const uint8_t*>(L.B) + (long long)e * total * 512;
+    for (int at = lo + (rank * kHiddenThreads + tid) * 8; at < hi; at += cs * kHiddenThreads * 8) bulk_prefetch(b + (long long)at * 512, (uint32_t)min(8, hi - at) * 512u);
+  }
+  const bool two = cnt > 8;
+  for (int v = rank * kHiddenWarps + warp; v < kHiddenSplit; v += cs * kHiddenWarps) {
+    uint32_t z0[4] = {0u, 0u, 0u, 0u}, z1[4] = {0u, 0u, 0u, 0u};   // fp32 or int32 sums; zero is the same word
+    const int st_lo = steps * v / kHiddenSplit, st_hi = steps * (v + 1) / kHiddenSplit;
+    if (int8) hidden_walk<true>(r0, r1, x0, x1, two, st_lo, st_hi, pitch, c, z0, z1);
+    else hidden_walk<false>(r0, r1, x0, x1, two, st_lo, st_hi, pitch, c, z0, z1);
+    const uint32_t to = cluster_map(smem_u32(&red[v][0][0]), 0);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint32_t at = to + 4u * ((g + (u >> 1) * 8) * 17 + 2 * c + (u & 1));
+      asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(z0[u]) : "memory");
+      if (two) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(at + 32u), "r"(z1[u]) : "memory");
+    }
+  }
+  cluster_sync_all();
+  if (rank == 0) {
+    const int row = tid & 15, col = tid >> 4;
+    if (col < cnt && j0 + row < r) {
+      unsigned m = mine;
+      for (int k = 0; k < col; ++k) m &= m - 1;
+      const int t = __ffs(m) - 1;
+      if (int8) {
+        int a = 0;
+#pragma unroll
+        for (int w = 0; w < kHiddenSplit; ++w) a += (int)red[w][row][col];
+        L.h_int[(long long)t * r + j0 + row] = a;
+      } else {
+        float a = 0.f;
+#pragma unroll
+        for (int w = 0; w < kHiddenSplit; ++w) a += __uint_as_float(red[w][row][col]);
+        store_h(L, t, j0 + row, a);
+      }
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// k_decode_main.  A CTA walks its share of the units in passes of up to kMaxPassUnits units of one linear.  The sign bits
+// of a pass sit in shared memory as [chunk of 128 k][feature of the pass][16 bytes]; with the streaming layout they arrive
+// by bulk copies, one pass ahead, otherwise through registers.  1-bit product: a warp works on two tiles of 16 features and a
+// slice of the contraction; the slices' sums (integers) are added up in shared memory.  Expert product: the rows of B_e of
+// one tile are one contiguous piece, fetched by a bulk copy over the sign bits (used by then); a warp takes whole (expert,
+// tile) items.
+// ---------------------------------------------------------------------------
+struct DecodePass { int l, unit, nu; };   // linear; first unit within it; units (0: no pass)
+
+// Chunks [c_lo, c_hi) of the pass's sign bits, tiles of 16 features at row0 and (T = 2) row0 + 16, against the codes; q: fragments
+// whose first chunk is q_c0, q_chunks of them per group of eight tokens.  G: groups of eight tokens.  Shared memory bounds this
+// loop (a 16-byte load of a warp takes four of the cycles the SM has for all its warps, however few different bytes it reads):
+// hence one weight word per lane and two tiles per set of codes.
+template <int G, int T>
+__device__ __forceinline__ void main_bits(const uint32_t* bits_s, int rows, int row0, const uint4* q, int q_c0, int q_chunks, int M, int c_lo, int c_hi, int lane,
+                                          int (&a1)[T][G][4], int (&a16)[T][G][4]) {
+  const int g = lane >> 2, c = lane & 3;
+  const uint32_t* w = bits_s + ((size_t)c_lo * rows + row0 + g) * 4 + c;
+  const int mg0 = min(8, M), mg1 = M - 8;
+  const uint4* q0 = q + (size_t)(c_lo - q_c0) * 2 * mg0 * 4 + min(g, mg0 - 1) * 4 + c;
+  const uint4* q1 = G > 1 ? q + (size_t)q_chunks * 64 + (size_t)(c_lo - q_c0) * 2 * mg1 * 4 + min(g, mg1 - 1) * 4 + c : q;
+#pragma unroll 2
+  for (int ch = c_lo; ch < c_hi; ++ch) {
+    uint32_t u[T], v[T];
+#pragma unroll
+    for (int t = 0; t < T; ++t) { u[t] = w[t * 64]; v[t] = w[t * 64 + 32]; }
+    w += rows * 4;
+    uint4 qq[G][2];
+    qq[0][0] = q0[0]; qq[0][1] = q0[mg0 * 4];
+    q0 += mg0 * 8;
+    if (G > 1) { qq[G - 1][0] = q1[0]; qq[G - 1][1] = q1[mg1 * 4]; q1 += mg1 * 8; }
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+      uint32_t m1[4][2], m16[4][2];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const uint32_t x = u[t] >> b, y = v[t] >> b;
+        m1[b][0] = x & 0x01010101u; m1[b][1] = y & 0x01010101u;
+        m16[b][0] = x & 0x10101010u; m16[b][1] = y & 0x10101010u;
+      }
+      const uint32_t A0[4] = {m1[0][0], m1[0][1], m1[1][0], m1[1][1]}, A1[4] = {m1[2][0], m1[2][1], m1[3][0], m1[3][1]};
+      const uint32_t B0[4] = {m16[0][0], m16[0][1], m16[1][0], m16[1][1]}, B1[4] = {m16[2][0], m16[2][1], m16[3][0], m16[3][1]};
+#pragma unroll
+      for (int G_ = 0; G_ < G; ++G_) {
+        mma_u8s8(a1[t][G_], A0, qq[G_][0].x, qq[G_][0].y);
+        mma_u8s8(a16[t][G_], B0, qq[G_][1].x, qq[G_][1].y);
+        mma_u8s8(a1[t][G_], A1, qq[G_][0].z, qq[G_][0].w);
+        mma_u8s8(a16[t][G_], B1, qq[G_][1].z, qq[G_][1].w);
+      }
+    }
+  }
+}
+
+// One (expert, tile) item of the expert product: b_s = the expert's rows of the tile (16 rows of r values), order[0 .. cnt) =
+// its tokens.  The columns of the product are those tokens; up to four of them sit beside one another with the leading halves of
+// h in columns 0-3 and the trailing ones in 4-7, more take two products per step.  A token has one expert, so its sums go
+// straight to out[token][16 features].
+__device__ __forceinline__ void main_expert(const uint4* b_s, int r, const uint8_t* order, int cnt, const uint4* h_s, int lane, float* out) {
+  const int g = lane >> 2, c = lane & 3;
+  const int steps = (r + 31) >> 5, r8 = r >> 3;
+  const bool packed = cnt <= 4;
+  const uint4 *r0 = b_s + g * r8 + c, *r1 = b_s + (g + 8) * r8 + c;
+  for (int first = 0; first < cnt; first += 8) {
+    const int n = min(8, cnt - first), col = packed ? g & 3 : g;
+    const bool in = col < n;
+    // h of token t, plane: piece ((t / 8) * 2 + plane) * steps * 32 + step * 32 + 4 (t % 8) + c
+    const int t = in ? order[first + col] : 0;
+    const uint4* h0 = h_s + (((t >> 3) * 2 + (packed ? g >> 2 : 0)) * steps) * 32 + 4 * (t & 7) + c;
+    const uint4* h1 = h0 + steps * 32;
+    float z0[4] = {0.f, 0.f, 0.f, 0.f}, z1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+    for (int st = 0; st < steps; ++st) {
+      uint4 w0 = make_uint4(0u, 0u, 0u, 0u), w1 = w0, hh = w0, hl = w0;
+      if (4 * st + c < r8) {
+        w0 = r0[4 * st]; w1 = r1[4 * st];
+        if (in) { hh = h0[st * 32]; if (!packed) hl = h1[st * 32]; }
+      }
+      mma_bf16(z0, w0.x, w1.x, w0.y, w1.y, hh.x, hh.y);
+      mma_bf16(z1, w0.z, w1.z, w0.w, w1.w, hh.z, hh.w);
+      if (!packed) {
+        mma_bf16(z0, w0.x, w1.x, w0.y, w1.y, hl.x, hl.y);
+        mma_bf16(z1, w0.z, w1.z, w0.w, w1.w, hl.z, hl.w);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {                              // columns 2 c and 2 c + 1; features g and g + 8
+      float v0 = z0[u] + z1[u], v1 = z0[u + 2] + z1[u + 2];
+      if (packed) { v0 += __shfl_xor_sync(0xffffffffu, v0, 2); v1 += __shfl_xor_sync(0xffffffffu, v1, 2); }
+      if (2 * c + u < n) {
+        float* o = out + order[first + 2 * c + u] * 16 + g;
+        o[0] = v0; o[8] = v1;
+      }
+    }
+  }
+}
+
+// G: groups of eight tokens the launch's linears have at most; a linear of a single group runs the one-group code
+template <int CAP, int G>
+__global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatch<CAP> bp) {
   extern __shared__ __align__(128) uint8_t smem[];
-  // barriers: token info; slot, q and expert-row rings, a full/empty pair per buffer
-  __shared__ __align__(8) uint64_t bars[1 + 2 * kDecodeMaxSlots + 2 * kDecodeMaxQ + 2 * kDecodeMaxRing];
+  __shared__ DecodeLinear lin_sh[2];       // records of the current linear and the next one (linear l in slot l & 1)
+  __shared__ __align__(8) uint64_t bars[2 + kMaxRows];     // sign bits (two buffers), expert rows
+  __shared__ DecodeTokInfo tok[kDecodeMaxTokens];
+  __shared__ float gh_sh[kDecodeMaxTokens], deq_sh[kDecodeMaxTokens];
+  // the linear's experts in use, in ascending order: index, first token in `order_sh`, number of tokens
+  __shared__ int used_sh, expert_sh[kDecodeMaxTokens], first_sh[kDecodeMaxTokens], count_sh[kDecodeMaxTokens];
+  __shared__ uint8_t order_sh[kDecodeMaxTokens];
+  __shared__ float be_sh[kMaxPassUnits * kUnit], al_sh[kMaxPassUnits * kUnit];
   __shared__ int fail_sh;
-  volatile int* fail = &fail_sh;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t bar0 = smem_u32(&bars[0]);
-  const uint32_t info_full = bar0;
-  auto slot_full = [&](int s) { return bar0 + 8u * (1 + s); };
-  auto slot_empty = [&](int s) { return bar0 + 8u * (1 + kDecodeMaxSlots + s); };
-  auto q_full = [&](int i) { return bar0 + 8u * (1 + 2 * kDecodeMaxSlots + i); };
-  auto q_empty = [&](int i) { return bar0 + 8u * (1 + 2 * kDecodeMaxSlots + kDecodeMaxQ + i); };
-  auto ring_full = [&](int i) { return bar0 + 8u * (1 + 2 * kDecodeMaxSlots + 2 * kDecodeMaxQ + i); };
-  auto ring_empty = [&](int i) { return bar0 + 8u * (1 + 2 * kDecodeMaxSlots + 2 * kDecodeMaxQ + kDecodeMaxRing + i); };
-  if (threadIdx.x == 0) {
-    fail_sh = 0;
-    mbar_init(info_full, 1);
-    for (int s = 0; s < bp.nslot; ++s) { mbar_init(slot_full(s), 1); mbar_init(slot_empty(s), bp.nwarps); }
-    for (int s = 0; s < bp.nq; ++s) { mbar_init(q_full(s), 1); mbar_init(q_empty(s), bp.nwarps); }
-    for (int s = 0; s < bp.nring; ++s) { mbar_init(ring_full(s), 1); mbar_init(ring_empty(s), bp.nwarps); }
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int u_lo = (int)((long long)bp.units * blockIdx.x / gridDim.x), u_hi = (int)((long long)bp.units * (blockIdx.x + 1) / gridDim.x);
+  int l_at = 0;
+  while (bp.unit0[l_at + 1] <= u_lo) ++l_at;
+  copy_record(&lin_sh[l_at & 1], bp, l_at);
+  if (l_at + 1 < bp.n && bp.unit0[l_at + 1] < u_hi) copy_record(&lin_sh[(l_at + 1) & 1], bp, l_at + 1);
+  const int nbuf = bp.nbuf, buf_bytes = bp.buf_bytes, q_chunks = bp.q_chunks, MT = bp.red_tokens, off_h = bp.off_h;
+  if (tid == 0) fail_sh = 0;
+  if (tid < 2 + kMaxRows) {
+    mbar_init(smem_u32(&bars[tid]), 1);
     mbar_fence_init();
   }
-  pdl_launch_dependents();
   __syncthreads();
-  if (warp != bp.nwarps) pdl_wait();   // the producer waits later: weights do not depend on the previous kernel
-
-  // token info of every linear of the batch sits at the start; a slot holds, for one linear, the sign bits
-  // of this CTA's features | the h fragments (both groups)
-  auto info_ptr = [&](int l) { return reinterpret_cast<const DecodeTokInfo*>(smem + l * kDecodeMetaBytes); };
-  auto slot_ptr = [&](int s) { return smem + bp.off_slots + (size_t)s * bp.slot_bytes; };
+  pdl_launch_dependents();
+  // the pass that begins at launch-wide unit u, known to belong to linear l or a later one
+  auto pass_at = [&](int u, int l) {
+    DecodePass p{l, 0, 0};
+    if (u >= u_hi) return p;
+    while (bp.unit0[p.l + 1] <= u) ++p.l;
+    const DecodeLinear& L = lin_sh[p.l & 1];
+    const int cap = max(1, min(kMaxPassUnits, buf_bytes / (256 * ((L.K + 127) >> 7))));
+    const int rem = min(u_hi, bp.unit0[p.l + 1]) - u, npass = (rem + cap - 1) / cap;
+    p.unit = u - bp.unit0[p.l];
+    p.nu = (rem + npass - 1) / npass;
+    return p;
+  };
+  // bulk copies of a pass's sign bits, issued by all warps; a pass is one or two runs within 128-feature groups, one copy per
+  // chunk and run
+  auto fetch_bits = [&](const DecodePass& p, int b) {
+    if (p.nu == 0) return;
+    const DecodeLinear& L = lin_sh[p.l & 1];
+    if (!L.bits_il) return;
+    const int C = (L.K + 127) >> 7;
+    const uint32_t dst = smem_u32(smem) + (uint32_t)b * buf_bytes, bar = smem_u32(&bars[b]);
+    if (tid == 0) mbar_expect_tx(bar, (uint32_t)p.nu * 256u * (uint32_t)C);   // (copies may land before: the phase completes when both agree)
+    for (int done = 0; done < p.nu;) {
+      const int unit = p.unit + done, run = min(p.nu - done, 8 - (unit & 7));
+      const uint4* src = L.bits_il + (long long)(unit >> 3) * C * 128 + (unit & 7) * 16;
+      for (int c = warp + kMainWarps * lane; c < C; c += 32 * kMainWarps)
+        bulk_load(dst + ((uint32_t)c * p.nu + done) * 256u, src + (long long)c * 128, (uint32_t)run * 256u, bar);
+      done += run;
+    }
+  };
+  // per-feature factors of a pass
+  auto load_scales = [&](const DecodePass& p) {
+    const DecodeLinear& L = lin_sh[p.l & 1];
+    if (p.nu == 0) return;
+    if (tid < p.nu * kUnit) be_sh[tid] = __ldg(L.beta + (long long)(p.unit * kUnit + tid) * L.sstride);
+    else if (tid >= 256 && tid - 256 < p.nu * kUnit && L.r > 0) al_sh[tid - 256] = __ldg(L.alpha + (long long)(p.unit * kUnit + tid - 256) * L.sstride);
+  };
+  DecodePass cur = pass_at(u_lo, l_at);
+  int u_next = u_lo + cur.nu;
+  DecodePass nxt = nbuf > 1 ? pass_at(u_next, cur.l) : DecodePass{0, 0, 0};
+  fetch_bits(cur, 0);
+  if (nbuf > 1) fetch_bits(nxt, 1);
+  load_scales(cur);
+  bool waited = false;                     // for the kernel before this one
+  if (!bp.early) { pdl_wait(); waited = true; }
+  const uint4* q_loaded = nullptr;
+  uint32_t phase[2] = {0u, 0u}, row_phase = 0u;
   uint4* q_s = reinterpret_cast<uint4*>(smem + bp.off_q);
-  uint8_t* ring = smem + bp.off_ring;
-
-  if (warp == bp.nwarps) {
-    // ------------------------------------------------------------------ producer (one thread issues everything)
-    if (lane != 0) return;
-    // The sign bits of the first linears (as many as there are slots) go out before the previous kernel, which
-    // prepares this one's tokens, is known to have finished: weights are not its output.
-    int early = 0;
+  uint4* h_s = reinterpret_cast<uint4*>(smem + off_h);
+  int8_t* qh_s = reinterpret_cast<int8_t*>(smem + off_h);
+  int* red_i = reinterpret_cast<int*>(smem + bp.off_red);        // [tile][token][16 features]
+  float* red_z = reinterpret_cast<float*>(red_i + kMaxPassUnits * MT * 16);   // [tile][token][16]
+  int loaded_l = -1;
+  for (int b = 0; cur.nu > 0;) {
+    const DecodeLinear& L = lin_sh[cur.l & 1];
+    const int M = L.M, K = L.K, N = L.N, r = L.r;
+    const int C = (K + 127) >> 7, rsteps = (r + 31) >> 5;
+    const int rows = cur.nu * kUnit, n0 = cur.unit * kUnit;
+    uint8_t* bits_s = smem + (size_t)b * buf_bytes;
+    const float lam = __ldg(L.w_scales);
+    const bool whole = q_chunks >= C;
+    // codes of the chunks [ch0, ch1) into shared memory: group 0 first, group 1 at q_chunks * 64
+    auto load_codes = [&](int ch0, int ch1) {
+      const int mg0 = min(8, M), n0q = (ch1 - ch0) * mg0 * 8, n1q = (ch1 - ch0) * (M - 8) * 8;
+      const uint4 *s0 = L.qfrag + (long long)ch0 * mg0 * 8, *s1 = L.qfrag + (long long)C * 64 + (long long)ch0 * (M - 8) * 8;
+      const int n = n0q + (M > 8 ? n1q : 0);
+      for (int i0 = tid; i0 < n; i0 += 4 * kMainThreads) {
+        uint4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u * kMainThreads;
+          v[u] = i < n0q ? __ldcg(s0 + i) : i < n ? __ldcg(s1 + i - n0q) : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u * kMainThreads;
+          if (i < n) q_s[i < n0q ? i : q_chunks * 64 + i - n0q] = v[u];
+        }
+      }
+    };
+    const bool new_linear = cur.l != loaded_l;
+    loaded_l = cur.l;
+    if (new_linear && warp == kMainWarps - 1) {
+      DecodeTokInfo t{-1, 0.f, 1.f, 0};
+      if (lane < M) {
+        const int4 a = __ldcg(reinterpret_cast<const int4*>(L.info) + lane);
+        t = DecodeTokInfo{a.x & 15, __int_as_float(a.y), __int_as_float(a.z), a.w};
+        tok[lane] = t;
+        deq_sh[lane] = __fdiv_rn(lam, t.gamma);
+      }
+      // tokens by expert: a token's place is the number of tokens with a lower expert, or the same one and a lower index
+      int place = 0;
+      const unsigned used = __reduce_or_sync(0xffffffffu, lane < M ? 1u << t.expert : 0u);
+      for (int i = 0; i < M; ++i) {
+        const int e = __shfl_sync(0xffffffffu, t.expert, i);
+        place += e < t.expert || (e == t.expert && i < lane);
+      }
+      const unsigned same = __match_any_sync(0xffffffffu, t.expert);
+      if (lane < M) {
+        order_sh[place] = (uint8_t)lane;
+        if ((same & ((1u << lane) - 1u)) == 0u) {                // the expert's first token
+          const int k = __popc(used & ((1u << t.expert) - 1u));
+          expert_sh[k] = t.expert; first_sh[k] = place; count_sh[k] = __popc(same);
+        }
+      }
+      if (lane == 0) used_sh = r > 0 ? __popc(used) : 0;
+    }
+    if (whole && q_loaded != L.qfrag) { load_codes(0, C); q_loaded = L.qfrag; }
+    for (int i = tid; i < cur.nu * MT * 16; i += kMainThreads) red_i[i] = 0;
+    if (!L.bits_il) {
+      // natural layout [N, K/32]: four lanes take four consecutive chunks of a row
+      const int KW = K >> 5;
+      for (int i = tid; i < rows * ((C + 3) & ~3); i += kMainThreads) {
+        const int ci = i & 3, row = (i >> 2) % rows, c = ((i >> 2) / rows) * 4 + ci;
+        if (c < C) {
+          const uint32_t* src = L.bits + (long long)(n0 + row) * KW + 4 * c;
+          uint32_t w[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) w[u] = 4 * c + u < KW ? __ldg(src + u) : 0u;
+          reinterpret_cast<uint4*>(bits_s)[(size_t)c * rows + row] = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+      }
+    }
+    __syncthreads();
+    // ---- 1-bit product
+    const int tiles = cur.nu, pairs = (tiles + 1) >> 1, S = kMainWarps / pairs;   // at most 4 pairs of tiles
+    const int sl = warp / pairs, tile = 2 * (warp - sl * pairs);
+    if (L.bits_il) {
+      decode_wait(smem_u32(&bars[b]), phase[b], &fail_sh);
+      phase[b] ^= 1u;
+    }
     {
-      DecodeCursor c0;
-      for (int l = 0; l < bp.n && early < bp.nslot; ++l) {
-        const DecodeLinear& L = bp.lin[l];
-        int n_lo, n_hi;
-        decode_range(blockIdx.x, L, n_lo, n_hi);
-        const int ncols = n_hi - n_lo;
-        if (ncols == 0) continue;
-        const uint32_t bits_bytes = (uint32_t)ncols * (uint32_t)(L.K >> 3);
-        const uint32_t h_bytes = L.r > 0 ? (uint32_t)(((L.M + 7) >> 3) * 2 * ((L.r + 31) >> 5)) * 512u : 0u;
-        mbar_expect_tx(slot_full(c0.idx), bits_bytes + h_bytes);
-        bulk_load(smem_u32(slot_ptr(c0.idx)), L.bits + (long long)n_lo * (L.K >> 5), bits_bytes, slot_full(c0.idx));
-        c0.next(bp.nslot);
-        ++early;
-      }
-    }
-    pdl_wait();
-    // The routing of every linear's tokens first: it decides which expert rows are fetched, and with it in
-    // hand nothing below waits for data, only for free buffers, so the loads run as far ahead as the rings allow.
-    mbar_expect_tx(info_full, (uint32_t)bp.n * kDecodeMetaBytes);
-    for (int l = 0; l < bp.n; ++l) bulk_load(smem_u32(smem + l * kDecodeMetaBytes), bp.lin[l].info, kDecodeMetaBytes, info_full);
-    decode_wait(info_full, 0, fail);
-    if (*fail) return;                                       // nothing below may be issued from data that never arrived
-    DecodeCursor cs, cq, cr;
-    for (int l = 0; l < bp.n; ++l) {
-      const DecodeLinear& L = bp.lin[l];
-      int n_lo, n_hi;
-      decode_range(blockIdx.x, L, n_lo, n_hi);
-      const int ncols = n_hi - n_lo;
-      if (ncols == 0) continue;
-      {
-        const uint32_t bits_bytes = (uint32_t)ncols * (uint32_t)(L.K >> 3);
-        const uint32_t h_bytes = L.r > 0 ? (uint32_t)(((L.M + 7) >> 3) * 2 * ((L.r + 31) >> 5)) * 512u : 0u;
-        if (early > 0) {
-          --early;                                          // bits already on their way
-        } else {
-          decode_wait(slot_empty(cs.idx), cs.phase ^ 1u, fail);
-          if (*fail) return;
-          mbar_expect_tx(slot_full(cs.idx), bits_bytes + h_bytes);
-          bulk_load(smem_u32(slot_ptr(cs.idx)), L.bits + (long long)n_lo * (L.K >> 5), bits_bytes, slot_full(cs.idx));
-        }
-        if (h_bytes) bulk_load(smem_u32(slot_ptr(cs.idx) + bp.off_slot_h), L.hfrag, h_bytes, slot_full(cs.idx));
-        cs.next(bp.nslot);
-      }
-      const int npairs = ((L.K >> 5) + 1) >> 1;
-      const uint32_t row_bytes = (uint32_t)L.r * 2u;
-      const int ngroups = (L.M + 7) >> 3;
-      for (int G = 0; G < ngroups; ++G) {
-        const uint32_t q_bytes = (uint32_t)(npairs * min(8, L.M - 8 * G)) * 64u;
-        decode_wait(q_empty(cq.idx), cq.phase ^ 1u, fail);
-        if (*fail) return;
-        mbar_expect_tx(q_full(cq.idx), q_bytes);
-        bulk_load(smem_u32(q_s) + cq.idx * bp.q_bytes, L.qfrag + (long long)G * npairs * 32, q_bytes, q_full(cq.idx));
-        cq.next(bp.nq);
-        unsigned emask = L.r > 0 ? decode_expert_mask(info_ptr(l), L.M, G) : 0u;
-        for (; emask; emask &= emask - 1) {
-          const int e = __ffs(emask) - 1;
-          decode_wait(ring_empty(cr.idx), cr.phase ^ 1u, fail);
-          if (*fail || e >= L.E) return;
-          mbar_expect_tx(ring_full(cr.idx), (uint32_t)ncols * row_bytes);
-          bulk_load(smem_u32(ring + cr.idx * bp.ring_stage_bytes), L.B + ((long long)e * L.N + n_lo) * L.r,
-                    (uint32_t)ncols * row_bytes, ring_full(cr.idx));
-          cr.next(bp.nring);
-        }
-      }
-    }
-    return;
-  }
-
-  // -------------------------------------------------------------------- consumers
-  // The work of a CTA is a list of items (linear, token group, tile of 16 features), in that order; item i
-  // belongs to warp i mod nwarps, which contracts over all of K, adds the expert product and writes the 16 x 8
-  // outputs: no warp waits for another.  Every warp walks every buffer of the three rings in the producer's
-  // order, waits for it to be full and hands it back exactly once (the empty barriers count nwarps arrivals),
-  // whether it used it or not: a warp that skipped ahead without waiting could arrive twice in one phase.
-  const int g = lane >> 2, c = lane & 3;
-  DecodeCursor cs, cq, cr;
-  decode_wait(info_full, 0, fail);
-  int base_mod = 0;                                          // (items before the current (linear, group)) mod nwarps
-  for (int l = 0; l < bp.n; ++l) {
-    const DecodeLinear& L = bp.lin[l];
-    int n_lo, n_hi;
-    decode_range(blockIdx.x, L, n_lo, n_hi);
-    const int ncols = n_hi - n_lo;
-    if (ncols == 0) continue;
-    const int ntile = (ncols + 15) >> 4;                     // <= nwarps (checked by the host)
-    const int nks = L.K >> 5, npairs = (nks + 1) >> 1;
-    const int rsteps = (L.r + 31) >> 5;                      // 32 hidden values per step of the expert product
-    const uint32_t row_bytes = (uint32_t)L.r * 2u;
-    const int ngroups = (L.M + 7) >> 3;
-    const DecodeTokInfo* tok = info_ptr(l);
-    const int s = cs.idx;
-    decode_wait(slot_full(s), cs.phase, fail);
-    cs.next(bp.nslot);
-    const uint32_t* bits_s = reinterpret_cast<const uint32_t*>(slot_ptr(s));
-    const uint4* h_all = reinterpret_cast<const uint4*>(slot_ptr(s) + bp.off_slot_h);
-
-    for (int G = 0; G < ngroups; ++G) {
-      int my_tile = warp - base_mod;                         // tile j of this (linear, group) is item base + j
-      if (my_tile < 0) my_tile += bp.nwarps;
-      const bool mine = my_tile < ntile;
-      base_mod += ntile;
-      if (base_mod >= bp.nwarps) base_mod -= bp.nwarps;
-      unsigned emask = L.r > 0 ? decode_expert_mask(tok, L.M, G) : 0u;
-      const int qb = cq.idx;
-      const uint32_t q_phase = cq.phase;
-      cq.next(bp.nq);
-      if (!mine) {
-        // nothing of this group is this warp's: hand its buffers back as they arrive
-        decode_wait(q_full(qb), q_phase, fail);
-        if (lane == 0) mbar_arrive(q_empty(qb));
-        for (; emask; emask &= emask - 1) {
-          decode_wait(ring_full(cr.idx), cr.phase, fail);
-          if (lane == 0) mbar_arrive(ring_empty(cr.idx));
-          cr.next(bp.nring);
-        }
-        continue;
-      }
-      const int row0 = 16 * my_tile + g, row1 = row0 + 8;    // this thread's two features (local index)
-      const bool has0 = row0 < ncols, has1 = row1 < ncols;
-      // per-feature factors of the epilogue, fetched before anything is waited for
-      float lam = L.w_scales[0];
-      float be0 = 0.f, be1 = 0.f, al0 = 0.f, al1 = 0.f;
-      if (has0) { be0 = L.beta[(n_lo + row0) * L.sstride]; if (L.r > 0) al0 = L.alpha[(n_lo + row0) * L.sstride]; }
-      if (has1) { be1 = L.beta[(n_lo + row1) * L.sstride]; if (L.r > 0) al1 = L.alpha[(n_lo + row1) * L.sstride]; }
-      const int mg = min(8, L.M - 8 * G);
-      decode_wait(q_full(qb), q_phase, fail);
-      // the epilogue's factors are in registers from here on: their loads were issued before the wait and must not
-      // be moved down to their first use, where a warp would sit out a trip to global memory per tile
-      asm volatile("" : "+f"(lam), "+f"(be0), "+f"(be1), "+f"(al0), "+f"(al1));
-
-      // ---- 1-bit product: masked sums, weight 1 and weight 16; two independent chains of accumulators.
-      // Threads of tokens that do not exist read the last token's fragments (their results are never stored),
-      // threads of features beyond the range read feature 0.
-      int acc1[4] = {0, 0, 0, 0}, acc16[4] = {0, 0, 0, 0}, bcc1[4] = {0, 0, 0, 0}, bcc16[4] = {0, 0, 0, 0};
-      {
-        const uint4* qp = reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(q_s) + qb * bp.q_bytes) + min(g, mg - 1) * 4 + c;
-        const int qstep = mg * 4;
-        const uint32_t* w0 = bits_s + (has0 ? row0 : 0) * nks;
-        const uint32_t* w1 = bits_s + (has1 ? row1 : 0) * nks;
-        auto mac = [&](uint32_t x00, uint32_t x01, uint32_t x10, uint32_t x11, const uint4& qv, int (&x1)[4], int (&x16)[4]) {
-          const uint32_t t00 = x00 >> c, t01 = x01 >> c, t10 = x10 >> c, t11 = x11 >> c;
-          const uint32_t a1[4] = {t00 & 0x01010101u, t10 & 0x01010101u, t01 & 0x01010101u, t11 & 0x01010101u};
-          const uint32_t a16[4] = {t00 & 0x10101010u, t10 & 0x10101010u, t01 & 0x10101010u, t11 & 0x10101010u};
-          mma_u8s8(x1, a1, qv.x, qv.y);
-          mma_u8s8(x16, a16, qv.z, qv.w);
-        };
-        if ((nks & 1) == 0) {
-          // Rows are 8-byte aligned: one load per pair of weight words.  Software pipeline without branches:
-          // two register sets of four steps each; while one is multiplied the other is being loaded (the
-          // loads past the end are clamped to the last step and never used).
-          const uint2* v0 = reinterpret_cast<const uint2*>(w0);
-          const uint2* v1 = reinterpret_cast<const uint2*>(w1);
-          struct Set { uint2 a[4], b[4]; uint4 q[4]; };
-          const int last = npairs - 1;
-          auto fetch = [&](Set& f, int ip) {
+      auto bits = [&](auto groups, auto per_warp) {
+        constexpr int GG = decltype(groups)::value, T = decltype(per_warp)::value;
+        int a1[T][GG][4], a16[T][GG][4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const int i = min(ip + j, last);
-              f.a[j] = v0[i]; f.b[j] = v1[i]; f.q[j] = qp[i * qstep];
+        for (int t = 0; t < T; ++t)
+#pragma unroll
+          for (int G_ = 0; G_ < GG; ++G_)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) { a1[t][G_][u] = 0; a16[t][G_][u] = 0; }
+        for (int ch0 = 0; ch0 < C; ch0 += q_chunks) {            // once, unless the codes of all of K do not fit
+          const int ch1 = min(C, ch0 + q_chunks);
+          if (!whole) {
+            __syncthreads();
+            load_codes(ch0, ch1);
+            __syncthreads();
+          }
+          if (sl < S)
+            main_bits<GG, T>(reinterpret_cast<const uint32_t*>(bits_s), rows, tile * 16, q_s, ch0, q_chunks, M, ch0 + (ch1 - ch0) * sl / S,
+                             ch0 + (ch1 - ch0) * (sl + 1) / S, lane, a1, a16);
+        }
+        const int g = lane >> 2, c = lane & 3;
+        if (sl < S) {
+#pragma unroll
+          for (int t = 0; t < T; ++t) {
+            if (tile + t < tiles) {
+#pragma unroll
+              for (int G_ = 0; G_ < GG; ++G_)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                  const int m = 8 * G_ + 2 * c + (u & 1);
+                  // the weight-16 sums are exact multiples of 16; integer sums do not depend on the order of the slices
+                  if (m < M) atomicAdd(red_i + ((tile + t) * MT + m) * 16 + g + (u >> 1) * 8, a1[t][G_][u] + (a16[t][G_][u] >> 4));
+                }
             }
-          };
-          auto macs = [&](const Set& f) {
-            mac(f.a[0].x, f.a[0].y, f.b[0].x, f.b[0].y, f.q[0], acc1, acc16);
-            mac(f.a[1].x, f.a[1].y, f.b[1].x, f.b[1].y, f.q[1], bcc1, bcc16);
-            mac(f.a[2].x, f.a[2].y, f.b[2].x, f.b[2].y, f.q[2], acc1, acc16);
-            mac(f.a[3].x, f.a[3].y, f.b[3].x, f.b[3].y, f.q[3], bcc1, bcc16);
-          };
-          Set A, B;
-          int ip = 0;
-          fetch(A, 0);
-          for (; ip + 8 <= npairs; ip += 8) {
-            fetch(B, ip + 4);
-            macs(A);
-            fetch(A, ip + 8);
-            macs(B);
-          }
-          // fewer than eight steps left; A holds steps ip .. ip + 3 (clamped)
-          if (ip + 4 <= npairs) { macs(A); ip += 4; fetch(A, ip); }
-          for (int j = 0; ip + j < npairs; ++j) {
-            if (j == 0) mac(A.a[0].x, A.a[0].y, A.b[0].x, A.b[0].y, A.q[0], acc1, acc16);
-            if (j == 1) mac(A.a[1].x, A.a[1].y, A.b[1].x, A.b[1].y, A.q[1], bcc1, bcc16);
-            if (j == 2) mac(A.a[2].x, A.a[2].y, A.b[2].x, A.b[2].y, A.q[2], acc1, acc16);
-          }
-        } else {
-          for (int ip = 0; ip < npairs; ++ip) {
-            const int i0 = 2 * ip, i1 = min(2 * ip + 1, nks - 1);   // the odd last word pairs with zeros of q
-            mac(w0[i0], w0[i1], w1[i0], w1[i1], qp[ip * qstep], acc1, acc16);
           }
         }
+      };
+      using One = std::integral_constant<int, 1>;
+      using Two = std::integral_constant<int, 2>;
+      if (G > 1 && M > 8) { if (tiles > 1) bits(std::integral_constant<int, G>{}, Two{}); else bits(std::integral_constant<int, G>{}, One{}); }
+      else { if (tiles > 1) bits(One{}, Two{}); else bits(One{}, One{}); }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // what plain stores filled may be overwritten by bulk copies
+    __syncthreads();                                             // the sign bits of this pass have been used
+    // ---- expert product.  The rows of B_e go over what has been used: this pass's sign bits, and in the CTA's last pass all
+    // buffers and the codes.  Every warp has slots of its own and takes every W-th (expert, tile) item.
+    const bool last = u_next >= u_hi && (nbuf == 1 || nxt.nu == 0), rows_now = r > 0 && !L.A8;
+    uint8_t* ring = last ? smem : bits_s;
+    const uint32_t item_bytes = 32u * (uint32_t)max(r, 1);
+    const int slots = min(kMaxRows, (int)((uint32_t)(last ? off_h : buf_bytes) / item_bytes));
+    const int W = min(kMainWarps, slots), per = rows_now ? min(kWarpRows, slots / W) : 1, items = rows_now && warp < W ? used_sh * tiles : 0;
+    auto issue = [&](int i, int j) {                             // item i into this warp's slot j
+      if (lane == 0) {
+        const int ei = i / tiles, t = i - ei * tiles;
+        const uint32_t bar = smem_u32(&bars[2 + warp * kWarpRows + j]);   // barriers belong to a warp, whatever the slots of a pass
+        mbar_expect_tx(bar, item_bytes);
+        bulk_load(smem_u32(ring) + (uint32_t)(warp * per + j) * item_bytes, L.B + ((long long)expert_sh[ei] * N + n0 + t * 16) * r, item_bytes, bar);
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(q_empty(qb));              // this warp is done with the q fragments
-      // ---- expert product z = B_e h, tokens of other experts masked out; four independent chains
-      float z0[4] = {0.f, 0.f, 0.f, 0.f}, z1[4] = {0.f, 0.f, 0.f, 0.f}, z2[4] = {0.f, 0.f, 0.f, 0.f}, z3[4] = {0.f, 0.f, 0.f, 0.f};
-      const int my_tok = 8 * G + g;                          // the token whose h this thread feeds
-      const int my_tok_e = my_tok < L.M ? tok[my_tok].expert : -1;
-      const uint4* h_hi = h_all + (size_t)(G * 2) * rsteps * 32;
-      const uint4* h_lo = h_hi + (size_t)rsteps * 32;
-      for (; emask; emask &= emask - 1) {
-        const int e = __ffs(emask) - 1;
-        const int stage = cr.idx;
-        decode_wait(ring_full(stage), cr.phase, fail);
-        cr.next(bp.nring);
-        const uint8_t* rows = ring + stage * bp.ring_stage_bytes;
-        const uint4* r0p = reinterpret_cast<const uint4*>(rows + (has0 ? row0 : 0) * row_bytes);
-        const uint4* r1p = reinterpret_cast<const uint4*>(rows + (has1 ? row1 : 0) * row_bytes);
-        const bool feeds = my_tok_e == e;
-        for (int st = 0; st < rsteps; ++st) {
-          const int chunk = 4 * st + c;
-          const bool in = chunk * 8 < L.r;
-          uint4 b0 = make_uint4(0, 0, 0, 0), b1 = b0, hh = b0, hl = b0;
-          if (in) { b0 = r0p[chunk]; b1 = r1p[chunk]; }
-          if (feeds && in) { hh = h_hi[st * 32 + lane]; hl = h_lo[st * 32 + lane]; }
-          mma_bf16(z0, b0.x, b1.x, b0.y, b1.y, hh.x, hh.y);
-          mma_bf16(z1, b0.z, b1.z, b0.w, b1.w, hh.z, hh.w);
-          mma_bf16(z2, b0.x, b1.x, b0.y, b1.y, hl.x, hl.y);
-          mma_bf16(z3, b0.z, b1.z, b0.w, b1.w, hl.z, hl.w);
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(ring_empty(stage));      // this warp is done with the buffer
+    };
+    for (int j = 0; j < per && warp + W * j < items; ++j) issue(warp + W * j, j);
+    if (!waited) { pdl_wait(); waited = true; }                  // h
+    if (new_linear) {
+      if (rows_now) {
+        // only the pieces of tokens that exist
+        const int n = ((M + 7) >> 3) * 2 * rsteps * 32;
+        for (int i = tid; i < n; i += kMainThreads)
+          if (((i & 31) >> 2) + (i >= 2 * rsteps * 32 ? 8 : 0) < M) h_s[i] = __ldcg(L.hfrag + i);
       }
-
-      // ---- epilogue (Eq. 10-11)
+      if (L.A8) {
+        // the hidden activation enters the second 8-bit product quantised per token from its exact integers (Eq. 7-9)
+        for (int t = warp; t < M; t += kMainWarps) {
+          float v[8];
+          float amax = 0.f;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        // accumulator u: feature row0 (u < 2) or row1, token 8G + 2c + (u & 1)
-        const int nl = (u < 2) ? row0 : row1, t = 8 * G + 2 * c + (u & 1);
-        if (nl < ncols && t < L.M) {
-          const int n = n_lo + nl;
-          const int m = (acc1[u] + bcc1[u]) + ((acc16[u] + bcc16[u]) >> 4);   // the weight-16 sums are exact multiples of 16
-          const int acc = 2 * m - tok[t].rowsum;
-          float y = ((u < 2) ? be0 : be1) * __fdiv_rn(lam, tok[t].gamma) * (float)acc;
-          if (L.r > 0) y = fmaf(((u < 2) ? al0 : al1) * tok[t].gate, (z0[u] + z1[u]) + (z2[u] + z3[u]), y);
-          L.Y[(long long)t * L.N + n] = __bfloat16_as_ushort(__float2bfloat16_rn(y));
-          if (L.acc_dump) L.acc_dump[(long long)t * L.N + n] = acc;
+          for (int u = 0; u < 8; ++u) {
+            v[u] = lane + 32 * u < r ? (float)__ldcg(L.h_int + (long long)t * r + lane + 32 * u) : 0.f;
+            amax = fmaxf(amax, fabsf(v[u]));
+          }
+          for (int d = 16; d > 0; d >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, d));
+          const float gh = __fdiv_rn(kActQmax, fmaxf(amax, kActAmaxFloor));
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            if (lane + 32 * u < r) qh_s[t * r + lane + 32 * u] = (int8_t)quant_code(v[u], gh);
+          if (lane == 0) gh_sh[t] = gh;
+        }
+      }
+      __syncthreads();                                           // h is visible
+    }
+    for (int i = warp, j = 0; i < items; i += W) {
+      const int ei = i / tiles, t = i - ei * tiles;
+      decode_wait(smem_u32(&bars[2 + warp * kWarpRows + j]), (row_phase >> j) & 1u, &fail_sh);
+      row_phase ^= 1u << j;
+      main_expert(reinterpret_cast<const uint4*>(ring + (size_t)(warp * per + j) * item_bytes), r, order_sh + first_sh[ei], count_sh[ei], h_s, lane, red_z + (size_t)t * MT * 16);
+      __syncwarp();
+      if (i + W * per < items) issue(i + W * per, j);
+      if (++j == per) j = 0;
+    }
+    if (last) q_loaded = nullptr;
+    if (L.A8) {
+      // INT8 branch: z_int = B8_e qh (exact), z = z_int / (gamma_B gamma_h gamma_A gamma_t).  An item is (tile, token): lanes l and
+      // l + 16 share feature l of the tile and take alternate pieces of 16 hidden values
+      const int r16 = r >> 4, G32 = ((N + 127) >> 7) * 4, half = lane >> 4, f = lane & 15;
+      for (int i = warp; i < tiles * M; i += kMainWarps) {
+        const int t = i / tiles, un = i - t * tiles, e = tok[t].expert, at = cur.unit + un;
+        const uint4* bp8 = L.B8_il + ((long long)e * G32 + (at >> 1)) * r16 * 32 + (at & 1) * 16 + f;
+        const uint4* qv = reinterpret_cast<const uint4*>(qh_s + t * r);
+        uint4 w[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) w[u] = 2 * u + half < r16 ? __ldg(bp8 + (2 * u + half) * 32) : make_uint4(0u, 0u, 0u, 0u);
+        int zi = 0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          if (2 * u + half < r16) {
+            const uint4 q = qv[2 * u + half];
+            zi = __dp4a((int)w[u].x, (int)q.x, zi); zi = __dp4a((int)w[u].y, (int)q.y, zi);
+            zi = __dp4a((int)w[u].z, (int)q.z, zi); zi = __dp4a((int)w[u].w, (int)q.w, zi);
+          }
+        }
+        zi += __shfl_xor_sync(0xffffffffu, zi, 16);
+        const float den = __fmul_rn(__fmul_rn(__fmul_rn(__ldg(L.hp_scales + 2 * e + 1), gh_sh[t]), __ldg(L.hp_scales + 2 * e)), tok[t].gamma);
+        if (half == 0) {
+          red_z[(un * MT + t) * 16 + f] = __fdiv_rn((float)zi, den);
+          if (L.zint_dump) L.zint_dump[(long long)t * N + n0 + un * 16 + f] = zi;
         }
       }
     }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(slot_empty(s));               // this warp is done with the slot of linear l
+    __syncthreads();
+    // ---- epilogue (Eq. 10-11), two features per thread
+    for (int o = tid; o < (rows >> 1) * M; o += kMainThreads) {
+      const int t = o / (rows >> 1), f = 2 * (o - t * (rows >> 1));
+      const int at = ((f >> 4) * MT + t) * 16 + (f & 15);
+      const int2 v = *reinterpret_cast<const int2*>(red_i + at);
+      const int a0 = 2 * v.x - tok[t].rowsum, a1 = 2 * v.y - tok[t].rowsum;
+      const float deq = deq_sh[t];
+      float y0 = be_sh[f] * deq * (float)a0, y1 = be_sh[f + 1] * deq * (float)a1;
+      if (r > 0) {
+        const float2 z = *reinterpret_cast<const float2*>(red_z + at);
+        y0 = fmaf(al_sh[f] * tok[t].gate, z.x, y0); y1 = fmaf(al_sh[f + 1] * tok[t].gate, z.y, y1);
+      }
+      *reinterpret_cast<uint32_t*>(L.Y + (long long)t * N + n0 + f) = pack_bf16x2(y0, y1);
+      if (L.acc_dump) { L.acc_dump[(long long)t * N + n0 + f] = a0; L.acc_dump[(long long)t * N + n0 + f + 1] = a1; }
+    }
+    // ---- the buffer is free: the pass after the next one
+    const int was = cur.l;
+    cur = nbuf > 1 ? nxt : pass_at(u_next, cur.l);
+    u_next += cur.nu;
+    if (cur.nu == 0) break;
+    __syncthreads();                                             // the sums, factors and records of this pass have been used
+    if (cur.l != was && cur.l + 1 < bp.n && bp.unit0[cur.l + 1] < u_hi) {
+      copy_record(&lin_sh[(cur.l + 1) & 1], bp, cur.l + 1);
+      __syncthreads();
+    }
+    if (nbuf > 1) {
+      nxt = pass_at(u_next, cur.l);
+      fetch_bits(nxt, b);
+      b ^= 1;
+    } else {
+      fetch_bits(cur, 0);
+    }
+    load_scales(cur);
   }
+  if (!waited) pdl_wait();
 }
 
 // ---------------------------------------------------------------------------
@@ -650,22 +932,22 @@ __global__ void __launch_bounds__(kDecodeMainThreads) k_decode_main(const __grid
 static inline size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 
 size_t decode_workspace_bytes(int M, int K, int N, int r, bool dump) {
-  const size_t npairs = ((size_t)K / 32 + 1) / 2;
+  const size_t halves = 2 * (((size_t)K + 127) / 128);
   size_t b = up256(sizeof(DecodeTokInfo) * kDecodeMaxTokens);
-  b += up256(2 * npairs * 32 * sizeof(uint4));
+  b += up256((size_t)(M > 8 ? 2 : 1) * halves * 32 * sizeof(uint4));
   b += up256((size_t)2 * 2 * ((r + 31) / 32 > 0 ? (r + 31) / 32 : 1) * 512);
   if (dump) b += up256(sizeof(int) * (size_t)M * N);
+  b += up256((size_t)M * K * 2);                           // normalised tokens, or codes in natural order
   return b;
 }
 
 DecodeViewPtrs decode_view(int M, int K, int N, int r, void* ws, bool dump) {
   uint8_t* w = static_cast<uint8_t*>(ws);
-  const size_t npairs = ((size_t)K / 32 + 1) / 2;
+  const size_t halves = 2 * (((size_t)K + 127) / 128);
   DecodeViewPtrs v{w, nullptr};
-  w += up256(sizeof(DecodeTokInfo) * kDecodeMaxTokens) + up256(2 * npairs * 32 * sizeof(uint4)) +
-       up256((size_t)2 * 2 * ((r + 31) / 32 > 0 ? (r + 31) / 32 : 1) * 512);
+  w += up256(sizeof(DecodeTokInfo) * kDecodeMaxTokens) + up256((size_t)(M > 8 ? 2 : 1) * halves * 32 * sizeof(uint4)) + up256((size_t)2 * 2 * ((r + 31) / 32 > 0 ? (r + 31) / 32 : 1) * 512);
   if (dump) v.acc = reinterpret_cast<int*>(w);
-  (void)M; (void)N;
+  (void)N;
   return v;
 }
 
@@ -680,153 +962,161 @@ static int decode_sm_count() {
   return n;
 }
 
-constexpr size_t kDecodeMainSmemLimit = 226 * 1024;   // dynamic shared memory of k_decode_main (its barriers are static)
-constexpr size_t kDecodePrepSmemLimit = 200 * 1024;   // K bf16 values of one token
+constexpr size_t kDecodeMainSmemLimit = 220 * 1024;   // dynamic shared memory of k_decode_main (it has a few KB of its own)
+constexpr size_t kDecodePrepSmemLimit = 200 * 1024;
 
-// One launch pair for up to kDecodeMaxBatch independent linears.
-static int decode_launch_with(const DecodeItemArgs* items, int n, int nwarps, cudaStream_t st) {
+template <int CAP>
+static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st) {
   static int sms = decode_sm_count();
-  // One CTA per SM.  Eight consumer warps keep up with what the buffer rings can hold in flight (measured: more warps,
-  // or two smaller CTAs per SM, are not faster); sixteen only when a CTA's feature range needs more than eight tiles.
-  const int nctas = sms;
-  const size_t smem_limit = kDecodeMainSmemLimit;
-  DecodeBatch bp{};
-  bp.n = n; bp.nwarps = nwarps;
-  size_t slot_bits = 0, slot_h = 0, q_bytes = 0, ring_stage = 0, prep_smem = 0;
-  int max_slices = 1, max_m = 1, max_k = 0;
+  DecodeBatch<CAP> bp;
+  bp.n = n;
+  size_t h_bytes = 0, x_bytes = 0, slot_bytes = 0;
+  int max_m = 1, max_e = 1, units = 0, max_c = 1;
+  bool any_norm = false;
+  bp.hidden_groups = 0;
   for (int i = 0; i < n; ++i) {
     const DecodeItemArgs& it = items[i];
     const int M = it.a.T, K = it.a.K, N = it.a.N, r = it.a.r;
     DecodeLinear& L = bp.lin[i];
     uint8_t* w = static_cast<uint8_t*>(it.ws);
-    const size_t npairs = ((size_t)K / 32 + 1) / 2;
+    const size_t rsteps = std::max(1, (r + 31) / 32);
     L.info = reinterpret_cast<DecodeTokInfo*>(w); w += up256(sizeof(DecodeTokInfo) * kDecodeMaxTokens);
-    L.qfrag = reinterpret_cast<uint4*>(w); w += up256(2 * npairs * 32 * sizeof(uint4));
-    L.hfrag = reinterpret_cast<uint4*>(w); w += up256((size_t)2 * 2 * ((r + 31) / 32 > 0 ? (r + 31) / 32 : 1) * 512);
+    L.qfrag = reinterpret_cast<uint4*>(w); w += up256((size_t)(M > 8 ? 2 : 1) * (((size_t)K + 127) / 128) * 64 * sizeof(uint4));
+    L.hfrag = reinterpret_cast<uint4*>(w); w += up256((size_t)2 * 2 * rsteps * 512);
     L.acc_dump = it.dump ? reinterpret_cast<int*>(w) : nullptr;
+    if (it.dump) w += up256(sizeof(int) * (size_t)M * N);
+    L.xn = reinterpret_cast<uint16_t*>(w);
+    any_norm = any_norm || it.norm_weight;
     L.X = reinterpret_cast<const uint4*>(it.X); L.Wr = reinterpret_cast<const uint4*>(it.a.Wr); L.A = it.a.A; L.B = it.a.B;
-    L.bits = it.bits; L.w_scales = it.a.w_scales; L.alpha = it.a.alpha; L.beta = it.a.beta; L.Y = it.Y;
+    L.bits = it.bits; L.bits_il = reinterpret_cast<const uint4*>(it.bits_il);
+    L.w_scales = it.a.w_scales; L.alpha = it.a.alpha; L.beta = it.a.beta; L.Y = it.Y;
     L.norm_w = reinterpret_cast<const uint4*>(it.norm_weight); L.norm_eps = it.norm_eps;
     L.M = M; L.K = K; L.N = N; L.r = r; L.E = (r > 0 && it.a.E > 1) ? it.a.E : 1; L.sstride = it.a.scale_stride;
-    if (M > max_m) max_m = M;
-    const int groups = N / 8;
-    L.grp_base = groups / nctas; L.grp_rem = groups % nctas;
-    const int max_cols = ((groups + nctas - 1) / nctas) * 8;
-    if (max_cols > 16 * nwarps) return PQ_ERR_UNSUPPORTED;       // at most one tile of 16 features per warp and token group
-    slot_bits = std::max(slot_bits, up256((size_t)max_cols * (K / 8)));
-    slot_h = std::max(slot_h, r > 0 ? up256((size_t)((M + 7) / 8) * 2 * ((r + 31) / 32) * 512) : (size_t)0);   // token groups in use only
-    q_bytes = std::max(q_bytes, up256(npairs * (size_t)std::min(M, 8) * 64));
-    ring_stage = std::max(ring_stage, up256((size_t)max_cols * r * 2));
-    max_k = std::max(max_k, K);
-  }
-  // Buffer rings: at least two slots, one activation buffer and (with experts) two expert-row buffers; then
-  // deeper, in turn, while shared memory lasts, so that the loads of several linears are in flight at once.
-  const size_t slot_bytes = slot_bits + slot_h;
-  const size_t fixed = (size_t)n * kDecodeMetaBytes + 128;
-  const bool experts = ring_stage > 0;
-  bp.nslot = 2; bp.nq = 1; bp.nring = experts ? 2 : 1;
-  auto total = [&](int ns, int nq, int nr) { return fixed + ns * slot_bytes + nq * q_bytes + nr * ring_stage; };
-  for (bool grew = true; grew;) {
-    grew = false;
-    if (bp.nslot < kDecodeMaxSlots && total(bp.nslot + 1, bp.nq, bp.nring) <= smem_limit) { ++bp.nslot; grew = true; }
-    if (experts && bp.nring < kDecodeMaxRing && total(bp.nslot, bp.nq, bp.nring + 1) <= smem_limit) { ++bp.nring; grew = true; }
-    if (bp.nq < kDecodeMaxQ && bp.nq < bp.nslot * ((max_m + 7) / 8) && total(bp.nslot, bp.nq + 1, bp.nring) <= smem_limit) { ++bp.nq; grew = true; }
-  }
-  size_t off = (size_t)n * kDecodeMetaBytes;
-  bp.off_slots = (int)off; bp.off_slot_h = (int)slot_bits; bp.slot_bytes = (int)slot_bytes;
-  off += bp.nslot * slot_bytes;
-  bp.q_bytes = (int)q_bytes;
-  bp.off_q = (int)off; off += bp.nq * q_bytes;
-  bp.ring_stage_bytes = (int)ring_stage;
-  bp.off_ring = (int)off; off += bp.nring * ring_stage;
-  const size_t smem_main = off + 128;
-  if (smem_main > smem_limit) {
-    return PQ_ERR_UNSUPPORTED;
-  }
-  // token preparation: the token and up to eight rows (router rows, then rows of A_e) of K bf16 values each
-  bp.prep_rows = (int)std::min<size_t>(8, (kDecodePrepSmemLimit - (size_t)max_k * 2) / ((size_t)max_k * 2)) & ~1;   // two buffers
-  if (bp.prep_rows < 2) return PQ_ERR_UNSUPPORTED;
-  prep_smem = (size_t)max_k * 2 * (1 + bp.prep_rows);
-  // Slices of the hidden rows: whole rounds of rows, as many slices as keep the grid within
-  // one wave of resident CTAs (every slice repeats the token's absmax and router, and rounds run one after another).
-  const int resident = sms * std::max<int>(1, (int)((227 * 1024) / (prep_smem + 1024)));
-  int total_tokens = 0;
-  for (int i = 0; i < n; ++i) total_tokens += items[i].a.T;
-  for (int i = 0; i < n; ++i) {
-    DecodeLinear& L = bp.lin[i];
-    L.slices = 1; L.rows_per_slice = 1;
-    if (L.r > 0) {
-      int slices = std::max(1, resident / std::max(1, total_tokens));
-      slices = std::min(slices, (L.r + 7) / 8);
-      const int round_rows = bp.prep_rows / 2;
-      L.rows_per_slice = ((L.r + slices - 1) / slices + round_rows - 1) / round_rows * round_rows;
-      L.slices = (L.r + L.rows_per_slice - 1) / L.rows_per_slice;
+    L.A8 = it.A8; L.B8_il = it.A8 ? reinterpret_cast<const uint4*>(it.B_il) : nullptr; L.hp_scales = it.hp_scales;
+    L.h_int = L.zint_dump = nullptr;
+    if (it.A8) {
+      decode_stream_view(M, K, N, r, it.ws, it.dump, &L.h_int, &L.zint_dump);
+      h_bytes = std::max(h_bytes, up256((size_t)M * r));
+    } else if (r > 0) {
+      h_bytes = std::max(h_bytes, up256((size_t)((M + 7) / 8) * 2 * rsteps * 512));
+      slot_bytes = std::max(slot_bytes, (size_t)32 * r);
     }
-    max_slices = std::max(max_slices, L.slices);
+    L.unit0 = units;
+    bp.unit0[i] = units;
+    units += N / kUnit;
+    L.hidden0 = bp.hidden_groups;
+    if (r > 0) bp.hidden_groups += std::min(L.E, M) * ((r + 15) / 16);
+    max_m = std::max(max_m, M); max_e = std::max(max_e, L.E); max_c = std::max(max_c, (K + 127) / 128);
+    x_bytes = std::max(x_bytes, up256((size_t)K * 2));
   }
-  // The opt-in limits are set once, to the largest request this file can make: a launch recorded in a CUDA graph
-  // keeps its own shared-memory size, and a later call with a smaller one must not lower the limit under it.
-  static const bool limits_set =
-      cudaFuncSetAttribute(k_decode_main, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeMainSmemLimit) == cudaSuccess &&
-      cudaFuncSetAttribute(k_decode_prep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodePrepSmemLimit) == cudaSuccess;
-  if (!limits_set) return PQ_ERR_CUDA;
+  for (int i = n; i <= CAP; ++i) bp.unit0[i] = units;
+  bp.units = units;
 
-  cudaLaunchAttribute attr[1];
+  // ---- k_decode_main: one CTA per SM (fewer when there is less than a unit for each)
+  const int ctas = std::min(sms, units), share = (units + ctas - 1) / ctas;
+  bp.red_tokens = max_m > 8 ? 16 : 8;
+  const size_t red_bytes = (size_t)2 * kMaxPassUnits * bp.red_tokens * 16 * 4;
+  const size_t unit_bytes = (size_t)256 * max_c, fixed = h_bytes + red_bytes;
+  const size_t chunk_bytes = (size_t)128 * max_m;            // codes of one chunk of k
+  const size_t buf_min = std::max(unit_bytes, up256(slot_bytes));
+  if (buf_min + chunk_bytes + fixed > kDecodeMainSmemLimit) return PQ_ERR_UNSUPPORTED;
+  bp.q_chunks = (int)std::min<size_t>(max_c, (kDecodeMainSmemLimit - buf_min - fixed) / chunk_bytes);
+  const size_t q_bytes = up256(bp.q_chunks * chunk_bytes);
+  const size_t room = kDecodeMainSmemLimit - fixed - q_bytes;
+  int pass_units = std::min(share, kMaxPassUnits);
+  bp.nbuf = (n == 1 && share <= pass_units) ? 1 : 2;
+  if (2 * buf_min > room) bp.nbuf = 1;
+  while (pass_units > 1 && bp.nbuf * std::max(pass_units * unit_bytes, buf_min) > room) --pass_units;
+  bp.buf_bytes = (int)std::max(pass_units * unit_bytes, buf_min);
+  if ((size_t)bp.nbuf * bp.buf_bytes > room) return PQ_ERR_UNSUPPORTED;
+  size_t off = (size_t)bp.nbuf * bp.buf_bytes;
+  bp.off_q = (int)off; off += q_bytes;
+  bp.off_h = (int)off; off += h_bytes;
+  bp.off_red = (int)off; off += red_bytes;
+  const size_t smem_main = off;
+
+  // ---- k_decode_prep
+  bp.off_wr = (int)x_bytes;
+  bp.off_gain = (int)(x_bytes + (max_e > 8 ? 2 : max_e > 1 ? 1 : 0) * x_bytes);
+  bp.early = bp.hidden_groups > 0;
+  // one CTA per SM, if that leaves any of the contraction's parallelism; otherwise three per SM, and k_decode_main's follow them
+  bp.hidden_cluster = 4 * bp.hidden_groups <= sms ? 4 : 2 * bp.hidden_groups <= 3 * sms ? 2 : 1;
+  const size_t smem_prep = bp.off_gain + (any_norm ? x_bytes : 0);
+  if (smem_prep > kDecodePrepSmemLimit) return PQ_ERR_UNSUPPORTED;
+
+  using Kern = void (*)(DecodeBatch<CAP>);
+  const Kern prep = k_decode_prep<CAP>, hidden = k_decode_hidden<CAP>;
+  const Kern main = max_m > 8 ? (Kern)k_decode_main<CAP, 2> : (Kern)k_decode_main<CAP, 1>;
+  // The opt-in limits are set once, to the largest request this file can make: a launch recorded in a CUDA graph
+  // keeps its own shared-memory size, and a later call with a smaller one must not lower the limit under it.  All kernels ask
+  // for the same split of an SM's memory: CTAs that want different splits cannot be resident together.
+  static const bool attributes_set = [] {
+    const Kern all[4] = {k_decode_prep<CAP>, k_decode_hidden<CAP>, k_decode_main<CAP, 1>, k_decode_main<CAP, 2>};
+    const size_t limit[4] = {kDecodePrepSmemLimit, 0, kDecodeMainSmemLimit, kDecodeMainSmemLimit};
+    for (int i = 0; i < 4; ++i) {
+      if (limit[i] && cudaFuncSetAttribute(all[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit[i]) != cudaSuccess) return false;
+      if (cudaFuncSetAttribute(all[i], cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess) return false;
+    }
+    return true;
+  }();
+  if (!attributes_set) return PQ_ERR_CUDA;
+
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg{};
   cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = g_decode_pdl ? 1 : 0;
   {
-    cfg.gridDim = dim3(max_slices, max_m, n); cfg.blockDim = dim3(256, 1, 1); cfg.dynamicSmemBytes = prep_smem;
+    cfg.gridDim = dim3(kPrepCluster, max_m, n); cfg.blockDim = dim3(kPrepThreads, 1, 1); cfg.dynamicSmemBytes = smem_prep;
     LaunchScope ls(KID_DECODE_PREP, st);
-    if (cudaLaunchKernelEx(&cfg, k_decode_prep, bp) != cudaSuccess) return PQ_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, prep, bp) != cudaSuccess) return PQ_ERR_CUDA;
+  }
+  if (bp.hidden_groups > 0) {
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = bp.hidden_cluster; attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    if (!g_decode_pdl) attr[0] = attr[1];
+    cfg.numAttrs = g_decode_pdl ? 2 : 1;
+    cfg.gridDim = dim3(bp.hidden_groups * bp.hidden_cluster, 1, 1); cfg.blockDim = dim3(kHiddenThreads, 1, 1); cfg.dynamicSmemBytes = 0;
+    LaunchScope ls(KID_DECODE_PREP, st);
+    if (cudaLaunchKernelEx(&cfg, hidden, bp) != cudaSuccess) return PQ_ERR_CUDA;
+    cfg.numAttrs = g_decode_pdl ? 1 : 0;
   }
   {
-    cfg.gridDim = dim3(nctas, 1, 1); cfg.blockDim = dim3(32 * nwarps + 32, 1, 1); cfg.dynamicSmemBytes = smem_main;
+    cfg.gridDim = dim3(ctas, 1, 1); cfg.blockDim = dim3(kMainThreads, 1, 1); cfg.dynamicSmemBytes = smem_main;
     LaunchScope ls(KID_DECODE_MAIN, st);
-    if (cudaLaunchKernelEx(&cfg, k_decode_main, bp) != cudaSuccess) return PQ_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, main, bp) != cudaSuccess) return PQ_ERR_CUDA;
   }
   return PQ_OK;
 }
 
+// the descriptors are copied with every launch: small groups carry a small table
 static int decode_launch(const DecodeItemArgs* items, int n, cudaStream_t st) {
-  const int rc = decode_launch_with(items, n, 8, st);
-  return rc == PQ_ERR_UNSUPPORTED ? decode_launch_with(items, n, kDecodeMaxConsumerWarps, st) : rc;
+  if (n <= 2) return decode_launch_as<2>(items, n, st);
+  if (n <= 16) return decode_launch_as<16>(items, n, st);
+  return decode_launch_as<kDecodeMaxBatch>(items, n, st);
 }
 
-// the launch groups of the streaming kernel are larger than those of the two-kernel path (defined in pq_decode_stream.cu)
-int decode_stream_max_batch();
+int decode_stream_max_batch();   // pq_decode_stream.cu
 
 int decode_batch(const DecodeItemArgs* items, int n, cudaStream_t st) {
   int i = 0;
   while (i < n) {
-    // The streaming kernel takes a group whose items all carry its weight layout, where it pays.  (Measured on the 3B
-    // shapes: its grid barrier and its longer chain of dependent steps cost about as much as eight linears' worth of
-    // streaming, so small groups, and mid-sized groups of many tokens, stay on the two kernels above.)
-    const int mode_opt = decode_stream_mode();
-    int m = std::min(n - i, decode_stream_max_batch());
-    bool all = true, hp8 = false;
-    int max_m = 1, run = 0;
-    for (int k = 0; k < m; ++k) {
-      if (!items[i + k].bits_il) { all = false; break; }
-      ++run;
-      hp8 = hp8 || items[i + k].A8 != nullptr;
-      max_m = std::max(max_m, items[i + k].a.T);
-    }
-    int rc = PQ_ERR_UNSUPPORTED;
-    if (!all) m = run;                                       // the items in front that carry the layout, if any
-    const int mode = hp8 ? 2 : mode_opt;
-    if (m > 0 && mode > 0 && (mode > 1 || hp8 || m >= 12 || (m >= 6 && max_m <= 2))) {
-      rc = decode_stream_launch(items + i, m, st);
-      if (hp8 && rc == PQ_ERR_UNSUPPORTED) return rc;        // the INT8 branch exists on the streaming kernel only
-    }
+    // The streaming kernel takes a run of items that all carry its weight layout, where it pays.
+    const int mode = decode_stream_mode();
+    const int most = std::min(n - i, std::min(decode_stream_max_batch(), kDecodeMaxBatch));
+    int run = 0, max_m = 1;
+    while (run < most && items[i + run].bits_il) max_m = std::max(max_m, items[i + run++].a.T);
+    int rc = PQ_ERR_UNSUPPORTED, m = run;
+    if (run > 0 && (mode > 1 || (mode == 1 && (run >= 12 || (run >= 6 && max_m <= 2))))) rc = decode_stream_launch(items + i, run, st);
     if (rc == PQ_ERR_UNSUPPORTED) {
-      // the two-kernel path: the same run of items that carry the layout, or the run in front that does not
-      if (m == 0)
-        while (i + m < n && m < kDecodeMaxBatch && !items[i + m].bits_il) ++m;
-      m = std::min(m, kDecodeMaxBatch);
-      for (int k = 0; k < m; ++k)
-        if (items[i + k].A8) return PQ_ERR_UNSUPPORTED;
+      // the three kernels above take items with and without the layout together, unless the streaming kernel is asked for
+      // wherever it can run
+      m = most;
+      if (mode > 1) {
+        m = run;
+        if (run == 0)
+          while (m < most && !items[i + m].bits_il) ++m;
+      }
       rc = decode_launch(items + i, m, st);
     }
     if (rc) return rc;
