@@ -160,129 +160,178 @@ __global__ void __launch_bounds__(256) k_row_rms(const uint4* __restrict__ X, in
 }
 
 // ---------------------------------------------------------------------------
-// K4a: router (Sec. 3.3).  One warp per token (or per two).  Logits in fp32 with a fixed
-// summation order -- lane j owns the 8-element chunks c with c mod 32 == j,
-// ascending k, fused multiply-add; lanes combined by the xor butterfly
-// 16, 8, 4, 2, 1 -- so that the top-1 index is reproducible bit for bit.
-// Softmax in fp32; ties go to the lowest index.  Also counts tokens per
-// expert for each block of kRouterTokensPerBlock consecutive tokens.
+// K4a: router (Sec. 3.3).  Logits in fp32 with a fixed summation order -- lane j owns the 8-element
+// chunks c with c mod 32 == j, ascending k, fused multiply-add; lanes combined by the xor butterfly
+// 16, 8, 4, 2, 1 -- so that the top-1 index is reproducible bit for bit.  Softmax in fp32; ties go to
+// the lowest index.  Also counts tokens per expert for each block of kRouterTokensPerBlock tokens.
+//
+// Bound by the fused multiply-adds (T K E of them; with the unpacking about 350 issue slots of a scheduler per
+// 16 tokens x 256 elements x 8 experts) and, about equally, by reading X.  The order above leaves one lane's
+// chain per (token, expert) and no way to split K over threads, so what keeps the chip busy is many small CTAs, each
+// with enough of X in flight: 16 tokens per CTA, four per warp, and a ring of kRouterStages steps of 256 elements
+// filled by 16-byte asynchronous copies (X of the warp's tokens, and the CTA's Wr, unpacked once per four tokens).
+// Two experts share one instruction (fma.rn.f32x2: two independent roundings, the same values).
+// Measured with eight experts, before (32 tokens per CTA, one step prefetched in registers, scalar fma) and now: 8192 tokens
+// x 2048 29 -> 13.8 us, x 5632 56 -> 31 us, 2048 tokens x 3200 41 -> 10.2 us.  Three stages and four CTAs per SM beat five
+// and three (31 against 33 us); scalar fma 41; two tokens per warp 39.
 // ---------------------------------------------------------------------------
-// EMAX: compile-time bound on E (the loops over experts are unrolled to it); TPW: tokens per warp -- the warp
-// walks the chunks once and applies each unpacked piece of Wr to TPW tokens.  Neither changes any token's
-// arithmetic: a lane's partial sum of (token, expert) is the same chain of fused multiply-adds.
-template <int EMAX, int TPW>
-__global__ void __launch_bounds__(32 * kRouterTokensPerBlock / TPW, TPW >= 4 ? 2 : 1) k_router(const uint4* __restrict__ X, const uint4* __restrict__ Wr, int T, int K,
-                                                                             int E, int* __restrict__ expert, float* __restrict__ gate_tok,
-                                                                             float* __restrict__ probs_tok, int* __restrict__ block_counts,
-                                                                             const uint4* __restrict__ norm_w, const float* __restrict__ rms) {
+constexpr int kRouterWarps = 4, kRouterTpw = kRouterTokensPerBlock / kRouterWarps, kRouterStages = 3;
+
+template <int EMAX>
+constexpr int router_smem() { return kRouterStages * (kRouterTokensPerBlock + EMAX) * 32 * (int)sizeof(uint4); }
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {   // invalid: zeros
+  const int n = valid ? 16 : 0;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
+  uint64_t v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+  return v;
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+
+// EMAX: compile-time bound on E, a power of two (experts past E have zero weights and are left out at the end)
+template <int EMAX>
+__global__ void __launch_bounds__(32 * kRouterWarps, EMAX <= 8 ? 4 : 2) k_router(const uint4* __restrict__ X, const uint4* __restrict__ Wr, int T, int K, int E,
+                                                              int* __restrict__ expert, float* __restrict__ gate_tok, float* __restrict__ probs_tok,
+                                                              int* __restrict__ block_counts, const uint4* __restrict__ norm_w,
+                                                              const float* __restrict__ rms) {
   pdl_launch_dependents();   // launched with programmatic stream serialisation: see launch_pdl
-  pdl_wait();
-  __shared__ int cnt[kMaxExperts];
-  if (threadIdx.x < kMaxExperts) cnt[threadIdx.x] = 0;
-  __syncthreads();
+  constexpr int TPW = kRouterTpw, S = kRouterStages, ROWS = kRouterTokensPerBlock + EMAX;
+  extern __shared__ uint4 ring[];                       // [stage][token or expert][32 chunks]
+  __shared__ __align__(16) float logit[kRouterTokensPerBlock * EMAX];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int chunks = K >> 3;
+  const int chunks = K >> 3, steps = (chunks + 31) >> 5;
   const int t0 = blockIdx.x * kRouterTokensPerBlock + warp * TPW;   // this warp's first token
-  if (t0 < T) {
-    float acc[TPW][EMAX];
+  pdl_wait();
+  // a token past the end repeats the last one, unused
+  auto fetch = [&](int step) {
+    if (step < steps) {
+      const int c = step * 32 + lane;
+      const bool in = c < chunks;
+      const uint32_t dst = smem_u32(ring + (step % S) * ROWS * 32 + lane);
 #pragma unroll
-    for (int u = 0; u < TPW; ++u)
+      for (int u = 0; u < TPW; ++u)
+        cp_async16(dst + (warp * TPW + u) * 512, X + (long long)min(t0 + u, T - 1) * chunks + (in ? c : 0), in);
 #pragma unroll
-      for (int e = 0; e < EMAX; ++e) acc[u][e] = 0.f;
-    const uint4* xrow[TPW];
-#pragma unroll
-    for (int u = 0; u < TPW; ++u) xrow[u] = X + (long long)min(t0 + u, T - 1) * chunks;   // a token past the end repeats the last one, unused
-    auto fold = [&](const uint4 (&xv)[TPW], const uint4 (&wr)[EMAX]) {
-      float x[TPW][8];
-#pragma unroll
-      for (int u = 0; u < TPW; ++u) {
-        x[u][0] = bf16lo(xv[u].x); x[u][1] = bf16hi(xv[u].x); x[u][2] = bf16lo(xv[u].y); x[u][3] = bf16hi(xv[u].y);
-        x[u][4] = bf16lo(xv[u].z); x[u][5] = bf16hi(xv[u].z); x[u][6] = bf16lo(xv[u].w); x[u][7] = bf16hi(xv[u].w);
+      for (int i = 0; i < EMAX / kRouterWarps; ++i) {
+        const int e = warp + i * kRouterWarps;
+        cp_async16(dst + (kRouterTokensPerBlock + e) * 512, Wr + (long long)(e < E ? e : 0) * chunks + (in ? c : 0), in && e < E);
       }
-#pragma unroll
-      for (int e = 0; e < EMAX; ++e) {
-        if (e < E) {
-          const uint4 wv = wr[e];
-          const float w[8] = {bf16lo(wv.x), bf16hi(wv.x), bf16lo(wv.y), bf16hi(wv.y), bf16lo(wv.z), bf16hi(wv.z), bf16lo(wv.w), bf16hi(wv.w)};
-#pragma unroll
-          for (int u = 0; u < TPW; ++u) {
-            float a = acc[u][e];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) a = fmaf(x[u][i], w[i], a);
-            acc[u][e] = a;
-          }
-        }
-      }
-    };
-    // the tokens' chunks in ascending order; the next chunk of every row and this chunk's pieces of Wr are
-    // requested before the current chunk is folded in
-    float srow[TPW];
-#pragma unroll
-    for (int u = 0; u < TPW; ++u) srow[u] = norm_w ? rms[min(t0 + u, T - 1)] : 1.0f;
-    auto fetch_x = [&](int u, int cc) {
-      if (cc >= chunks) return make_uint4(0u, 0u, 0u, 0u);
-      const uint4 v = __ldg(xrow[u] + cc);
-      return norm_w ? rms_apply(v, srow[u], __ldg(norm_w + cc)) : v;      // the router sees the normalised token
-    };
-    int c = lane;
-    uint4 xc[TPW];
-#pragma unroll
-    for (int u = 0; u < TPW; ++u) xc[u] = fetch_x(u, c);
-    while (c < chunks) {
-      const int cn = c + 32;
-      uint4 xn[TPW];
-#pragma unroll
-      for (int u = 0; u < TPW; ++u) xn[u] = fetch_x(u, cn);
-      uint4 wr[EMAX];
-#pragma unroll
-      for (int e = 0; e < EMAX; ++e) wr[e] = e < E ? __ldg(Wr + (long long)e * chunks + c) : make_uint4(0u, 0u, 0u, 0u);
-      fold(xc, wr);
-#pragma unroll
-      for (int u = 0; u < TPW; ++u) xc[u] = xn[u];
-      c = cn;
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float srow[TPW];
+#pragma unroll
+  for (int u = 0; u < TPW; ++u) srow[u] = norm_w ? __ldcg(rms + min(t0 + u, T - 1)) : 1.0f;
+  uint64_t acc[TPW][EMAX / 2];
+#pragma unroll
+  for (int u = 0; u < TPW; ++u)
+#pragma unroll
+    for (int e = 0; e < EMAX / 2; ++e) acc[u][e] = 0ull;
+#pragma unroll
+  for (int i = 0; i < S - 1; ++i) fetch(i);
+  for (int step = 0; step < steps; ++step) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(S - 2) : "memory");
+    __syncthreads();
+    fetch(step + S - 1);                                // into the stage every warp has left
+    const uint4* st = ring + (step % S) * ROWS * 32 + lane;
+    uint4 g = make_uint4(0u, 0u, 0u, 0u);
+    if (norm_w && step * 32 + lane < chunks) g = __ldg(norm_w + step * 32 + lane);
+    uint64_t x[TPW][8];
 #pragma unroll
     for (int u = 0; u < TPW; ++u) {
-      const int t = t0 + u;
-      if (t >= T) break;
+      uint4 v = st[(warp * TPW + u) * 32];
+      if (norm_w) v = rms_apply(v, srow[u], g);         // the router sees the normalised token
+      const float f[8] = {bf16lo(v.x), bf16hi(v.x), bf16lo(v.y), bf16hi(v.y), bf16lo(v.z), bf16hi(v.z), bf16lo(v.w), bf16hi(v.w)};
 #pragma unroll
-      for (int e = 0; e < EMAX; ++e) {
-        if (e < E) {
-          float a = acc[u][e];
-          for (int d = 16; d > 0; d >>= 1) a = a + __shfl_xor_sync(0xffffffffu, a, d);
-          acc[u][e] = a;
+      for (int i = 0; i < 8; ++i) x[u][i] = pack_f32x2(f[i], f[i]);
+    }
+#pragma unroll
+    for (int e = 0; e < EMAX / 2; ++e) {
+      const uint4 a = st[(kRouterTokensPerBlock + 2 * e) * 32], b = st[(kRouterTokensPerBlock + 2 * e + 1) * 32];
+      const uint64_t w[8] = {pack_f32x2(bf16lo(a.x), bf16lo(b.x)), pack_f32x2(bf16hi(a.x), bf16hi(b.x)), pack_f32x2(bf16lo(a.y), bf16lo(b.y)),
+                             pack_f32x2(bf16hi(a.y), bf16hi(b.y)), pack_f32x2(bf16lo(a.z), bf16lo(b.z)), pack_f32x2(bf16hi(a.z), bf16hi(b.z)),
+                             pack_f32x2(bf16lo(a.w), bf16lo(b.w)), pack_f32x2(bf16hi(a.w), bf16hi(b.w))};
+#pragma unroll
+      for (int u = 0; u < TPW; ++u)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc[u][e] = fma_f32x2(x[u][i], w[i], acc[u][e]);
+    }
+  }
+  // butterfly 16, 8, 4, 2, 1 over the lanes; a lane keeps half of its sums at each level (the same additions)
+  constexpr int NV = TPW * EMAX;
+  float v[NV];
+#pragma unroll
+  for (int u = 0; u < TPW; ++u)
+#pragma unroll
+    for (int e = 0; e < EMAX / 2; ++e) {
+      v[u * EMAX + 2 * e] = __uint_as_float((uint32_t)acc[u][e]);
+      v[u * EMAX + 2 * e + 1] = __uint_as_float((uint32_t)(acc[u][e] >> 32));
+    }
+  int n = NV, idx = 0;
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) {
+    if (n > 1) {
+      n >>= 1;
+      const bool up = lane & d;
+      idx += up ? n : 0;
+#pragma unroll
+      for (int i = 0; i < NV / 2; ++i) {
+        if (i < n) {
+          const float keep = up ? v[i + n] : v[i], send = up ? v[i] : v[i + n];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, d);
         }
       }
-      // every lane now holds all logits; lane 0 finishes the token
-      int best = 0;
-      float lmax = acc[u][0];
+    } else {
+      v[0] = v[0] + __shfl_xor_sync(0xffffffffu, v[0], d);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < (NV > 32 ? NV / 32 : 1); ++i) logit[warp * NV + idx + i] = v[i];
+  __syncthreads();
+  // a lane of the first warp per token
+  if (warp == 0) {
+    const int t = blockIdx.x * kRouterTokensPerBlock + lane;
+    const bool own = lane < kRouterTokensPerBlock && t < T;
+    int best = -1;
+    if (own) {
+      float l[EMAX];
+      const float4* row = reinterpret_cast<const float4*>(logit + lane * EMAX);
+#pragma unroll
+      for (int e = 0; e < EMAX; e += 4) { const float4 q = row[e >> 2]; l[e] = q.x; l[e + 1] = q.y; l[e + 2] = q.z; l[e + 3] = q.w; }
+      best = 0;
+      float lmax = l[0];
 #pragma unroll
       for (int e = 1; e < EMAX; ++e)
-        if (e < E && acc[u][e] > lmax) { lmax = acc[u][e]; best = e; }
+        if (e < E && l[e] > lmax) { lmax = l[e]; best = e; }
       float den = 0.f;
-      float pe[EMAX];
 #pragma unroll
       for (int e = 0; e < EMAX; ++e) {
-        pe[e] = (e < E) ? expf(acc[u][e] - lmax) : 0.f;
-        den += pe[e];
+        l[e] = e < E ? expf(l[e] - lmax) : 0.f;
+        den += l[e];
       }
       const float inv = 1.0f / den;
-      if (lane == 0) {
-        expert[t] = best;
-        atomicAdd(&cnt[best], 1);
-      }
+      expert[t] = best;
 #pragma unroll
       for (int e = 0; e < EMAX; ++e) {
         if (e < E) {
-          const float pr = pe[e] * inv;
-          if (lane == 0) probs_tok[(long long)t * E + e] = pr;
-          if (e == best && lane == 0) gate_tok[t] = pr;
+          const float pr = l[e] * inv;
+          probs_tok[(long long)t * E + e] = pr;
+          if (e == best) gate_tok[t] = pr;
         }
       }
     }
+    for (int e = 0; e < E; ++e) {
+      const int cnt = __popc(__ballot_sync(0xffffffffu, best == e));
+      if (lane == 0) block_counts[e * gridDim.x + blockIdx.x] = cnt;
+    }
   }
-  __syncthreads();
-  if (threadIdx.x < E) block_counts[blockIdx.x * E + threadIdx.x] = cnt[threadIdx.x];
 }
 
 // ---------------------------------------------------------------------------
@@ -292,14 +341,16 @@ __global__ void __launch_bounds__(32 * kRouterTokensPerBlock / TPW, TPW >= 4 ? 2
 // relative to the tile).  Items are sorted by tile and therefore by expert.
 // One block; the work is a few hundred integers.
 // ---------------------------------------------------------------------------
-// Items of one 128-row tile [r0, r1) of the sorted order: experts e0 <= e < E whose non-empty range
-// [off[e], off[e+1]) meets the tile.  Returns the number of items; calls f(k, e, lo, hi) for the k-th.
-template <class F>
-__device__ __forceinline__ int tile_items(const int* off, int Ee, int r0, int r1, F f) {
+// All of it is latency (a few thousand integers), so nothing is carried from step to step: a warp takes an expert,
+// 512 blocks of tokens loaded and scanned together; and the number of items before a tile has a closed form,
+// so every table entry is one thread's own sum over the experts.  Measured at 8192 tokens, eight experts: 5.6 us with the
+// blocks 32 at a time and block-wide scans over the tiles, 4.4 us now.
+// items in the tiles before `tile`, tiles of `rows` rows: a non-empty expert has one in every tile that it meets
+__device__ __forceinline__ int items_before(const int* off, int Ee, int rows_log2, int tile) {
   int n = 0;
   for (int e = 0; e < Ee; ++e) {
-    const int lo = max(off[e], r0), hi = min(off[e + 1], r1);
-    if (hi > lo) { f(n, e, lo, hi); ++n; }
+    const int lo = off[e], hi = off[e + 1];
+    if (hi > lo) n += max(0, min(tile - 1, (hi - 1) >> rows_log2) - (lo >> rows_log2) + 1);
   }
   return n;
 }
@@ -308,99 +359,81 @@ __global__ void __launch_bounds__(512) k_route_scan(int T, int E, int nblocks, c
                                                     int* __restrict__ block_base, int* __restrict__ offsets, RoutingTables rt) {
   pdl_launch_dependents();   // launched with programmatic stream serialisation: see launch_pdl
   pdl_wait();
+  constexpr int kPer = 16, kTileLog2 = 7;
+  static_assert(kTileRows == 1 << kTileLog2 && kMaxExperts <= 16, "a warp per expert");
   __shared__ int off[kMaxExperts + 1];
   __shared__ int total[kMaxExperts];
-  __shared__ int warp_sums[16];
-  __shared__ int carry_sh;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int Ee = E < 1 ? 1 : E;
   if (E > 1 && warp < E) {
-    // exclusive scan of this expert's per-block counts, 32 blocks at a time
+    // exclusive scan of this expert's per-block counts
     int carry = 0;
-    for (int b0 = 0; b0 < nblocks; b0 += 32) {
-      const int b = b0 + lane;
-      const int v = b < nblocks ? block_counts[b * E + warp] : 0;
-      int inc = v;
+    for (int b0 = 0; b0 < nblocks; b0 += 32 * kPer) {
+      const int* src = block_counts + (long long)warp * nblocks + b0 + lane;
+      int* dst = block_base + (long long)warp * nblocks + b0 + lane;
+      int v[kPer], inc[kPer];
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) v[i] = inc[i] = b0 + 32 * i + lane < nblocks ? __ldcg(src + 32 * i) : 0;
+#pragma unroll
       for (int d = 1; d < 32; d <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, inc, d);
-        if (lane >= d) inc += u;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+          const int u = __shfl_up_sync(0xffffffffu, inc[i], d);
+          if (lane >= d) inc[i] += u;
+        }
       }
-      if (b < nblocks) block_base[b * E + warp] = carry + inc - v;
-      carry += __shfl_sync(0xffffffffu, inc, 31);
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        if (b0 + 32 * i + lane < nblocks) dst[32 * i] = carry + inc[i] - v[i];
+        carry += __shfl_sync(0xffffffffu, inc[i], 31);
+      }
     }
     if (lane == 0) total[warp] = carry;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    if (E <= 1) {
-      off[0] = 0; off[1] = T;
-    } else {
-      int run = 0;
-      for (int e = 0; e < E; ++e) { off[e] = run; run += total[e]; }
-      off[E] = run;
-    }
-    carry_sh = 0;
+  if (threadIdx.x <= Ee) {
+    int run = threadIdx.x > 0 && E <= 1 ? T : 0;
+    if (E > 1)
+      for (int e = 0; e < threadIdx.x; ++e) run += total[e];
+    off[threadIdx.x] = offsets[threadIdx.x] = run;
   }
   __syncthreads();
-  if (threadIdx.x <= Ee) offsets[threadIdx.x] = off[threadIdx.x];
 
-  // items: one thread per tile counts its items, a block-wide scan places them
-  const int mtiles = (T + kTileRows - 1) / kTileRows;
-  auto scan_tiles = [&](int ntiles, int rows, auto place) {
-    for (int base = 0; base < ntiles; base += blockDim.x) {
-      const int tile = base + threadIdx.x;
-      const int r0 = tile * rows, r1 = min(T, r0 + rows);
-      const int cnt = tile < ntiles ? tile_items(off, Ee, r0, r1, [](int, int, int, int) {}) : 0;
-      int inc = cnt;
-      for (int d = 1; d < 32; d <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, inc, d);
-        if (lane >= d) inc += u;
-      }
-      if (lane == 31) warp_sums[warp] = inc;
-      __syncthreads();
-      int before = carry_sh;
-      for (int w = 0; w < warp; ++w) before += warp_sums[w];
-      const int first = before + inc - cnt;
-      if (tile < ntiles) place(tile, r0, r1, first);
-      __syncthreads();
-      if (threadIdx.x == blockDim.x - 1) carry_sh = first + cnt;
-      __syncthreads();
+  const int mtiles = (T + kTileRows - 1) / kTileRows, mpairs = (mtiles + 1) / 2;
+  for (int tile = threadIdx.x; tile <= mtiles; tile += blockDim.x) {
+    int k = items_before(off, Ee, kTileLog2, tile);
+    rt.tile_item_begin[tile] = k;
+    if (tile == mtiles) { rt.n_items[0] = k; break; }
+    const int r0 = tile * kTileRows, r1 = min(T, r0 + kTileRows);
+    for (int e = 0; e < Ee; ++e) {
+      const int lo = max(off[e], r0), hi = min(off[e + 1], r1);
+      if (hi > lo) rt.items[k++] = make_int4(tile, e, lo - r0, hi - r0);
     }
-  };
-  scan_tiles(mtiles, kTileRows, [&](int tile, int r0, int r1, int first) {
-    rt.tile_item_begin[tile] = first;
-    tile_items(off, Ee, r0, r1, [&](int k, int e, int lo, int hi) { rt.items[first + k] = make_int4(tile, e, lo - r0, hi - r0); });
-  });
-  const int n_items = carry_sh;
-  if (threadIdx.x == 0) { rt.tile_item_begin[mtiles] = n_items; rt.n_items[0] = n_items; }
+  }
   // first item of each expert: the first item of the tile holding its first row, plus the items of the
   // non-empty experts below it in that tile; an empty expert points at its successor's first item
-  if (threadIdx.x <= Ee) {
-    int e = threadIdx.x;
+  if (threadIdx.x >= 480 && threadIdx.x - 480 <= Ee) {
+    const int i = threadIdx.x - 480;
+    int e = i;
     while (e < Ee && off[e + 1] == off[e]) ++e;
-    int idx = n_items;
-    if (e < Ee) {
-      const int tile = off[e] / kTileRows, r0 = tile * kTileRows;
-      idx = rt.tile_item_begin[tile];   // written above by this block, ordered by the barriers of the loop
-      for (int f = 0; f < e; ++f)
-        if (min(off[f + 1], r0 + kTileRows) > max(off[f], r0)) ++idx;
-    }
-    rt.expert_item_begin[threadIdx.x] = idx;
+    const int tile = e < Ee ? off[e] >> kTileLog2 : mtiles;
+    int idx = items_before(off, Ee, kTileLog2, tile);
+    if (e < Ee)
+      for (int f = 0; f < e; ++f) idx += off[f + 1] > off[f] && off[f + 1] > tile * kTileRows;
+    rt.expert_item_begin[i] = idx;
   }
   // the same for pairs of tiles; the items of a tile are in expert order, so each expert of the pair takes the next one
-  __syncthreads();
-  if (threadIdx.x == 0) carry_sh = 0;
-  __syncthreads();
-  const int mpairs = (mtiles + 1) / 2;
-  scan_tiles(mpairs, 2 * kTileRows, [&](int pair, int r0, int r1, int first) {
-    const int mid = r0 + kTileRows;
-    int i0 = rt.tile_item_begin[2 * pair], i1 = mid < r1 ? rt.tile_item_begin[2 * pair + 1] : 0;
-    rt.pair_begin[pair] = first;
-    tile_items(off, Ee, r0, r1, [&](int k, int e, int lo, int hi) {
-      rt.pair_items[first + k] = make_int4(e, lo < mid ? i0++ : -1, hi > mid ? i1++ : -1, pair);
-    });
-  });
-  if (threadIdx.x == 0) rt.pair_begin[mpairs] = carry_sh;
+  for (int pair = (int)blockDim.x - 1 - (int)threadIdx.x; pair <= mpairs; pair += blockDim.x) {
+    int k = items_before(off, Ee, kTileLog2 + 1, pair);
+    rt.pair_begin[pair] = k;
+    if (pair == mpairs) break;
+    const int r0 = pair * 2 * kTileRows, r1 = min(T, r0 + 2 * kTileRows), mid = r0 + kTileRows;
+    int i0 = items_before(off, Ee, kTileLog2, 2 * pair), i1 = items_before(off, Ee, kTileLog2, 2 * pair + 1);
+    for (int e = 0; e < Ee; ++e) {
+      const int lo = max(off[e], r0), hi = min(off[e + 1], r1);
+      if (hi > lo) rt.pair_items[k++] = make_int4(e, lo < mid ? i0++ : -1, hi > mid ? i1++ : -1, pair);
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -458,10 +491,11 @@ __global__ void __launch_bounds__(256) k_act_quant(const uint4* __restrict__ X, 
   if (E > 1) {
     const int e = expert[t];
     const int blk = t / kRouterTokensPerBlock, first = blk * kRouterTokensPerBlock;
-    const int other = (first + lane < T) ? expert[first + lane] : -1;
+    const int other = lane < kRouterTokensPerBlock && first + lane < T ? expert[first + lane] : -1;
     const unsigned same = __ballot_sync(0xffffffffu, other == e);
     const int rank = __popc(same & ((1u << (t - first)) - 1u));
-    p = offsets[e] + block_base[blk * E + e] + rank;
+    const int nblocks = (T + kRouterTokensPerBlock - 1) / kRouterTokensPerBlock;
+    p = offsets[e] + block_base[(long long)e * nblocks + blk] + rank;
   }
   for (int d = 16; d > 0; d >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, d));
   if (WPR > 1) {
@@ -815,13 +849,17 @@ cudaError_t launch_route_and_quant(const uint16_t* X, const uint16_t* Wr, int T,
   const int nblocks = (T + kRouterTokensPerBlock - 1) / kRouterTokensPerBlock;
   if (E > 1) {
     LaunchScope ls(KID_ROUTER, st);
-    // two tokens per warp (half the loads and unpacking of Wr per token), 512 threads
-    if (E <= 4) launch_pdl(k_router<4, 4>, nblocks, 8 * kRouterTokensPerBlock, 0, st, reinterpret_cast<const uint4*>(X), reinterpret_cast<const uint4*>(Wr), T, K, E,
-                           sv.expert, sc.gate_tok, sc.probs_tok, sc.block_counts, nw, sc.rms);
-    else if (E <= 8) launch_pdl(k_router<8, 4>, nblocks, 8 * kRouterTokensPerBlock, 0, st, reinterpret_cast<const uint4*>(X), reinterpret_cast<const uint4*>(Wr), T, K, E,
-                                sv.expert, sc.gate_tok, sc.probs_tok, sc.block_counts, nw, sc.rms);
-    else launch_pdl(k_router<kMaxExperts, 2>, nblocks, 16 * kRouterTokensPerBlock, 0, st, reinterpret_cast<const uint4*>(X), reinterpret_cast<const uint4*>(Wr), T, K, E,
-                    sv.expert, sc.gate_tok, sc.probs_tok, sc.block_counts, nw, sc.rms);
+    auto kern = k_router<kMaxExperts>;
+    int smem = router_smem<kMaxExperts>();
+    if (E <= 4) { kern = k_router<4>; smem = router_smem<4>(); }
+    else if (E <= 8) { kern = k_router<8>; smem = router_smem<8>(); }
+    // One CTA per SM (two) where the grid needs no more: its CTAs become resident while the kernel before ends, and the SMs that
+    // end first would otherwise take all they can hold.  2048 tokens x 3200: 17 us without this, 10 with it.
+    if (nblocks <= 148) smem = 116 * 1024;
+    else if (nblocks <= 2 * 148) smem = 76 * 1024;
+    if (cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) return e;
+    launch_pdl(kern, nblocks, 32 * kRouterWarps, smem, st, reinterpret_cast<const uint4*>(X), reinterpret_cast<const uint4*>(Wr), T, K, E, sv.expert,
+               sc.gate_tok, sc.probs_tok, sc.block_counts, nw, sc.rms);
   }
   { LaunchScope ls(KID_ROUTE_SCAN, st);
   launch_pdl(k_route_scan, 1, 512, 0, st, T, E, nblocks, sc.block_counts, sc.block_base, sv.offsets, sv.rt); }

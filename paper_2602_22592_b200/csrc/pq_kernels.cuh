@@ -7,7 +7,7 @@
 namespace pq {
 
 constexpr int kMaxExperts = 16;
-constexpr int kRouterTokensPerBlock = 32;  // must equal the warp width (rank-in-block ballot)
+constexpr int kRouterTokensPerBlock = 16;  // at most the warp width (rank-in-block ballot); a multiple of the router's warps
 constexpr int kTileRows = 128;             // rows of one tensor-core tile
 constexpr int kPackPartials = 1024;        // fp64 partial sums of the weight reduction
 constexpr float kActQmax = 128.0f;         // 2^7 of Eq. 9
