@@ -224,7 +224,7 @@ def elementwise_bytes(L, routed):
     T, K, N = L.T, L.K, L.N
     return {"pack_sums": 4 * N * K, "binarize_pack": 4 * N * K + N * K + N * K // 8,
             "act_quant": 2 * T * K + T * K + 2 * T * K + (2 * T * K if routed else 0),
-            "router": 2 * T * K, "scatter_rows": 4 * T * N, "scaled_sign": N * K + 2 * N * K}
+            "router": 2 * T * K, "scaled_sign": N * K + 2 * N * K + (4 * T * N if routed else 0)}
 
 
 def measure_mlp(ctx, E, steps, warmup, engine, full):
@@ -238,7 +238,7 @@ def measure_mlp(ctx, E, steps, warmup, engine, full):
     ctx.barrier()
     ctx.check_status("during warm-up")
 
-    # dominant kernel: the dW GEMM (contraction over tokens), timed live with events on the launch stream
+    # dominant kernel: the products of the backward (one launch), timed live with events on the launch stream
     kid = pqb.KERNEL_IDS["bwd_dw"]
     ev = [[(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in layers] for _ in range(steps)]
     for row in ev:
@@ -266,13 +266,10 @@ def measure_mlp(ctx, E, steps, warmup, engine, full):
     peak, peak_key, peak_why = pick_bf16_peak(ctx.peaks, ctx.peak_kind, elapsed_ms * 1e-3, clocks)
 
     dw_ms = float(np.mean([a.elapsed_time(b) for row in ev for a, b in row]))
-    # algorithmic flops of the launch: dW = dY^T . (q/gamma).  (The HP tiles dB, dA and the router gradient are a
-    # launch of their own, profile id hp_db, and are not counted here.)  The launch shares the GPU with the chain
-    # scaled sign -> HP gradient GEMM -> dX on the library's helper stream, so its event time includes SMs it
-    # had to wait for.
-    dw_flops = float(np.mean([2.0 * L.T * L.N * L.K for L in layers]))
+    # algorithmic flops of the launch: dW = dY^T . (q/gamma), dX = dY . S, and the experts' dH, its share of dX, dB and dA
+    dw_flops = float(np.mean([4.0 * L.T * L.N * L.K + 4.0 * L.T * L.r * (L.N + L.K) for L in layers]))
     achieved = dw_flops / (dw_ms * 1e-3) / 1e12
-    roofline = {"kernel": "k_gemm_bwd_dw (dW = dY^T . q/gamma, bf16 tcgen05, fp32 accumulate)", "bound": "tensor",
+    roofline = {"kernel": "k_gemm_bwd (dW, dX and the experts' gradients, bf16 tcgen05, fp32 accumulate)", "bound": "tensor",
                 "achieved": round(achieved, 1), "peak": peak, "unit": "TFLOP/s", "frac": round(achieved / peak, 4),
                 "peak_source": peak_why, "avg_launch_ms": round(dw_ms, 4),
                 "frac_of_burst": round(achieved / ctx.peaks["bf16_tflops"], 4),
@@ -334,12 +331,12 @@ def measure_mlp(ctx, E, steps, warmup, engine, full):
 
 def breakdown(ctx, layers, routed):
     """Per-kernel device time: mean over a few extra (untimed) steps, every kernel on one stream (helper stream off) so
-    that each pair of events brackets one kernel running alone; the weight gradient is then a single launch again.
+    that each pair of events brackets one kernel running alone.
     Second result: achieved GB/s of the memory-bound kernels over their algorithmic bytes."""
     torch, pqb = ctx.torch, ctx.pqb
     pqb.pq_set_option(pqb.PQ_OPT_SIDE_STREAM, 0)
-    names = ["pack_sums", "binarize_pack", "router", "route_scan", "act_quant", "hp_up", "fwd", "scatter_rows", "scaled_sign",
-             "hp_dh", "bwd_dx", "bwd_dw", "hp_db", "sum_partials", "sum_scalar"]
+    names = ["pack_sums", "binarize_pack", "router", "route_scan", "act_quant", "hp_up", "fwd", "scaled_sign", "bwd_dw",
+             "sum_partials", "sum_scalar"]
     bev = {n: (torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for n in names}
     total = {n: 0.0 for n in names}
     algo = {}

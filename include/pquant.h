@@ -19,8 +19,8 @@
  *     caller's memory between calls.  What it does keep, per process: a few
  *     small file-scope device variables (a status word, the spin limit, the
  *     64 KiB array of pq_pack_weights_static), and -- unless PQ_OPT_SIDE_STREAM
- *     is 0 -- one helper stream and three events per (device, caller stream)
- *     that has called pq_linear_forward / pq_linear_backward, created on first
+ *     is 0 -- one helper stream and two events per (device, caller stream)
+ *     that has called pq_linear_forward, created on first
  *     use and kept until the process exits;
  *   - work is only enqueued on `stream` (a cudaStream_t passed as void*) and on
  *     that helper stream, which is joined back into `stream` inside the same
@@ -382,14 +382,11 @@ int pq_device_status(void* stream, int* code, int* where);
  *   PQ_OPT_DECODE_PDL (default 1): launch the decode kernels with programmatic stream
  *   serialisation, so that a kernel's prologue (barrier set-up, the copy of the sign bits)
  *   overlaps the tail of the kernel before it in the stream.  0 = plain stream order.
- *   PQ_OPT_SIDE_STREAM (default 1): pq_linear_forward (dense layer with an HP branch) and
- *   pq_linear_backward run kernels that do not depend on one another side by side, on a helper
- *   stream the library keeps per caller stream (created on first use, never during a stream
- *   capture); the helper's work is joined back inside the same call, so the caller's stream
- *   order is unchanged and a stream capture records one graph with a fork and a join.  In the
- *   backward pass the weight-gradient tiles that need only dY and q/gamma are one launch
- *   (profile id bwd_dw) and the HP tiles (dB, dA, router) a second one (id hp_db).
- *   0 = every kernel on the caller's stream, the weight gradient as one launch.
+ *   PQ_OPT_SIDE_STREAM (default 1): pq_linear_forward (dense layer with an HP branch) runs the
+ *   activation quantisation beside the HP up-projection, on a helper stream the library keeps per
+ *   caller stream (created on first use, never during a stream capture); the helper's work is joined
+ *   back inside the same call, so the caller's stream order is unchanged and a stream capture records
+ *   one graph with a fork and a join.  0 = every kernel on the caller's stream.
  *   PQ_OPT_SPIN_CYCLES: limit of every device-side spin-wait in SM clock cycles (value <= 0 restores
  *   the default of 4e9, about two seconds).  A test hook: with a limit of a few cycles the first wait
  *   that does not succeed at once runs out, the kernel stops issuing work, lets copies and MMAs in
@@ -417,10 +414,10 @@ long long pq_kernel_launches(void);
  * bracketed by cudaEventRecord(start_event) / cudaEventRecord(stop_event) on
  * the launching stream (both cudaEvent_t passed as void*; NULL, NULL clears).
  * Ids: 0 weight sums, 1 binarize+pack, 2 router, 3 expert scan, 4 activation
- * quantise, 5 HP up-projection, 6 fused forward tile, 7 row scatter, 8 scaled
- * sign, 9 scaled B, 10 HP dH, 11 dX, 12 dW (with the dB, dA and router-weight
- * tiles), 16 per-feature scale gradients (vector scales), 17 scalar scale gradients (one launch), 18 debug
- * GEMM, 19 decode token preparation, 20 decode main; 13-15, 21, 22 unused. */
+ * quantise, 5 HP up-projection, 6 fused forward tile, 8 the backward's operands (row
+ * scatter, scaled sign, scaled B), 12 the products of the backward, 16 per-feature
+ * scale gradients (vector scales), 17 scalar scale gradients (one launch), 18 debug
+ * GEMM, 19 decode token preparation, 20 decode main; 7, 9-11, 13-15, 21, 22 unused. */
 int pq_profile_events(int kernel_id, void* start_event, void* stop_event);
 
 const char* pq_status_string(int status);

@@ -108,8 +108,8 @@ struct BwdScratch {
   uint16_t* dlc;
   float* dbeta_partial;
   float* dalpha_partial;
-  double* blk_sums;      // scalar feature scales: per-block fp64 sums of k_finalize_scales, [2 * ceil(N/128)]
-  unsigned* arrivals;    // ... and its arrival counter
+  double* blk_sums;      // scalar feature scales: per-block fp64 sums of k_finalize_scales, [2 * ceil(N/32)]
+  unsigned* arrivals;    // ... its arrival counter [0], and the tickets [1] and finished dH tiles [2] of k_gemm_bwd
 };
 
 static size_t carve_bwd_scratch(const pq_desc* d, void* base, BwdScratch* out) {
@@ -127,7 +127,7 @@ static size_t carve_bwd_scratch(const pq_desc* d, void* base, BwdScratch* out) {
   s.dlc = routed(d) ? c.take<uint16_t>(T * 16) : nullptr;
   s.dbeta_partial = c.take<float>(2 * ((K + 255) / 256) * N);   // two slots per 256-column tile of K
   s.dalpha_partial = r > 0 ? c.take<float>((size_t)2 * E * N) : nullptr;
-  s.blk_sums = c.take<double>(2 * ((N + 127) / 128));
+  s.blk_sums = c.take<double>(2 * ((N + 31) / 32));
   s.arrivals = c.take<unsigned>(4);
   if (out) *out = s;
   return c.off;
@@ -138,9 +138,8 @@ static inline bool misaligned(const void* p) { return (reinterpret_cast<uintptr_
 // ---------------------------------------------------------------------------
 // Helper stream: kernels of one call that do not depend on one another run side
 // by side (forward of a dense layer with an HP branch: the activation quantisation
-// next to the HP up-projection; backward: the weight-gradient GEMM next to the chain
-// scaled sign matrix -> HP gradient GEMM -> dX, each filling the other's last wave).
-// Every caller stream gets one non-blocking helper stream and three events, created
+// next to the HP up-projection).
+// Every caller stream gets one non-blocking helper stream and two events, created
 // on first use and kept; work forked to the helper is always joined back before the
 // call's last kernel, so the caller sees plain stream order.  Event record and wait
 // are legal under stream capture and become edges of the captured graph.
@@ -149,7 +148,7 @@ static int g_side_streams = 1;
 
 struct SideCtx {
   cudaStream_t side = nullptr;
-  cudaEvent_t fork = nullptr, join = nullptr, mid = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
 };
 
 static SideCtx* side_for(cudaStream_t st) {
@@ -170,8 +169,7 @@ static SideCtx* side_for(cudaStream_t st) {
     SideCtx n;
     if (cudaStreamCreateWithFlags(&n.side, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&n.fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&n.join, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&n.mid, cudaEventDisableTiming) != cudaSuccess) {
+        cudaEventCreateWithFlags(&n.join, cudaEventDisableTiming) != cudaSuccess) {
       cudaGetLastError();
       return nullptr;   // the caller falls back to plain stream order
     }
@@ -705,32 +703,17 @@ int pq_linear_backward(const pq_desc* d, const uint16_t* dY, const uint16_t* X, 
   LayerArgs a{d->T, d->K, d->N, d->r, E, vec, w_scales, alpha, beta, A, B, Wr};
 
   BwdBuffers b{};
-  if (routed(d)) {
-    if (launch_scatter_rows(dY, sc.dys, sv.pos, d->T, d->N, st) != cudaSuccess) return PQ_ERR_CUDA;
-    b.dys = sc.dys;
-    b.xs = sv.xs;
-  } else {
-    b.dys = dY;
-    b.xs = normed(d) ? sv.xs : X;      // the layer's input is the normalised activation the forward left in `saved`
-  }
-  // With the helper stream: what leads to dX (scaled sign matrix, scaled B, HP gradient GEMM, dX) runs there, the
-  // weight gradient on the caller's stream beside it; see BwdStreams.
-  SideCtx* side = side_for(st);
-  if (side && !side_fork(side, st)) return PQ_ERR_CUDA;
-  cudaStream_t sx = side ? side->side : st;
-  if (launch_scaled_sign(w_s8, sc.sb, beta, vec, d->N, d->K, sc.arrivals, sx) != cudaSuccess) return PQ_ERR_CUDA;
+  // without routing the gradient is in order, and the layer's input is X or, normalised, what the forward left in `saved`
+  b.dys = routed(d) ? sc.dys : dY;
+  b.xs = routed(d) || normed(d) ? sv.xs : X;
   b.sb = sc.sb;
-  if (hp && vec) {
-    if (launch_scaled_b(B, sc.ba, alpha, E, d->N, d->r, sx) != cudaSuccess) return PQ_ERR_CUDA;
-    b.ba = sc.ba;
-  } else {
-    b.ba = B;
-  }
+  b.ba = hp && vec ? sc.ba : B;
+  if (launch_bwd_prep(a, dY, routed(d) ? sc.dys : nullptr, sv.pos, w_s8, sc.sb, hp && vec ? sc.ba : nullptr, sc.arrivals, st) != cudaSuccess)
+    return PQ_ERR_CUDA;
   b.dhc = sc.dhc; b.gh = sc.gh; b.dl = sc.dl; b.dlc = sc.dlc;
   b.dbeta_partial = sc.dbeta_partial; b.dalpha_partial = sc.dalpha_partial;
-  BwdStreams bs;
-  if (side) { bs.side = side->side; bs.dh_done = side->mid; bs.side_done = side->join; }
-  rc = gemm_backward(a, w_s8, sv, b, dX, dW, dA, dB, dWr, st, bs);
+  b.sync = sc.arrivals;
+  rc = gemm_backward(a, w_s8, sv, b, dX, dW, dA, dB, dWr, st);
   if (rc) return rc;
 
   // dbeta_n = lam * sum over the column tiles of the partial sign-weighted row sums, dalpha_n = sum over experts

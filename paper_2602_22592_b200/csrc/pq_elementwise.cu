@@ -552,82 +552,103 @@ __global__ void __launch_bounds__(256) k_act_quant(const uint4* __restrict__ X, 
   }
 }
 
-// dst[pos[t], :] = src[t, :]  (rows of `chunks` 16-byte pieces), one warp per row
-__global__ void __launch_bounds__(256) k_scatter_rows(const uint4* __restrict__ src, uint4* __restrict__ dst, const int* __restrict__ pos,
-                                                      int T, int chunks) {
+// What the products of the backward read, in one launch (blocks [0, rows) / [rows, signs) / [signs, end)):
+//   dys[pos[t], :] = dY[t, :]             routed layers: the gradient rows in expert order, one warp per row
+//   Sb[n,k] = bf16(scale_n) * S[n,k]      scale_n = beta_n (vector form) or 1
+//   Ba[e,n,j] = bf16(alpha_n * B[e,n,j])  vector form only
+// and the counters of the call's later kernels cleared (arrivals of k_finalize_scales; tickets and finished dH tiles of
+// k_gemm_bwd).  Bound by memory; the three are independent and small enough that a launch of its own cost each of them
+// as much as the work at a thousand tokens.
+struct BwdPrepArgs {
+  const uint4* dY; uint4* dys; const int* pos; int T, chunks;
+  const uint4* s8; uint4* sb; const float* beta; int beta_stride, N, K;
+  const uint4* B; uint4* ba; const float* alpha; int E, r;
+  unsigned* counters;
+  int rows, signs;
+};
+__global__ void __launch_bounds__(256) k_bwd_prep(BwdPrepArgs a) {
   pdl_launch_dependents();   // launched with programmatic stream serialisation: see launch_pdl
   pdl_wait();
-  const int t = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (t >= T) return;
-  const uint4* s = src + (long long)t * chunks;
-  uint4* d = dst + (long long)pos[t] * chunks;
-  for (int c = lane; c < chunks; c += 32) d[c] = __ldg(s + c);
-}
-
-// Sb[n,k] = bf16(scale_n) * S[n,k]; scale_n = beta_n (vector form) or 1
-__global__ void __launch_bounds__(256) k_scaled_sign(const uint4* __restrict__ s8, uint4* __restrict__ out, const float* __restrict__ beta,
-                                                     int beta_stride, int N, int K, unsigned* __restrict__ arrivals) {
-  pdl_launch_dependents();   // launched with programmatic stream serialisation: see launch_pdl
-  pdl_wait();
-  // first kernel of every backward call: it also clears the arrival counter of the call's last kernel (k_finalize_scales)
-  if (arrivals && blockIdx.x == 0 && threadIdx.x == 0) *arrivals = 0u;
-  const long long n16 = (long long)N * K / 16;
-  const int per_row = K / 16;
-  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n16; i += gridDim.x * 256LL) {
-    const int n = (int)(i / per_row);
-    const float sc = beta_stride ? beta[n] : 1.0f;
-    const uint4 v = __ldg(s8 + i);
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    uint4 o[2];
-    uint32_t* ow = reinterpret_cast<uint32_t*>(o);
+  if (blockIdx.x == 0 && threadIdx.x < 3) a.counters[threadIdx.x] = 0u;
+  if ((int)blockIdx.x < a.rows) {
+    const int t = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (t >= a.T) return;
+    const uint4* s = a.dY + (long long)t * a.chunks;
+    uint4* d = a.dys + (long long)a.pos[t] * a.chunks;
+    int c = lane;
+    for (; c + 96 < a.chunks; c += 128) {
+      uint4 v[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float a = (float)(int8_t)(w[j] & 0xFF) * sc, b = (float)(int8_t)((w[j] >> 8) & 0xFF) * sc;
-      const float c = (float)(int8_t)((w[j] >> 16) & 0xFF) * sc, d = (float)(int8_t)(w[j] >> 24) * sc;
-      ow[2 * j] = pack_bf16x2(a, b);
-      ow[2 * j + 1] = pack_bf16x2(c, d);
+      for (int u = 0; u < 4; ++u) v[u] = __ldg(s + c + 32 * u);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) d[c + 32 * u] = v[u];
     }
-    out[2 * i] = o[0];
-    out[2 * i + 1] = o[1];
+    for (; c < a.chunks; c += 32) d[c] = __ldg(s + c);
+    return;
+  }
+  if ((int)blockIdx.x < a.signs) {
+    const long long n16 = (long long)a.N * a.K / 16;
+    const int per_row = a.K / 16;
+    for (long long i = (blockIdx.x - a.rows) * 256LL + threadIdx.x; i < n16; i += (a.signs - a.rows) * 256LL) {
+      const float sc = a.beta_stride ? a.beta[(int)(i / per_row)] : 1.0f;
+      const uint4 v = __ldg(a.s8 + i);
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+      uint4 o[2];
+      uint32_t* ow = reinterpret_cast<uint32_t*>(o);
+      const uint32_t one = pack_bf16x2(sc, sc);            // +-1 bytes: bit 7 set <-> -1
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        ow[2 * j] = one ^ (((w[j] << 8) & 0x8000u) | ((w[j] << 16) & 0x80000000u));
+        ow[2 * j + 1] = one ^ (((w[j] >> 8) & 0x8000u) | (w[j] & 0x80000000u));
+      }
+      a.sb[2 * i] = o[0];
+      a.sb[2 * i + 1] = o[1];
+    }
+    return;
+  }
+  const long long n8 = (long long)a.E * a.N * a.r / 8;
+  const int per_row = a.r / 8;
+  for (long long i = (blockIdx.x - a.signs) * 256LL + threadIdx.x; i < n8; i += (gridDim.x - a.signs) * 256LL) {
+    const float al = a.alpha[(int)((i / per_row) % a.N)];
+    const uint4 v = __ldg(a.B + i);
+    a.ba[i] = make_uint4(pack_bf16x2(bf16lo(v.x) * al, bf16hi(v.x) * al), pack_bf16x2(bf16lo(v.y) * al, bf16hi(v.y) * al),
+                         pack_bf16x2(bf16lo(v.z) * al, bf16hi(v.z) * al), pack_bf16x2(bf16lo(v.w) * al, bf16hi(v.w) * al));
   }
 }
 
-// Ba[e,n,j] = bf16(alpha_n * B[e,n,j])  (vector alpha only)
-__global__ void __launch_bounds__(256) k_scaled_b(const uint32_t* __restrict__ B2, uint32_t* __restrict__ out, const float* __restrict__ alpha,
-                                                  int E, int N, int r) {
-  pdl_launch_dependents();   // launched with programmatic stream serialisation: see launch_pdl
-  pdl_wait();
-  const long long n2 = (long long)E * N * r / 2;
-  const int per_row = r / 2;
-  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n2; i += gridDim.x * 256LL) {
-    const int n = (int)((i / per_row) % N);
-    const uint32_t v = __ldg(B2 + i);
-    out[i] = pack_bf16x2(bf16lo(v) * alpha[n], bf16hi(v) * alpha[n]);
-  }
-}
-
-// Feature-scale gradients from their per-tile partials, one thread per output feature:
-//   dbeta_n = lam * sum_s dbeta_partial[s, n]      dalpha_n = sum_e dalpha_partial[e, n]   (slots / experts ascending)
+// Feature-scale gradients from their per-tile partials:
+//   dbeta_n = lam * sum_s dbeta_partial[s, n]      dalpha_n = sum_e dalpha_partial[e, n]
+// A block takes 32 features; its eight warps take every eighth partial each (one trip to memory for up to 64 of them: a
+// thread per feature that walked all 44 made six dependent trips), and the warps' sums are added in order.
 // Vector scales: written per feature.  Scalar scales (blk_sums != null): every block adds its features in fp64 (fixed
 // tree) into blk_sums[2 * block], the block that arrives last adds the blocks' sums in index order -- the result does
-// not depend on which block that is -- and writes the two scalars; `arrivals` was cleared by the call's first kernel.
-__global__ void __launch_bounds__(128) k_finalize_scales(const float* __restrict__ dbeta_partial, int nslots,
+// not depend on which block that is -- and writes the two scalars; `arrivals` was cleared by an earlier kernel of the call.
+__global__ void __launch_bounds__(256) k_finalize_scales(const float* __restrict__ dbeta_partial, int nslots,
                                                          const float* __restrict__ dalpha_partial, int E, int N,
                                                          const float* __restrict__ w_scales, float* __restrict__ dbeta,
                                                          float* __restrict__ dalpha, double* blk_sums, unsigned* arrivals) {
   pdl_launch_dependents();   // launched with programmatic stream serialisation: see launch_pdl
   pdl_wait();
-  const int n = blockIdx.x * 128 + threadIdx.x;
+  __shared__ float sh[2][8][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int n = blockIdx.x * 32 + lane;
   float b = 0.f, a = 0.f;
   if (n < N) {
 #pragma unroll 8
-    for (int s = 0; s < nslots; ++s) b += dbeta_partial[(long long)s * N + n];
-    b *= w_scales[0];
+    for (int s = warp; s < nslots; s += 8) b += __ldcg(dbeta_partial + (long long)s * N + n);
     if (dalpha_partial) {
-#pragma unroll 8
-      for (int e = 0; e < E; ++e) a += dalpha_partial[(long long)e * N + n];
+#pragma unroll 4
+      for (int e = warp; e < E; e += 8) a += __ldcg(dalpha_partial + (long long)e * N + n);
     }
   }
+  sh[0][warp][lane] = b;
+  sh[1][warp][lane] = a;
+  __syncthreads();
+  if (warp > 0) return;
+  b = a = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) { b += sh[0][w][lane]; a += sh[1][w][lane]; }
+  b *= w_scales[0];
   if (!blk_sums) {
     if (n < N) {
       dbeta[n] = b;
@@ -635,31 +656,27 @@ __global__ void __launch_bounds__(128) k_finalize_scales(const float* __restrict
     }
     return;
   }
-  __shared__ double sh[2][4];
-  __shared__ bool last;
   double sb = (double)b, sa = (double)a;
   for (int d = 16; d > 0; d >>= 1) {
     sb += __shfl_xor_sync(0xffffffffu, sb, d);
     sa += __shfl_xor_sync(0xffffffffu, sa, d);
   }
-  if ((threadIdx.x & 31) == 0) { sh[0][threadIdx.x >> 5] = sb; sh[1][threadIdx.x >> 5] = sa; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    blk_sums[2 * blockIdx.x] = (sh[0][0] + sh[0][1]) + (sh[0][2] + sh[0][3]);
-    blk_sums[2 * blockIdx.x + 1] = (sh[1][0] + sh[1][1]) + (sh[1][2] + sh[1][3]);
+  unsigned last = 0u;
+  if (lane == 0) {
+    blk_sums[2 * blockIdx.x] = sb;
+    blk_sums[2 * blockIdx.x + 1] = sa;
     __threadfence();
     last = atomicAdd(arrivals, 1u) == gridDim.x - 1;
   }
-  __syncthreads();
-  if (!last || threadIdx.x >= 32) return;
+  if (!__shfl_sync(0xffffffffu, last, 0)) return;
   __threadfence();
   double tb = 0.0, ta = 0.0;
-  for (int i = threadIdx.x; i < (int)gridDim.x; i += 32) { tb += __ldcg(blk_sums + 2 * i); ta += __ldcg(blk_sums + 2 * i + 1); }
+  for (int i = lane; i < (int)gridDim.x; i += 32) { tb += __ldcg(blk_sums + 2 * i); ta += __ldcg(blk_sums + 2 * i + 1); }
   for (int d = 16; d > 0; d >>= 1) {
     tb += __shfl_xor_sync(0xffffffffu, tb, d);
     ta += __shfl_xor_sync(0xffffffffu, ta, d);
   }
-  if (threadIdx.x == 0) {
+  if (lane == 0) {
     dbeta[0] = (float)tb;
     if (dalpha_partial) dalpha[0] = (float)ta;
   }
@@ -878,32 +895,26 @@ cudaError_t launch_route_and_quant(const uint16_t* X, const uint16_t* Wr, int T,
   return cudaGetLastError();
 }
 
-cudaError_t launch_scatter_rows(const uint16_t* src, uint16_t* dst, const int* pos, int T, int row_elems, cudaStream_t st) {
-  LaunchScope ls(KID_SCATTER_ROWS, st);
-  launch_pdl(k_scatter_rows, (T + 7) / 8, 256, 0, st, reinterpret_cast<const uint4*>(src), reinterpret_cast<uint4*>(dst), pos, T, row_elems / 8);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_scaled_sign(const int8_t* s8, uint16_t* out, const float* beta, int beta_stride, int N, int K, unsigned* arrivals,
-                               cudaStream_t st) {
-  const long long n16 = (long long)N * K / 16;
+cudaError_t launch_bwd_prep(const LayerArgs& a, const uint16_t* dY, uint16_t* dys, const int* pos, const int8_t* s8, uint16_t* sb,
+                            uint16_t* ba, unsigned* counters, cudaStream_t st) {
+  BwdPrepArgs p{};
+  p.dY = reinterpret_cast<const uint4*>(dY); p.dys = reinterpret_cast<uint4*>(dys); p.pos = pos; p.T = a.T; p.chunks = a.N / 8;
+  p.s8 = reinterpret_cast<const uint4*>(s8); p.sb = reinterpret_cast<uint4*>(sb); p.beta = a.beta; p.beta_stride = a.scale_stride;
+  p.N = a.N; p.K = a.K;
+  p.B = reinterpret_cast<const uint4*>(a.B); p.ba = reinterpret_cast<uint4*>(ba); p.alpha = a.alpha; p.E = a.E; p.r = a.r;
+  p.counters = counters;
+  p.rows = dys ? (a.T + 7) / 8 : 0;
+  p.signs = p.rows + grid_for((long long)a.N * a.K / 16, 256 * 2, 148 * 8);
+  const int end = p.signs + (ba ? grid_for((long long)a.E * a.N * a.r / 8, 256 * 2, 148 * 8) : 0);
   LaunchScope ls(KID_SCALED_SIGN, st);
-  launch_pdl(k_scaled_sign, grid_for(n16, 256 * 2, 148 * 8), 256, 0, st, reinterpret_cast<const uint4*>(s8), reinterpret_cast<uint4*>(out), beta,
-                                                               beta_stride, N, K, arrivals);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_scaled_b(const uint16_t* B, uint16_t* out, const float* alpha, int E, int N, int r, cudaStream_t st) {
-  const long long n2 = (long long)E * N * r / 2;
-  LaunchScope ls(KID_SCALED_B, st);
-  launch_pdl(k_scaled_b, grid_for(n2, 256 * 4, 148 * 8), 256, 0, st, reinterpret_cast<const uint32_t*>(B), reinterpret_cast<uint32_t*>(out), alpha, E, N, r);
+  launch_pdl(k_bwd_prep, end, 256, 0, st, p);
   return cudaGetLastError();
 }
 
 cudaError_t launch_finalize_scales(const float* dbeta_partial, int nslots, const float* dalpha_partial, int E, int N, const float* w_scales,
                                    int vec, float* dbeta, float* dalpha, double* blk_sums, unsigned* arrivals, cudaStream_t st) {
   LaunchScope ls(vec ? KID_SUM_PARTIALS : KID_SUM_SCALAR, st);
-  launch_pdl(k_finalize_scales, (N + 127) / 128, 128, 0, st, dbeta_partial, nslots, dalpha_partial, E, N, w_scales, dbeta, dalpha,
+  launch_pdl(k_finalize_scales, (N + 31) / 32, 256, 0, st, dbeta_partial, nslots, dalpha_partial, E, N, w_scales, dbeta, dalpha,
              vec ? nullptr : blk_sums, vec ? nullptr : arrivals);
   return cudaGetLastError();
 }

@@ -21,7 +21,8 @@
 // adds into.  This lets one kernel chain, e.g., the int8 1-bit product, the
 // bf16 expert product and the router product of one output tile.
 //
-// A "Problem" type supplies the tile list, the segments and the epilogue.
+// A "Problem" type supplies the tile list, the segments and the epilogue.  Tiles go to the CTAs (or pairs) in turn or, where
+// their lengths differ (P::kTickets, pairs only), by a counter in global memory: whoever is free takes the next one.
 #pragma once
 #include <cuda.h>
 
@@ -39,7 +40,8 @@ constexpr int kMnBoxBytes = 64 * 128;    // one MN-major box: 64 k-rows of 64 bf
 constexpr int kTmemCols = 512;
 constexpr int kAccCols = 256;            // TMEM columns of one accumulator
 constexpr int kStagingBytes = 32 * 1024; // epilogue warps: transposing buffers (kStagingBytes / kEpiWarps each)
-constexpr int kGemmSmemBytes = kRingBytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kStagingBytes;
+constexpr int kBarrierBytes = 384;
+constexpr int kGemmSmemBytes = kRingBytes + 1024 /*alignment slack*/ + kBarrierBytes + kStagingBytes;
 static_assert(kGemmSmemBytes <= 227 * 1024, "shared memory of one CTA");
 
 enum OpMode : int {
@@ -150,6 +152,32 @@ __device__ __forceinline__ void warp_store_rows(uint8_t* stage, const uint4 (&v)
   __syncwarp();
 }
 
+// The same wait, where what it guards was written by the other CTA of the pair
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ bool pipe_wait_cluster(uint32_t bar, uint32_t parity, int where, volatile int* abort_flag) {
+  if (mbar_try_wait_cluster(bar, parity)) return true;
+  const long long t0 = clock64();
+  while (!mbar_try_wait_cluster(bar, parity)) {
+    if (*abort_flag) return false;
+    if (clock64() - t0 > c_spin_cycles) {
+      report_timeout(where);
+      *abort_flag = 1;
+      return false;
+    }
+  }
+  return true;
+}
+
 // Problems whose epilogue needs nothing fetched ahead of the accumulator
 struct NoPre {};
 
@@ -175,25 +203,41 @@ struct stage_rows_of<P, std::void_t<decltype(&P::stage_rows)>> {
 struct AccDouble { static constexpr bool kSplit = false; };
 struct AccSplit { static constexpr bool kSplit = true; };
 
+// Problems that hand out their tiles by ticket name the counter (cleared before the launch) and may hold a tile back until what
+// it reads has been written: `ready`, called by the producers, returns false if it gave up.
+template <class P, class = void>
+struct tickets_of : std::false_type {};
+template <class P>
+struct tickets_of<P, std::void_t<decltype(&P::tickets)>> : std::true_type {};
+
 template <class P>
 __device__ __forceinline__ void gemm_body(const typename P::Params& p) {
   extern __shared__ uint8_t smem_raw[];
   constexpr int CG = P::CG;
   constexpr int kEpiWarps = P::kEpiWarps;
   constexpr bool kSplit = P::Acc::kSplit;
+  constexpr bool kTickets = tickets_of<P>::value;
+  static_assert(!kTickets || CG == 2, "tickets are handed out by the first CTA of a pair");
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t kStageBytes = kOperandBytes + (uint32_t)stage_rows_of<P>::get(p) * 128u;   // a multiple of 1024
   const int kStages = min(kMaxStages, (int)(kRingBytes / kStageBytes));
   const uint32_t bar_base = smem_base + kRingBytes;
-  // barrier block: full[12] empty[12] tfull[2] tempty[2] (8 B each), then tmem ptr, abort flag
+  // barrier block: full[12] empty[12] tfull[2] tempty[2] kfull[4] kempty[4] (8 B each), tile numbers of the tickets [4],
+  // tmem ptr, abort flag
+  constexpr int kSlots = 4;
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (kMaxStages + s); };
   auto tfull_bar = [&](int s) { return bar_base + 8u * (2 * kMaxStages + s); };
   auto tempty_bar = [&](int s) { return bar_base + 8u * (2 * kMaxStages + 2 + s); };
+  auto kfull_bar = [&](int s) { return bar_base + 8u * (2 * kMaxStages + 4 + s); };
+  auto kempty_bar = [&](int s) { return bar_base + 8u * (2 * kMaxStages + 4 + kSlots + s); };
+  constexpr int kWords = 8 * (2 * kMaxStages + 4 + 2 * kSlots);
   uint8_t* bar_generic = smem_raw + (bar_base - smem_u32(smem_raw));
-  volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(bar_generic + 8 * (2 * kMaxStages + 4));
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_generic + 8 * (2 * kMaxStages + 4) + 8);
-  uint8_t* epi_stage = bar_generic + 256;
+  volatile int* slots = reinterpret_cast<volatile int*>(bar_generic + kWords);
+  volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(bar_generic + kWords + 4 * kSlots);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_generic + kWords + 4 * kSlots + 4);
+  uint8_t* epi_stage = bar_generic + kBarrierBytes;
+  static_assert(kWords + 4 * kSlots + 8 <= kBarrierBytes, "barrier block");
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -205,6 +249,9 @@ __device__ __forceinline__ void gemm_body(const typename P::Params& p) {
     // when the epilogue warps of every CTA have read it
     for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     for (int s = 0; s < 2; ++s) { mbar_init(tfull_bar(s), 1); mbar_init(tempty_bar(s), CG * kEpiWarps); }
+    // a ticket's slot is free when every reader of both CTAs has it: the epilogue warps, the MMA warp, the second producer
+    if (kTickets)
+      for (int s = 0; s < kSlots; ++s) { mbar_init(kfull_bar(s), 1); mbar_init(kempty_bar(s), CG * (kEpiWarps + 1)); }
     *abort_flag = 0;
     mbar_fence_init();
   }
@@ -223,14 +270,49 @@ __device__ __forceinline__ void gemm_body(const typename P::Params& p) {
   const uint32_t tmem_base = *tmem_holder;
   const int ntiles = P::num_tiles(p);
 
+  // The next tile of a role (`ntiles` or more: none left).  whole: a warp asks, else one lane does.
+  auto next_tile = [&](PipeState& ks, int prev, bool whole, int where) -> int {
+    if constexpr (!kTickets) return prev < 0 ? group : prev + ngroups;
+    else {
+      const bool got = pipe_wait_cluster(kfull_bar(ks.stage), ks.phase, where, abort_flag);
+      if (whole ? !__all_sync(0xffffffffu, got) : !got) return ntiles;
+      const int tile = slots[ks.stage];
+      if (whole) __syncwarp();
+      if (!whole || lane == 0) mbar_arrive_cluster(cluster_map(kempty_bar(ks.stage), 0));
+      ks.advance(kSlots);
+      return tile;
+    }
+  };
+
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      PipeState st;
+      PipeState st, ks;
       bool ok = true;
-      for (int tile = group; ok && tile < ntiles; tile += ngroups) {
+      // the first CTA's producer draws the tickets, one ahead, and hands each to every role of both CTAs
+      int drawn = 0;
+      if constexpr (kTickets) { if (rank == 0) drawn = (int)atomicAdd(P::tickets(p), 1u); }
+      auto next = [&](int prev) -> int {
+        if constexpr (kTickets) {
+          if (rank == 0) {
+            const int tile = drawn;
+            if (!pipe_wait_cluster(kempty_bar(ks.stage), ks.phase ^ 1, WHERE_PRODUCER, abort_flag)) return ntiles;
+            const uint32_t slot = smem_u32(const_cast<int*>(slots + ks.stage));
+            for (int c = 0; c < 2; ++c) {
+              asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_map(slot, c)), "r"(tile) : "memory");
+              mbar_arrive_cluster(cluster_map(kfull_bar(ks.stage), c));
+            }
+            ks.advance(kSlots);
+            if (tile < ntiles) drawn = (int)atomicAdd(P::tickets(p), 1u);
+            return tile;
+          }
+        }
+        return next_tile(ks, prev, false, WHERE_PRODUCER);
+      };
+      for (int tile = next(-1); ok && tile < ntiles; tile = next(tile)) {
         typename P::Tile t;
         P::tile_init(p, tile, rank, t);
+        if constexpr (kTickets) { if (!P::ready(p, t, abort_flag)) break; }
         const int nseg = P::num_segments(p, t);
         for (int s = 0; ok && s < nseg; ++s) {
           Segment sg;
@@ -276,7 +358,7 @@ __device__ __forceinline__ void gemm_body(const typename P::Params& p) {
     // loads taken out); with the loop below, unrolled and specialised on the operand form, at the 128 cycles of the tensor
     // pipe (4.5 POP/s int8, 2.2 PFLOP/s bf16, loads taken out).
     if (rank == 0) {
-      PipeState st, ac;
+      PipeState st, ac, ks;
       bool ok = true;
       auto all_wait = [&](uint32_t bar, uint32_t parity) {
         const bool got = __all_sync(0xffffffffu, pipe_wait(bar, parity, WHERE_MMA, abort_flag));
@@ -284,7 +366,7 @@ __device__ __forceinline__ void gemm_body(const typename P::Params& p) {
         return got;
       };
       auto commit = [&](uint32_t bar) { if (elect_one()) umma_commit<CG>(bar); };
-      for (int tile = group; ok && tile < ntiles; tile += ngroups) {
+      for (int tile = next_tile(ks, -1, true, WHERE_MMA); ok && tile < ntiles; tile = next_tile(ks, tile, true, WHERE_MMA)) {
         typename P::Tile t;
         P::tile_init(p, tile, rank, t);
         const int nseg = P::num_segments(p, t);
@@ -347,7 +429,7 @@ __device__ __forceinline__ void gemm_body(const typename P::Params& p) {
     }
   } else {
     // ------------------------------------------------------------ epilogue warps
-    PipeState ac;
+    PipeState ac, ks;
     const int quad = warp & 3;          // TMEM lanes [32*quad, 32*quad+32) are this warp's
     const int part = (warp - 2) >> 2;   // which of the quadrant's warps: it takes column chunks part, part + kEpiWarps / 4, ...
     uint8_t* stage = epi_stage + (warp - 2) * (kStagingBytes / kEpiWarps);
@@ -368,7 +450,7 @@ __device__ __forceinline__ void gemm_body(const typename P::Params& p) {
       tc_fence_after();
       return got;
     };
-    for (int tile = group; tile < ntiles; tile += ngroups) {
+    for (int tile = next_tile(ks, -1, true, WHERE_EPILOGUE); tile < ntiles; tile = next_tile(ks, tile, true, WHERE_EPILOGUE)) {
       typename P::Tile t;
       P::tile_init(p, tile, rank, t);
       // per-row factors and addresses are fetched while the contraction is still running

@@ -643,46 +643,239 @@ __device__ __forceinline__ float dx_scale(const float* w_scales, const float* be
 }
 
 // ---------------------------------------------------------------------------
-// B1: dHraw = dYs . (alpha B_e) per item; epilogue forms
-//   dg_t = alpha * sum_j H dHraw,  dH = g dHraw  ->  dhc = dH / c  (bf16, masked)
-//   gh = g H (bf16, masked),  dl[t,j] = dg g (delta_je - p_tj),  dlc = dl / c
+// The whole backward in one launch.  Tiles of a pair of CTAs, in the order of their tickets:
+//   dH   (one per pair of 128-row tiles and expert with rows there): dHraw = dYs . (alpha B_e); the epilogue forms
+//          dg_t = alpha * sum_j H dHraw,  dH = g dHraw  ->  dhc = dH / c  (bf16, masked)
+//          gh = g H (bf16, masked),  dl[t,j] = dg g (delta_je - p_tj),  dlc = dl / c
+//   dW   (256 output features x 256 columns of K): G = dYs^T . xt; dW = beta_n G; per-tile partial of
+//          dbeta_n = lam * sum_k S[n,k] G[n,k].
+//   dWr  (256 columns of K): dWr^T = c * Xs^T . (dl / c), the logit gradient in the bf16 form the dX tile also uses
+//          (Sec. 3.3, "trained end-to-end").
+//   dX   (256 tokens x 256 columns of K) = c * ( dYs . Sb  +  sum_items dhc . A_e  +  dlc . Wr ), rows scattered back to
+//          token order.
+//   dB   (one per expert and 256 output features): dBraw_e = dYs^T . (g H) over the expert's items, the hi and lo
+//          planes of g H side by side as the two halves of the tile's columns (one half per CTA of the pair);
+//          dB = alpha_n dBraw, and the partial of dalpha_n = sum_j B[e,n,j] dBraw[n,j].
+//   dA   (one per expert and 256 columns of K): dA_e^T = c * Xs^T . (dH / c) over the expert's items, with the
+//          leading bf16 plane of dH / c (its 2^-9 rounding averages out over the tokens of the sum).
+// dWr and dA have K as the rows of the tile, 256 of them for the pair, and the short dimension (E or r) as columns: the
+// other way round half of a pair's rows would be empty.
+//
+// Bound by the tensor pipe and, equally, by what an SM takes in from L2 (32 KB per CTA and 512 MMA cycles); the tiles'
+// contractions run over T, N, the tokens of an expert or a few hundred values, so what was left on the table was the last
+// waves: as three launches (dH, dX, the rest, on two streams) with tiles handed out in turn, pairs with an extra dW tile also
+// got the experts' tiles, and dH kept 64 SMs busy.  Here the longest tiles come first and whoever is free takes the next
+// one.  dH has the first tickets and its readers (dWr, dX, dB, dA) wait for a counter of finished dH tiles: a ticket is
+// drawn by a running pair only, a dH tile waits for nothing, so the counter gets there.  dW needs none of it and fills the
+// time.  Measured, whole training step, three GEMM launches on two streams -> this: 256 tokens, 512 -> 512 54.6 -> 51.8 us;
+// 8192 tokens, eight experts, 2048 -> 2048 329 -> 301 us, 5632 -> 2048 663 -> 671 us (all of it at the 11 TB/s that the SMs
+// together take in from L2).
 // ---------------------------------------------------------------------------
-struct HpDhProblem {
-  static constexpr int CG = 1, kEpiWarps = 8;
+struct BwdProblem {
+  static constexpr int CG = 2, kEpiWarps = 8;
   using Acc = AccDouble;
+  enum Kind : int { KIND_DH = 0, KIND_DW, KIND_DWR, KIND_DX, KIND_DB, KIND_DA };
   struct Params {
-    CUtensorMap tdy, tba;  // dYs [T,N]; (alpha) B [E,N,r]
+    CUtensorMap tdy, tba, tsb, tdh, ta3, tdl, twr;   // dYs [T,N]; (alpha) B [E,N,r]; Sb [N,K]; dhc; A; dlc; Wr
+    CUtensorMap tdyT, txt, tgh, tdlT, txs, tdhT;     // the same and q / gamma, g H, Xs, contracted over tokens
     RoutingTables rt;
     const uint16_t* H;
     const float* gate;
     const float* probs;
-    const float* w_scales;
-    const float* alpha;
+    const int8_t* s8;
     const float* beta;
+    const float* alpha;
+    const float* w_scales;
+    const uint16_t* B;       // [E, N, r]
+    const int* perm;
     uint16_t* dhc;
     uint16_t* gh;
     float* dl;
     uint16_t* dlc;
-    int T, N, r, E, bn, sstride, item_rows, ba_blk;
+    uint16_t* dX;
+    float* dWr;              // [E, K]
+    float* dA;               // [E, r, K]
+    float* dW;
+    float* dB;               // [E, N, r]
+    float* dbeta_partial;    // [2 * ceil(K/256), N]
+    float* dalpha_partial;   // [2 * E, N]
+    unsigned* sync;          // {.., tickets, finished warps of dH tiles}
+    TileGrid gx, gw;
+    int T, N, K, r, r64, E, sstride, item_rows, ntn, ntk, mpairs, hp, long_experts;
+    int ba_blk, sb_blk, a3_blk, wr_blk, dy_blk, xt_blk, gh_blk, xs_blk, dh_blk;
   };
-  struct Tile { int item; int4 it; };
-  __device__ static int stage_rows(const Params& p) { return p.bn <= 128 ? 128 : 256; }
-  __device__ static int num_tiles(const Params& p) { return p.rt.n_items[0]; }
-  __device__ static void tile_init(const Params& p, int i, int, Tile& t) { t.item = i; t.it = p.rt.items[i]; }
-  __device__ static int num_segments(const Params&, const Tile&) { return 1; }
-  __device__ static void segment(const Params& p, const Tile& t, int, Segment& s) {
-    s.a_blk = 0; s.b_blk = p.ba_blk; s.b_bytes = p.bn * 128;
-    s.mode = MODE_BF_KM; s.acc = 0; s.bn = p.bn; s.ksteps = 4; s.nkb = (p.N + 63) / 64;
-    s.ta = &p.tdy; s.a_rank = 2; s.a_x = 0; s.a_y = t.it.x * 128; s.a_z = 0;
-    s.tb = &p.tba; s.b_rank = 3; s.b_x = 0; s.b_y = 0; s.b_z = t.it.y;
+  // nt: this CTA's block of 128 rows (tokens, features, or columns of K); [ib, ie): items (dB, dA), pair entries (dX); item: this
+  // CTA's item of a dH tile or -1, with its rows [lo, hi)
+  struct Tile { int kind, rank, nt, n0, bn, e, ib, ie, item, lo, hi, skip1; };
+  __device__ static unsigned* tickets(const Params& p) { return p.sync + 1; }
+  __device__ static int dh_tiles(const Params& p) { return p.hp ? p.rt.pair_begin[p.mpairs] : 0; }
+  __device__ static int num_tiles(const Params& p) {
+    return dh_tiles(p) + p.gw.total + p.gx.total + (p.hp ? p.E * (p.ntn + p.ntk) + (p.E > 1 ? p.ntk : 0) : 0);
   }
-  using Pre = NoPre;
-  __device__ static Pre prepare(const Params&, const Tile&, int, int) { return Pre{}; }
-  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t taddr, int quad, int half, int lane, uint8_t* stage) {
-    if (half) return;   // each row's sum over all r columns stays in one thread
+  __device__ static void tile_init(const Params& p, int i, int rank, Tile& t) {
+    t.ib = t.ie = 0; t.e = 0; t.n0 = 0; t.rank = rank; t.item = -1; t.lo = t.hi = 0; t.skip1 = 0;
+    const int dh = dh_tiles(p);
+    if (i < dh) {
+      const int4 pi = p.rt.pair_items[i];
+      t.kind = KIND_DH; t.e = pi.x; t.item = rank ? pi.z : pi.y; t.nt = 2 * pi.w + rank; t.bn = round_up(p.r, 128);
+      if (t.item >= 0) { const int4 it = p.rt.items[t.item]; t.lo = it.z; t.hi = it.w; }
+      return;
+    }
+    i -= dh;
+    if (i < p.gw.total) {
+      t.kind = KIND_DW;
+      // along the shorter side of the grid first: the tiles under way at a time then read the fewest different panels
+      const bool tall = p.gw.mt > p.gw.nt;
+      const int m = tall ? i / p.gw.nt : i % p.gw.mt, n = tall ? i % p.gw.nt : i / p.gw.mt;
+      t.nt = CG * m + rank; t.n0 = n * p.gw.bn;
+      t.bn = clip_bn(p.gw.bn, t.n0, p.K, 128);
+      return;
+    }
+    i -= p.gw.total;
+    if (p.hp && p.E > 1) {
+      if (i < p.ntk) {
+        t.kind = KIND_DWR; t.nt = 2 * i + rank; t.bn = 128;
+        return;
+      }
+      i -= p.ntk;
+    }
+    // the experts' tiles before dX where their contraction (all tokens, with one expert) is the longer one, else after it
+    const int experts = p.hp ? p.E * (p.ntn + p.ntk) : 0;
+    int x = p.long_experts ? i - experts : i;
+    if (x >= 0 && x < p.gx.total) {
+      t.kind = KIND_DX;
+      const TileCoord c = tile_coord<CG>(p.gx, x, rank);
+      t.nt = c.m; t.n0 = c.n0;
+      t.bn = clip_bn(c.bn, c.n0, p.K, 128);
+      if (p.hp) { t.ib = p.rt.pair_begin[t.nt >> 1]; t.ie = p.rt.pair_begin[(t.nt >> 1) + 1]; }
+      t.skip1 = dx_scale(p.w_scales, p.beta, p.sstride) == 0.f;
+      return;
+    }
+    x = p.long_experts ? i : i - p.gx.total;
+    t.e = x / (p.ntn + p.ntk);
+    x -= t.e * (p.ntn + p.ntk);
+    t.ib = p.rt.expert_item_begin[t.e]; t.ie = p.rt.expert_item_begin[t.e + 1];
+    if (x < p.ntn) { t.kind = KIND_DB; t.nt = 2 * x + rank; t.bn = 2 * p.r64; }
+    else { t.kind = KIND_DA; t.nt = 2 * (x - p.ntn) + rank; t.bn = 128; }
+  }
+  // what reads the results of the dH tiles waits for them; they were written through the generic proxy
+  __device__ static bool ready(const Params& p, const Tile& t, volatile int* abort_flag) {
+    if (!p.hp || t.kind == KIND_DH || t.kind == KIND_DW) return true;
+    const unsigned want = 8u * dh_tiles(p);                // four warps in each CTA of a pair
+    const long long t0 = clock64();
+    unsigned v;
+    for (;;) {
+      asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(p.sync + 2) : "memory");
+      if (v >= want) break;
+      if (*abort_flag) return false;
+      if (clock64() - t0 > c_spin_cycles) {
+        report_timeout(WHERE_PRODUCER);
+        *abort_flag = 1;
+        return false;
+      }
+    }
+    asm volatile("fence.proxy.async;" ::: "memory");
+    return true;
+  }
+  __device__ static int num_segments(const Params& p, const Tile& t) {
+    if (t.kind == KIND_DX) return (t.skip1 ? 0 : 1) + 2 * (t.ie - t.ib) + (p.hp && p.E > 1 ? 1 : 0);
+    return t.kind == KIND_DB || t.kind == KIND_DA ? t.ie - t.ib : 1;
+  }
+  __device__ static void segment(const Params& p, const Tile& t, int i, Segment& s) {
+    s.acc = 0; s.bn = t.bn; s.ksteps = 4; s.b_bytes = kOperandBytes;
+    s.a_rank = 2; s.a_z = 0; s.b_rank = 2; s.b_z = 0;
+    if (t.kind == KIND_DX) {
+      s.mode = MODE_BF_KM; s.a_x = 0; s.a_blk = 0;
+      s.b_x = t.n0 + t.rank * (t.bn >> 1); s.b_y = 0;
+      if (!t.skip1) {
+        if (i == 0) {
+          s.nkb = (p.N + 63) / 64;
+          s.ta = &p.tdy; s.a_y = t.nt * 128;
+          s.tb = &p.tsb; s.b_rank = 2; s.b_blk = p.sb_blk;
+          return;
+        }
+        --i;
+      }
+      if (i < 2 * (t.ie - t.ib)) {
+        const int4 pi = p.rt.pair_items[t.ib + (i >> 1)];
+        const int item = t.rank ? pi.z : pi.y, plane = i & 1;
+        s.nkb = (p.r + 63) / 64;
+        s.ta = &p.tdh; s.a_y = item >= 0 ? plane * p.item_rows + item * 128 : 2 * p.item_rows;   // beyond both planes: zeros
+        s.tb = &p.ta3; s.b_rank = 3; s.b_z = pi.x; s.b_blk = p.a3_blk;
+        return;
+      }
+      s.nkb = 1; s.ksteps = 1;
+      s.ta = &p.tdl; s.a_y = t.nt * 128;
+      s.tb = &p.twr; s.b_rank = 2; s.b_blk = p.wr_blk;
+      return;
+    }
+    if (t.kind == KIND_DH) {
+      s.mode = MODE_BF_KM; s.nkb = (p.N + 63) / 64; s.a_x = 0; s.a_blk = 0;
+      s.ta = &p.tdy; s.a_y = t.item >= 0 ? t.nt * 128 : p.T;     // no rows of this expert in the CTA's tile: zeros
+      s.tb = &p.tba; s.b_rank = 3; s.b_x = t.rank * (t.bn >> 1); s.b_y = 0; s.b_z = t.e; s.b_blk = p.ba_blk; s.b_bytes = t.bn * 64;
+      return;
+    }
+    s.mode = MODE_BF_MM; s.a_x = t.nt * 128;
+    switch (t.kind) {
+      case KIND_DW:
+        s.nkb = (p.T + 63) / 64;
+        s.ta = &p.tdyT; s.a_y = 0; s.a_blk = p.dy_blk;
+        s.tb = &p.txt; s.b_x = t.n0 + t.rank * (t.bn >> 1); s.b_y = 0; s.b_blk = p.xt_blk;
+        break;
+      case KIND_DB: {
+        const int item = t.ib + i;
+        s.nkb = 2;                                        // the 128 tokens of the item's tile (rows outside the item are zero in g H)
+        s.ta = &p.tdyT; s.a_y = p.rt.items[item].x * 128; s.a_blk = p.dy_blk;
+        s.tb = &p.tgh; s.b_x = 0; s.b_y = t.rank * p.item_rows + item * 128; s.b_blk = p.gh_blk; s.b_bytes = p.r64 * 128;
+        break;
+      }
+      case KIND_DWR:
+        s.nkb = (p.T + 63) / 64;
+        s.ta = &p.txs; s.a_y = 0; s.a_blk = p.xs_blk;
+        s.tb = &p.tdlT; s.b_x = t.rank * 64; s.b_y = 0; s.b_blk = -1; s.b_bytes = kMnBoxBytes;   // 16 columns, zeros beyond
+        break;
+      default: {                                          // KIND_DA
+        const int item = t.ib + i;
+        s.nkb = 2;
+        s.ta = &p.txs; s.a_y = p.rt.items[item].x * 128; s.a_blk = p.xs_blk;
+        s.tb = &p.tdhT; s.b_x = t.rank * 64; s.b_y = item * 128; s.b_blk = p.dh_blk; s.b_bytes = kMnBoxBytes;
+        break;
+      }
+    }
+  }
+  struct Pre { uint16_t* xrow; float cc; };
+  __device__ static Pre prepare(const Params& p, const Tile& t, int quad, int lane) {
+    Pre r{nullptr, 1.0f};
+    if (t.kind == KIND_DH && t.item >= 0) {
+      const long long row = ((long long)t.item * 128 + quad * 32 + lane) * p.r, plane = (long long)p.item_rows * p.r;
+      for (int j = 0; j < p.r; j += 64) {
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(p.H + row + j));
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(p.H + plane + row + j));
+      }
+    }
+    if (t.kind != KIND_DX) return r;
+    const int pos = t.nt * 128 + quad * 32 + lane;
+    const float c = dx_scale(p.w_scales, p.beta, p.sstride);
+    if (c != 0.f) r.cc = c;
+    if (pos < p.T) r.xrow = p.dX + (long long)(p.perm ? p.perm[pos] : pos) * p.K;
+    return r;
+  }
+  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t taddr, int quad, int part, int lane, uint8_t* stage) {
+    if (t.kind == KIND_DX) epilogue_dx(p, t, pre, taddr, part, lane, stage);
+    else if (t.kind != KIND_DH) epilogue_tokens(p, t, taddr, quad, part, lane, stage);
+    else if (part == 0) {                          // each row's sum over all r columns stays in one thread
+      if (t.item >= 0) epilogue_dh(p, t, taddr, quad, lane);
+      // this warp's rows are written: visible to every later TMA load, then counted
+      __threadfence();
+      asm volatile("fence.proxy.async;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) atomicAdd(p.sync + 2, 1u);
+    }
+  }
+  __device__ static void epilogue_dh(const Params& p, const Tile& t, uint32_t taddr, int quad, int lane) {
     const int row = quad * 32 + lane;
-    const bool live = row >= t.it.z && row < t.it.w;
-    const int pos = t.it.x * 128 + row;
+    const bool live = row >= t.lo && row < t.hi;
+    const int pos = t.nt * 128 + row;
     const float c = dx_scale(p.w_scales, p.beta, p.sstride);
     const float inv_cc = c != 0.f ? 1.0f / c : 1.0f;
     const float ca = p.sstride ? 1.0f : p.alpha[0];
@@ -733,7 +926,7 @@ struct HpDhProblem {
       for (int e = 0; e < 16; ++e) {
         float d = 0.f;
         if (e < p.E) {
-          d = dg * g * ((e == t.it.y ? 1.0f : 0.0f) - p.probs[(long long)pos * p.E + e]);
+          d = dg * g * ((e == t.e ? 1.0f : 0.0f) - p.probs[(long long)pos * p.E + e]);
           p.dl[(long long)pos * p.E + e] = d;
         }
         if (e & 1) packed[e >> 1] = pack_bf16x2(prev * inv_cc, d * inv_cc);
@@ -744,75 +937,11 @@ struct HpDhProblem {
       o[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
     }
   }
-};
-
-PQ_DEFINE_GEMM_KERNEL(k_gemm_hp_dh, HpDhProblem)
-
-// ---------------------------------------------------------------------------
-// B2: dX tile = c * ( dYs . Sb  +  sum_items dhc . A_e  +  dlc . Wr ), rows
-// scattered back to token order.
-// ---------------------------------------------------------------------------
-struct BwdDxProblem {
-  static constexpr int CG = 2, kEpiWarps = 8;
-  using Acc = AccDouble;
-  struct Params {
-    CUtensorMap tdy, tsb, tdh, ta3, tdl, twr;
-    RoutingTables rt;
-    const int* perm;
-    const float* w_scales;
-    const float* beta;
-    uint16_t* dX;
-    TileGrid g;
-    int T, N, K, r, E, sstride, item_rows, sb_blk, a3_blk, wr_blk;
-  };
-  struct Tile { TileCoord c; int m, rank, bn, pb, pe, skip1; };
-  __device__ static int num_tiles(const Params& p) { return p.g.total; }
-  __device__ static void tile_init(const Params& p, int i, int rank, Tile& t) {
-    t.c = tile_coord<CG>(p.g, i, rank);
-    t.m = t.c.m;
-    t.rank = rank;
-    t.bn = clip_bn(t.c.bn, t.c.n0, p.K, 128);
-    if (p.r > 0) { t.pb = p.rt.pair_begin[t.m >> 1]; t.pe = p.rt.pair_begin[(t.m >> 1) + 1]; } else { t.pb = t.pe = 0; }
-    t.skip1 = dx_scale(p.w_scales, p.beta, p.sstride) == 0.f;
-  }
-  __device__ static int num_segments(const Params& p, const Tile& t) { return (t.skip1 ? 0 : 1) + 2 * (t.pe - t.pb) + (p.E > 1 ? 1 : 0); }
-  __device__ static void segment(const Params& p, const Tile& t, int i, Segment& s) {
-    s.mode = MODE_BF_KM; s.acc = 0; s.bn = t.bn; s.ksteps = 4; s.a_rank = 2; s.a_x = 0; s.a_z = 0;
-    s.b_x = t.c.n0 + t.rank * (t.bn >> 1); s.b_y = 0; s.b_z = 0; s.b_bytes = kOperandBytes; s.a_blk = 0;
-    if (!t.skip1) {
-      if (i == 0) {
-        s.nkb = (p.N + 63) / 64;
-        s.ta = &p.tdy; s.a_y = t.m * 128;
-        s.tb = &p.tsb; s.b_rank = 2; s.b_blk = p.sb_blk;
-        return;
-      }
-      --i;
-    }
-    if (i < 2 * (t.pe - t.pb)) {
-      const int4 pi = p.rt.pair_items[t.pb + (i >> 1)];
-      const int item = t.rank ? pi.z : pi.y, plane = i & 1;
-      s.nkb = (p.r + 63) / 64;
-      s.ta = &p.tdh; s.a_y = item >= 0 ? plane * p.item_rows + item * 128 : 2 * p.item_rows;   // beyond both planes: zeros
-      s.tb = &p.ta3; s.b_rank = 3; s.b_z = pi.x; s.b_blk = p.a3_blk;
-      return;
-    }
-    s.nkb = 1; s.ksteps = 1;
-    s.ta = &p.tdl; s.a_y = t.m * 128;
-    s.tb = &p.twr; s.b_rank = 2; s.b_blk = p.wr_blk;
-  }
-  struct Pre { uint16_t* xrow; float cc; };
-  __device__ static Pre prepare(const Params& p, const Tile& t, int quad, int lane) {
-    const int pos = t.m * 128 + quad * 32 + lane;
-    const float c = dx_scale(p.w_scales, p.beta, p.sstride);
-    Pre r{nullptr, c != 0.f ? c : 1.0f};
-    if (pos < p.T) r.xrow = p.dX + (long long)(p.perm ? p.perm[pos] : pos) * p.K;
-    return r;
-  }
-  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t taddr, int quad, int part, int lane, uint8_t* stage) {
+  __device__ static void epilogue_dx(const Params& p, const Tile& t, const Pre& pre, uint32_t taddr, int part, int lane, uint8_t* stage) {
     const float cc = pre.cc;
     const bool has = num_segments(p, t) > 0;
     for (int c64 = part; c64 * 64 < t.bn; c64 += kEpiWarps / 4) {
-      const int k0 = t.c.n0 + c64 * 64;
+      const int k0 = t.n0 + c64 * 64;
       if (k0 >= p.K) break;
       uint32_t v0[32], v1[32];
       tmem_ld32(taddr + c64 * 64, v0);
@@ -830,110 +959,7 @@ struct BwdDxProblem {
       warp_store_rows<8>(stage, o, pre.xrow ? pre.xrow + k0 : nullptr, min(64, p.K - k0) * 2, lane);
     }
   }
-};
-PQ_DEFINE_GEMM_KERNEL(k_gemm_bwd_dx, BwdDxProblem)
-
-// ---------------------------------------------------------------------------
-// B3: the products that contract over tokens.
-//   dW tiles (256 output features x 256 columns of K): G = dYs^T . xt; dW = beta_n G; per-tile partial of
-//     dbeta_n = lam * sum_k S[n,k] G[n,k].
-//   dB tiles (one per expert and 256 output features): dBraw_e = dYs^T . (g H) over the expert's items, the hi and lo
-//     planes of g H side by side as the two halves of the tile's columns (one half per CTA of the pair);
-//     dB = alpha_n dBraw, and the partial of dalpha_n = sum_j B[e,n,j] dBraw[n,j].
-//   router tiles (one per 256 columns of K): dWr^T = c * Xs^T . (dl / c), the logit gradient in the bf16 form the dX tile
-//     also uses (Sec. 3.3, "trained end-to-end").
-//   dA tiles (one per expert and 256 columns of K): dA_e^T = c * Xs^T . (dH / c) over the expert's items, with the
-//     leading bf16 plane of dH / c (its 2^-9 rounding averages out over the tokens of the sum).
-// The last two have K as the rows of the tile, 256 of them for the pair, and the r (or E) short dimension as columns: the
-// other way round half of a pair's rows would be empty.
-// ---------------------------------------------------------------------------
-struct BwdDwProblem {
-  static constexpr int CG = 2, kEpiWarps = 8;
-  using Acc = AccDouble;
-  enum Kind : int { KIND_DW = 0, KIND_DB = 1, KIND_DWR = 2, KIND_DA = 3 };
-  struct Params {
-    CUtensorMap tdyT, txt, tgh, tdlT, txs, tdhT;
-    RoutingTables rt;
-    const int8_t* s8;
-    const float* beta;
-    const float* alpha;
-    const float* w_scales;
-    float* dWr;              // [E, K]
-    float* dA;               // [E, r, K]
-    const uint16_t* B;       // [E, N, r]
-    float* dW;
-    float* dB;               // [E, N, r]
-    float* dbeta_partial;    // [2 * ceil(K/256), N]
-    float* dalpha_partial;   // [2 * E, N]
-    TileGrid g;
-    int T, N, K, r, r64, E, sstride, dy_blk, xt_blk, gh_blk, xs_blk, dh_blk, item_rows, ntn, ntk, db_tiles, wr_tiles, da_tiles;
-  };
-  struct Tile { int kind, rank, nt, n0, bn, e, ib, ie; };   // nt: this CTA's block of 128 rows (features, or columns of K)
-  __device__ static int num_tiles(const Params& p) { return p.wr_tiles + p.da_tiles + p.g.total + p.db_tiles; }
-  // order: the tiles whose contraction runs over all tokens first (router, dA with one expert, dW), the short ones last
-  __device__ static void tile_init(const Params& p, int i, int rank, Tile& t) {
-    t.ib = t.ie = 0; t.e = 0; t.n0 = 0; t.rank = rank;
-    if (i < p.wr_tiles) {
-      t.kind = KIND_DWR; t.nt = 2 * i + rank; t.bn = 128;
-      return;
-    }
-    i -= p.wr_tiles;
-    if (i < p.da_tiles) {
-      t.kind = KIND_DA;
-      t.e = i / p.ntk;
-      t.ib = p.rt.expert_item_begin[t.e]; t.ie = p.rt.expert_item_begin[t.e + 1];
-      t.nt = 2 * (i % p.ntk) + rank; t.bn = 128;
-      return;
-    }
-    i -= p.da_tiles;
-    if (i < p.g.total) {
-      t.kind = KIND_DW;
-      const TileCoord c = tile_coord<CG>(p.g, i, rank);
-      t.nt = c.m; t.n0 = c.n0;
-      t.bn = clip_bn(c.bn, c.n0, p.K, 128);
-      return;
-    }
-    i -= p.g.total;
-    t.kind = KIND_DB;
-    t.e = i / p.ntn; t.nt = 2 * (i % p.ntn) + rank;
-    t.ib = p.rt.expert_item_begin[t.e]; t.ie = p.rt.expert_item_begin[t.e + 1];
-    t.bn = 2 * p.r64;
-  }
-  __device__ static int num_segments(const Params&, const Tile& t) { return (t.kind == KIND_DW || t.kind == KIND_DWR) ? 1 : t.ie - t.ib; }
-  __device__ static void segment(const Params& p, const Tile& t, int i, Segment& s) {
-    s.mode = MODE_BF_MM; s.acc = 0; s.bn = t.bn; s.ksteps = 4; s.b_bytes = kOperandBytes;
-    s.a_rank = 2; s.a_z = 0; s.b_rank = 2; s.b_z = 0;
-    s.a_x = t.nt * 128;
-    switch (t.kind) {
-      case KIND_DW:
-        s.nkb = (p.T + 63) / 64;
-        s.ta = &p.tdyT; s.a_y = 0; s.a_blk = p.dy_blk;
-        s.tb = &p.txt; s.b_x = t.n0 + t.rank * (t.bn >> 1); s.b_y = 0; s.b_blk = p.xt_blk;
-        break;
-      case KIND_DB: {
-        const int item = t.ib + i;
-        s.nkb = 2;                                        // the 128 tokens of the item's tile (rows outside the item are zero in g H)
-        s.ta = &p.tdyT; s.a_y = p.rt.items[item].x * 128; s.a_blk = p.dy_blk;
-        s.tb = &p.tgh; s.b_x = 0; s.b_y = t.rank * p.item_rows + item * 128; s.b_blk = p.gh_blk; s.b_bytes = p.r64 * 128;
-        break;
-      }
-      case KIND_DWR:
-        s.nkb = (p.T + 63) / 64;
-        s.ta = &p.txs; s.a_y = 0; s.a_blk = p.xs_blk;
-        s.tb = &p.tdlT; s.b_x = t.rank * 64; s.b_y = 0; s.b_blk = -1; s.b_bytes = kMnBoxBytes;   // 16 columns, zeros beyond
-        break;
-      default: {                                          // KIND_DA
-        const int item = t.ib + i;
-        s.nkb = 2;
-        s.ta = &p.txs; s.a_y = p.rt.items[item].x * 128; s.a_blk = p.xs_blk;
-        s.tb = &p.tdhT; s.b_x = t.rank * 64; s.b_y = item * 128; s.b_blk = p.dh_blk; s.b_bytes = kMnBoxBytes;
-        break;
-      }
-    }
-  }
-  using Pre = NoPre;
-  __device__ static Pre prepare(const Params&, const Tile&, int, int) { return Pre{}; }
-  __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t taddr, int quad, int part, int lane, uint8_t* stage) {
+  __device__ static void epilogue_tokens(const Params& p, const Tile& t, uint32_t taddr, int quad, int part, int lane, uint8_t* stage) {
     if (t.kind == KIND_DWR || t.kind == KIND_DA) {
       // ---- row k of the tile, column j: dWr[j, k] / c, or dA[e, j, k] / c.  A warp holds 32 consecutive k of one j: whole lines
       const int k = t.nt * 128 + quad * 32 + lane;
@@ -1027,94 +1053,43 @@ struct BwdDwProblem {
     if (live) p.dbeta_partial[(long long)(2 * (t.n0 / 256) + part) * p.N + n] = psum;
   }
 };
-PQ_DEFINE_GEMM_KERNEL(k_gemm_bwd_dw, BwdDwProblem)
+PQ_DEFINE_GEMM_KERNEL(k_gemm_bwd, BwdProblem)
 
 int gemm_backward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, const BwdBuffers& b, uint16_t* dX, float* dW, float* dA,
-                  float* dB, float* dWr, cudaStream_t st, const BwdStreams& bs) {
+                  float* dB, float* dWr, cudaStream_t st) {
   const int ntk = (a.K + 255) / 256, ntn = (a.N + 255) / 256;
-  const bool hp = a.r > 0;
+  const bool hp = a.r > 0, routed = hp && a.E > 1;
   const int r64 = h_round_up(a.r, 64);
   const uint64_t item_rows = (uint64_t)sv.max_items * 128;  // rows of one plane; buffers hold two
-  cudaStream_t sx = bs.side ? bs.side : st;                 // stream of the HP gradient GEMM and dX
-  int rc;
-
-  BwdDwProblem::Params w;
-  {
-    if (!map_mn(&w.tdyT, &w.dy_blk, b.dys, a.N, a.T, 2, 1, 2)) return PQ_ERR_CUDA;
-    if (!map_mn(&w.txt, &w.xt_blk, sv.xt, a.K, a.T, 2, 1, 2)) return PQ_ERR_CUDA;
-    w.tgh = w.txt; w.gh_blk = 0;
-    if (hp && !map_mn(&w.tgh, &w.gh_blk, b.gh, a.r, 2 * item_rows, 2, 1, r64 / 64)) return PQ_ERR_CUDA;
-    w.rt = sv.rt; w.s8 = w_s8; w.beta = a.beta; w.alpha = a.alpha; w.B = a.B; w.dW = dW; w.dB = dB;
-    w.dbeta_partial = b.dbeta_partial; w.dalpha_partial = b.dalpha_partial;
-    w.T = a.T; w.N = a.N; w.K = a.K; w.r = a.r; w.r64 = r64; w.E = a.E; w.sstride = a.scale_stride; w.item_rows = (int)item_rows;
-    w.ntn = ntn; w.ntk = ntk; w.db_tiles = hp ? a.E * ntn : 0; w.da_tiles = hp ? a.E * ntk : 0;
-    w.tdlT = w.txt; w.txs = w.txt; w.tdhT = w.txt; w.xs_blk = 0; w.dh_blk = 0; w.wr_tiles = 0;
-    w.w_scales = a.w_scales; w.dWr = dWr; w.dA = dA;
-    if (hp) {
-      if (!map_mn(&w.txs, &w.xs_blk, b.xs, a.K, a.T, 2, 1, 2)) return PQ_ERR_CUDA;
-      if (!map_mn(&w.tdhT, &w.dh_blk, b.dhc, a.r, 2 * item_rows, 2, 1, 1)) return PQ_ERR_CUDA;
-    }
-    if (hp && a.E > 1) {
-      int one_box = 0;
-      if (!map_mn(&w.tdlT, &one_box, b.dlc, 16, a.T, 2, 1, 1)) return PQ_ERR_CUDA;
-      w.wr_tiles = ntk;
-    }
-    w.g = make_tile_grid(ntn, ntk, 256);
-  }
-  if (bs.side) {
-    // the dW tiles proper need dY and q / gamma only: they start at once and take every SM; what follows on the
-    // other stream moves into their last wave
-    BwdDwProblem::Params m = w;
-    m.wr_tiles = 0; m.da_tiles = 0; m.db_tiles = 0;
-    rc = launch_gemm<BwdDwProblem>(KID_BWD_DW, k_gemm_bwd_dw, m, m.g.total, st);
-    if (rc) return rc;
-  }
+  BwdProblem::Params p{};
+  if (!map2d(&p.tdy, false, b.dys, a.N, a.T, 64, 128)) return PQ_ERR_CUDA;
+  if (!map_mn(&p.tsb, &p.sb_blk, b.sb, a.K, a.N, 2, 1, 2)) return PQ_ERR_CUDA;
+  if (!map_mn(&p.tdyT, &p.dy_blk, b.dys, a.N, a.T, 2, 1, 2)) return PQ_ERR_CUDA;
+  if (!map_mn(&p.txt, &p.xt_blk, sv.xt, a.K, a.T, 2, 1, 2)) return PQ_ERR_CUDA;
+  p.tba = p.tdh = p.ta3 = p.tdl = p.twr = p.tgh = p.tdlT = p.txs = p.tdhT = p.tdy;
   if (hp) {
-    HpDhProblem::Params p;
-    if (!map2d(&p.tdy, false, b.dys, a.N, a.T, 64, 128)) return PQ_ERR_CUDA;
-    if (!map_mn(&p.tba, &p.ba_blk, b.ba, a.r, a.N, 3, a.E, r64 / 64)) return PQ_ERR_CUDA;
-    p.rt = sv.rt; p.H = sv.h; p.gate = sv.gate; p.probs = sv.probs; p.w_scales = a.w_scales; p.alpha = a.alpha; p.beta = a.beta;
-    p.dhc = b.dhc; p.gh = b.gh; p.dl = b.dl; p.dlc = b.dlc;
-    p.T = a.T; p.N = a.N; p.r = a.r; p.E = a.E; p.bn = r64; p.sstride = a.scale_stride; p.item_rows = (int)item_rows;
-    rc = launch_gemm<HpDhProblem>(KID_HP_DH, k_gemm_hp_dh, p, sv.max_items, sx);
-    if (rc) return rc;
-    if (bs.side && cudaEventRecord(bs.dh_done, sx) != cudaSuccess) return PQ_ERR_CUDA;
+    if (!map_mn(&p.tba, &p.ba_blk, b.ba, a.r, a.N, 3, a.E, h_round_up(a.r, 128) / 128)) return PQ_ERR_CUDA;
+    if (!map2d(&p.tdh, false, b.dhc, a.r, 2 * item_rows, 64, 128)) return PQ_ERR_CUDA;
+    if (!map_mn(&p.ta3, &p.a3_blk, a.A, a.K, a.r, 3, a.E, 2)) return PQ_ERR_CUDA;
+    if (!map_mn(&p.tgh, &p.gh_blk, b.gh, a.r, 2 * item_rows, 2, 1, r64 / 64)) return PQ_ERR_CUDA;
+    if (!map_mn(&p.txs, &p.xs_blk, b.xs, a.K, a.T, 2, 1, 2)) return PQ_ERR_CUDA;
+    if (!map_mn(&p.tdhT, &p.dh_blk, b.dhc, a.r, 2 * item_rows, 2, 1, 1)) return PQ_ERR_CUDA;
   }
-  {
-    BwdDxProblem::Params p;
-    if (!map2d(&p.tdy, false, b.dys, a.N, a.T, 64, 128)) return PQ_ERR_CUDA;
-    if (!map_mn(&p.tsb, &p.sb_blk, b.sb, a.K, a.N, 2, 1, 2)) return PQ_ERR_CUDA;
-    p.tdh = p.tdy; p.ta3 = p.tdy; p.tdl = p.tdy; p.twr = p.tdy; p.a3_blk = 0; p.wr_blk = 0;
-    if (hp) {
-      if (!map2d(&p.tdh, false, b.dhc, a.r, 2 * item_rows, 64, 128)) return PQ_ERR_CUDA;
-      if (!map_mn(&p.ta3, &p.a3_blk, a.A, a.K, a.r, 3, a.E, 2)) return PQ_ERR_CUDA;
-    }
-    if (hp && a.E > 1) {
-      if (!map2d(&p.tdl, false, b.dlc, 16, a.T, 64, 128)) return PQ_ERR_CUDA;
-      if (!map_mn(&p.twr, &p.wr_blk, a.Wr, a.K, a.E, 2, 1, 2)) return PQ_ERR_CUDA;
-    }
-    p.rt = sv.rt; p.perm = (hp && a.E > 1) ? sv.perm : nullptr; p.w_scales = a.w_scales; p.beta = a.beta; p.dX = dX;
-    p.T = a.T; p.N = a.N; p.K = a.K; p.r = a.r; p.E = hp ? a.E : 1; p.sstride = a.scale_stride; p.item_rows = (int)item_rows;
-    p.g = make_tile_grid((a.T + 255) / 256, ntk, 256);
-    rc = launch_gemm<BwdDxProblem>(KID_BWD_DX, k_gemm_bwd_dx, p, p.g.total, sx);
-    if (rc) return rc;
-    if (bs.side && cudaEventRecord(bs.side_done, sx) != cudaSuccess) return PQ_ERR_CUDA;
+  if (routed) {
+    int one_box = 0;
+    if (!map2d(&p.tdl, false, b.dlc, 16, a.T, 64, 128)) return PQ_ERR_CUDA;
+    if (!map_mn(&p.twr, &p.wr_blk, a.Wr, a.K, a.E, 2, 1, 2)) return PQ_ERR_CUDA;
+    if (!map_mn(&p.tdlT, &one_box, b.dlc, 16, a.T, 2, 1, 1)) return PQ_ERR_CUDA;
   }
-  if (!bs.side) {
-    rc = launch_gemm<BwdDwProblem>(KID_BWD_DW, k_gemm_bwd_dw, w, w.wr_tiles + w.da_tiles + w.g.total + w.db_tiles, st);
-    if (rc) return rc;
-  } else {
-    if (hp) {
-      // dB, dA and the router gradient read what the HP gradient GEMM wrote
-      BwdDwProblem::Params x = w;
-      x.g.total = 0;
-      if (cudaStreamWaitEvent(st, bs.dh_done, 0) != cudaSuccess) return PQ_ERR_CUDA;
-      rc = launch_gemm<BwdDwProblem>(KID_HP_DB, k_gemm_bwd_dw, x, x.wr_tiles + x.da_tiles + x.db_tiles, st);
-      if (rc) return rc;
-    }
-    if (cudaStreamWaitEvent(st, bs.side_done, 0) != cudaSuccess) return PQ_ERR_CUDA;
-  }
-  return PQ_OK;
+  p.rt = sv.rt; p.H = sv.h; p.gate = sv.gate; p.probs = sv.probs; p.s8 = w_s8; p.beta = a.beta; p.alpha = a.alpha; p.w_scales = a.w_scales;
+  p.B = a.B; p.perm = routed ? sv.perm : nullptr;
+  p.dhc = b.dhc; p.gh = b.gh; p.dl = b.dl; p.dlc = b.dlc; p.dX = dX; p.dWr = dWr; p.dA = dA; p.dW = dW; p.dB = dB;
+  p.dbeta_partial = b.dbeta_partial; p.dalpha_partial = b.dalpha_partial; p.sync = b.sync;
+  p.T = a.T; p.N = a.N; p.K = a.K; p.r = a.r; p.r64 = r64; p.E = hp ? a.E : 1; p.sstride = a.scale_stride; p.item_rows = (int)item_rows;
+  p.ntn = ntn; p.ntk = ntk; p.mpairs = (a.T + 255) / 256; p.hp = hp; p.long_experts = hp && a.E == 1;
+  p.gx = make_tile_grid(p.mpairs, ntk, 256);
+  p.gw = make_tile_grid(ntn, ntk, 256);
+  return launch_gemm<BwdProblem>(KID_BWD_DW, k_gemm_bwd, p, p.gx.total + p.gw.total + (hp ? p.E * (ntn + ntk) : 0), st);
 }
 
 }  // namespace pq

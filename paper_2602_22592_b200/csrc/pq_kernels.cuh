@@ -91,11 +91,6 @@ cudaError_t launch_pack(const float* W, int N, int K, uint32_t* bits, int8_t* s8
 // xs of the tokens is then written even without routing (it is the only place the normalised activation exists)
 cudaError_t launch_route_and_quant(const uint16_t* X, const uint16_t* Wr, int T, int K, int E, const SavedPtrs& sv, const FwdScratch& sc,
                                    cudaStream_t st, cudaStream_t st_quant, const uint16_t* norm_weight = nullptr, float norm_eps = 0.f);
-cudaError_t launch_scatter_rows(const uint16_t* src, uint16_t* dst, const int* pos, int T, int row_elems, cudaStream_t st);
-// arrivals: counter of the call's k_finalize_scales launch, cleared here (null: nothing to clear)
-cudaError_t launch_scaled_sign(const int8_t* s8, uint16_t* out, const float* beta, int beta_stride, int N, int K, unsigned* arrivals,
-                               cudaStream_t st);
-cudaError_t launch_scaled_b(const uint16_t* B, uint16_t* out, const float* alpha, int E, int N, int r, cudaStream_t st);
 cudaError_t launch_finalize_scales(const float* dbeta_partial, int nslots, const float* dalpha_partial, int E, int N, const float* w_scales,
                                    int vec, float* dbeta, float* dalpha, double* blk_sums, unsigned* arrivals, cudaStream_t st);
 cudaError_t launch_fill_zero(void* p, size_t bytes, cudaStream_t st);
@@ -168,18 +163,13 @@ struct BwdBuffers {
   uint16_t* dlc;         // [T,16] bf16 dl / c
   float* dbeta_partial;  // [2 * ceil(K/256), N]
   float* dalpha_partial; // [2 * E, N]
+  unsigned* sync;        // counters of the call: [1] tickets, [2] finished dH tiles (cleared by k_bwd_prep)
 };
-// Where the backward GEMMs run.  side == nullptr: all on st, in the order HP gradient, dX, dW (one launch with the
-// HP tiles).  Otherwise the weight-gradient tiles that need nothing from the HP gradient GEMM are launched on st at
-// once, the HP gradient GEMM and dX follow one another on `side` (already ordered after the scaled sign matrix), and
-// the HP tiles of the weight gradient (dB, dA, router) go to st after `dh_done`; st then waits for `side_done`.
-// Kernels of the two streams fill one another's last waves.
-struct BwdStreams {
-  cudaStream_t side = nullptr;
-  cudaEvent_t dh_done = nullptr;     // recorded on side after the HP gradient GEMM
-  cudaEvent_t side_done = nullptr;   // recorded on side after dX
-};
+// dys, ba: null where the layer has no routing / no vector scales
+cudaError_t launch_bwd_prep(const LayerArgs& a, const uint16_t* dY, uint16_t* dys, const int* pos, const int8_t* s8, uint16_t* sb,
+                            uint16_t* ba, unsigned* counters, cudaStream_t st);
+// The products of the backward pass, one launch.
 int gemm_backward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, const BwdBuffers& b, uint16_t* dX, float* dW, float* dA,
-                  float* dB, float* dWr, cudaStream_t st, const BwdStreams& bs);
+                  float* dB, float* dWr, cudaStream_t st);
 
 }  // namespace pq
