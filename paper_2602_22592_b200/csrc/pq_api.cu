@@ -391,10 +391,14 @@ static int check_decode_item(const pq_desc* d, const uint16_t* X, const uint32_t
 }
 
 // hp_scales != nullptr: INT8 HP branch, A and B are int8 codes (training path only)
+// What the FFN form asks of a forward beyond a linear's: a second 1-bit matrix on the same codes, or an input that is still the
+// gate projection X and the up projection `up` (the product of the two is left in `mid`)
+struct FfnParts { SecondWeight second; const uint16_t* up = nullptr; uint16_t* mid = nullptr; };
+
 static int forward_impl(const pq_desc* d, const uint16_t* X, const uint32_t* w_bits, const int8_t* w_s8, const float* w_scales,
                         const uint16_t* A, const uint16_t* B, const float* hp_scales, const uint16_t* Wr, const float* alpha, const float* beta,
                         uint16_t* Y, void* saved, size_t saved_bytes, void* ws, size_t ws_bytes, void* stream, bool hp_ext = false,
-                        const uint16_t* norm_weight = nullptr, float norm_eps = 0.f) {
+                        const uint16_t* norm_weight = nullptr, float norm_eps = 0.f, const FfnParts& ffn = FfnParts{}) {
   if (!d || !X || !w_scales || !beta || !Y) return PQ_ERR_NULL;
   if (!w_s8) {
     if (hp_scales) return PQ_ERR_UNSUPPORTED;
@@ -451,11 +455,12 @@ static int forward_impl(const pq_desc* d, const uint16_t* X, const uint32_t* w_b
   // (with a fused norm the up-projection reads the normalised copy the quantiser writes, so it follows it)
   SideCtx* side = (d->r > 0 && !routed(d) && !hp_scales && !norm_weight) ? side_for(st) : nullptr;
   if (side && !side_fork(side, st)) return PQ_ERR_CUDA;
-  if (launch_route_and_quant(X, Wr, d->T, d->K, routed(d) ? E : 1, sv, sc, st, side ? side->side : st, norm_weight, norm_eps) != cudaSuccess)
+  if (launch_route_and_quant(X, Wr, d->T, d->K, routed(d) ? E : 1, sv, sc, st, side ? side->side : st, norm_weight, norm_eps,
+                             ffn.up, ffn.mid) != cudaSuccess)
     return PQ_ERR_CUDA;
   if (side && cudaEventRecord(side->join, side->side) != cudaSuccess) return PQ_ERR_CUDA;
   const uint16_t* xs = (routed(d) || norm_weight) ? sv.xs : X;
-  return gemm_forward(a, w_s8, sv, xs, Y, st, side ? side->join : nullptr);
+  return gemm_forward(a, w_s8, sv, xs, Y, st, side ? side->join : nullptr, ffn.second);
 }
 
 int pq_linear_forward(const pq_desc* d, const uint16_t* X, const uint32_t* w_bits, const int8_t* w_s8, const float* w_scales,
@@ -579,9 +584,11 @@ int pq_ffn_forward(const pq_ffn_desc* d, const uint16_t* X, const int8_t* g_s8, 
   if (rc) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const pq_desc dx = ffn_linear_desc(d, d->D, d->F1, 0), dd = ffn_linear_desc(d, d->F1, d->D, d->r);
-  // 1-bit FFN, gate projection: also leaves the int8 codes of x and the tile table in saved_x
+  // 1-bit FFN, gate and up projections: also leaves the int8 codes of x and the tile table in saved_x
+  FfnParts gate_up;
+  gate_up.second = SecondWeight{u_s8, u_scales, c.U1};
   rc = forward_impl(&dx, X, nullptr, g_s8, g_scales, nullptr, nullptr, nullptr, nullptr, nullptr, one, c.G1, c.saved_x, c.saved_x_bytes,
-                    c.ws_fwd, c.ws_fwd_bytes, stream);
+                    c.ws_fwd, c.ws_fwd_bytes, stream, false, nullptr, 0.f, gate_up);
   if (rc) return rc;
   // INT8 FFN: exact sums of its gate and up projections on those codes, then its hidden activation as codes, written
   // where the fused down projection expects the codes of h
@@ -589,21 +596,16 @@ int pq_ffn_forward(const pq_ffn_desc* d, const uint16_t* X, const int8_t* g_s8, 
   carve_saved(&dx, c.saved_x, &sx);
   carve_saved(&dd, c.saved_d, &sd);
   LayerArgs a8{d->T, d->D, d->D, d->r, 1, 0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  rc = gemm_hp_up8(a8, sx, G8, c.g_int, st);
-  if (rc) return rc;
-  rc = gemm_hp_up8(a8, sx, U8, c.u_int, st);
+  rc = gemm_hp_up8(a8, sx, G8, c.g_int, st, U8, c.u_int);
   if (rc) return rc;
   int8_t* qm = reinterpret_cast<int8_t*>(sd.h);
   float* gamma_m = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(sd.h) + align_up((size_t)sd.max_items * kTileRows * d->r));
   if (launch_ffn8_act(c.g_int, c.u_int, sx.gamma, hp_scales, d->T, d->r, qm, gamma_m, st) != cudaSuccess) return PQ_ERR_CUDA;
-  // 1-bit FFN, up projection and gate
-  rc = forward_impl(&dx, X, nullptr, u_s8, u_scales, nullptr, nullptr, nullptr, nullptr, nullptr, one, c.U1, c.saved_x, c.saved_x_bytes,
-                    c.ws_fwd, c.ws_fwd_bytes, stream);
-  if (rc) return rc;
-  if (launch_swiglu(c.G1, c.U1, c.M1, (long long)d->T * d->F1, st) != cudaSuccess) return PQ_ERR_CUDA;
+  FfnParts down;
+  down.up = c.U1; down.mid = c.M1;
   // down projections of both FFNs in one fused tile: beta (lam / gamma) (q(M1) . S_d) + alpha (D8 qm) / (gamma_D gamma_m)
-  return forward_impl(&dd, c.M1, nullptr, d_s8, d_scales, reinterpret_cast<const uint16_t*>(D8), reinterpret_cast<const uint16_t*>(D8),
-                      hp_scales + 1, nullptr, alpha, beta, Y, c.saved_d, c.saved_d_bytes, c.ws_fwd, c.ws_fwd_bytes, stream, true);
+  return forward_impl(&dd, c.G1, nullptr, d_s8, d_scales, reinterpret_cast<const uint16_t*>(D8), reinterpret_cast<const uint16_t*>(D8),
+                      hp_scales + 1, nullptr, alpha, beta, Y, c.saved_d, c.saved_d_bytes, c.ws_fwd, c.ws_fwd_bytes, stream, true, nullptr, 0.f, down);
 }
 
 int pq_decode_pack_bytes(const pq_desc* d, size_t* bits_il_bytes, size_t* b_il_bytes) {

@@ -443,17 +443,34 @@ __global__ void __launch_bounds__(512) k_route_scan(int T, int E, int nblocks, c
 // stable): q (int8), xt = q / gamma (bf16, the backward's operand) and, with
 // routing, a bf16 copy of the row itself plus its gate and probabilities.
 // ---------------------------------------------------------------------------
+// Hidden activation of the 1-bit FFN (Eq. 11): bf16(silu(g) * u), element by element (fp32)
+__device__ __forceinline__ uint4 swiglu8(const uint4& g, const uint4& u) {
+  const uint32_t gw[4] = {g.x, g.y, g.z, g.w}, uw[4] = {u.x, u.y, u.z, u.w};
+  uint32_t o[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float g0 = bf16lo(gw[j]), g1 = bf16hi(gw[j]);
+    o[j] = pack_bf16x2(g0 / (1.0f + __expf(-g0)) * bf16lo(uw[j]), g1 / (1.0f + __expf(-g1)) * bf16hi(uw[j]));
+  }
+  return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+// SWIGLU: the row is made from gate and up (X = gate) on the way in and left in `mid`, instead of by a kernel that writes it for
+// this one to read back: 2048 tokens x 5504 13.9 + 11.3 us as two launches, 22.5 us as one.
 // WPR warps share one token row.  CH > 0: every lane keeps its CH 16-byte pieces of the row in registers
 // between the absmax pass and the quantising pass (rows of up to 256 * CH * WPR elements), so X is read
 // once; CH = 0 reads the row twice.
-template <int CH, int WPR>
-__global__ void __launch_bounds__(256) k_act_quant(const uint4* __restrict__ X, int T, int K, int E, const int* __restrict__ expert,
+// Bound by memory (routed training layer: 7 bytes written and 2 read per value), and to reach it by the rows in flight: four
+// pieces per lane and as many warps per row as that takes leave room for five blocks per SM.  Eight pieces per lane (two blocks)
+// and four, routed: 8192 x 2048 21.2 -> 17.3 us, 8192 x 5632 67 -> 58 us (5.6 TB/s); with the SwiGLU 38 -> 22.5 us.
+template <int CH, int WPR, bool SWIGLU = false>
+__global__ void __launch_bounds__(256, CH > 0 ? 5 : 2) k_act_quant(const uint4* __restrict__ X, int T, int K, int E, const int* __restrict__ expert,
                                                    const int* __restrict__ block_base, const int* __restrict__ offsets,
                                                    const float* __restrict__ gate_tok, const float* __restrict__ probs_tok,
                                                    uint2* __restrict__ q, uint4* __restrict__ xt, uint4* __restrict__ xs,
                                                    float* __restrict__ gamma_s, float* __restrict__ gate_s, float* __restrict__ probs_s,
                                                    int* __restrict__ perm, int* __restrict__ pos, const uint4* __restrict__ norm_w,
-                                                   const float* __restrict__ rms) {
+                                                   const float* __restrict__ rms, const uint4* __restrict__ up, uint4* __restrict__ mid) {
   pdl_launch_dependents();   // launched with programmatic stream serialisation: see launch_pdl
   pdl_wait();
   __shared__ float amax_sh[8];
@@ -468,6 +485,11 @@ __global__ void __launch_bounds__(256) k_act_quant(const uint4* __restrict__ X, 
   const float srow = norm_w ? rms[t] : 1.0f;
   auto fetch_x = [&](int c) {                      // with a fused RMSNorm every later step sees the normalised token
     const uint4 v = __ldg(xrow + c);
+    if (SWIGLU) {
+      const uint4 m = swiglu8(v, __ldg(up + (long long)t * chunks + c));
+      if (valid) mid[(long long)t * chunks + c] = m;
+      return m;
+    }
     return norm_w ? rms_apply(v, srow, __ldg(norm_w + c)) : v;
   };
   uint4 held[CH > 0 ? CH : 1];
@@ -754,25 +776,9 @@ cudaError_t launch_pack_experts(const uint16_t* A, const uint16_t* B, int E, int
 }
 
 // ---------------------------------------------------------------------------
-// FFN-level decoupling (Eq. 11): the two small kernels between the projections.
+// FFN-level decoupling (Eq. 11): the small kernel between the INT8 FFN's projections (the 1-bit FFN's is part of
+// the quantiser).
 // ---------------------------------------------------------------------------
-// Hidden activation of the 1-bit FFN: M = bf16(silu(G) * U), element by element (fp32).
-__global__ void __launch_bounds__(256) k_swiglu(const uint4* __restrict__ G, const uint4* __restrict__ U, uint4* __restrict__ M, long long n8) {
-  pdl_launch_dependents();
-  pdl_wait();
-  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n8; i += gridDim.x * 256LL) {
-    const uint4 g = __ldg(G + i), u = __ldg(U + i);
-    const uint32_t gw[4] = {g.x, g.y, g.z, g.w}, uw[4] = {u.x, u.y, u.z, u.w};
-    uint32_t o[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float g0 = bf16lo(gw[j]), g1 = bf16hi(gw[j]);
-      o[j] = pack_bf16x2(g0 / (1.0f + __expf(-g0)) * bf16lo(uw[j]), g1 / (1.0f + __expf(-g1)) * bf16hi(uw[j]));
-    }
-    M[i] = make_uint4(o[0], o[1], o[2], o[3]);
-  }
-}
-
 // Hidden activation of the INT8 FFN, one warp per token: from the exact sums g_int = G8 q, u_int = U8 q
 //   g = fl(fl(g_int) * fl(1 / fl(gamma_G gamma_t))), u likewise, m = fl(fl(g * s) * u) with the logistic factor s taken
 //   in fp64 and rounded once to fp32 (an fp32 exponential would not be reproducible, and m feeds a quantiser),
@@ -808,15 +814,6 @@ __global__ void __launch_bounds__(256) k_ffn8_act(const int* __restrict__ g_int,
     const int j = lane + 32 * k;
     if (j < r) qm[(long long)t * r + j] = (int8_t)max(-128, min(127, __float2int_rn(__fmul_rn(m[k], gm))));
   }
-}
-
-cudaError_t launch_swiglu(const uint16_t* G, const uint16_t* U, uint16_t* M, long long n, cudaStream_t st) {
-  const long long n8 = n / 8;
-  long long g = (n8 + 1023) / 1024;
-  launch_pdl(k_swiglu, (int)(g < 1 ? 1 : (g > 148 * 8 ? 148 * 8 : g)), 256, 0, st, reinterpret_cast<const uint4*>(G), reinterpret_cast<const uint4*>(U),
-             reinterpret_cast<uint4*>(M), n8);
-  ++g_launches;
-  return cudaGetLastError();
 }
 
 cudaError_t launch_ffn8_act(const int* g_int, const int* u_int, const float* gamma, const float* hp_scales, int T, int r, int8_t* qm,
@@ -855,7 +852,7 @@ cudaError_t launch_pack(const float* W, int N, int K, uint32_t* bits, int8_t* s8
 }
 
 cudaError_t launch_route_and_quant(const uint16_t* X, const uint16_t* Wr, int T, int K, int E, const SavedPtrs& sv, const FwdScratch& sc,
-                                   cudaStream_t st, cudaStream_t st_quant, const uint16_t* norm_weight, float norm_eps) {
+                                   cudaStream_t st, cudaStream_t st_quant, const uint16_t* norm_weight, float norm_eps, const uint16_t* up, uint16_t* mid) {
   if (E > 1) st_quant = st;   // the sorted position of a token comes from the router and the scan
   const uint4* nw = reinterpret_cast<const uint4*>(norm_weight);
   if (nw) {
@@ -882,16 +879,17 @@ cudaError_t launch_route_and_quant(const uint16_t* X, const uint16_t* Wr, int T,
   launch_pdl(k_route_scan, 1, 512, 0, st, T, E, nblocks, sc.block_counts, sc.block_base, sv.offsets, sv.rt); }
   LaunchScope ls(KID_ACT_QUANT, st_quant);
   const int per_lane = (K / 8 + 31) / 32;   // 16-byte pieces of a row per lane if one warp took the whole row
-  auto kern = k_act_quant<0, 1>;
+  auto kern = up ? k_act_quant<0, 1, true> : k_act_quant<0, 1>;
   int wpr = 1;
-  if (per_lane <= 4) kern = k_act_quant<4, 1>;
-  else if (per_lane <= 8) kern = k_act_quant<8, 1>;
-  else if (per_lane <= 16) { kern = k_act_quant<8, 2>; wpr = 2; }
-  else if (per_lane <= 32) { kern = k_act_quant<8, 4>; wpr = 4; }
+  if (per_lane <= 4) kern = up ? k_act_quant<4, 1, true> : k_act_quant<4, 1>;
+  else if (per_lane <= 8) { kern = up ? k_act_quant<4, 2, true> : k_act_quant<4, 2>; wpr = 2; }
+  else if (per_lane <= 16) { kern = up ? k_act_quant<4, 4, true> : k_act_quant<4, 4>; wpr = 4; }
+  else if (per_lane <= 32) { kern = up ? k_act_quant<4, 8, true> : k_act_quant<4, 8>; wpr = 8; }
   const int rows_per_block = 8 / wpr;
   launch_pdl(kern, (T + rows_per_block - 1) / rows_per_block, 256, 0, st_quant, reinterpret_cast<const uint4*>(X), T, K, E, sv.expert, sc.block_base, sv.offsets, sc.gate_tok,
                                     sc.probs_tok, reinterpret_cast<uint2*>(sv.q), reinterpret_cast<uint4*>(sv.xt),
-                                    reinterpret_cast<uint4*>(sv.xs), sv.gamma, sv.gate, sv.probs, sv.perm, sv.pos, nw, sc.rms);
+                                    reinterpret_cast<uint4*>(sv.xs), sv.gamma, sv.gate, sv.probs, sv.perm, sv.pos, nw, sc.rms,
+                                    reinterpret_cast<const uint4*>(up), reinterpret_cast<uint4*>(mid));
   return cudaGetLastError();
 }
 

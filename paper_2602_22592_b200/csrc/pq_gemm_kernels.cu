@@ -287,29 +287,33 @@ struct HpUp8Problem {
   static constexpr int CG = 1, kEpiWarps = 8;
   using Acc = AccDouble;
   struct Params {
-    CUtensorMap tq, ta;  // q sorted [T,K] s8; A8 [E,r,K] s8
+    CUtensorMap tq, ta, tb;  // q sorted [T,K] s8; A8 [E,r,K] s8, twice
     RoutingTables rt;
     int8_t* qh;
     float* gamma_h;
     int* raw;            // not null: write the exact sums h_int [items*128, r] instead of codes (the caller quantises later)
+    int* rawb;           // sums of the second matrix (an FFN's gate and up projections in one launch), or null
     int K, r, rp, bn;
   };
-  struct Tile { int item; int4 it; };
+  struct Tile { int item, second; int4 it; };
   __device__ static int stage_rows(const Params& p) { return p.bn <= 128 ? 128 : 256; }
-  __device__ static int num_tiles(const Params& p) { return p.rt.n_items[0]; }
-  __device__ static void tile_init(const Params& p, int i, int, Tile& t) { t.item = i; t.it = p.rt.items[i]; }
+  __device__ static int num_tiles(const Params& p) { return p.rt.n_items[0] * (p.rawb ? 2 : 1); }
+  __device__ static void tile_init(const Params& p, int i, int, Tile& t) {
+    const int n = p.rt.n_items[0];
+    t.second = i >= n; t.item = t.second ? i - n : i; t.it = p.rt.items[t.item];
+  }
   __device__ static int num_segments(const Params&, const Tile&) { return 1; }
   __device__ static void segment(const Params& p, const Tile& t, int, Segment& s) {
     s.mode = MODE_I8_KK; s.acc = 0; s.bn = p.bn; s.ksteps = 4; s.nkb = (p.K + 127) / 128;
     s.ta = &p.tq; s.a_rank = 2; s.a_x = 0; s.a_y = t.it.x * 128; s.a_z = 0;
-    s.tb = &p.ta; s.b_rank = 3; s.b_x = 0; s.b_y = 0; s.b_z = t.it.y;
+    s.tb = t.second ? &p.tb : &p.ta; s.b_rank = 3; s.b_x = 0; s.b_y = 0; s.b_z = t.it.y;
     s.b_bytes = p.bn * 128; s.a_blk = 0; s.b_blk = 0;
   }
   using Pre = NoPre;
   __device__ static Pre prepare(const Params&, const Tile&, int, int) { return Pre{}; }
   __device__ static void epilogue(const Params& p, const Tile& t, const Pre& pre, uint32_t taddr, int quad, int half, int lane, uint8_t* stage) {
     if (p.raw) {
-      int* out = p.raw + ((long long)t.item * 128 + quad * 32 + lane) * p.r;
+      int* out = (t.second ? p.rawb : p.raw) + ((long long)t.item * 128 + quad * 32 + lane) * p.r;
       for (int c = half; c * 32 < p.r; c += 2) {
         uint32_t v[32];
         tmem_ld32(taddr + c * 32, v);
@@ -376,7 +380,7 @@ struct FwdProblem {
   static constexpr int CG = 2, kEpiWarps = HP ? 16 : 8;
   using Acc = typename std::conditional<HP, AccSplit, AccDouble>::type;
   struct Params {
-    CUtensorMap tq, ts, th, tb;  // q [T,K] s8; S [N,K] s8; H [items*128,r]; B [E,N,r]
+    CUtensorMap tq, ts, ts2, th, tb;  // q [T,K] s8; S [N,K] s8, of a second matrix too; H [items*128,r]; B [E,N,r]
     RoutingTables rt;
     TileGrid g;
     const int* perm;
@@ -391,13 +395,18 @@ struct FwdProblem {
     const float* gamma_h;    // [items*128], null for the bf16 branch
     const float* hp_scales;  // [E][2] = {gamma_A, gamma_B}
     int hp_ext;              // the codes of h and gamma_h were written by the caller
-    int T, N, K, r, sstride, item_rows;
+    // without an HP branch: a second matrix of the same sizes, whose column tiles follow those of the first (`tiles1` of them)
+    const float* w_scales2;
+    uint16_t* Y2;
+    int T, N, K, r, sstride, item_rows, tiles1;
   };
-  struct Tile { TileCoord c; int bn, pb, pe, rank; };
+  struct Tile { TileCoord c; int bn, pb, pe, rank, second; };
   __device__ static int num_tiles(const Params& p) { return p.g.total; }
   __device__ static void tile_init(const Params& p, int i, int rank, Tile& t) {
     t.c = tile_coord<CG>(p.g, i, rank);
     t.rank = rank;
+    t.second = !HP && t.c.n0 >= p.tiles1 * p.g.bn;
+    if (t.second) t.c.n0 -= p.tiles1 * p.g.bn;
     t.bn = clip_bn(t.c.bn, t.c.n0, p.N, 32);
     if (HP) { t.pb = p.rt.pair_begin[t.c.m >> 1]; t.pe = p.rt.pair_begin[(t.c.m >> 1) + 1]; } else { t.pb = t.pe = 0; }
   }
@@ -410,7 +419,7 @@ struct FwdProblem {
     if (i == t.pe - t.pb) {
       s.mode = MODE_I8_KK; s.acc = 0; s.nkb = (p.K + 127) / 128;
       s.ta = &p.tq; s.a_rank = 2; s.a_x = 0; s.a_y = t.c.m * 128;
-      s.tb = &p.ts; s.b_rank = 2;
+      s.tb = t.second ? &p.ts2 : &p.ts; s.b_rank = 2;
     } else {
       const int4 pi = p.rt.pair_items[t.pb + i];
       const int item = t.rank ? pi.z : pi.y;
@@ -453,8 +462,8 @@ struct FwdProblem {
     Pre r{nullptr, 0.f, 0.f};
     if (pos < p.T) {
       const int token = p.perm ? p.perm[pos] : pos;
-      r.yrow = p.Y + (long long)token * p.N;
-      r.cb = __fdiv_rn(p.w_scales[0], p.gamma[pos]);
+      r.yrow = (t.second ? p.Y2 : p.Y) + (long long)token * p.N;
+      r.cb = __fdiv_rn((t.second ? p.w_scales2 : p.w_scales)[0], p.gamma[pos]);
       if (HP) r.ca = p.gate[pos];
       if (HP && p.gamma_h) {
         // the item of this row: its expert's weight scales and the row's own hidden scale
@@ -571,11 +580,13 @@ static inline float* hp8_gamma_h(const SavedPtrs& sv, int r) {
 // the fused output tile of a layer, with or without an HP branch
 template <bool HP, bool GEN>
 static int launch_forward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, uint16_t* Y, void (*kernel)(typename FwdProblem<HP, GEN>::Params),
-                          cudaStream_t st) {
+                          cudaStream_t st, const SecondWeight& second) {
   using P = FwdProblem<HP, GEN>;
   typename P::Params f;
   if (!map2d(&f.tq, true, sv.q, a.K, a.T, 128, 128)) return PQ_ERR_CUDA;
   if (!map2d(&f.ts, true, w_s8, a.K, a.N, 128, 128)) return PQ_ERR_CUDA;
+  f.ts2 = f.ts; f.w_scales2 = second.w_scales; f.Y2 = second.Y;
+  if (second.w_s8 && !map2d(&f.ts2, true, second.w_s8, a.K, a.N, 128, 128)) return PQ_ERR_CUDA;
   f.th = f.tq; f.tb = f.tq;
   f.gamma_h = nullptr; f.hp_scales = a.hp_scales; f.hp_ext = a.hp_ext ? 1 : 0;
   if (HP && a.hp_scales) {
@@ -591,23 +602,26 @@ static int launch_forward(const LayerArgs& a, const int8_t* w_s8, const SavedPtr
   f.rt = sv.rt; f.perm = (HP && a.E > 1) ? sv.perm : nullptr; f.gamma = sv.gamma; f.gate = sv.gate; f.w_scales = a.w_scales;
   f.alpha = a.alpha; f.beta = a.beta; f.Y = Y; f.T = a.T; f.N = a.N; f.K = a.K; f.r = a.r; f.sstride = a.scale_stride;
   f.item_rows = sv.max_items * 128;
-  f.g = make_tile_grid((a.T + 255) / 256, (a.N + 255) / 256, 256);
+  f.tiles1 = (a.N + 255) / 256;
+  f.g = make_tile_grid((a.T + 255) / 256, f.tiles1 * (second.w_s8 ? 2 : 1), 256);
   return launch_gemm<P>(KID_FWD, kernel, f, f.g.total, st);
 }
 
 // h_int = q A8_e^T per item.  raw == nullptr: codes and scales of h into the saved h region; otherwise the exact sums
 // [items*128, r] into `raw` (A8 [E, r, K] int8).
-int gemm_hp_up8(const LayerArgs& a, const SavedPtrs& sv, const void* A8, int* raw, cudaStream_t st) {
+int gemm_hp_up8(const LayerArgs& a, const SavedPtrs& sv, const void* A8, int* raw, cudaStream_t st, const void* A8b, int* rawb) {
   HpUp8Problem::Params p;
-  p.rt = sv.rt; p.qh = reinterpret_cast<int8_t*>(sv.h); p.gamma_h = raw ? nullptr : hp8_gamma_h(sv, a.r); p.raw = raw;
+  p.rt = sv.rt; p.qh = reinterpret_cast<int8_t*>(sv.h); p.gamma_h = raw ? nullptr : hp8_gamma_h(sv, a.r); p.raw = raw; p.rawb = rawb;
   p.K = a.K; p.r = a.r; p.rp = a.r; p.bn = h_round_up(a.r, 16);
   if (!map2d(&p.tq, true, sv.q, a.K, a.T, 128, 128)) return PQ_ERR_CUDA;
   if (!map3d_i8(&p.ta, A8, a.K, a.K, a.r, a.E, p.bn)) return PQ_ERR_CUDA;
-  return launch_gemm<HpUp8Problem>(KID_HP_UP, k_gemm_hp_up8, p, sv.max_items, st);
+  p.tb = p.ta;
+  if (rawb && !map3d_i8(&p.tb, A8b, a.K, a.K, a.r, a.E, p.bn)) return PQ_ERR_CUDA;
+  return launch_gemm<HpUp8Problem>(KID_HP_UP, k_gemm_hp_up8, p, sv.max_items * (rawb ? 2 : 1), st);
 }
 
 int gemm_forward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, const uint16_t* xs, uint16_t* Y, cudaStream_t st,
-                 cudaEvent_t before_main) {
+                 cudaEvent_t before_main, const SecondWeight& second) {
   if (a.r > 0 && a.hp_scales) {
     if (!a.hp_ext) {
       const int rc = gemm_hp_up8(a, sv, a.A, nullptr, st);
@@ -624,8 +638,8 @@ int gemm_forward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, co
   if (before_main && cudaStreamWaitEvent(st, before_main, 0) != cudaSuccess) return PQ_ERR_CUDA;
   const bool general = a.scale_stride != 0 || a.K >= 32768;
   if (a.r > 0)
-    return general ? launch_forward<true, true>(a, w_s8, sv, Y, k_gemm_fwd_hp_general, st) : launch_forward<true, false>(a, w_s8, sv, Y, k_gemm_fwd_hp, st);
-  return general ? launch_forward<false, true>(a, w_s8, sv, Y, k_gemm_fwd_1bit_general, st) : launch_forward<false, false>(a, w_s8, sv, Y, k_gemm_fwd_1bit, st);
+    return general ? launch_forward<true, true>(a, w_s8, sv, Y, k_gemm_fwd_hp_general, st, second) : launch_forward<true, false>(a, w_s8, sv, Y, k_gemm_fwd_hp, st, second);
+  return general ? launch_forward<false, true>(a, w_s8, sv, Y, k_gemm_fwd_1bit_general, st, second) : launch_forward<false, false>(a, w_s8, sv, Y, k_gemm_fwd_1bit, st, second);
 }
 
 

@@ -90,11 +90,11 @@ cudaError_t launch_pack(const float* W, int N, int K, uint32_t* bits, int8_t* s8
 // norm_weight != nullptr: X is un-normalised and RMSNorm (gain [K] bf16, epsilon) is applied on the fly; the sorted copy
 // xs of the tokens is then written even without routing (it is the only place the normalised activation exists)
 cudaError_t launch_route_and_quant(const uint16_t* X, const uint16_t* Wr, int T, int K, int E, const SavedPtrs& sv, const FwdScratch& sc,
-                                   cudaStream_t st, cudaStream_t st_quant, const uint16_t* norm_weight = nullptr, float norm_eps = 0.f);
+                                   cudaStream_t st, cudaStream_t st_quant, const uint16_t* norm_weight = nullptr, float norm_eps = 0.f,
+                                   const uint16_t* up = nullptr, uint16_t* mid = nullptr);   // up: X is silu's side of a SwiGLU, left in mid
 cudaError_t launch_finalize_scales(const float* dbeta_partial, int nslots, const float* dalpha_partial, int E, int N, const float* w_scales,
                                    int vec, float* dbeta, float* dalpha, double* blk_sums, unsigned* arrivals, cudaStream_t st);
 cudaError_t launch_fill_zero(void* p, size_t bytes, cudaStream_t st);
-cudaError_t launch_swiglu(const uint16_t* G, const uint16_t* U, uint16_t* M, long long n, cudaStream_t st);
 cudaError_t launch_ffn8_act(const int* g_int, const int* u_int, const float* gamma, const float* hp_scales, int T, int r, int8_t* qm,
                             float* gamma_m, cudaStream_t st);
 cudaError_t launch_concat_experts(const uint16_t* B, int E, int N, int r, uint16_t* out, cudaStream_t st);
@@ -117,9 +117,12 @@ struct LayerArgs {
 
 int gemm_debug(int mode, int M, int N, int K, const void* A, const void* B, void* D, int tile_n, cudaStream_t st);
 // before_main: an event the fused forward GEMM waits for (work on another stream that feeds it), or nullptr
-int gemm_hp_up8(const LayerArgs& a, const SavedPtrs& sv, const void* A8, int* raw, cudaStream_t st);
+// A8b, rawb: a second matrix of the same sizes and its sums, or null
+int gemm_hp_up8(const LayerArgs& a, const SavedPtrs& sv, const void* A8, int* raw, cudaStream_t st, const void* A8b = nullptr, int* rawb = nullptr);
+// a second 1-bit matrix of the same sizes beside the first
+struct SecondWeight { const int8_t* w_s8 = nullptr; const float* w_scales = nullptr; uint16_t* Y = nullptr; };
 int gemm_forward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, const uint16_t* xs, uint16_t* Y, cudaStream_t st,
-                 cudaEvent_t before_main);
+                 cudaEvent_t before_main, const SecondWeight& second = SecondWeight{});
 
 // decode path (pq_decode.cu)
 size_t decode_workspace_bytes(int M, int K, int N, int r, bool dump);
