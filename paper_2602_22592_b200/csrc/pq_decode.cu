@@ -1101,13 +1101,22 @@ int decode_stream_max_batch();   // pq_decode_stream.cu
 int decode_batch(const DecodeItemArgs* items, int n, cudaStream_t st) {
   int i = 0;
   while (i < n) {
-    // The streaming kernel takes a run of items that all carry its weight layout, where it pays.
+    // The streaming kernel takes a run of items that all carry its weight layout, where it pays.  Measured on linears of 3200 x
+    // 8640, eight experts of 160, small-group kernels against streaming (us): 3 linears, M = 1 / 4 / 8 / 16: 27/27 32/39 47/60
+    // 98/89; 6 linears: 44/30 64/57 95/86 190/132; 12 linears: 84/41 115/86 154/130 361/220.  INT8 experts, 3 linears: 24/28
+    // 29/37 39/56 64/80; 6 linears: 39/31 49/52 65/72 128/114; 12 linears: 66/39 100/78 113/103 239/205.
     const int mode = decode_stream_mode();
     const int most = std::min(n - i, std::min(decode_stream_max_batch(), kDecodeMaxBatch));
     int run = 0, max_m = 1;
-    while (run < most && items[i + run].bits_il) max_m = std::max(max_m, items[i + run++].a.T);
+    bool int8 = false;
+    while (run < most && items[i + run].bits_il) {
+      max_m = std::max(max_m, items[i + run].a.T);
+      if (items[i + run].A8) int8 = true;
+      ++run;
+    }
+    const bool pays = run >= 12 || (run >= 6 && (!int8 || max_m <= 2 || max_m > 8)) || (run >= 3 && !int8 && max_m > 8);
     int rc = PQ_ERR_UNSUPPORTED, m = run;
-    if (run > 0 && (mode > 1 || (mode == 1 && (run >= 12 || (run >= 6 && max_m <= 2))))) rc = decode_stream_launch(items + i, run, st);
+    if (run > 0 && (mode > 1 || (mode == 1 && pays))) rc = decode_stream_launch(items + i, run, st);
     if (rc == PQ_ERR_UNSUPPORTED) {
       // the three kernels above take items with and without the layout together, unless the streaming kernel is asked for
       // wherever it can run

@@ -2,12 +2,15 @@
 straddle them."""
 import numpy as np
 import pytest
+import torch
 
 from oracle import pquant_oracle as O
+from paper_2602_22592_b200 import binding as pqb
 from paper_2602_22592_b200 import inputs as I
+from paper_2602_22592_b200.layer import PQLinear
 from test_gpu_backward import check_backward, run_fwd_bwd
 from test_gpu_ffn import test_ffn_decoupled_forward_matches_oracle as check_ffn
-from test_gpu_forward import check_forward, run_forward
+from test_gpu_forward import check_forward, check_status, run_forward
 
 pytestmark = pytest.mark.gpu
 
@@ -54,3 +57,54 @@ def test_forward_of_long_rows_uses_the_general_tile():
     c["W"][:16] = np.abs(c["W"][:16]) + 0.01
     f = O.linear_forward(c["X"], c["W"], c["A"], c["B"], c["Wr"], c["alpha"], c["beta"])
     check_forward(c, run_forward(c, False), f)
+
+
+def _decode_layers(shapes):
+    layers = []
+    for i, kw in enumerate(shapes):
+        kw = dict(kw)
+        hp8, stream = kw.pop("hp8", False), kw.pop("stream", True)
+        c = I.make_linear_case(kw["T"], kw["K"], kw["N"], kw["r"], kw["E"], seed=60 + i, exact_quota=False, with_grad=False)
+        L = PQLinear(c["T"], c["K"], c["N"], c["r"], c["E"], training=False, dump_acc=True).load_case(c)
+        PQLinear.stream_decode = stream
+        try:
+            L.pack(bits_only=True)
+        finally:
+            PQLinear.stream_decode = True
+        if hp8:
+            L.pack_decode_hp8()
+        layers.append((L, c))
+    return layers
+
+
+@pytest.mark.parametrize("shapes", [
+    # both sides of the lines between the small-group kernels and the streaming one
+    *[[dict(T=M, K=256, N=96, r=32, E=4, hp8=hp8)] * n for n, M, hp8 in
+      [(2, 9, False), (3, 9, False), (5, 4, False), (6, 4, False), (5, 2, True), (6, 2, True), (6, 8, True), (6, 9, True), (12, 8, True)]],
+    # the small-group kernels: codes of a row too long to be in shared memory at once; one unit; ragged hidden widths; the INT8
+    # branch beside linears with and without the streaming layout
+    [dict(T=16, K=16384, N=64, r=32, E=2)], [dict(T=16, K=16384, N=64, r=40, E=2, stream=False)],
+    [dict(T=1, K=32, N=32, r=8, E=16), dict(T=8, K=4128, N=1056, r=48, E=2, hp8=True), dict(T=5, K=96, N=160, r=72, E=3, stream=False)],
+])
+def test_decode_dispatch_and_small_groups(shapes):
+    # the exact integers and the outputs of the oracle; for INT8 experts the outputs of the streaming kernel
+    from test_gpu_decode import check_decode
+    layers = _decode_layers(shapes)
+    pqb.pq_decode_batch(pqb.make_decode_items([L.decode_entry() for L, _ in layers]))
+    torch.cuda.synchronize()
+    check_status()
+    for (L, c), kw in zip(layers, shapes):
+        if kw.get("hp8"):
+            q, gamma = O.act_quant(c["X"])
+            assert np.array_equal(L.decode_view()["code_sum"].cpu().numpy(), q.astype(np.int64).sum(axis=1))
+            y = L.Y.clone()
+            pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 2)          # the streaming kernel is checked against the oracle elsewhere
+            try:
+                L.decode()
+                torch.cuda.synchronize()
+            finally:
+                pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 1)
+            # integer sums on both sides, de-quantised by the same factors: at most the rounding of the bf16 output
+            assert torch.all((y.float() - L.Y.float()).abs() <= 2.0 ** -7 * L.Y.float().abs() + 1e-6)
+        else:
+            check_decode(c, L)
