@@ -178,10 +178,10 @@ int pq_pack_experts(const pq_desc* d, const uint16_t* A, const uint16_t* B, int8
  *   training (w_s8 != NULL): tensor-core path; fills `saved` (may be NULL when
  *     no backward follows).  A, B may be NULL iff r == 0; Wr NULL iff E <= 1.
  *   decode (w_s8 == NULL): T <= 16 tokens straight from the packed bits w_bits
- *     (App. A): two kernels bound by the bytes of the weights.  `saved` is ignored,
+ *     (App. A): three overlapped kernels.  `saved` is ignored,
  *     ws needs pq_workspace_bytes(d, PQ_PHASE_DECODE) bytes.  r <= 256; K and N such
  *     that one SM's share of the bits and expert rows fits its shared memory
- *     (PQ_ERR_UNSUPPORTED otherwise; the 3B-shaped 3200 x 8640 layers fit).  The two
+ *     (PQ_ERR_UNSUPPORTED otherwise; the 3B-shaped 3200 x 8640 layers fit).  The
  *     kernels are launched with programmatic stream serialisation, so consecutive
  *     decode calls on one stream overlap their prologues. */
 int pq_linear_forward(const pq_desc* d, const uint16_t* X, const uint32_t* w_bits,
@@ -262,20 +262,19 @@ typedef struct pq_decode_token {
 typedef struct pq_decode_view {
   pq_decode_token* tokens; /* [T] (device)                                                        */
   int32_t* acc;            /* [T,N] sum_k S[n,k] q[t,k] when PQ_DECODE_DUMP_ACC is set, else NULL */
-  /* INT8 branch on the streaming kernel (pq_decode_item.A8): the exact integers it went through */
+  /* INT8 branch (pq_decode_item.A8): the exact integers it went through */
   int32_t* hp_h_int;       /* [T,r] h_int = A8_e q                                                 */
   int32_t* hp_z_int;       /* [T,N] z_int = B8_e qh when PQ_DECODE_DUMP_ACC is set, else NULL       */
 } pq_decode_view;
 int pq_decode_view_init(const pq_desc* d, void* ws, pq_decode_view* out);
 
-/* Decode forward of several INDEPENDENT linears in one launch pair (App. A: at batch size
+/* Decode forward of several INDEPENDENT linears in one group of launches (App. A: at batch size
  * one the weights' bytes are the cost, so linears that do not depend on each other -- the
  * gate and up projections of a block, the q/k/v projections, other sequences -- should
  * stream their weights back to back instead of paying a launch and a pipeline fill each).
  * Each item is what pq_linear_forward takes in its decode form; results are identical to n
  * separate calls.  `items` is a HOST array, read before the call returns.  1 <= n <= 4096
- * (PQ_ERR_SHAPE otherwise; launched in groups of up to 96 consecutive items on the streaming kernel, of 16 on the
- * two-kernel path); every item needs its own ws. */
+ * (PQ_ERR_SHAPE otherwise; launched in groups of up to 96 consecutive items); every item needs its own ws. */
 typedef struct pq_decode_item {
   pq_desc desc;            /* T <= 16 */
   const uint16_t* X;       /* [T,K] bf16 */
@@ -303,7 +302,7 @@ typedef struct pq_decode_item {
    * (PQ_OPT_DECODE_STREAM), the group runs as ONE cooperative kernel that
    * streams each weight byte once with coalesced loads; results: the same integers (codes, routing, sums over k),
    * Y within the tolerance of the float epilogue (the expert product is summed in another order).  Otherwise, and
-   * for shapes that kernel does not take (r not a multiple of 8), the two-kernel path is used.  Items of one launch
+   * for shapes that kernel does not take (r not a multiple of 8), the small-group kernels are used.  Items of one launch
    * group that read the same X (same pointer, T, K and norm) are quantised once.  w_bits, A and B
    * are needed in both cases (the rows of A_e are read in their natural layout). */
   const uint32_t* w_bits_il;
@@ -312,7 +311,7 @@ typedef struct pq_decode_item {
    * hp_scales [E][2] from pq_pack_experts, B8_il from pq_pack_decode_hp8.  The branch multiplies the token's int8 codes:
    *   h_int = A8_e q (int32, exact);  qh, gamma_h = Eq. 7-9 on h_int;  z_int = B8_e qh (int32, exact);
    *   z = z_int / (gamma_B gamma_h gamma_A gamma_t)
-   * -- the arithmetic of pq_linear_forward_hp8.  It runs on the streaming kernel only, whatever the group's size:
+   * -- the arithmetic of pq_linear_forward_hp8.  On either path (PQ_OPT_DECODE_STREAM);
    * w_bits_il is required (PQ_ERR_NULL), r a multiple of 16 (PQ_ERR_SHAPE); A, B and B_il are not read. */
   const int8_t* A8;
   const int8_t* B8_il;
