@@ -385,10 +385,11 @@ __device__ __forceinline__ void mma_s8s8(int (&c)[4], uint32_t a0, uint32_t a1, 
 }
 // Steps [st_lo, st_hi) of 64 bytes per row.  Rows of `pitch` 16-byte pieces; r0, r1, x0, x1 point at this lane's piece of step 0
 // (x0, x1: its columns' tokens, null for columns without one).
-template <bool INT8>
-__device__ __forceinline__ void hidden_walk(const uint4* r0, const uint4* r1, const uint4* x0, const uint4* x1, bool two, int st_lo, int st_hi, int last, int c,
+// TWO: the expert has more than eight tokens.
+template <bool INT8, bool TWO>
+__device__ __forceinline__ void hidden_walk(const uint4* r0, const uint4* r1, const uint4* x0, const uint4* x1, int st_lo, int st_hi, int last, int c,
                                             uint32_t (&z0)[4], uint32_t (&z1)[4]) {
-  constexpr int U = 4;                                         // steps in flight
+  constexpr int U = TWO ? 3 : 4;                               // steps in flight, as many as 80 registers hold
   const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
   auto mma = [](uint32_t (&z)[4], const uint4& a, const uint4& b, const uint4& v) {
     if (INT8) {
@@ -402,21 +403,20 @@ __device__ __forceinline__ void hidden_walk(const uint4* r0, const uint4* r1, co
     }
   };
   for (int st = st_lo; st < st_hi; st += U) {
-    uint4 w0[U], w1[U], v[U];
+    uint4 w0[U], w1[U], v[U], v1[TWO ? U : 1];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const bool in = st + u < st_hi && (st + u) * 4 + c < last;   // a row's last step may be half a step (INT8, K % 64 = 32)
       w0[u] = in ? __ldg(r0 + (st + u) * 4) : zero;
       w1[u] = in ? __ldg(r1 + (st + u) * 4) : zero;
       v[u] = in && x0 ? __ldcg(x0 + (st + u) * 4) : zero;
+      if (TWO) v1[u] = in && x1 ? __ldcg(x1 + (st + u) * 4) : zero;
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) mma(z0, w0[u], w1[u], v[u]);
-    if (two) {
+    if (TWO) {
 #pragma unroll
-      for (int u = 0; u < U; ++u) v[u] = st + u < st_hi && (st + u) * 4 + c < last && x1 ? __ldcg(x1 + (st + u) * 4) : zero;
-#pragma unroll
-      for (int u = 0; u < U; ++u) mma(z1, w0[u], w1[u], v[u]);
+      for (int u = 0; u < U; ++u) mma(z1, w0[u], w1[u], v1[u]);
     }
   }
 }
@@ -479,8 +479,13 @@ __global__ void __maxnreg__(80) k_decode_hidden(const __grid_constant__ DecodeBa
   for (int v = rank * kHiddenWarps + warp; v < kHiddenSplit; v += cs * kHiddenWarps) {
     uint32_t z0[4] = {0u, 0u, 0u, 0u}, z1[4] = {0u, 0u, 0u, 0u};   // fp32 or int32 sums; zero is the same word
     const int st_lo = steps * v / kHiddenSplit, st_hi = steps * (v + 1) / kHiddenSplit;
-    if (int8) hidden_walk<true>(r0, r1, x0, x1, two, st_lo, st_hi, pitch, c, z0, z1);
-    else hidden_walk<false>(r0, r1, x0, x1, two, st_lo, st_hi, pitch, c, z0, z1);
+    if (int8) {
+      if (two) hidden_walk<true, true>(r0, r1, x0, x1, st_lo, st_hi, pitch, c, z0, z1);
+      else hidden_walk<true, false>(r0, r1, x0, x1, st_lo, st_hi, pitch, c, z0, z1);
+    } else {
+      if (two) hidden_walk<false, true>(r0, r1, x0, x1, st_lo, st_hi, pitch, c, z0, z1);
+      else hidden_walk<false, false>(r0, r1, x0, x1, st_lo, st_hi, pitch, c, z0, z1);
+    }
     const uint32_t to = cluster_map(smem_u32(&red[v][0][0]), 0);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -975,7 +980,7 @@ static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st)
   DecodeBatch<CAP> bp;
   bp.n = n;
   size_t h_bytes = 0, x_bytes = 0, slot_bytes = 0;
-  int max_m = 1, max_e = 1, units = 0, max_c = 1;
+  int max_m = 1, max_e = 1, units = 0, max_c = 1, row_bytes = 0;
   bool any_norm = false;
   bp.hidden_groups = 0;
   for (int i = 0; i < n; ++i) {
@@ -1009,6 +1014,7 @@ static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st)
     bp.unit0[i] = units;
     units += N / kUnit;
     L.hidden0 = bp.hidden_groups;
+    if (r > 0) row_bytes = std::max(row_bytes, it.A8 ? K : 2 * K);
     if (r > 0) bp.hidden_groups += std::min(L.E, M) * ((r + 15) / 16);
     max_m = std::max(max_m, M); max_e = std::max(max_e, L.E); max_c = std::max(max_c, (K + 127) / 128);
     x_bytes = std::max(x_bytes, up256((size_t)K * 2));
@@ -1043,8 +1049,10 @@ static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st)
   bp.off_wr = (int)x_bytes;
   bp.off_gain = (int)(x_bytes + (max_e > 8 ? 2 : max_e > 1 ? 1 : 0) * x_bytes);
   bp.early = bp.hidden_groups > 0;
-  // one CTA per SM, if that leaves any of the contraction's parallelism; otherwise three per SM, and k_decode_main's follow them
-  bp.hidden_cluster = 4 * bp.hidden_groups <= sms ? 4 : 2 * bp.hidden_groups <= 3 * sms ? 2 : 1;
+  // One CTA per SM; with rows of A_e beyond 4 KB, whose contraction is worth more than room for k_decode_main's CTAs beside it, up to
+  // three.  Per call, one CTA per cluster against two where two are more than the SMs hold: M = 11, 1056 x 7552 18.6 / 21.7 us, M = 4,
+  // INT8, 3200 x 8640 16.9 / 18.3; M = 13, 2816 x 4960 22.1 / 20.7, M = 16, 3200 x 8640 37.2 / 31.4.
+  bp.hidden_cluster = 4 * bp.hidden_groups <= sms ? 4 : 2 * bp.hidden_groups <= (row_bytes > 4096 ? 3 * sms : sms) ? 2 : 1;
   const size_t smem_prep = bp.off_gain + (any_norm ? x_bytes : 0);
   if (smem_prep > kDecodePrepSmemLimit) return PQ_ERR_UNSUPPORTED;
 
