@@ -37,7 +37,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # projection) from an ncu capture, stamped with the hash of the files that kernel is compiled from (the tensor-core engine,
 # the GEMM kernels, the shared device helpers): once one of them changes the stamp no longer matches and the bench line
 # reports null until the kernel is captured again.
-NCU_TRAFFIC = {"bwd_dw": {"bytes": 218562048, "sources_sha16": "e1887889fce22bf8", "files": ("pq_gemm.cuh", "pq_gemm_kernels.cu", "pq_common.cuh")}}
+NCU_TRAFFIC = {"bwd_dw": {"bytes": 634162688, "sources_sha16": "fd80037ecb1a2c21", "files": ("pq_gemm.cuh", "pq_gemm_kernels.cu", "pq_common.cuh")}}
 
 
 def sources_sha16(files) -> str:
@@ -490,7 +490,7 @@ def subrecords(args, ctx, engine):
                 "batched_all: all 78 linears of the step handed to one pq_decode_batch call (one launch: the kernel's fixed costs -- "
                 "token work, grid barrier, launch gap -- are paid once); "
                 "pairs: what one sequence's model allows (gate + up of a block together); serial: one call per linear, each after "
-                "the previous one -- both on the two-kernel path, which the library picks for small groups"),
+                "the previous one -- both on the small-group kernels, which the library picks for them"),
                 "kernels": ctx.decode_kernels}
             for M in (1, 4, 16):
                 d = measure_decode(ctx, M, max(5, min(args.steps, 20)), weights, full=True)
@@ -880,7 +880,7 @@ def main():
     ap.add_argument("--decode-batch", type=int, default=16, help="independent decode linears per pq_decode_batch call")
     ap.add_argument("--decode-kernels", default="auto", choices=["auto", "stream", "pair"],
                     help="auto: the library picks per launch group; stream: the cooperative streaming kernel wherever the items allow; "
-                         "pair: the two-kernel path on the plain layout")
+                         "pair: the small-group kernels on the plain layout")
     ap.add_argument("--decode-interleave", type=int, default=1, choices=[0, 1, 2], help="streaming decode kernel: side-by-side walk of its two work lists (0 never, 1 auto, 2 always)")
     ap.add_argument("--decode-hp8", action="store_true", help="decode with the INT8 high-precision branch (int8 experts: half the expert bytes)")
     ap.add_argument("--decode-mma-from", type=int, default=5, help="streaming decode kernel: token groups of at least this size use the tensor-core bit product")

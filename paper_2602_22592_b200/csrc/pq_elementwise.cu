@@ -823,12 +823,6 @@ cudaError_t launch_ffn8_act(const int* g_int, const int* u_int, const float* gam
   return cudaGetLastError();
 }
 
-__global__ void k_fill_zero(uint4* p, long long n16) {
-  pdl_launch_dependents();   // launched with programmatic stream serialisation: see launch_pdl
-  pdl_wait();
-  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n16; i += gridDim.x * 256LL) p[i] = make_uint4(0, 0, 0, 0);
-}
-
 // ---------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------
@@ -914,13 +908,6 @@ cudaError_t launch_finalize_scales(const float* dbeta_partial, int nslots, const
   LaunchScope ls(vec ? KID_SUM_PARTIALS : KID_SUM_SCALAR, st);
   launch_pdl(k_finalize_scales, (N + 31) / 32, 256, 0, st, dbeta_partial, nslots, dalpha_partial, E, N, w_scales, dbeta, dalpha,
              vec ? nullptr : blk_sums, vec ? nullptr : arrivals);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_fill_zero(void* p, size_t bytes, cudaStream_t st) {
-  const long long n16 = (long long)(bytes / 16);
-  if (n16 == 0) return cudaSuccess;
-  launch_pdl(k_fill_zero, grid_for(n16, 256 * 4, 148 * 4), 256, 0, st, reinterpret_cast<uint4*>(p), n16);
   return cudaGetLastError();
 }
 

@@ -94,7 +94,6 @@ cudaError_t launch_route_and_quant(const uint16_t* X, const uint16_t* Wr, int T,
                                    const uint16_t* up = nullptr, uint16_t* mid = nullptr);   // up: X is silu's side of a SwiGLU, left in mid
 cudaError_t launch_finalize_scales(const float* dbeta_partial, int nslots, const float* dalpha_partial, int E, int N, const float* w_scales,
                                    int vec, float* dbeta, float* dalpha, double* blk_sums, unsigned* arrivals, cudaStream_t st);
-cudaError_t launch_fill_zero(void* p, size_t bytes, cudaStream_t st);
 cudaError_t launch_ffn8_act(const int* g_int, const int* u_int, const float* gamma, const float* hp_scales, int T, int r, int8_t* qm,
                             float* gamma_m, cudaStream_t st);
 cudaError_t launch_concat_experts(const uint16_t* B, int E, int N, int r, uint16_t* out, cudaStream_t st);
