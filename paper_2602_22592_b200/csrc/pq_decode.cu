@@ -15,8 +15,8 @@
 // with the codes and the experts' rows of B on their way when h arrives.
 //
 // Measured, two kernels with the hidden rows in the first (INT8 experts: the streaming kernel) -> these three: one 2048 x 2048
-// linear, one token 13.8 -> 10.8 us; 26 layers of gate + up, then down of 3200 x 8640, one token 1010 -> 788 us, sixteen 1759 -> 1609
-// us; 8 layers, four tokens, INT8 experts 572 -> 301 us.
+// linear, one token 13.8 -> 10.8 us; 26 layers of gate + up, then down of 3200 x 8640, one token 1010 -> 790 us, sixteen 1767 -> 1591
+// us; 8 layers, four tokens, INT8 experts 573 -> 278 us.  A dense branch with nine to fourteen tokens loses 1 us a call.
 //
 // The sum over k of q S is evaluated as 2 * (sum over the set bits of q) - (sum of q): the bit
 // words feed the tensor cores as 0/1 masks without expansion to +-1.
