@@ -2,6 +2,8 @@
 // binarize-and-pack (Eq. 3, 4, 6), router (Sec. 3.3), expert sort, activation
 // quantisation (Eq. 7-9), and the small gather / scale / reduce helpers of the
 // backward pass.
+#include <mutex>
+
 #include "pq_kernels.cuh"
 
 namespace pq {
@@ -845,6 +847,26 @@ cudaError_t launch_pack(const float* W, int N, int K, uint32_t* bits, int8_t* s8
   return cudaGetLastError();
 }
 
+// The router's opt-in limit is set once per device, to the largest request: it belongs to the kernel, not to a launch, so that a
+// call which set a smaller one would take it from under a call of another thread, or from under a launch recorded in a CUDA graph.
+constexpr int kRouterSmemLimit = 116 * 1024;
+static_assert(router_smem<kMaxExperts>() <= kRouterSmemLimit, "the bare ring fits too");
+static cudaError_t router_limits() {
+  constexpr int kMaxDevices = 64;
+  static std::once_flag done[kMaxDevices];
+  static cudaError_t result[kMaxDevices] = {};
+  int dev = 0;
+  if (const cudaError_t e = cudaGetDevice(&dev)) return e;
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  std::call_once(done[dev], [&] {
+    auto set = [](auto k) { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kRouterSmemLimit); };
+    result[dev] = set(k_router<4>);
+    if (result[dev] == cudaSuccess) result[dev] = set(k_router<8>);
+    if (result[dev] == cudaSuccess) result[dev] = set(k_router<kMaxExperts>);
+  });
+  return result[dev];
+}
+
 cudaError_t launch_route_and_quant(const uint16_t* X, const uint16_t* Wr, int T, int K, int E, const SavedPtrs& sv, const FwdScratch& sc,
                                    cudaStream_t st, cudaStream_t st_quant, const uint16_t* norm_weight, float norm_eps, const uint16_t* up, uint16_t* mid) {
   if (E > 1) st_quant = st;   // the sorted position of a token comes from the router and the scan
@@ -863,14 +885,17 @@ cudaError_t launch_route_and_quant(const uint16_t* X, const uint16_t* Wr, int T,
     else if (E <= 8) { kern = k_router<8>; smem = router_smem<8>(); }
     // One CTA per SM (two) where the grid needs no more: its CTAs become resident while the kernel before ends, and the SMs that
     // end first would otherwise take all they can hold.  2048 tokens x 3200: 17 us without this, 10 with it.
-    if (nblocks <= 148) smem = 116 * 1024;
+    if (nblocks <= 148) smem = kRouterSmemLimit;
     else if (nblocks <= 2 * 148) smem = 76 * 1024;
-    if (cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) return e;
-    launch_pdl(kern, nblocks, 32 * kRouterWarps, smem, st, reinterpret_cast<const uint4*>(X), reinterpret_cast<const uint4*>(Wr), T, K, E, sv.expert,
-               sc.gate_tok, sc.probs_tok, sc.block_counts, nw, sc.rms);
+    if (const cudaError_t e = router_limits()) return e;
+    const cudaError_t e = launch_pdl(kern, nblocks, 32 * kRouterWarps, smem, st, reinterpret_cast<const uint4*>(X), reinterpret_cast<const uint4*>(Wr), T, K,
+                                     E, sv.expert, sc.gate_tok, sc.probs_tok, sc.block_counts, nw, sc.rms);
+    if (e != cudaSuccess) return e;   // the kernels behind this one store where its counts say
   }
-  { LaunchScope ls(KID_ROUTE_SCAN, st);
-  launch_pdl(k_route_scan, 1, 512, 0, st, T, E, nblocks, sc.block_counts, sc.block_base, sv.offsets, sv.rt); }
+  {
+    LaunchScope ls(KID_ROUTE_SCAN, st);
+    if (const cudaError_t e = launch_pdl(k_route_scan, 1, 512, 0, st, T, E, nblocks, sc.block_counts, sc.block_base, sv.offsets, sv.rt)) return e;
+  }
   LaunchScope ls(KID_ACT_QUANT, st_quant);
   const int per_lane = (K / 8 + 31) / 32;   // 16-byte pieces of a row per lane if one warp took the whole row
   auto kern = up ? k_act_quant<0, 1, true> : k_act_quant<0, 1>;

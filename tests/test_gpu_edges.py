@@ -59,6 +59,40 @@ def test_forward_of_long_rows_uses_the_general_tile():
     check_forward(c, run_forward(c, False), f)
 
 
+def test_router_calls_of_two_threads_at_once():
+    # the router asks for 116, 76 or 36 KB of shared memory by the number of blocks of tokens; the kernel's limit belongs to the
+    # process, so a call must not lower it between another thread's look at it and that thread's launch
+    import threading
+    layers = []
+    for T in (2048, 4096, 8192):
+        c = I.make_linear_case(T, 64, 64, 16, 8, seed=T, with_grad=False)
+        L = PQLinear(T, 64, 64, 16, 8).load_case(c)
+        L.pack()
+        L.forward()
+        layers.append(L)
+    torch.cuda.synchronize()
+    want = [(L.Y.clone(), L.saved_view()["perm"].clone()) for L in layers]
+    failed = []
+
+    def calls(L):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(300):
+                    L.forward()
+        except Exception as e:      # noqa: BLE001 -- reported by the main thread
+            failed.append(e)
+    threads = [threading.Thread(target=calls, args=(L,)) for L in layers]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    check_status()
+    assert not failed
+    for L, (y, perm) in zip(layers, want):
+        assert torch.equal(L.Y, y) and torch.equal(L.saved_view()["perm"], perm)
+
+
 def _decode_layers(shapes):
     layers = []
     for i, kw in enumerate(shapes):
