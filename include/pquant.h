@@ -391,8 +391,8 @@ int pq_device_status(void* stream, int* code, int* where);
  *   that does not succeed at once runs out, the kernel stops issuing work, lets copies and MMAs in
  *   flight finish, releases its TMEM and returns; pq_device_status then reports PQ_ERR_TIMEOUT and the
  *   outputs of that call are undefined.  Applies to the current device; blocks until the device's
- *   earlier work has finished.  Meant for pq_debug_gemm; do not shorten the limit around the decode
- *   entry points, whose later stages read indices an abandoned stage has not delivered.
+ *   earlier work has finished.  For tests of a single call; not around pq_linear_forward of training size, whose
+ *   results a backward call would go on from.
  *   PQ_OPT_DECODE_STREAM (default 1): which launch groups of pq_decode_batch (up to 96 consecutive items) run on the
  *   streaming kernel when their items carry w_bits_il / B_il.  1 = those for which it is the faster of the two paths
  *   (six or more linears, with INT8 experts and three to eight tokens twelve; three or more bf16 ones with more than eight

@@ -134,11 +134,15 @@ __device__ __forceinline__ void copy_record(DecodeLinear* dst, const DecodeBatch
 }
 
 // Wait with a bound.  Once any wait of the CTA has run out, every later wait returns at once, so that
-// all threads keep the same control flow and the kernel ends (with an error status and undefined output).
+// all threads keep the same control flow and the kernel ends (with an error status and undefined output): no copy is
+// issued any more, and decode_drain lets those in flight land before the CTA's shared memory passes to another.
+// A copy takes a microsecond or two, less than the hardware may suspend a waiting thread for: a limit as short as that is polled.
 __device__ __forceinline__ void decode_wait(uint32_t bar, uint32_t parity, volatile int* fail) {
-  if (mbar_try_wait(bar, parity)) return;
+  const bool poll = c_spin_cycles < 1000;
+  auto done = [&] { return poll ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity); };
+  if (done()) return;
   const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity)) {
+  while (!done()) {
     if (*fail) return;
     if (clock64() - t0 > c_spin_cycles) {
       report_timeout(WHERE_OTHER);
@@ -146,6 +150,11 @@ __device__ __forceinline__ void decode_wait(uint32_t bar, uint32_t parity, volat
       return;
     }
   }
+}
+
+__device__ __forceinline__ void decode_drain(volatile int* fail) {
+  if (*fail)
+    for (int i = 0; i < 200; ++i) __nanosleep(1000);
 }
 
 __device__ __forceinline__ int quant_code(float x, float gamma) { return max(-128, min(127, __float2int_rn(__fmul_rn(x, gamma)))); }
@@ -365,8 +374,9 @@ __global__ void __cluster_dims__(kPrepCluster, 1, 1) __maxnreg__(80) k_decode_pr
       if (w >= routed) tot += sum_sh[rk][w];
     }
     for (int d = 16; d > 0; d >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, d);
-    if (lane == 0) L.info[m] = DecodeTokInfo{best, gate, gamma, tot};
+    if (lane == 0) L.info[m] = DecodeTokInfo{best, gate, gamma, tot};   // after a failed wait too: an expert that exists
   }
+  decode_drain(&fail_sh);
 }
 
 // ---------------------------------------------------------------------------
@@ -814,7 +824,8 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
       else { if (tiles > 1) bits(One{}, Two{}); else bits(One{}, One{}); }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // what plain stores filled may be overwritten by bulk copies
-    __syncthreads();                                             // the sign bits of this pass have been used
+    // the sign bits of this pass have been used; after a failed wait nothing is issued over copies that may be in flight
+    if (__syncthreads_or(*(volatile int*)&fail_sh)) break;
     // ---- expert product.  The rows of B_e go over what has been used: this pass's sign bits, and in the CTA's last pass all
     // buffers and the codes.  Every warp has slots of its own and takes every W-th (expert, tile) item.
     const bool last = u_next >= u_hi && (nbuf == 1 || nxt.nu == 0), rows_now = r > 0 && !L.A8;
@@ -865,7 +876,7 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
       row_phase ^= 1u << j;
       main_expert(reinterpret_cast<const uint4*>(ring + (size_t)(warp * per + j) * item_bytes), r, order_sh + first_sh[ei], count_sh[ei], h_s, lane, red_z + (size_t)t * MT * 16);
       __syncwarp();
-      if (i + W * per < items) issue(i + W * per, j);
+      if (i + W * per < items && !*(volatile int*)&fail_sh) issue(i + W * per, j);
       if (++j == per) j = 0;
     }
     if (last) q_loaded = nullptr;
@@ -897,7 +908,7 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
         }
       }
     }
-    __syncthreads();
+    if (__syncthreads_or(*(volatile int*)&fail_sh)) break;
     // ---- epilogue (Eq. 10-11), two features per thread
     for (int o = tid; o < (rows >> 1) * M; o += kMainThreads) {
       const int t = o / (rows >> 1), f = 2 * (o - t * (rows >> 1));
@@ -933,6 +944,7 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
     load_scales(cur);
   }
   if (!waited) pdl_wait();
+  decode_drain(&fail_sh);
 }
 
 // ---------------------------------------------------------------------------

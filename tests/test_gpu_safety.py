@@ -77,6 +77,75 @@ def test_grid_barrier_of_the_streaming_decode_kernel_runs_out_and_recovers():
         pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 1)
 
 
+def test_waits_of_the_small_group_decode_kernels_run_out_and_recover():
+    # The waits are for router rows, sign bits and expert rows on their way to shared memory.  With up to sixteen
+    # experts in use a pass waits for expert rows that it has just asked for.  Under a limit of one cycle the first that is not
+    # there yet gives up: no further copy is issued, those in flight land before the CTA ends, and every index a later
+    # stage reads is one that exists.  The next calls are exact.
+    c = I.make_linear_case(16, 1024, 8640, 256, 16, seed=55, zipf=False, exact_quota=False, with_grad=False)
+    layers = [PQLinear(16, 1024, 8640, 256, 16, training=False, dump_acc=True, guard=True).load_case(c) for _ in range(2)]
+    for L in layers:
+        L.pack(bits_only=True)
+    items = pqb.make_decode_items([L.decode_entry() for L in layers])
+    pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 0)
+    try:
+        pqb.pq_decode_batch(items)
+        torch.cuda.synchronize()
+        check_status()
+        want = [(L.Y.clone(), L.decode_view()["acc"].clone()) for L in layers]
+        pqb.pq_set_option(pqb.PQ_OPT_SPIN_CYCLES, 1)
+        try:
+            pqb.pq_decode_batch(items)
+            code, where = pqb.pq_device_status()
+        finally:
+            pqb.pq_set_option(pqb.PQ_OPT_SPIN_CYCLES, 0)
+        assert code == pqb.PQ_ERR_TIMEOUT and where == 4
+        assert pqb.pq_device_status() == (0, 0)
+        for _ in range(2):
+            for L in layers:
+                L.Y.zero_()
+            pqb.pq_decode_batch(items)
+            torch.cuda.synchronize()
+            check_status()
+            for L, (y, acc) in zip(layers, want):
+                assert torch.equal(L.Y, y) and torch.equal(L.decode_view()["acc"], acc)
+                assert L.check_guards() == 0
+    finally:
+        pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 1)
+
+
+@pytest.mark.parametrize("T,K,N,r,E", [(16384, 256, 256, 0, 0), (1000, 512, 768, 64, 1), (1000, 512, 768, 64, 8)])
+def test_waits_of_the_backward_kernel_run_out_and_recover(T, K, N, r, E):
+    # The tickets, the tiles held back until the experts' gradients are there, the operand ring and the accumulators: under a
+    # limit of one cycle the first of these waits that does not succeed at once gives up (without experts: the epilogue's, for
+    # a contraction over all tokens), every role of both CTAs of a pair leaves, and the next call gives what it gave before.
+    c = I.make_linear_case(T, K, N, r, E, seed=57)
+    L = PQLinear(T, K, N, r, E, guard=True).load_case(c)
+    L.pack()
+    L.forward()
+    L.backward()
+    torch.cuda.synchronize()
+    check_status()
+    names = ["dX", "dW", "dbeta"] + (["dA", "dB", "dalpha"] if r else []) + (["dWr"] if E > 1 else [])
+    want = {n: getattr(L, n).clone() for n in names}
+    pqb.pq_set_option(pqb.PQ_OPT_SPIN_CYCLES, 1)
+    try:
+        L.backward()
+        code, where = pqb.pq_device_status()
+    finally:
+        pqb.pq_set_option(pqb.PQ_OPT_SPIN_CYCLES, 0)
+    assert code == pqb.PQ_ERR_TIMEOUT and where in (1, 2, 3)
+    assert pqb.pq_device_status() == (0, 0)
+    for _ in range(2):
+        for n in names:
+            getattr(L, n).zero_()
+        L.backward()
+        torch.cuda.synchronize()
+        check_status()
+        assert all(torch.equal(getattr(L, n), w) for n, w in want.items())
+        assert L.check_guards() == 0
+
+
 @pytest.mark.parametrize("shape", [dict(T=333, K=384, N=544, r=64, E=1), dict(T=1000, K=512, N=768, r=128, E=8),
                                    dict(T=200, K=256, N=320, r=0, E=0), dict(T=130, K=5632, N=96, r=16, E=4)])
 def test_training_kernels_stay_inside_their_buffers(shape):
