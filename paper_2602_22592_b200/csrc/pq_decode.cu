@@ -921,7 +921,13 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
         const float2 z = *reinterpret_cast<const float2*>(red_z + at);
         y0 = fmaf(al_sh[f] * tok[t].gate, z.x, y0); y1 = fmaf(al_sh[f + 1] * tok[t].gate, z.y, y1);
       }
-      *reinterpret_cast<uint32_t*>(L.Y + (long long)t * N + n0 + f) = pack_bf16x2(y0, y1);
+      uint16_t* y = L.Y + (long long)t * N + n0 + f;
+      const uint32_t both = pack_bf16x2(y0, y1);
+      if ((reinterpret_cast<uintptr_t>(L.Y) & 3) == 0) {         // rows have an even number of features
+        *reinterpret_cast<uint32_t*>(y) = both;
+      } else {                                                   // an output that starts at an odd element
+        y[0] = (uint16_t)both; y[1] = (uint16_t)(both >> 16);
+      }
       if (L.acc_dump) { L.acc_dump[(long long)t * N + n0 + f] = a0; L.acc_dump[(long long)t * N + n0 + f + 1] = a1; }
     }
     // ---- the buffer is free: the pass after the next one

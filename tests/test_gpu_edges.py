@@ -10,7 +10,7 @@ from paper_2602_22592_b200 import inputs as I
 from paper_2602_22592_b200.layer import PQLinear
 from test_gpu_backward import check_backward, run_fwd_bwd
 from test_gpu_ffn import test_ffn_decoupled_forward_matches_oracle as check_ffn
-from test_gpu_forward import check_forward, check_status, run_forward
+from test_gpu_forward import TOL_BF16, check_forward, check_status, f32, rel_err, run_forward
 
 pytestmark = pytest.mark.gpu
 
@@ -142,3 +142,22 @@ def test_decode_dispatch_and_small_groups(shapes):
             assert torch.all((y.float() - L.Y.float()).abs() <= 2.0 ** -7 * L.Y.float().abs() + 1e-6)
         else:
             check_decode(c, L)
+
+
+@pytest.mark.parametrize("mode", [0, 2])
+def test_decode_output_that_starts_at_an_odd_element(mode):
+    # outputs are stored two features at a time where the output allows it, else one by one
+    M, N = 5, 96
+    c = I.make_linear_case(M, 256, N, 32, 4, seed=11, exact_quota=False, with_grad=False)
+    L = PQLinear(M, 256, N, 32, 4, training=False).load_case(c)
+    L.pack(bits_only=True)
+    buf = torch.full((M * N + 2,), 7.0, dtype=torch.bfloat16, device="cuda")
+    pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, mode)
+    try:
+        L.decode()
+        L.decode(Y=buf[1:-1])
+        torch.cuda.synchronize()
+    finally:
+        pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 1)
+    check_status()
+    assert torch.equal(buf[1:-1].view(M, N), L.Y) and buf[0] == 7.0 and buf[-1] == 7.0
