@@ -179,9 +179,9 @@ int pq_pack_experts(const pq_desc* d, const uint16_t* A, const uint16_t* B, int8
  *     no backward follows).  A, B may be NULL iff r == 0; Wr NULL iff E <= 1.
  *   decode (w_s8 == NULL): T <= 16 tokens straight from the packed bits w_bits
  *     (App. A): three overlapped kernels.  `saved` is ignored,
- *     ws needs pq_workspace_bytes(d, PQ_PHASE_DECODE) bytes.  r <= 256; K and N such
- *     that one SM's share of the bits and expert rows fits its shared memory
- *     (PQ_ERR_UNSUPPORTED otherwise; the 3B-shaped 3200 x 8640 layers fit).  The
+ *     ws needs pq_workspace_bytes(d, PQ_PHASE_DECODE) bytes.  r <= 256; K such that one SM's shared memory holds a
+ *     token and a router row (4 K bytes, 2 K without routing, of 200 KiB), and the sign bits of 16 features
+ *     (2 K bytes) beside codes, hidden values and sums (PQ_ERR_UNSUPPORTED otherwise).  The
  *     kernels are launched with programmatic stream serialisation, so consecutive
  *     decode calls on one stream overlap their prologues. */
 int pq_linear_forward(const pq_desc* d, const uint16_t* X, const uint32_t* w_bits,

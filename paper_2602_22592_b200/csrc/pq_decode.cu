@@ -111,7 +111,6 @@ static_assert(sizeof(DecodeLinear) % 16 == 0, "copied in 16-byte pieces");
 template <int CAP>
 struct DecodeBatch {
   int n, units;             // linears; units of 16 features of all of them
-  int off_wr, off_gain;     // k_decode_prep: router rows of the CTA, the norm's gains
   int early;                // k_decode_hidden runs in between: k_decode_main may read prep's results before it waits
   int hidden_groups, hidden_cluster;   // k_decode_hidden: clusters of all linears, CTAs of each
   // k_decode_main: buffers of sign bits, their size, and the carve-up of shared memory behind them
@@ -186,8 +185,26 @@ __device__ __forceinline__ void store_h(const DecodeLinear& L, int m, int j, flo
   base[pos + rsteps * 32 * 8] = __bfloat16_as_ushort(lo);
 }
 
-// grid (8, M, linears), one cluster per token.  Dynamic shared memory: the token's K bf16 values, the router rows of this CTA's
-// experts, the norm's gains.
+// Shared memory of k_decode_prep: the token's K bf16 values, the router rows of the CTA's experts, the norm's gains.  Where the three do
+// not fit (rows of 25,600 values with more than eight experts and a norm), the gains stay in global memory and a CTA's two
+// router rows take turns.
+struct PrepPlan { uint32_t row, off_gain; int slots; bool lean; size_t bytes; };
+constexpr size_t kDecodePrepSmemLimit = 200 * 1024;
+__host__ __device__ inline PrepPlan prep_plan(int K, int E, bool norm) {
+  PrepPlan p{};
+  p.row = ((uint32_t)K * 2u + 255u) / 256u * 256u;             // the token, and what follows it
+  p.slots = E > kPrepCluster ? 2 : E > 1 ? 1 : 0;
+  p.off_gain = p.row * (1u + p.slots);
+  p.bytes = p.off_gain + (norm ? p.row : 0u);
+  p.lean = p.bytes > kDecodePrepSmemLimit;
+  if (p.lean) {
+    p.slots = E > 1 ? 1 : 0;
+    p.bytes = p.row * (size_t)(1 + p.slots);
+  }
+  return p;
+}
+
+// grid (8, M, linears), one cluster per token
 template <int CAP>
 __global__ void __cluster_dims__(kPrepCluster, 1, 1) __maxnreg__(80) k_decode_prep(const __grid_constant__ DecodeBatch<CAP> bp) {
   extern __shared__ __align__(128) uint8_t prep_smem[];
@@ -201,7 +218,6 @@ __global__ void __cluster_dims__(kPrepCluster, 1, 1) __maxnreg__(80) k_decode_pr
   const int m = blockIdx.y, rank = blockIdx.x;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   copy_record(&L, bp, blockIdx.z);
-  const int off_wr = bp.off_wr, off_gain = bp.off_gain;
   if (tid == 0) {
     fail_sh = 0;
     mbar_init(smem_u32(&wr_bar), 1);
@@ -214,8 +230,11 @@ __global__ void __cluster_dims__(kPrepCluster, 1, 1) __maxnreg__(80) k_decode_pr
   const int chunks = K >> 3;
   const uint32_t row_bytes = (uint32_t)K * 2u;
   uint4* xs4 = reinterpret_cast<uint4*>(prep_smem);
-  uint4* gain4 = reinterpret_cast<uint4*>(prep_smem + off_gain);
+  const PrepPlan plan = prep_plan(K, E, L.norm_w != nullptr);
+  const uint32_t off_wr = plan.row;
+  uint4* gain4 = reinterpret_cast<uint4*>(prep_smem + plan.off_gain);   // unless plan.lean
   const int my_experts = E > 1 && rank < E ? (E - rank + kPrepCluster - 1) / kPrepCluster : 0;   // rank, rank + 8
+  const int my_warps = min(my_experts, plan.slots);             // warps that multiply router rows
   // weights start towards L2 while the previous kernel is still running
   if (m == 0) {
     if (tid < my_experts) bulk_prefetch(L.Wr + (long long)(rank + tid * kPrepCluster) * chunks, row_bytes);
@@ -224,8 +243,8 @@ __global__ void __cluster_dims__(kPrepCluster, 1, 1) __maxnreg__(80) k_decode_pr
   pdl_wait();                // X may come from the previous kernel; the buffers written here may still be read by it
   pdl_launch_dependents();   // from here on the kernels behind this one may start: what they read early is final
   if (tid == 0 && my_experts > 0) {
-    mbar_expect_tx(smem_u32(&wr_bar), (uint32_t)my_experts * row_bytes);
-    for (int i = 0; i < my_experts; ++i)
+    mbar_expect_tx(smem_u32(&wr_bar), (uint32_t)my_warps * row_bytes);
+    for (int i = 0; i < my_warps; ++i)
       bulk_load(smem_u32(prep_smem + off_wr) + (uint32_t)i * row_bytes, L.Wr + (long long)(rank + i * kPrepCluster) * chunks, row_bytes, smem_u32(&wr_bar));
   }
 
@@ -244,14 +263,14 @@ __global__ void __cluster_dims__(kPrepCluster, 1, 1) __maxnreg__(80) k_decode_pr
       for (int u = 0; u < 4; ++u) {
         const bool in = c0 + u * kPrepThreads < chunks;
         v[u] = in ? __ldcg(x4 + c0 + u * kPrepThreads) : make_uint4(0u, 0u, 0u, 0u);
-        if (L.norm_w && in) g[u] = __ldcg(L.norm_w + c0 + u * kPrepThreads);
+        if (L.norm_w && in && !plan.lean) g[u] = __ldcg(L.norm_w + c0 + u * kPrepThreads);
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         if (c0 + u * kPrepThreads < chunks) {
           xs4[c0 + u * kPrepThreads] = v[u];
           if (L.norm_w) {
-            gain4[c0 + u * kPrepThreads] = g[u];
+            if (!plan.lean) gain4[c0 + u * kPrepThreads] = g[u];
             ss += sum_squares(v[u]);
           } else {
             fold_amax(v[u]);
@@ -272,7 +291,7 @@ __global__ void __cluster_dims__(kPrepCluster, 1, 1) __maxnreg__(80) k_decode_pr
     for (int w = 0; w < kPrepWarps; ++w) tot += red_d[w];
     const float s = (float)(1.0 / sqrt(tot / (double)K + (double)L.norm_eps));
     for (int c = tid; c < chunks; c += kPrepThreads) {   // each thread reads back the chunks it wrote itself
-      const uint4 v = rms_apply(xs4[c], s, gain4[c]);
+      const uint4 v = rms_apply(xs4[c], s, plan.lean ? __ldcg(L.norm_w + c) : gain4[c]);
       xs4[c] = v;
       fold_amax(v);
     }
@@ -288,32 +307,41 @@ __global__ void __cluster_dims__(kPrepCluster, 1, 1) __maxnreg__(80) k_decode_pr
   asm volatile("barrier.cluster.wait.aligned;" ::: "memory");  // every CTA of the cluster is running
   // router: the same pinned fp32 order as the training path (lane j owns the chunks c = j mod 32, ascending,
   // fused multiply-add; butterfly 16, 8, 4, 2, 1), one warp per expert of this CTA; the cluster exchanges the logits
-  if (warp < my_experts) {
-    decode_wait(smem_u32(&wr_bar), 0, &fail_sh);
+  if (warp < my_warps) {
     const uint4* wrow = reinterpret_cast<const uint4*>(prep_smem + off_wr) + (size_t)warp * chunks;
-    float acc = 0.f;
-    auto fold = [&](const uint4& xv, const uint4& wv) {
-      acc = fmaf(bf16lo(xv.x), bf16lo(wv.x), acc); acc = fmaf(bf16hi(xv.x), bf16hi(wv.x), acc);
-      acc = fmaf(bf16lo(xv.y), bf16lo(wv.y), acc); acc = fmaf(bf16hi(xv.y), bf16hi(wv.y), acc);
-      acc = fmaf(bf16lo(xv.z), bf16lo(wv.z), acc); acc = fmaf(bf16hi(xv.z), bf16hi(wv.z), acc);
-      acc = fmaf(bf16lo(xv.w), bf16lo(wv.w), acc); acc = fmaf(bf16hi(xv.w), bf16hi(wv.w), acc);
-    };
-    int c = lane;
-    for (; c + 96 < chunks; c += 128) {
-      uint4 wv[4], xv[4];
+    for (int k = warp; k < my_experts; k += my_warps) {           // once, unless two rows share a place
+      decode_wait(smem_u32(&wr_bar), k == warp ? 0 : 1, &fail_sh);
+      float acc = 0.f;
+      auto fold = [&](const uint4& xv, const uint4& wv) {
+        acc = fmaf(bf16lo(xv.x), bf16lo(wv.x), acc); acc = fmaf(bf16hi(xv.x), bf16hi(wv.x), acc);
+        acc = fmaf(bf16lo(xv.y), bf16lo(wv.y), acc); acc = fmaf(bf16hi(xv.y), bf16hi(wv.y), acc);
+        acc = fmaf(bf16lo(xv.z), bf16lo(wv.z), acc); acc = fmaf(bf16hi(xv.z), bf16hi(wv.z), acc);
+        acc = fmaf(bf16lo(xv.w), bf16lo(wv.w), acc); acc = fmaf(bf16hi(xv.w), bf16hi(wv.w), acc);
+      };
+      int c = lane;
+      for (; c + 96 < chunks; c += 128) {
+        uint4 wv[4], xv[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) { wv[u] = wrow[c + 32 * u]; xv[u] = xs4[c + 32 * u]; }
+        for (int u = 0; u < 4; ++u) { wv[u] = wrow[c + 32 * u]; xv[u] = xs4[c + 32 * u]; }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) fold(xv[u], wv[u]);
+        for (int u = 0; u < 4; ++u) fold(xv[u], wv[u]);
+      }
+      for (; c < chunks; c += 32) fold(xs4[c], wrow[c]);
+      for (int d = 16; d > 0; d >>= 1) acc = acc + __shfl_xor_sync(0xffffffffu, acc, d);
+      if (lane == 0)
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_map(smem_u32(&logit_sh[rank + k * kPrepCluster]), 0)), "f"(acc) : "memory");
+      if (k + my_warps < my_experts) {
+        __syncwarp();
+        if (lane == 0 && !*(volatile int*)&fail_sh) {
+          mbar_expect_tx(smem_u32(&wr_bar), row_bytes);
+          bulk_load(smem_u32(wrow), L.Wr + (long long)(rank + (k + my_warps) * kPrepCluster) * chunks, row_bytes, smem_u32(&wr_bar));
+        }
+      }
     }
-    for (; c < chunks; c += 32) fold(xs4[c], wrow[c]);
-    for (int d = 16; d > 0; d >>= 1) acc = acc + __shfl_xor_sync(0xffffffffu, acc, d);
-    if (lane == 0)
-      asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_map(smem_u32(&logit_sh[rank + warp * kPrepCluster]), 0)), "f"(acc) : "memory");
   } else {
     // meanwhile the other warps: this CTA's eighth of the token's codes (Eq. 7-9), in fragment order -- an item is one 16-byte
     // piece (chunk and half, quad index) -- and, for the INT8 branch, in natural order
-    const int nhalves = 2 * ((K + 127) >> 7), first = my_experts * 32, nthr = kPrepThreads - first;
+    const int nhalves = 2 * ((K + 127) >> 7), first = my_warps * 32, nthr = kPrepThreads - first;
     const int group = m >> 3, g = m & 7, mg = min(8, L.M - 8 * group);
     const int i_lo = nhalves * 4 * rank / kPrepCluster, i_hi = nhalves * 4 * (rank + 1) / kPrepCluster;
     uint4* dst = L.qfrag + (long long)group * nhalves * 32 + g * 4;
@@ -371,7 +399,7 @@ __global__ void __cluster_dims__(kPrepCluster, 1, 1) __maxnreg__(80) k_decode_pr
     for (int i = 0; i < kPrepCluster * kPrepWarps / 32; ++i) {
       const int k = i * 32 + lane, rk = k / kPrepWarps, w = k % kPrepWarps;
       const int routed = E > 1 && rk < E ? (E - rk + kPrepCluster - 1) / kPrepCluster : 0;
-      if (w >= routed) tot += sum_sh[rk][w];
+      if (w >= min(routed, plan.slots)) tot += sum_sh[rk][w];
     }
     for (int d = 16; d > 0; d >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, d);
     if (lane == 0) L.info[m] = DecodeTokInfo{best, gate, gamma, tot};   // after a failed wait too: an expert that exists
@@ -990,16 +1018,14 @@ static int decode_sm_count() {
 }
 
 constexpr size_t kDecodeMainSmemLimit = 220 * 1024;   // dynamic shared memory of k_decode_main (it has a few KB of its own)
-constexpr size_t kDecodePrepSmemLimit = 200 * 1024;
 
 template <int CAP>
 static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st) {
   static int sms = decode_sm_count();
   DecodeBatch<CAP> bp;
   bp.n = n;
-  size_t h_bytes = 0, x_bytes = 0, slot_bytes = 0;
-  int max_m = 1, max_e = 1, units = 0, max_c = 1, row_bytes = 0;
-  bool any_norm = false;
+  size_t h_bytes = 0, smem_prep = 0, slot_bytes = 0;
+  int max_m = 1, units = 0, max_c = 1, row_bytes = 0;
   bp.hidden_groups = 0;
   for (int i = 0; i < n; ++i) {
     const DecodeItemArgs& it = items[i];
@@ -1013,7 +1039,6 @@ static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st)
     L.acc_dump = it.dump ? reinterpret_cast<int*>(w) : nullptr;
     if (it.dump) w += up256(sizeof(int) * (size_t)M * N);
     L.xn = reinterpret_cast<uint16_t*>(w);
-    any_norm = any_norm || it.norm_weight;
     L.X = reinterpret_cast<const uint4*>(it.X); L.Wr = reinterpret_cast<const uint4*>(it.a.Wr); L.A = it.a.A; L.B = it.a.B;
     L.bits = it.bits; L.bits_il = reinterpret_cast<const uint4*>(it.bits_il);
     L.w_scales = it.a.w_scales; L.alpha = it.a.alpha; L.beta = it.a.beta; L.Y = it.Y;
@@ -1034,8 +1059,8 @@ static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st)
     L.hidden0 = bp.hidden_groups;
     if (r > 0) row_bytes = std::max(row_bytes, it.A8 ? K : 2 * K);
     if (r > 0) bp.hidden_groups += std::min(L.E, M) * ((r + 15) / 16);
-    max_m = std::max(max_m, M); max_e = std::max(max_e, L.E); max_c = std::max(max_c, (K + 127) / 128);
-    x_bytes = std::max(x_bytes, up256((size_t)K * 2));
+    max_m = std::max(max_m, M); max_c = std::max(max_c, (K + 127) / 128);
+    smem_prep = std::max(smem_prep, prep_plan(K, L.E, L.norm_w != nullptr).bytes);
   }
   for (int i = n; i <= CAP; ++i) bp.unit0[i] = units;
   bp.units = units;
@@ -1064,14 +1089,11 @@ static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st)
   const size_t smem_main = off;
 
   // ---- k_decode_prep
-  bp.off_wr = (int)x_bytes;
-  bp.off_gain = (int)(x_bytes + (max_e > 8 ? 2 : max_e > 1 ? 1 : 0) * x_bytes);
   bp.early = bp.hidden_groups > 0;
   // One CTA per SM; with rows of A_e beyond 4 KB, whose contraction is worth more than room for k_decode_main's CTAs beside it, up to
   // three.  Per call, one CTA per cluster against two where two are more than the SMs hold: M = 11, 1056 x 7552 18.6 / 21.7 us, M = 4,
   // INT8, 3200 x 8640 16.9 / 18.3; M = 13, 2816 x 4960 22.1 / 20.7, M = 16, 3200 x 8640 37.2 / 31.4.
   bp.hidden_cluster = 4 * bp.hidden_groups <= sms ? 4 : 2 * bp.hidden_groups <= (row_bytes > 4096 ? 3 * sms : sms) ? 2 : 1;
-  const size_t smem_prep = bp.off_gain + (any_norm ? x_bytes : 0);
   if (smem_prep > kDecodePrepSmemLimit) return PQ_ERR_UNSUPPORTED;
 
   using Kern = void (*)(DecodeBatch<CAP>);

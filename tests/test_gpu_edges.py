@@ -161,3 +161,58 @@ def test_decode_output_that_starts_at_an_odd_element(mode):
         pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 1)
     check_status()
     assert torch.equal(buf[1:-1].view(M, N), L.Y) and buf[0] == 7.0 and buf[-1] == 7.0
+
+
+def _decode_case(T, K, N, r, E, norm, seed=17):
+    c = I.make_linear_case(T, K, N, r, E, seed=seed, exact_quota=False, with_grad=False)
+    L = PQLinear(T, K, N, r, E, training=False, dump_acc=True).load_case(c)
+    w = None
+    if norm:
+        w = I.bf16_values(1.0 + 0.1 * np.random.default_rng(5).standard_normal(K).astype(np.float32))
+        L.norm_weight, L.norm_eps = torch.from_numpy(w).cuda().to(torch.bfloat16), 1e-5
+    L.pack(bits_only=True)
+    return c, L, w
+
+
+def _check_long_row(c, L, w):
+    mu, lam = O.weight_scales(c["W"])
+    f = O.decode_forward(c["X"], O.pack_bits(O.binarize(c["W"], mu)), lam, c["A"], c["B"], c["Wr"], c["alpha"], c["beta"],
+                         **(dict(norm_weight=w, norm_eps=1e-5) if w is not None else {}))
+    v = L.decode_view()
+    assert np.array_equal(v["expert"].cpu().numpy(), f["idx"])
+    assert np.array_equal(v["code_sum"].cpu().numpy(), f["q"].astype(np.int64).sum(axis=1))
+    assert np.array_equal(v["acc"].cpu().numpy().astype(np.int64), f["acc"])
+    assert rel_err(f32(L.Y), f["Y"]) <= TOL_BF16
+
+
+@pytest.mark.parametrize("K,E,norm", [
+    (25600, 16, True), (25632, 16, True),     # token, two router rows and gains: as many as fit, and one group of 32 values more
+    (34112, 16, False), (34112, 8, True), (34144, 8, True), (32768, 1, True),
+])
+def test_decode_of_rows_that_fill_shared_memory(K, E, norm):
+    c, L, w = _decode_case(3, K, 64, 16, E, norm)
+    L.decode()
+    torch.cuda.synchronize()
+    check_status()
+    _check_long_row(c, L, w)
+
+
+@pytest.mark.parametrize("shapes", [
+    [(1, 32768, 32, 16, 1, True), (16, 64, 32, 16, 16, False)],        # the longest row, the most experts and the norm in different linears
+])
+def test_decode_batch_of_linears_that_fit_one_by_one(shapes):
+    layers = [_decode_case(*s, seed=18 + i)[1] for i, s in enumerate(shapes)]
+    pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 0)
+    try:
+        for L in layers:
+            L.decode()
+        torch.cuda.synchronize()
+        want = [L.Y.clone() for L in layers]
+        for L in layers:
+            L.Y.zero_()
+        pqb.pq_decode_batch(pqb.make_decode_items([L.decode_entry() for L in layers]))
+        torch.cuda.synchronize()
+    finally:
+        pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 1)
+    check_status()
+    assert all(torch.equal(L.Y, y) for L, y in zip(layers, want))
