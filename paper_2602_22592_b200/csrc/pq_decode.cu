@@ -1179,6 +1179,8 @@ int decode_batch(const DecodeItemArgs* items, int n, cudaStream_t st) {
           while (m < most && !items[i + m].bits_il) ++m;
       }
       rc = decode_launch(items + i, m, st);
+      // shared memory is laid out for the largest of everything in a launch: what does not fit together may fit apart
+      while (rc == PQ_ERR_UNSUPPORTED && m > 1) rc = decode_launch(items + i, m /= 2, st);
     }
     if (rc) return rc;
     i += m;

@@ -199,6 +199,7 @@ def test_decode_of_rows_that_fill_shared_memory(K, E, norm):
 
 @pytest.mark.parametrize("shapes", [
     [(1, 32768, 32, 16, 1, True), (16, 64, 32, 16, 16, False)],        # the longest row, the most experts and the norm in different linears
+    [(1, 100000, 32, 16, 1, False), (16, 64, 32, 256, 2, False)],      # no room for both in one launch
 ])
 def test_decode_batch_of_linears_that_fit_one_by_one(shapes):
     layers = [_decode_case(*s, seed=18 + i)[1] for i, s in enumerate(shapes)]
