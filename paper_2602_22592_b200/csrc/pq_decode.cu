@@ -388,7 +388,8 @@ __global__ void __cluster_dims__(kPrepCluster, 1, 1) __maxnreg__(80) k_decode_pr
       float lmax = lg;
       for (int d = 16; d > 0; d >>= 1) lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, d));
       best = __ffs(__ballot_sync(0xffffffffu, lane < E && lg == lmax)) - 1;
-      if (best < 0) best = 0;                                  // no logit is a number
+      // as the training path's comparison of one logit after the other has it: expert 0 if its own logit is not a number
+      if (best < 0 || isnan(logit_sh[0])) best = 0;
       const float pe = lane < E ? expf(lg - lmax) : 0.f;
       float den = pe;
       for (int d = 16; d > 0; d >>= 1) den += __shfl_xor_sync(0xffffffffu, den, d);

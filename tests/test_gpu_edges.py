@@ -217,3 +217,23 @@ def test_decode_batch_of_linears_that_fit_one_by_one(shapes):
         pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 1)
     check_status()
     assert all(torch.equal(L.Y, y) for L, y in zip(layers, want))
+
+
+@pytest.mark.parametrize("mode", [0, 2])
+def test_decode_expert_when_the_first_logit_is_not_a_number(mode):
+    # one logit is compared after the other, from expert 0 on: nothing is greater than a logit that is not a number
+    c = I.make_linear_case(3, 256, 96, 16, 4, seed=23, exact_quota=False, with_grad=False)
+    c["Wr"][0, 5] = np.nan
+    D = PQLinear(3, 256, 96, 16, 4, training=False).load_case(c)
+    L = PQLinear(3, 256, 96, 16, 4).load_case(c)
+    pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, mode)
+    try:
+        D.pack(bits_only=True)
+        D.decode()
+        L.pack()
+        L.forward()
+        torch.cuda.synchronize()
+    finally:
+        pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 1)
+    check_status()
+    assert D.decode_view()["expert"].tolist() == L.saved_view()["expert"].tolist() == [0, 0, 0]
