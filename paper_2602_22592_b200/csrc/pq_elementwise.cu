@@ -463,10 +463,11 @@ __device__ __forceinline__ uint4 swiglu8(const uint4& g, const uint4& u) {
 // between the absmax pass and the quantising pass (rows of up to 256 * CH * WPR elements), so X is read
 // once; CH = 0 reads the row twice.
 // Bound by memory (routed training layer: 7 bytes written and 2 read per value), and to reach it by the rows in flight: four
-// pieces per lane and as many warps per row as that takes leave room for five blocks per SM.  Eight pieces per lane (two blocks)
+// pieces per lane and as many warps per row as that takes leave room for five blocks per SM; for rows of one warp, four: held to 48
+// registers that form went to memory with 52 bytes a thread (8192 x 1024 with the forward tile 23.2 us, 21.3 so).  Eight pieces per lane (two blocks)
 // and four, routed: 8192 x 2048 21.2 -> 17.3 us, 8192 x 5632 67 -> 58 us (5.6 TB/s); with the SwiGLU 38 -> 22.5 us.
 template <int CH, int WPR, bool SWIGLU = false>
-__global__ void __launch_bounds__(256, CH > 0 ? 5 : 2) k_act_quant(const uint4* __restrict__ X, int T, int K, int E, const int* __restrict__ expert,
+__global__ void __launch_bounds__(256, CH == 0 ? 2 : WPR == 1 ? 4 : 5) k_act_quant(const uint4* __restrict__ X, int T, int K, int E, const int* __restrict__ expert,
                                                    const int* __restrict__ block_base, const int* __restrict__ offsets,
                                                    const float* __restrict__ gate_tok, const float* __restrict__ probs_tok,
                                                    uint2* __restrict__ q, uint4* __restrict__ xt, uint4* __restrict__ xs,
