@@ -317,36 +317,48 @@ __device__ __forceinline__ void gemm_body(const typename P::Params& p) {
         for (int s = 0; ok && s < nseg; ++s) {
           Segment sg;
           P::segment(p, t, s, sg);
-          const int a_step = (sg.mode == MODE_I8_KK) ? 128 : 64;
-          for (int kb = 0; kb < sg.nkb; ++kb) {
-            if (!pipe_wait(empty_bar(st.stage), st.phase ^ 1, WHERE_PRODUCER, abort_flag)) { ok = false; break; }
-            // the barrier of the issuing CTA counts the bytes of both
-            uint32_t bar = full_bar(st.stage);
-            if (rank == 0) mbar_expect_tx(bar, CG * (kOperandBytes + sg.b_bytes));
-            if (CG == 2) bar = cluster_map(bar, 0);
-            const uint32_t sa = smem_base + st.stage * kStageBytes, sb = sa + kOperandBytes;
-            if (a_is_mn(sg.mode)) {
-              if (sg.a_blk > 0) {
-                tma_fetch_blocked<CG>(sa, sg.ta, bar, sg.a_rank, sg.a_y + kb * 64, sg.a_x >> 6, sg.a_z);
+          // LOADS: how a step's operands come, chosen once per segment -- 0: both K-major, 1: B MN-major through a blocked map,
+          // 2: both MN-major through blocked maps, 3: as the segment says.  With these tests inside the loop, a step of a problem
+          // whose segments differ (the backward) cost the one issuing lane more than the 512 cycles that its MMAs take: one 256 x 256
+          // tile of dW over 8192 and 16384 tokens 60 and 103 us; as it is now 52 and 87 (537 cycles a step).
+          auto produce = [&](auto loads) {
+            constexpr int LOADS = decltype(loads)::value;
+            const int a_step = (sg.mode == MODE_I8_KK) ? 128 : 64;
+            const uint32_t bytes = CG * (kOperandBytes + sg.b_bytes);
+            for (int kb = 0; kb < sg.nkb; ++kb) {
+              if (!pipe_wait(empty_bar(st.stage), st.phase ^ 1, WHERE_PRODUCER, abort_flag)) { ok = false; break; }
+              // the barrier of the issuing CTA counts the bytes of both
+              uint32_t bar = full_bar(st.stage);
+              if (rank == 0) mbar_expect_tx(bar, bytes);
+              if (CG == 2) bar = cluster_map(bar, 0);
+              const uint32_t sa = smem_base + st.stage * kStageBytes, sb = sa + kOperandBytes;
+              if (LOADS == 2 || (LOADS == 3 && a_is_mn(sg.mode))) {
+                if (LOADS == 2 || sg.a_blk > 0) {
+                  tma_fetch_blocked<CG>(sa, sg.ta, bar, LOADS == 2 ? 2 : sg.a_rank, sg.a_y + kb * 64, sg.a_x >> 6, sg.a_z);
+                } else {
+                  tma_fetch<CG>(sa, sg.ta, bar, sg.a_rank, sg.a_x, sg.a_y + kb * 64, sg.a_z);
+                  tma_fetch<CG>(sa + kMnBoxBytes, sg.ta, bar, sg.a_rank, sg.a_x + 64, sg.a_y + kb * 64, sg.a_z);
+                }
               } else {
-                tma_fetch<CG>(sa, sg.ta, bar, sg.a_rank, sg.a_x, sg.a_y + kb * 64, sg.a_z);
-                tma_fetch<CG>(sa + kMnBoxBytes, sg.ta, bar, sg.a_rank, sg.a_x + 64, sg.a_y + kb * 64, sg.a_z);
+                tma_fetch<CG>(sa, sg.ta, bar, sg.a_rank, sg.a_x + kb * a_step, sg.a_y, sg.a_z);
               }
-            } else {
-              tma_fetch<CG>(sa, sg.ta, bar, sg.a_rank, sg.a_x + kb * a_step, sg.a_y, sg.a_z);
-            }
-            if (b_is_mn(sg.mode)) {
-              if (sg.b_blk > 0) {
-                tma_fetch_blocked<CG>(sb, sg.tb, bar, sg.b_rank, sg.b_y + kb * 64, sg.b_x >> 6, sg.b_z);
+              if (LOADS == 1 || LOADS == 2 || (LOADS == 3 && b_is_mn(sg.mode))) {
+                if (LOADS != 3 || sg.b_blk > 0) {
+                  tma_fetch_blocked<CG>(sb, sg.tb, bar, sg.b_rank, sg.b_y + kb * 64, sg.b_x >> 6, sg.b_z);
+                } else {
+                  for (int b = 0; b < -sg.b_blk; ++b)
+                    tma_fetch<CG>(sb + b * kMnBoxBytes, sg.tb, bar, sg.b_rank, sg.b_x + 64 * b, sg.b_y + kb * 64, sg.b_z);
+                }
               } else {
-                for (int b = 0; b < -sg.b_blk; ++b)
-                  tma_fetch<CG>(sb + b * kMnBoxBytes, sg.tb, bar, sg.b_rank, sg.b_x + 64 * b, sg.b_y + kb * 64, sg.b_z);
+                tma_fetch<CG>(sb, sg.tb, bar, sg.b_rank, sg.b_x + kb * a_step, sg.b_y, sg.b_z);
               }
-            } else {
-              tma_fetch<CG>(sb, sg.tb, bar, sg.b_rank, sg.b_x + kb * a_step, sg.b_y, sg.b_z);
+              st.advance(kStages);
             }
-            st.advance(kStages);
-          }
+          };
+          if (sg.mode <= MODE_BF_KK) produce(std::integral_constant<int, 0>{});
+          else if (sg.mode == MODE_BF_KM && sg.b_blk > 0) produce(std::integral_constant<int, 1>{});
+          else if (sg.mode == MODE_BF_MM && sg.a_blk > 0 && sg.b_blk > 0 && sg.a_rank == 2) produce(std::integral_constant<int, 2>{});
+          else produce(std::integral_constant<int, 3>{});
         }
       }
     }
