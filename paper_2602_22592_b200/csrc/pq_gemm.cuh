@@ -203,8 +203,8 @@ struct stage_rows_of<P, std::void_t<decltype(&P::stage_rows)>> {
 struct AccDouble { static constexpr bool kSplit = false; };
 struct AccSplit { static constexpr bool kSplit = true; };
 
-// Problems that hand out their tiles by ticket name the counter (cleared before the launch) and may hold a tile back until what
-// it reads has been written: `ready`, called by the producers, returns false if it gave up.
+// Problems that hand out their tiles by ticket name the counter (cleared before the launch) and may hold a segment back until what
+// it reads has been written: `ready`, called by the producers before each, returns false if it gave up.
 template <class P, class = void>
 struct tickets_of : std::false_type {};
 template <class P>
@@ -314,10 +314,10 @@ __device__ __forceinline__ void gemm_body(const typename P::Params& p) {
       for (int tile = next(-1); ok && tile < ntiles; tile = next(tile)) {
         typename P::Tile t;
         P::tile_init(p, tile, rank, t);
-        if constexpr (kTickets) { if (!P::ready(p, t, abort_flag)) break; }
         const int nseg = P::num_segments(p, t);
         if (nseg == 0) draw();
         for (int s = 0; ok && s < nseg; ++s) {
+          if constexpr (kTickets) { if (!P::ready(p, t, s, abort_flag)) { ok = false; break; } }
           Segment sg;
           P::segment(p, t, s, sg);
           // LOADS: how a step's operands come, chosen once per segment -- 0: both K-major, 1: B MN-major through a blocked map,

@@ -715,7 +715,7 @@ struct BwdProblem {
     float* dalpha_partial;   // [2 * E, N]
     unsigned* sync;          // {.., tickets, finished warps of dH tiles}
     TileGrid gx, gw;
-    int T, N, K, r, r64, E, sstride, item_rows, ntn, ntk, mpairs, hp, long_experts;
+    int T, N, K, r, r64, E, sstride, item_rows, ntn, ntk, mpairs, hp, long_experts, early_dx;
     int ba_blk, sb_blk, a3_blk, wr_blk, dy_blk, xt_blk, gh_blk, xs_blk, dh_blk;
   };
   // nt: this CTA's block of 128 rows (tokens, features, or columns of K); [ib, ie): items (dB, dA), pair entries (dX); item: this
@@ -772,9 +772,10 @@ struct BwdProblem {
     if (x < p.ntn) { t.kind = KIND_DB; t.nt = 2 * x + rank; t.bn = 2 * p.r64; }
     else { t.kind = KIND_DA; t.nt = 2 * (x - p.ntn) + rank; t.bn = 128; }
   }
-  // what reads the results of the dH tiles waits for them; they were written through the generic proxy
-  __device__ static bool ready(const Params& p, const Tile& t, volatile int* abort_flag) {
-    if (!p.hp || t.kind == KIND_DH || t.kind == KIND_DW) return true;
+  // What reads the results of the dH tiles waits for them; they were written through the generic proxy.  In a dX tile that is every
+  // segment but the first, the product with Sb; where it is long and the tiles are few (see early_dx) the wait comes after it.
+  __device__ static bool ready(const Params& p, const Tile& t, int i, volatile int* abort_flag) {
+    if (!p.hp || t.kind == KIND_DH || t.kind == KIND_DW || i != (t.kind == KIND_DX && !t.skip1 && p.early_dx ? 1 : 0)) return true;
     const unsigned want = 8u * dh_tiles(p);                // four warps in each CTA of a pair
     const long long t0 = clock64();
     unsigned v;
@@ -1101,6 +1102,10 @@ int gemm_backward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, c
   p.dbeta_partial = b.dbeta_partial; p.dalpha_partial = b.dalpha_partial; p.sync = b.sync;
   p.T = a.T; p.N = a.N; p.K = a.K; p.r = a.r; p.r64 = r64; p.E = hp ? a.E : 1; p.sstride = a.scale_stride; p.item_rows = (int)item_rows;
   p.ntn = ntn; p.ntk = ntk; p.mpairs = (a.T + 255) / 256; p.hp = hp; p.long_experts = hp && a.E == 1;
+  // A dX tile that has done its first product beside the dH tiles has little left when they are finished; one of many, drawn by pairs
+  // that the dH tiles need the L2 of, only slows them.  Backward, waiting before and after: 512 tokens, 1024 -> 4096, one / eight experts
+  // 68 / 83 and 56 / 71 us; 1024 tokens, 1024 -> 1024, eight experts 51 and 47; 8192 tokens, 2048 -> 2048, one / eight 134 / 161 and 137 / 166.
+  p.early_dx = routed ? a.N >= a.T : a.N > a.T;
   p.gx = make_tile_grid(p.mpairs, ntk, 256);
   p.gw = make_tile_grid(ntn, ntk, 256);
   return launch_gemm<BwdProblem>(KID_BWD_DW, k_gemm_bwd, p, p.gx.total + p.gw.total + (hp ? p.E * (ntn + ntk) : 0), st);
