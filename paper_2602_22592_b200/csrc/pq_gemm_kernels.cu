@@ -371,13 +371,14 @@ PQ_DEFINE_GEMM_KERNEL(k_gemm_hp_up8, HpUp8Problem)
 // ---------------------------------------------------------------------------
 // GEN = false: scalar feature scales and K < 32768; GEN = true: anything (the extra addresses and branches cost registers the
 // common form does not have to spare).
-template <bool HP, bool GEN>
+// CG_: a pair of CTAs per 256 rows, or one CTA per 128 (see gemm_forward).
+template <bool HP, bool GEN, int CG_>
 struct FwdProblem {
   // With the HP branch a tile holds an int32 and an fp32 accumulator of 256 columns each, all of TMEM.  Sixteen epilogue
   // warps, 64 columns of a row per thread: the fp32 accumulator waits in 64 registers while the int8 contraction runs, and
   // what the next tile's int8 contraction has to wait for is only the read of the int32 accumulator, which the next tile's
   // HP segments cover.
-  static constexpr int CG = 2, kEpiWarps = HP ? 16 : 8;
+  static constexpr int CG = CG_, kEpiWarps = HP ? 16 : 8;
   using Acc = typename std::conditional<HP, AccSplit, AccDouble>::type;
   struct Params {
     CUtensorMap tq, ts, ts2, th, tb;  // q [T,K] s8; S [N,K] s8, of a second matrix too; H [items*128,r]; B [E,N,r]
@@ -408,27 +409,33 @@ struct FwdProblem {
     t.second = !HP && t.c.n0 >= p.tiles1 * p.g.bn;
     if (t.second) t.c.n0 -= p.tiles1 * p.g.bn;
     t.bn = clip_bn(t.c.bn, t.c.n0, p.N, 32);
-    if (HP) { t.pb = p.rt.pair_begin[t.c.m >> 1]; t.pe = p.rt.pair_begin[(t.c.m >> 1) + 1]; } else { t.pb = t.pe = 0; }
+    const int* begin = CG == 2 ? p.rt.pair_begin : p.rt.tile_item_begin;   // entries of the pair of row tiles, or items of the row tile
+    if (HP) { t.pb = begin[t.c.m / CG]; t.pe = begin[t.c.m / CG + 1]; } else { t.pb = t.pe = 0; }
   }
   // The HP product uses the leading bf16 plane of H only: its 2^-9 relative rounding is of the size of the
   // output's own rounding to bf16; the second plane serves the backward pass, whose sums are longer.
   __device__ static int num_segments(const Params&, const Tile& t) { return (t.pe - t.pb) + 1; }
   __device__ static void segment(const Params& p, const Tile& t, int i, Segment& s) {
-    s.bn = t.bn; s.ksteps = 4; s.a_z = 0; s.b_z = 0; s.a_blk = 0; s.b_blk = 0; s.b_bytes = kOperandBytes;
-    s.b_x = 0; s.b_y = t.c.n0 + t.rank * (t.bn >> 1);
+    s.bn = t.bn; s.ksteps = 4; s.a_z = 0; s.b_z = 0; s.a_blk = 0; s.b_blk = 0; s.b_bytes = kOperandBytes * (2 / CG);
+    s.b_x = 0; s.b_y = t.c.n0 + t.rank * (t.bn / CG);
     if (i == t.pe - t.pb) {
       s.mode = MODE_I8_KK; s.acc = 0; s.nkb = (p.K + 127) / 128;
       s.ta = &p.tq; s.a_rank = 2; s.a_x = 0; s.a_y = t.c.m * 128;
       s.tb = t.second ? &p.ts2 : &p.ts; s.b_rank = 2;
     } else {
-      const int4 pi = p.rt.pair_items[t.pb + i];
-      const int item = t.rank ? pi.z : pi.y;
+      int item, expert;
+      if (CG == 2) {
+        const int4 pi = p.rt.pair_items[t.pb + i];
+        item = t.rank ? pi.z : pi.y; expert = pi.x;
+      } else {
+        item = t.pb + i; expert = p.rt.items[item].y;
+      }
       if (p.gamma_h) { s.mode = MODE_I8_KK; s.nkb = (p.r + 127) / 128; }
       else { s.mode = MODE_BF_KK; s.nkb = (p.r + 63) / 64; }
       s.acc = 1;
       s.ta = &p.th; s.a_rank = p.gamma_h ? 3 : 2; s.a_x = 0;
       s.a_y = item >= 0 ? item * 128 : 2 * p.item_rows;    // no rows of this expert here: beyond both planes of H, read as zeros
-      s.tb = &p.tb; s.b_rank = 3; s.b_z = pi.x;
+      s.tb = &p.tb; s.b_rank = 3; s.b_z = expert;
     }
   }
   // float of an accumulator of the 1-bit product, exactly.  |acc| <= 128 K: below K = 32768 the integer fits the mantissa of
@@ -562,14 +569,22 @@ struct FwdProblem {
   }
 };
 // (the macro takes one name per problem)
-using FwdHp = FwdProblem<true, false>;
-using FwdHpGen = FwdProblem<true, true>;
-using Fwd1 = FwdProblem<false, false>;
-using Fwd1Gen = FwdProblem<false, true>;
+using FwdHp = FwdProblem<true, false, 2>;
+using FwdHpGen = FwdProblem<true, true, 2>;
+using Fwd1 = FwdProblem<false, false, 2>;
+using Fwd1Gen = FwdProblem<false, true, 2>;
+using FwdHpSingle = FwdProblem<true, false, 1>;
+using FwdHpGenSingle = FwdProblem<true, true, 1>;
+using Fwd1Single = FwdProblem<false, false, 1>;
+using Fwd1GenSingle = FwdProblem<false, true, 1>;
 PQ_DEFINE_GEMM_KERNEL(k_gemm_fwd_hp, FwdHp)
 PQ_DEFINE_GEMM_KERNEL(k_gemm_fwd_hp_general, FwdHpGen)
 PQ_DEFINE_GEMM_KERNEL(k_gemm_fwd_1bit, Fwd1)
 PQ_DEFINE_GEMM_KERNEL(k_gemm_fwd_1bit_general, Fwd1Gen)
+PQ_DEFINE_GEMM_KERNEL(k_gemm_fwd_hp_single, FwdHpSingle)
+PQ_DEFINE_GEMM_KERNEL(k_gemm_fwd_hp_general_single, FwdHpGenSingle)
+PQ_DEFINE_GEMM_KERNEL(k_gemm_fwd_1bit_single, Fwd1Single)
+PQ_DEFINE_GEMM_KERNEL(k_gemm_fwd_1bit_general_single, Fwd1GenSingle)
 
 // INT8 branch: the saved h region holds the codes qh [items*128, r] and, behind them, gamma_h [items*128]
 static inline float* hp8_gamma_h(const SavedPtrs& sv, int r) {
@@ -578,32 +593,32 @@ static inline float* hp8_gamma_h(const SavedPtrs& sv, int r) {
 }
 
 // the fused output tile of a layer, with or without an HP branch
-template <bool HP, bool GEN>
-static int launch_forward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, uint16_t* Y, void (*kernel)(typename FwdProblem<HP, GEN>::Params),
+template <class P>
+static int launch_forward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, uint16_t* Y, void (*kernel)(typename P::Params), bool HP,
                           cudaStream_t st, const SecondWeight& second) {
-  using P = FwdProblem<HP, GEN>;
+  constexpr int rows_b = 256 / P::CG;                // features of a tile that one CTA loads
   typename P::Params f;
   if (!map2d(&f.tq, true, sv.q, a.K, a.T, 128, 128)) return PQ_ERR_CUDA;
-  if (!map2d(&f.ts, true, w_s8, a.K, a.N, 128, 128)) return PQ_ERR_CUDA;
+  if (!map2d(&f.ts, true, w_s8, a.K, a.N, 128, rows_b)) return PQ_ERR_CUDA;
   f.ts2 = f.ts; f.w_scales2 = second.w_scales; f.Y2 = second.Y;
-  if (second.w_s8 && !map2d(&f.ts2, true, second.w_s8, a.K, a.N, 128, 128)) return PQ_ERR_CUDA;
+  if (second.w_s8 && !map2d(&f.ts2, true, second.w_s8, a.K, a.N, 128, rows_b)) return PQ_ERR_CUDA;
   f.th = f.tq; f.tb = f.tq;
   f.gamma_h = nullptr; f.hp_scales = a.hp_scales; f.hp_ext = a.hp_ext ? 1 : 0;
   if (HP && a.hp_scales) {
     // INT8 branch: codes of h [items*128, r] and of B_e [E, N, r], one byte per value
     const uint64_t rows = (uint64_t)sv.max_items * 128;
     if (!map3d_i8(&f.th, sv.h, a.r, a.r, rows, 1, 128)) return PQ_ERR_CUDA;
-    if (!map3d_i8(&f.tb, a.B, a.r, a.r, a.N, a.E, 128)) return PQ_ERR_CUDA;
+    if (!map3d_i8(&f.tb, a.B, a.r, a.r, a.N, a.E, rows_b)) return PQ_ERR_CUDA;
     f.gamma_h = hp8_gamma_h(sv, a.r);
   } else if (HP) {
     if (!map2d(&f.th, false, sv.h, a.r, (uint64_t)sv.max_items * 256, 64, 128)) return PQ_ERR_CUDA;
-    if (!map3d(&f.tb, a.B, a.r, a.N, a.E, 64, 128)) return PQ_ERR_CUDA;
+    if (!map3d(&f.tb, a.B, a.r, a.N, a.E, 64, rows_b)) return PQ_ERR_CUDA;
   }
   f.rt = sv.rt; f.perm = (HP && a.E > 1) ? sv.perm : nullptr; f.gamma = sv.gamma; f.gate = sv.gate; f.w_scales = a.w_scales;
   f.alpha = a.alpha; f.beta = a.beta; f.Y = Y; f.T = a.T; f.N = a.N; f.K = a.K; f.r = a.r; f.sstride = a.scale_stride;
   f.item_rows = sv.max_items * 128;
   f.tiles1 = (a.N + 255) / 256;
-  f.g = make_tile_grid((a.T + 255) / 256, f.tiles1 * (second.w_s8 ? 2 : 1), 256);
+  f.g = make_tile_grid((a.T + 128 * P::CG - 1) / (128 * P::CG), f.tiles1 * (second.w_s8 ? 2 : 1), 256);
   return launch_gemm<P>(KID_FWD, kernel, f, f.g.total, st);
 }
 
@@ -637,9 +652,19 @@ int gemm_forward(const LayerArgs& a, const int8_t* w_s8, const SavedPtrs& sv, co
   }
   if (before_main && cudaStreamWaitEvent(st, before_main, 0) != cudaSuccess) return PQ_ERR_CUDA;
   const bool general = a.scale_stride != 0 || a.K >= 32768;
+  // A pair takes half of the operand bytes per MMA, but its two CTAs go through launch, accumulators and epilogue in step: worth it from
+  // a contraction of more than eight steps on.  Forward, single / pairs: 8192 tokens, 512 -> 2048, dense 33.9 / 39.5 us, 1024 -> 1024
+  // 31.1 / 33.2, 256 tokens, 512 -> 512 20.8 / 22.4; without experts 8192, 2048 -> 2048 50.5 / 47.0, 2048, 3200 -> 8640 54.7 / 50.1.
+  const bool pairs = a.K > 1024;
+  if (a.r > 0 && pairs)
+    return general ? launch_forward<FwdHpGen>(a, w_s8, sv, Y, k_gemm_fwd_hp_general, true, st, second) : launch_forward<FwdHp>(a, w_s8, sv, Y, k_gemm_fwd_hp, true, st, second);
   if (a.r > 0)
-    return general ? launch_forward<true, true>(a, w_s8, sv, Y, k_gemm_fwd_hp_general, st, second) : launch_forward<true, false>(a, w_s8, sv, Y, k_gemm_fwd_hp, st, second);
-  return general ? launch_forward<false, true>(a, w_s8, sv, Y, k_gemm_fwd_1bit_general, st, second) : launch_forward<false, false>(a, w_s8, sv, Y, k_gemm_fwd_1bit, st, second);
+    return general ? launch_forward<FwdHpGenSingle>(a, w_s8, sv, Y, k_gemm_fwd_hp_general_single, true, st, second)
+                   : launch_forward<FwdHpSingle>(a, w_s8, sv, Y, k_gemm_fwd_hp_single, true, st, second);
+  if (pairs)
+    return general ? launch_forward<Fwd1Gen>(a, w_s8, sv, Y, k_gemm_fwd_1bit_general, false, st, second) : launch_forward<Fwd1>(a, w_s8, sv, Y, k_gemm_fwd_1bit, false, st, second);
+  return general ? launch_forward<Fwd1GenSingle>(a, w_s8, sv, Y, k_gemm_fwd_1bit_general_single, false, st, second)
+                 : launch_forward<Fwd1Single>(a, w_s8, sv, Y, k_gemm_fwd_1bit_single, false, st, second);
 }
 
 

@@ -237,3 +237,14 @@ def test_decode_expert_when_the_first_logit_is_not_a_number(mode):
         pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 1)
     check_status()
     assert D.decode_view()["expert"].tolist() == L.saved_view()["expert"].tolist() == [0, 0, 0]
+
+
+@pytest.mark.parametrize("T,K,N,r,E,vector", [
+    (1, 32, 32, 8, 1, False), (257, 1024, 544, 72, 2, True),   # a lone tile; the longest contraction on single CTAs, rows left over in both forms
+    (257, 1056, 544, 72, 2, False),                            # the shortest on pairs
+    (513, 128, 288, 128, 16, False), (640, 512, 96, 0, 0, True),
+])
+def test_forward_on_single_ctas_and_on_pairs(T, K, N, r, E, vector):
+    c = I.make_linear_case(T, K, N, r, E, seed=T, scale_vector=vector, alpha=1.5, beta=0.5, with_grad=False)
+    f = O.linear_forward(c["X"], c["W"], c["A"], c["B"], c["Wr"], c["alpha"], c["beta"])
+    check_forward(c, run_forward(c, vector), f)
