@@ -753,6 +753,7 @@ int pq_set_option(int option, int value) {
       // the limit lives in constant memory of the current device; the copy is ordered after everything
       // already enqueued there (a blocking copy), so no running kernel sees it change
       const long long cycles = value > 0 ? (long long)value : kDefaultSpinCycles;
+      decode_set_poll(cycles < 1000);
       return cudaMemcpyToSymbol(c_spin_cycles, &cycles, sizeof(cycles)) == cudaSuccess ? PQ_OK : PQ_ERR_CUDA;
     }
     default: return PQ_ERR_UNSUPPORTED;

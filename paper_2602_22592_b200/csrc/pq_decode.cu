@@ -111,6 +111,7 @@ static_assert(sizeof(DecodeLinear) % 16 == 0, "copied in 16-byte pieces");
 template <int CAP>
 struct DecodeBatch {
   int n, units;             // linears; units of 16 features of all of them
+  int poll;                 // waits are polled
   int early;                // k_decode_hidden runs in between: k_decode_main may read prep's results before it waits
   int hidden_groups, hidden_cluster;   // k_decode_hidden: clusters of all linears, CTAs of each
   // k_decode_main: buffers of sign bits, their size, and the carve-up of shared memory behind them
@@ -135,9 +136,9 @@ __device__ __forceinline__ void copy_record(DecodeLinear* dst, const DecodeBatch
 // Wait with a bound.  Once any wait of the CTA has run out, every later wait returns at once, so that
 // all threads keep the same control flow and the kernel ends (with an error status and undefined output): no copy is
 // issued any more, and decode_drain lets those in flight land before the CTA's shared memory passes to another.
-// A copy takes a microsecond or two, less than the hardware may suspend a waiting thread for: a limit as short as that is polled.
-__device__ __forceinline__ void decode_wait(uint32_t bar, uint32_t parity, volatile int* fail) {
-  const bool poll = c_spin_cycles < 1000;
+// A copy takes a microsecond or two, less than the hardware may suspend a waiting thread for: a limit as short as that is polled
+// (`poll`, from the host: to look the limit up here is a trip to memory that no wait hides, 0.35 us a call).
+__device__ __forceinline__ void decode_wait(uint32_t bar, uint32_t parity, volatile int* fail, bool poll) {
   auto done = [&] { return poll ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity); };
   if (done()) return;
   const long long t0 = clock64();
@@ -218,6 +219,7 @@ __global__ void __cluster_dims__(kPrepCluster, 1, 1) __maxnreg__(80) k_decode_pr
   const int m = blockIdx.y, rank = blockIdx.x;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   copy_record(&L, bp, blockIdx.z);
+  const bool poll = bp.poll;
   if (tid == 0) {
     fail_sh = 0;
     mbar_init(smem_u32(&wr_bar), 1);
@@ -310,7 +312,7 @@ __global__ void __cluster_dims__(kPrepCluster, 1, 1) __maxnreg__(80) k_decode_pr
   if (warp < my_warps) {
     const uint4* wrow = reinterpret_cast<const uint4*>(prep_smem + off_wr) + (size_t)warp * chunks;
     for (int k = warp; k < my_experts; k += my_warps) {           // once, unless two rows share a place
-      decode_wait(smem_u32(&wr_bar), k == warp ? 0 : 1, &fail_sh);
+      decode_wait(smem_u32(&wr_bar), k == warp ? 0 : 1, &fail_sh, poll);
       float acc = 0.f;
       auto fold = [&](const uint4& xv, const uint4& wv) {
         acc = fmaf(bf16lo(xv.x), bf16lo(wv.x), acc); acc = fmaf(bf16hi(xv.x), bf16hi(wv.x), acc);
@@ -672,6 +674,7 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
   copy_record(&lin_sh[l_at & 1], bp, l_at);
   if (l_at + 1 < bp.n && bp.unit0[l_at + 1] < u_hi) copy_record(&lin_sh[(l_at + 1) & 1], bp, l_at + 1);
   const int nbuf = bp.nbuf, buf_bytes = bp.buf_bytes, q_chunks = bp.q_chunks, MT = bp.red_tokens, off_h = bp.off_h;
+  const bool poll = bp.poll;
   if (tid == 0) fail_sh = 0;
   if (tid < 2 + kMaxRows) {
     mbar_init(smem_u32(&bars[tid]), 1);
@@ -806,7 +809,7 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
     const int tiles = cur.nu, pairs = (tiles + 1) >> 1, S = kMainWarps / pairs;   // at most 4 pairs of tiles
     const int sl = warp / pairs, tile = 2 * (warp - sl * pairs);
     if (L.bits_il) {
-      decode_wait(smem_u32(&bars[b]), phase[b], &fail_sh);
+      decode_wait(smem_u32(&bars[b]), phase[b], &fail_sh, poll);
       phase[b] ^= 1u;
     }
     {
@@ -901,7 +904,7 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
     }
     for (int i = warp, j = 0; i < items; i += W) {
       const int ei = i / tiles, t = i - ei * tiles;
-      decode_wait(smem_u32(&bars[2 + warp * kWarpRows + j]), (row_phase >> j) & 1u, &fail_sh);
+      decode_wait(smem_u32(&bars[2 + warp * kWarpRows + j]), (row_phase >> j) & 1u, &fail_sh, poll);
       row_phase ^= 1u << j;
       main_expert(reinterpret_cast<const uint4*>(ring + (size_t)(warp * per + j) * item_bytes), r, order_sh + first_sh[ei], count_sh[ei], h_s, lane, red_z + (size_t)t * MT * 16);
       __syncwarp();
@@ -1010,6 +1013,8 @@ DecodeViewPtrs decode_view(int M, int K, int N, int r, void* ws, bool dump) {
 // Launch option: programmatic stream serialisation of the two decode kernels (on by default).
 static int g_decode_pdl = 1;
 void decode_set_pdl(int on) { g_decode_pdl = on ? 1 : 0; }
+static int g_decode_poll = 0;
+void decode_set_poll(int on) { g_decode_poll = on ? 1 : 0; }
 
 static int decode_sm_count() {
   int dev = 0, n = 0;
@@ -1025,6 +1030,7 @@ static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st)
   static int sms = decode_sm_count();
   DecodeBatch<CAP> bp;
   bp.n = n;
+  bp.poll = g_decode_poll;
   size_t h_bytes = 0, smem_prep = 0, slot_bytes = 0;
   int max_m = 1, units = 0, max_c = 1, row_bytes = 0;
   bp.hidden_groups = 0;

@@ -152,6 +152,7 @@ int decode_stream_mode();
 void decode_stream_reset();
 int decode_batch(const DecodeItemArgs* items, int n, cudaStream_t st);   // independent linears, launched together
 void decode_set_pdl(int on);
+void decode_set_poll(int on);           // waits without suspension (a spin limit of a few cycles)
 DecodeViewPtrs decode_view(int M, int K, int N, int r, void* ws, bool dump);
 
 struct BwdBuffers {
