@@ -135,26 +135,23 @@ __device__ __forceinline__ void copy_record(DecodeLinear* dst, const DecodeBatch
 
 // Wait with a bound.  Once any wait of the CTA has run out, every later wait returns at once, so that
 // all threads keep the same control flow and the kernel ends (with an error status and undefined output): no copy is
-// issued any more, and decode_drain lets those in flight land before the CTA's shared memory passes to another.
+// issued any more, and the thread whose wait ran out sleeps until those in flight have landed, before the CTA's shared memory passes to
+// another.  (Here, and plain barriers behind it: a look at `fail` at the end of each kernel and barriers that vote on it were 0.3 us a call.)
 // A copy takes a microsecond or two, less than the hardware may suspend a waiting thread for: a limit as short as that is polled
 // (`poll`, from the host: to look the limit up here is a trip to memory that no wait hides, 0.35 us a call).
 __device__ __forceinline__ void decode_wait(uint32_t bar, uint32_t parity, volatile int* fail, bool poll) {
   auto done = [&] { return poll ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity); };
-  if (done()) return;
+  if (done() || *fail) return;
   const long long t0 = clock64();
   while (!done()) {
     if (*fail) return;
     if (clock64() - t0 > c_spin_cycles) {
       report_timeout(WHERE_OTHER);
       *fail = 1;
+      for (int i = 0; i < 200; ++i) __nanosleep(1000);
       return;
     }
   }
-}
-
-__device__ __forceinline__ void decode_drain(volatile int* fail) {
-  if (*fail)
-    for (int i = 0; i < 200; ++i) __nanosleep(1000);
 }
 
 __device__ __forceinline__ int quant_code(float x, float gamma) { return max(-128, min(127, __float2int_rn(__fmul_rn(x, gamma)))); }
@@ -407,7 +404,6 @@ __global__ void __cluster_dims__(kPrepCluster, 1, 1) __maxnreg__(80) k_decode_pr
     for (int d = 16; d > 0; d >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, d);
     if (lane == 0) L.info[m] = DecodeTokInfo{best, gate, gamma, tot};   // after a failed wait too: an expert that exists
   }
-  decode_drain(&fail_sh);
 }
 
 // ---------------------------------------------------------------------------
@@ -856,8 +852,7 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
       else { if (tiles > 1) bits(One{}, Two{}); else bits(One{}, One{}); }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // what plain stores filled may be overwritten by bulk copies
-    // the sign bits of this pass have been used; after a failed wait nothing is issued over copies that may be in flight
-    if (__syncthreads_or(*(volatile int*)&fail_sh)) break;
+    __syncthreads();                                             // the sign bits of this pass have been used
     // ---- expert product.  The rows of B_e go over what has been used: this pass's sign bits, and in the CTA's last pass all
     // buffers and the codes.  Every warp has slots of its own and takes every W-th (expert, tile) item.
     const bool last = u_next >= u_hi && (nbuf == 1 || nxt.nu == 0), rows_now = r > 0 && !L.A8;
@@ -873,7 +868,8 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
         bulk_load(smem_u32(ring) + (uint32_t)(warp * per + j) * item_bytes, L.B + ((long long)expert_sh[ei] * N + n0 + t * 16) * r, item_bytes, bar);
       }
     };
-    for (int j = 0; j < per && warp + W * j < items; ++j) issue(warp + W * j, j);
+    if (!*(volatile int*)&fail_sh)                               // after a failed wait nothing goes over copies that may be in flight
+      for (int j = 0; j < per && warp + W * j < items; ++j) issue(warp + W * j, j);
     if (!waited) { pdl_wait(); waited = true; }                  // h
     if (new_linear) {
       if (rows_now) {
@@ -940,7 +936,7 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
         }
       }
     }
-    if (__syncthreads_or(*(volatile int*)&fail_sh)) break;
+    __syncthreads();
     // ---- epilogue (Eq. 10-11), two features per thread
     for (int o = tid; o < (rows >> 1) * M; o += kMainThreads) {
       const int t = o / (rows >> 1), f = 2 * (o - t * (rows >> 1));
@@ -968,6 +964,7 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
     u_next += cur.nu;
     if (cur.nu == 0) break;
     __syncthreads();                                             // the sums, factors and records of this pass have been used
+    if (*(volatile int*)&fail_sh) break;
     if (cur.l != was && cur.l + 1 < bp.n && bp.unit0[cur.l + 1] < u_hi) {
       copy_record(&lin_sh[(cur.l + 1) & 1], bp, cur.l + 1);
       __syncthreads();
@@ -982,7 +979,6 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
     load_scales(cur);
   }
   if (!waited) pdl_wait();
-  decode_drain(&fail_sh);
 }
 
 // ---------------------------------------------------------------------------
