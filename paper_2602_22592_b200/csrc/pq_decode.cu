@@ -40,6 +40,7 @@ constexpr int kUnit = 16;                 // output features of a unit of work (
 constexpr int kMaxPassUnits = 8;          // units a CTA works on at once (two warps or more each)
 constexpr int kWarpRows = 2;              // tiles of expert rows a warp of k_decode_main has in flight
 constexpr int kMaxRows = kWarpRows * kMainWarps;
+static_assert(kWarpRows == 2, "the host's choice of places");
 
 struct DecodeTokInfo {  // one per token
   int expert;
@@ -114,9 +115,12 @@ struct DecodeBatch {
   int poll;                 // waits are polled
   int early;                // k_decode_hidden runs in between: k_decode_main may read prep's results before it waits
   int hidden_groups, hidden_cluster;   // k_decode_hidden: clusters of all linears, CTAs of each
-  // k_decode_main: buffers of sign bits, their size, and the carve-up of shared memory behind them
-  int nbuf, buf_bytes, off_q, off_h, off_red;
+  // k_decode_main: buffers of sign bits, their size, the carve-up of shared memory behind them, and how many tiles of expert rows
+  // have a place apart (0: they go over used sign bits)
+  int nbuf, buf_bytes, off_q, off_h, off_red, off_rows, row_slots;
   int q_chunks;             // chunks of 128 values of k whose codes are in shared memory at once
+  int pass_units;           // units of a pass at most
+  int rows_early;           // k_decode_hidden brings the experts' rows of B into L2
   int red_tokens;
   int unit0[CAP + 1];
   DecodeLinear lin[CAP];
@@ -506,8 +510,8 @@ __global__ void __maxnreg__(80) k_decode_hidden(const __grid_constant__ DecodeBa
   const uint4* x1 = t1 >= 0 ? x + (long long)t1 * pitch : nullptr;
   const uint4* rows = base + e * expert_pitch + row0 + c;
   const uint4 *r0 = rows + (long long)g * pitch, *r1 = rows + (long long)(j0 + g + 8 < r ? g + 8 : g) * pitch;
-  // the rows of B_e that k_decode_main reads next start towards L2 (512-byte pieces)
-  if (!int8) {
+  // where k_decode_main asks for the rows of B_e late, they start towards L2 (512-byte pieces)
+  if (bp.rows_early && !int8) {
     const int total = (L.N >> 5) * (r >> 3), per = (total + tiles - 1) / tiles, lo = per * tile, hi = min(total, lo + per);
     const uint8_t* b = reinterpret_cast<const uint8_t*>(L.B) + (long long)e * total * 512;
     for (int at = lo + (rank * kHiddenThreads + tid) * 8; at < hi; at += cs * kHiddenThreads * 8) bulk_prefetch(b + (long long)at * 512, (uint32_t)min(8, hi - at) * 512u);
@@ -558,8 +562,7 @@ __global__ void __maxnreg__(80) k_decode_hidden(const __grid_constant__ DecodeBa
 // of a pass sit in shared memory as [chunk of 128 k][feature of the pass][16 bytes]; with the streaming layout they arrive
 // by bulk copies, one pass ahead, otherwise through registers.  1-bit product: a warp works on two tiles of 16 features and a
 // slice of the contraction; the slices' sums (integers) are added up in shared memory.  Expert product: the rows of B_e of
-// one tile are one contiguous piece, fetched by a bulk copy over the sign bits (used by then); a warp takes whole (expert,
-// tile) items.
+// one tile are one contiguous piece, fetched by a bulk copy; a warp takes whole (expert, tile) items.
 // ---------------------------------------------------------------------------
 struct DecodePass { int l, unit, nu; };   // linear; first unit within it; units (0: no pass)
 
@@ -684,7 +687,7 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
     if (u >= u_hi) return p;
     while (bp.unit0[p.l + 1] <= u) ++p.l;
     const DecodeLinear& L = lin_sh[p.l & 1];
-    const int cap = max(1, min(kMaxPassUnits, buf_bytes / (256 * ((L.K + 127) >> 7))));
+    const int cap = max(1, min(bp.pass_units, buf_bytes / (256 * ((L.K + 127) >> 7))));
     const int rem = min(u_hi, bp.unit0[p.l + 1]) - u, npass = (rem + cap - 1) / cap;
     p.unit = u - bp.unit0[p.l];
     p.nu = (rem + npass - 1) / npass;
@@ -728,7 +731,7 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
   uint4* h_s = reinterpret_cast<uint4*>(smem + off_h);
   int8_t* qh_s = reinterpret_cast<int8_t*>(smem + off_h);
   int* red_i = reinterpret_cast<int*>(smem + bp.off_red);        // [tile][token][16 features]
-  float* red_z = reinterpret_cast<float*>(red_i + kMaxPassUnits * MT * 16);   // [tile][token][16]
+  float* red_z = reinterpret_cast<float*>(red_i + bp.pass_units * MT * 16);   // [tile][token][16]
   int loaded_l = -1;
   for (int b = 0; cur.nu > 0;) {
     const DecodeLinear& L = lin_sh[cur.l & 1];
@@ -801,8 +804,29 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
       }
     }
     __syncthreads();
+    // Expert rows: every warp has places of its own and takes every W-th (expert, tile) item.  The places either lie apart, and the
+    // rows set out now, beside the 1-bit product; or over what the product has used by then -- this pass's sign bits, and in the CTA's
+    // last pass all buffers and the codes.
+    const bool rows_now = r > 0 && !L.A8, own = bp.row_slots > 0, last = u_next >= u_hi && (nbuf == 1 || nxt.nu == 0);
+    const uint32_t item_bytes = 32u * (uint32_t)max(r, 1);
+    const int tiles = cur.nu;
+    uint8_t* ring = smem + bp.off_rows;
+    int W = 1, per = 1, items = 0;                               // warps that take items, places of each, items
+    auto issue = [&](int i, int j) {                             // item i into this warp's place j
+      if (lane == 0) {
+        const int ei = i / tiles, t = i - ei * tiles;
+        const uint32_t bar = smem_u32(&bars[2 + warp * kWarpRows + j]);   // barriers belong to a warp, whatever the places of a pass
+        mbar_expect_tx(bar, item_bytes);
+        bulk_load(smem_u32(ring) + (uint32_t)(warp * per + j) * item_bytes, L.B + ((long long)expert_sh[ei] * N + n0 + t * 16) * r, item_bytes, bar);
+      }
+    };
+    auto ask = [&](int slots) {
+      W = min(kMainWarps, slots); per = slots < kMaxRows ? 1 : kWarpRows; items = warp < W ? used_sh * tiles : 0;
+      for (int j = 0; j < per && warp + W * j < items; ++j) issue(warp + W * j, j);
+    };
+    if (rows_now && own) ask(bp.row_slots);
     // ---- 1-bit product
-    const int tiles = cur.nu, pairs = (tiles + 1) >> 1, S = kMainWarps / pairs;   // at most 4 pairs of tiles
+    const int pairs = (tiles + 1) >> 1, S = kMainWarps / pairs;   // at most 4 pairs of tiles
     const int sl = warp / pairs, tile = 2 * (warp - sl * pairs);
     if (L.bits_il) {
       decode_wait(smem_u32(&bars[b]), phase[b], &fail_sh, poll);
@@ -853,23 +877,11 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // what plain stores filled may be overwritten by bulk copies
     __syncthreads();                                             // the sign bits of this pass have been used
-    // ---- expert product.  The rows of B_e go over what has been used: this pass's sign bits, and in the CTA's last pass all
-    // buffers and the codes.  Every warp has slots of its own and takes every W-th (expert, tile) item.
-    const bool last = u_next >= u_hi && (nbuf == 1 || nxt.nu == 0), rows_now = r > 0 && !L.A8;
-    uint8_t* ring = last ? smem : bits_s;
-    const uint32_t item_bytes = 32u * (uint32_t)max(r, 1);
-    const int slots = min(kMaxRows, (int)((uint32_t)(last ? off_h : buf_bytes) / item_bytes));
-    const int W = min(kMainWarps, slots), per = rows_now ? min(kWarpRows, slots / W) : 1, items = rows_now && warp < W ? used_sh * tiles : 0;
-    auto issue = [&](int i, int j) {                             // item i into this warp's slot j
-      if (lane == 0) {
-        const int ei = i / tiles, t = i - ei * tiles;
-        const uint32_t bar = smem_u32(&bars[2 + warp * kWarpRows + j]);   // barriers belong to a warp, whatever the slots of a pass
-        mbar_expect_tx(bar, item_bytes);
-        bulk_load(smem_u32(ring) + (uint32_t)(warp * per + j) * item_bytes, L.B + ((long long)expert_sh[ei] * N + n0 + t * 16) * r, item_bytes, bar);
-      }
-    };
-    if (!*(volatile int*)&fail_sh)                               // after a failed wait nothing goes over copies that may be in flight
-      for (int j = 0; j < per && warp + W * j < items; ++j) issue(warp + W * j, j);
+    // ---- expert product
+    if (rows_now && !own && !*(volatile int*)&fail_sh) {         // after a failed wait nothing goes over copies that may be in flight
+      ring = last ? smem : bits_s;
+      ask(min(kMaxRows, (int)((uint32_t)(last ? off_h : buf_bytes) / item_bytes)));
+    }
     if (!waited) { pdl_wait(); waited = true; }                  // h
     if (new_linear) {
       if (rows_now) {
@@ -907,7 +919,7 @@ __global__ void __maxnreg__(88) k_decode_main(const __grid_constant__ DecodeBatc
       if (i + W * per < items && !*(volatile int*)&fail_sh) issue(i + W * per, j);
       if (++j == per) j = 0;
     }
-    if (last) q_loaded = nullptr;
+    if (last && !own) q_loaded = nullptr;
     if (L.A8) {
       // INT8 branch: z_int = B8_e qh (exact), z = z_int / (gamma_B gamma_h gamma_A gamma_t).  An item is (tile, token): lanes l and
       // l + 16 share feature l of the tile and take alternate pieces of 16 hidden values
@@ -1020,6 +1032,7 @@ static int decode_sm_count() {
 }
 
 constexpr size_t kDecodeMainSmemLimit = 220 * 1024;   // dynamic shared memory of k_decode_main (it has a few KB of its own)
+constexpr size_t kDecodeMainSmemBeside = 185 * 1024;  // ... that leaves room for one CTA of k_decode_hidden on the SM
 
 template <int CAP>
 static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st) {
@@ -1028,7 +1041,7 @@ static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st)
   bp.n = n;
   bp.poll = g_decode_poll;
   size_t h_bytes = 0, smem_prep = 0, slot_bytes = 0;
-  int max_m = 1, units = 0, max_c = 1, row_bytes = 0;
+  int max_m = 1, units = 0, max_c = 1, row_bytes = 0, max_used = 1, min_c = 1 << 30;
   bp.hidden_groups = 0;
   for (int i = 0; i < n; ++i) {
     const DecodeItemArgs& it = items[i];
@@ -1055,6 +1068,7 @@ static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st)
     } else if (r > 0) {
       h_bytes = std::max(h_bytes, up256((size_t)((M + 7) / 8) * 2 * rsteps * 512));
       slot_bytes = std::max(slot_bytes, (size_t)32 * r);
+      max_used = std::max(max_used, std::min(L.E, M));
     }
     L.unit0 = units;
     bp.unit0[i] = units;
@@ -1062,7 +1076,7 @@ static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st)
     L.hidden0 = bp.hidden_groups;
     if (r > 0) row_bytes = std::max(row_bytes, it.A8 ? K : 2 * K);
     if (r > 0) bp.hidden_groups += std::min(L.E, M) * ((r + 15) / 16);
-    max_m = std::max(max_m, M); max_c = std::max(max_c, (K + 127) / 128);
+    max_m = std::max(max_m, M); max_c = std::max(max_c, (K + 127) / 128); min_c = std::min(min_c, (K + 127) / 128);
     smem_prep = std::max(smem_prep, prep_plan(K, L.E, L.norm_w != nullptr).bytes);
   }
   for (int i = n; i <= CAP; ++i) bp.unit0[i] = units;
@@ -1071,24 +1085,65 @@ static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st)
   // ---- k_decode_main: one CTA per SM (fewer when there is less than a unit for each)
   const int ctas = std::min(sms, units), share = (units + ctas - 1) / ctas;
   bp.red_tokens = max_m > 8 ? 16 : 8;
-  const size_t red_bytes = (size_t)2 * kMaxPassUnits * bp.red_tokens * 16 * 4;
-  const size_t unit_bytes = (size_t)256 * max_c, fixed = h_bytes + red_bytes;
-  const size_t chunk_bytes = (size_t)128 * max_m;            // codes of one chunk of k
-  const size_t buf_min = std::max(unit_bytes, up256(slot_bytes));
-  if (buf_min + chunk_bytes + fixed > kDecodeMainSmemLimit) return PQ_ERR_UNSUPPORTED;
-  bp.q_chunks = (int)std::min<size_t>(max_c, (kDecodeMainSmemLimit - buf_min - fixed) / chunk_bytes);
-  const size_t q_bytes = up256(bp.q_chunks * chunk_bytes);
-  const size_t room = kDecodeMainSmemLimit - fixed - q_bytes;
-  int pass_units = std::min(share, kMaxPassUnits);
-  bp.nbuf = (n == 1 && share <= pass_units) ? 1 : 2;
-  if (2 * buf_min > room) bp.nbuf = 1;
-  while (pass_units > 1 && bp.nbuf * std::max(pass_units * unit_bytes, buf_min) > room) --pass_units;
-  bp.buf_bytes = (int)std::max(pass_units * unit_bytes, buf_min);
-  if ((size_t)bp.nbuf * bp.buf_bytes > room) return PQ_ERR_UNSUPPORTED;
+  // Shared memory goes to sign bits (units of 16 features in a pass), codes (those of all of K, or of a slice of it), sums, and
+  // places for expert rows, apart from the rest or over it.  In microseconds, about: a pass is three of barriers and first trips, a
+  // further slice of the codes one, a round of expert rows (as many items as there are places) one, and one more where they set
+  // out only after the 1-bit product; a CTA that leaves no room for one of k_decode_hidden's beside it starts one and a half later.  The split
+  // with the least of these is taken.  Linears of different K share it: `units` are of the longest row, shorter ones have more in a pass.
+  // Places apart against places over used sign bits, us a call with eight experts of 160: 1056 x 7552, four tokens 12.9 / 19.6, sixteen
+  // 20.3 / 24.5; 2048 x 5632, twelve linears, eight tokens 74 / 98; two of 3200 x 8640, sixteen tokens 33.7 / 31.2.
+  const size_t unit_bytes = (size_t)256 * max_c, chunk_bytes = (size_t)128 * max_m;   // a unit's sign bits; codes of 128 values of k
+  struct Split { int nbuf, units, red_units, q_chunks, slots; size_t q_bytes, bytes; double cost; } best{};
+  const int most = std::min(share, kMaxPassUnits);
+  const bool one_pass = n == 1 && share <= kMaxPassUnits;        // sign bits of a single pass need no second buffer
+  auto places = [](size_t bytes, size_t each, int wanted) {      // two for each warp, one, or fewer than there are warps
+    const int fit = (int)(bytes / each);
+    return wanted > kMainWarps && fit >= kMaxRows ? kMaxRows : std::min({kMainWarps, wanted, fit});
+  };
+  auto rounds = [](int wanted, int slots) { return std::max(1.0, (double)wanted / slots); };
+  for (int nbuf = one_pass ? 1 : 2; nbuf >= 1 && best.units == 0; --nbuf) {
+    for (int units = most; units >= 1; --units) {
+      if (one_pass && units < share && best.units > 0) break;
+      int passes = 1;
+      for (int i = 0; i < n; ++i) {
+        const int cap = std::min(most, units * max_c / ((items[i].a.K + 127) / 128));
+        passes = std::max(passes, (std::min(share, items[i].a.N / kUnit) + cap - 1) / cap);
+      }
+      for (int slices = 1; slices <= max_c; ++slices) {
+        Split c{nbuf, units, nbuf == 1 && !one_pass ? units : most, (max_c + slices - 1) / slices, 0, 0, 0, 0.0};
+        c.q_bytes = up256(c.q_chunks * chunk_bytes);
+        const size_t red = (size_t)2 * c.red_units * bp.red_tokens * 16 * 4, buf = units * unit_bytes, used = nbuf * buf + c.q_bytes + h_bytes + red;
+        if (used > kDecodeMainSmemLimit) continue;
+        const int wanted = max_used * units;
+        auto offer = [&](int slots, double rows) {               // rows: what the expert rows of all passes cost
+          c.slots = slots; c.bytes = used + slots * slot_bytes;
+          c.cost = passes * (3.0 + (slices - 1)) + rows + (c.bytes > kDecodeMainSmemBeside ? 1.5 : 0.0);
+          if (best.units == 0 || c.cost < best.cost) best = c;
+        };
+        if (slot_bytes == 0) {
+          offer(0, 0.0);
+        } else {
+          for (size_t limit : {kDecodeMainSmemBeside, kDecodeMainSmemLimit})
+            if (const int s = used < limit ? places(limit - used, slot_bytes, wanted) : 0) offer(s, passes * rounds(wanted, s));
+          if (buf >= slot_bytes)
+            offer(0, passes + (passes - 1) * rounds(wanted, places(buf, slot_bytes, wanted)) +
+                         rounds(wanted, places(nbuf * buf + c.q_bytes, slot_bytes, wanted)));
+        }
+        if (slices >= 4 && best.units > 0) break;
+      }
+    }
+  }
+  if (best.units == 0) return PQ_ERR_UNSUPPORTED;
+  bp.nbuf = best.nbuf; bp.pass_units = best.red_units; bp.q_chunks = best.q_chunks; bp.row_slots = best.slots;
+  bp.buf_bytes = (int)(best.units * unit_bytes);
+  // One or two linears only: of more, the rows take the memory from those of A that k_decode_hidden is waiting for (twelve of 3200 x
+  // 8640, sixteen tokens 163 us with, 145 without; two 31.2 / 31.8).
+  bp.rows_early = best.slots == 0 && n <= 2;
   size_t off = (size_t)bp.nbuf * bp.buf_bytes;
-  bp.off_q = (int)off; off += q_bytes;
+  bp.off_q = (int)off; off += best.q_bytes;
   bp.off_h = (int)off; off += h_bytes;
-  bp.off_red = (int)off; off += red_bytes;
+  bp.off_red = (int)off; off += (size_t)2 * best.red_units * bp.red_tokens * 16 * 4;
+  bp.off_rows = (int)off; off += best.slots * slot_bytes;
   const size_t smem_main = off;
 
   // ---- k_decode_prep
@@ -1096,7 +1151,10 @@ static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st)
   // One CTA per SM; with rows of A_e beyond 4 KB, whose contraction is worth more than room for k_decode_main's CTAs beside it, up to
   // three.  Per call, one CTA per cluster against two where two are more than the SMs hold: M = 11, 1056 x 7552 18.6 / 21.7 us, M = 4,
   // INT8, 3200 x 8640 16.9 / 18.3; M = 13, 2816 x 4960 22.1 / 20.7, M = 16, 3200 x 8640 37.2 / 31.4.
-  bp.hidden_cluster = 4 * bp.hidden_groups <= sms ? 4 : 2 * bp.hidden_groups <= (row_bytes > 4096 ? 3 * sms : sms) ? 2 : 1;
+  // Up to four tokens and rows of one length, where pairs would be a few more than the SMs and a CTA of k_decode_main has room beside one
+  // of these, one: two linears of 3200 x 8640 (8640 x 3200), four tokens 21.2 (25.9) us, with pairs 24.8 (30.8).
+  const bool few_over = max_m <= 4 && 4 * bp.hidden_groups <= 2 * sms + sms / 2 && best.bytes <= kDecodeMainSmemBeside && min_c == max_c;
+  bp.hidden_cluster = 4 * bp.hidden_groups <= sms ? 4 : 2 * bp.hidden_groups <= (row_bytes > 4096 && !few_over ? 3 * sms : sms) ? 2 : 1;
   if (smem_prep > kDecodePrepSmemLimit) return PQ_ERR_UNSUPPORTED;
 
   using Kern = void (*)(DecodeBatch<CAP>);

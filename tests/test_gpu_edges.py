@@ -248,3 +248,28 @@ def test_forward_on_single_ctas_and_on_pairs(T, K, N, r, E, vector):
     c = I.make_linear_case(T, K, N, r, E, seed=T, scale_vector=vector, alpha=1.5, beta=0.5, with_grad=False)
     f = O.linear_forward(c["X"], c["W"], c["A"], c["B"], c["Wr"], c["alpha"], c["beta"])
     check_forward(c, run_forward(c, vector), f)
+
+
+@pytest.mark.parametrize("M,K,N,r,E", [
+    (4, 1056, 7552, 160, 8), (14, 1056, 7552, 160, 8),      # short rows of sign bits: more expert rows in a pass than those would hold
+    (16, 8640, 3200, 256, 8), (16, 3200, 8640, 160, 8),     # codes, sign bits and expert rows that do not fit at once
+    (1, 32, 37888, 8, 1), (9, 64, 4768, 8, 16),             # many units in a pass; a unit more than two for each SM
+])
+def test_decode_shapes_of_a_pass(M, K, N, r, E):
+    from test_gpu_decode import check_decode
+    c, L, _ = _decode_case(M, K, N, r, E, False, seed=31)
+    others = [_decode_case(M, 8640, 512, r, E, False, seed=32)[1], _decode_case(M, 96, 2048, r, E, False, seed=33)[1]]
+    pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 0)
+    try:
+        L.decode()
+        torch.cuda.synchronize()
+        check_decode(c, L)
+        y = L.Y.clone()
+        for beside in (others[:1], others):     # other splits of shared memory, the same bits
+            L.Y.zero_()
+            pqb.pq_decode_batch(pqb.make_decode_items([L.decode_entry()] + [o.decode_entry() for o in beside]))
+            torch.cuda.synchronize()
+            assert torch.equal(L.Y, y)
+    finally:
+        pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 1)
+    check_status()
