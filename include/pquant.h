@@ -395,8 +395,8 @@ int pq_device_status(void* stream, int* code, int* where);
  *   results a backward call would go on from.
  *   PQ_OPT_DECODE_STREAM (default 1): which launch groups of pq_decode_batch (up to 96 consecutive items) run on the
  *   streaming kernel when their items carry w_bits_il / B_il.  1 = those for which it is the faster of the two paths
- *   (six or more linears, with INT8 experts and three to eight tokens twelve; three or more bf16 ones with more than eight
- *   tokens); 2 = every group; 0 = none.
+ *   (many features per SM for few tokens: with experts about 19 units of 16 features per SM at one token, 44 at four, 75 at
+ *   six, never from seven tokens on); 2 = every group; 0 = none.
  *   PQ_OPT_DECODE_PREFETCH (default 1): the streaming decode kernel asks for the sign bits four chunks ahead of its
  *   bit product to be brought into L2.
  *   PQ_OPT_DECODE_MMA_FROM (default 5): the streaming decode kernel multiplies the sign bits of a group of at least this

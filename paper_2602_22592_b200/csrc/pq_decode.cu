@@ -1211,34 +1211,54 @@ static int decode_launch(const DecodeItemArgs* items, int n, cudaStream_t st) {
 
 int decode_stream_max_batch();   // pq_decode_stream.cu
 
+// The run of items at the front that all carry the streaming kernel's weight layout: its length, at most `most`, and whether that kernel
+// is the faster one for it.  It starts late (token work, then a barrier of the whole grid) and costs little per linear; what decides is
+// the number of units of 16 features per SM, the number of tokens and whether there are experts.
+struct StreamRun { int n; bool pays; };
+static StreamRun stream_run(const DecodeItemArgs* items, int most) {
+  StreamRun run{0, false};
+  static const int sms = decode_sm_count();
+  int max_m = 1;
+  long long units = 0;
+  bool experts = false, routed = false;
+  while (run.n < most && items[run.n].bits_il) {
+    const LayerArgs& a = items[run.n].a;
+    max_m = std::max(max_m, a.T);
+    units += a.N / kUnit;
+    experts = experts || a.r > 0;
+    routed = routed || (a.r > 0 && a.E > 1);
+    ++run.n;
+  }
+  // us a call, small-group kernels / streaming kernel: eight experts of 160, one token, 8 linears of 2048 x 5632 31 / 30, 6 of 3200 x
+  // 8640 33 / 31, 24 of 2048 x 2048 39 / 38; two tokens, 6 and 8 of 3200 x 8640 40 / 44, 50 / 47; three, 8 and 12 54 / 59, 75 / 70; four, 12 and
+  // 24 77 / 80, 148 / 128; six, 24 of 2048 x 5632 123 / 127, of 3200 x 8640 179 / 172; eight, 78 619 / 635; sixteen 935 / 1215.  A dense
+  // branch of 128, one token, 8 of 3200 x 8640 38 / 32; two, 12 53 / 50, 24 of 2048 x 5632 61 / 61; four, 78 of 3200 x 8640 283 / 317.  No
+  // branch, one token, 8 and 12 24 / 27, 34 / 32; two, 12 and 24 35 / 39, 65 / 57; four, 48 of 2048 x 5632 84 / 81.  INT8 experts as bf16 ones.
+  constexpr int kNever = 1 << 30;
+  const int least = routed ? (max_m <= 1 ? 19 : max_m <= 2 ? 29 : max_m <= 3 ? 40 : max_m <= 4 ? 44 : max_m <= 6 ? 75 : kNever)
+                    : experts ? (max_m <= 1 ? 19 : max_m <= 2 ? 50 : max_m <= 3 ? 150 : kNever)
+                              : (max_m <= 1 ? 37 : max_m <= 2 ? 65 : max_m <= 4 ? 114 : kNever);
+  run.pays = units >= (long long)least * sms;
+  return run;
+}
+
 int decode_batch(const DecodeItemArgs* items, int n, cudaStream_t st) {
+  const int mode = decode_stream_mode(), group = std::min(decode_stream_max_batch(), kDecodeMaxBatch);
   int i = 0;
   while (i < n) {
-    // The streaming kernel takes a run of items that all carry its weight layout, where it pays.  Measured on linears of 3200 x
-    // 8640, eight experts of 160, small-group kernels against streaming (us): 3 linears, M = 1 / 4 / 8 / 16: 27/27 32/39 47/60
-    // 98/89; 6 linears: 44/30 64/57 95/86 190/132; 12 linears: 84/41 115/86 154/130 361/220.  INT8 experts, 3 linears: 24/28
-    // 29/37 39/56 64/80; 6 linears: 39/31 49/52 65/72 128/114; 12 linears: 66/39 100/78 113/103 239/205.
-    const int mode = decode_stream_mode();
-    const int most = std::min(n - i, std::min(decode_stream_max_batch(), kDecodeMaxBatch));
-    int run = 0, max_m = 1;
-    bool int8 = false;
-    while (run < most && items[i + run].bits_il) {
-      max_m = std::max(max_m, items[i + run].a.T);
-      if (items[i + run].A8) int8 = true;
-      ++run;
-    }
-    const bool pays = run >= 12 || (run >= 6 && (!int8 || max_m <= 2 || max_m > 8)) || (run >= 3 && !int8 && max_m > 8);
-    int rc = PQ_ERR_UNSUPPORTED, m = run;
-    if (run > 0 && (mode > 1 || (mode == 1 && pays))) rc = decode_stream_launch(items + i, run, st);
+    const int most = std::min(n - i, group);
+    const StreamRun run = stream_run(items + i, most);
+    int rc = PQ_ERR_UNSUPPORTED, m = run.n;
+    if (run.n > 0 && (mode > 1 || (mode == 1 && run.pays))) rc = decode_stream_launch(items + i, run.n, st);
     if (rc == PQ_ERR_UNSUPPORTED) {
-      // the three kernels above take items with and without the layout together, unless the streaming kernel is asked for
-      // wherever it can run
-      m = most;
-      if (mode > 1) {
-        m = run;
-        if (run == 0)
-          while (m < most && !items[i + m].bits_il) ++m;
-      }
+      // The three kernels above take items with and without the layout together, up to the start of a run that the streaming kernel
+      // takes.
+      auto run_starts = [&](int k) {
+        if (mode == 0 || !items[i + k].bits_il || items[i + k - 1].bits_il) return false;
+        return mode > 1 || stream_run(items + i + k, std::min(n - i - k, group)).pays;
+      };
+      m = std::max(run.n, 1);
+      while (m < most && !(mode > 1 && run.n > 0) && !run_starts(m)) ++m;
       rc = decode_launch(items + i, m, st);
       // shared memory is laid out for the largest of everything in a launch: what does not fit together may fit apart
       while (rc == PQ_ERR_UNSUPPORTED && m > 1) rc = decode_launch(items + i, m /= 2, st);

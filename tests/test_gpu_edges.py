@@ -111,37 +111,94 @@ def _decode_layers(shapes):
     return layers
 
 
+def check_decode_int8(c, L):
+    # every integer the INT8 branch goes through, and the outputs, against the oracle
+    mu, lam = O.weight_scales(c["W"])
+    f = O.decode_forward(c["X"], O.pack_bits(O.binarize(c["W"], mu)), lam, c["A"], c["B"], c["Wr"], c["alpha"], c["beta"],
+                         hp_int8=O.quantize_experts(c["A"], c["B"]))
+    v = L.decode_view()
+    for name, want in (("expert", f["idx"]), ("acc", f["acc"]), ("hp_h_int", f["h_int"]), ("hp_z_int", f["z_int"])):
+        assert np.array_equal(v[name].cpu().numpy().astype(np.int64), want)
+    assert rel_err(f32(L.Y), f["Y"]) <= TOL_BF16
+
+
 @pytest.mark.parametrize("shapes", [
-    # both sides of the lines between the small-group kernels and the streaming one
-    *[[dict(T=M, K=256, N=96, r=32, E=4, hp8=hp8)] * n for n, M, hp8 in
-      [(2, 9, False), (3, 9, False), (5, 4, False), (6, 4, False), (5, 2, True), (6, 2, True), (6, 8, True), (6, 9, True), (12, 8, True)]],
-    # the small-group kernels: codes of a row too long to be in shared memory at once; one unit; ragged hidden widths; the INT8
-    # branch beside linears with and without the streaming layout
+    *[[dict(T=M, K=256, N=96, r=32, E=4, hp8=hp8)] * n for n, M, hp8 in [(2, 9, False), (6, 4, False), (2, 9, True), (6, 2, True), (12, 8, True)]],
+    # codes of a row too long to be in shared memory at once; one unit; ragged hidden widths; the INT8 branch beside linears
+    # with and without the streaming layout
     [dict(T=16, K=16384, N=64, r=32, E=2)], [dict(T=16, K=16384, N=64, r=40, E=2, stream=False)],
     [dict(T=1, K=32, N=32, r=8, E=16), dict(T=8, K=4128, N=1056, r=48, E=2, hp8=True), dict(T=5, K=96, N=160, r=72, E=3, stream=False)],
 ])
-def test_decode_dispatch_and_small_groups(shapes):
-    # the exact integers and the outputs of the oracle; for INT8 experts the outputs of the streaming kernel
+def test_decode_small_groups(shapes):
+    # the exact integers and the outputs of the oracle, in three launches
     from test_gpu_decode import check_decode
     layers = _decode_layers(shapes)
+    before = pqb.pq_kernel_launches()
     pqb.pq_decode_batch(pqb.make_decode_items([L.decode_entry() for L, _ in layers]))
+    assert pqb.pq_kernel_launches() - before == 3
     torch.cuda.synchronize()
     check_status()
     for (L, c), kw in zip(layers, shapes):
-        if kw.get("hp8"):
-            q, gamma = O.act_quant(c["X"])
-            assert np.array_equal(L.decode_view()["code_sum"].cpu().numpy(), q.astype(np.int64).sum(axis=1))
-            y = L.Y.clone()
-            pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 2)          # the streaming kernel is checked against the oracle elsewhere
-            try:
-                L.decode()
-                torch.cuda.synchronize()
-            finally:
-                pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 1)
-            # integer sums on both sides, de-quantised by the same factors: at most the rounding of the bf16 output
-            assert torch.all((y.float() - L.Y.float()).abs() <= 2.0 ** -7 * L.Y.float().abs() + 1e-6)
-        else:
-            check_decode(c, L)
+        (check_decode_int8 if kw.get("hp8") else check_decode)(c, L)
+
+
+def _layers_alike(n, M, r, E, hp8):
+    # n linears of 64 -> 8192 with the same weights and activations
+    c = I.make_linear_case(M, 64, 8192, r, E, seed=71, exact_quota=False, with_grad=False)
+    layers = []
+    for _ in range(n):
+        L = PQLinear(M, 64, 8192, r, E, training=False, dump_acc=True).load_case(c)
+        L.pack(bits_only=True)
+        if hp8:
+            L.pack_decode_hp8()
+        layers.append(L)
+    return c, layers
+
+
+def _linears_for(units_per_sm):
+    return -(-units_per_sm * torch.cuda.get_device_properties(0).multi_processor_count * 16 // 8192)
+
+
+@pytest.mark.parametrize("M,r,E,hp8,least", [
+    # units of 16 features per SM from which the streaming kernel takes a batch: by tokens and kind of branch
+    (1, 16, 4, False, 19), (1, 16, 4, True, 19), (2, 16, 4, False, 29), (3, 16, 2, False, 40), (4, 16, 4, True, 44), (6, 16, 4, False, 75),
+    (1, 16, 1, False, 19), (2, 16, 1, False, 50), (1, 0, 0, False, 37), (2, 0, 0, False, 65), (7, 16, 4, False, None),
+])
+def test_decode_dispatch_on_both_sides_of_its_lines(M, r, E, hp8, least):
+    from test_gpu_decode import check_decode
+    n = 48 if least is None else _linears_for(least)
+    c, layers = _layers_alike(n, M, r, E, hp8)
+    for take, launches in ((n - 1, 3 if r else 2), (n, (3 if r else 2) if least is None else 1)):
+        for L in layers:
+            L.Y.zero_()
+            L.ws_decode.zero_()
+        before = pqb.pq_kernel_launches()
+        pqb.pq_decode_batch(pqb.make_decode_items([L.decode_entry() for L in layers[:take]]))
+        assert pqb.pq_kernel_launches() - before == launches
+        torch.cuda.synchronize()
+        check_status()
+        (check_decode_int8 if hp8 else check_decode)(c, layers[take - 1])
+        assert all(torch.equal(L.Y, layers[0].Y) for L in layers[1:take])
+
+
+@pytest.mark.parametrize("plain,launches", [
+    ([0], 3 + 1), ([1], 3 + 1), ([2], 3 + 1),             # linears without the layout, alone or after one or two with it: up to the run that pays
+    ([-1], 1 + 3), ([0, -1], 3 + 1 + 3),
+])
+def test_decode_batch_of_a_run_that_pays_and_linears_without_the_layout(plain, launches):
+    n = _linears_for(19)
+    c, layers = _layers_alike(n + len(plain) + max(plain[0], 0), 1, 16, 4, False)
+    entries = [list(L.decode_entry()) for L in layers]
+    for k in plain:
+        entries[k][13] = entries[k][14] = None
+    before = pqb.pq_kernel_launches()
+    pqb.pq_decode_batch(pqb.make_decode_items([tuple(e) for e in entries]))
+    assert pqb.pq_kernel_launches() - before == launches
+    torch.cuda.synchronize()
+    check_status()
+    from test_gpu_decode import check_decode
+    for k in (0, len(layers) // 2, -1):
+        check_decode(c, layers[k])
 
 
 @pytest.mark.parametrize("mode", [0, 2])
