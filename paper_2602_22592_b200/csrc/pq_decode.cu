@@ -1085,6 +1085,21 @@ static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st)
   // ---- k_decode_main: one CTA per SM (fewer when there is less than a unit for each)
   const int ctas = std::min(sms, units), share = (units + ctas - 1) / ctas;
   bp.red_tokens = max_m > 8 ? 16 : 8;
+  // ---- k_decode_hidden: CTAs of a cluster
+  // One CTA per SM; with rows of A_e beyond 4 KB, whose contraction is worth more than room for k_decode_main's CTAs beside it, up to
+  // three.  Per call, one CTA per cluster against two where two are more than the SMs hold: M = 11, 1056 x 7552 18.6 / 21.7 us, M = 4,
+  // INT8, 3200 x 8640 16.9 / 18.3; M = 13, 2816 x 4960 22.1 / 20.7, M = 16, 3200 x 8640 37.2 / 31.4.
+  // Up to four tokens and rows of one length, where pairs would be a few more than the SMs and a CTA of k_decode_main has room beside one
+  // of these, one: two linears of 3200 x 8640 (8640 x 3200), four tokens 21.2 (25.9) us, with pairs 24.8 (30.8).
+  const bool few_over = max_m <= 4 && 4 * bp.hidden_groups <= 2 * sms + sms / 2 && min_c == max_c;
+  const int pairs_to = row_bytes > 4096 ? 3 * sms : sms;
+  bp.hidden_cluster = 4 * bp.hidden_groups <= sms ? 4 : 2 * bp.hidden_groups <= pairs_to ? 2 : 1;
+  // CTAs of k_decode_main that start beside k_decode_hidden's take room and memory requests from them: with more than eight tokens and rows
+  // of A_e beyond 4 KB, where those are more than the SMs but would all be resident without, they start only afterwards.  Beside / after,
+  // eight experts, sixteen tokens: 8640 x 3200 29.6 / 28.2 us, 2784 x 4960 21.8 / 20.8, two of 3200 x 8640 31.5 / 30.4.  Eight tokens:
+  // 8640 x 3200 20.6 / 22.6; shorter rows: three of 2048 x 2048, sixteen 24.1 / 26.1; more CTAs: twelve of 2048 x 5632, eight 72.4 / 73.5.
+  const int hidden_ctas = bp.hidden_groups * bp.hidden_cluster;
+  const bool apart = max_m > 8 && row_bytes > 4096 && hidden_ctas > sms && hidden_ctas <= 3 * sms;
   // Shared memory goes to sign bits (units of 16 features in a pass), codes (those of all of K, or of a slice of it), sums, and
   // places for expert rows, apart from the rest or over it.  In microseconds, about: a pass is three of barriers and first trips, a
   // further slice of the codes one, a round of expert rows (as many items as there are places) one, and one more where they set
@@ -1117,7 +1132,7 @@ static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st)
         const int wanted = max_used * units;
         auto offer = [&](int slots, double rows) {               // rows: what the expert rows of all passes cost
           c.slots = slots; c.bytes = used + slots * slot_bytes;
-          c.cost = passes * (3.0 + (slices - 1)) + rows + (c.bytes > kDecodeMainSmemBeside ? 1.5 : 0.0);
+          c.cost = passes * (3.0 + (slices - 1)) + rows + (c.bytes > kDecodeMainSmemBeside && !apart ? 1.5 : 0.0);
           if (best.units == 0 || c.cost < best.cost) best = c;
         };
         if (slot_bytes == 0) {
@@ -1136,6 +1151,7 @@ static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st)
   if (best.units == 0) return PQ_ERR_UNSUPPORTED;
   bp.nbuf = best.nbuf; bp.pass_units = best.red_units; bp.q_chunks = best.q_chunks; bp.row_slots = best.slots;
   bp.buf_bytes = (int)(best.units * unit_bytes);
+  if (few_over && best.bytes <= kDecodeMainSmemBeside && 2 * bp.hidden_groups > sms) bp.hidden_cluster = 1;
   // One or two linears only: of more, the rows take the memory from those of A that k_decode_hidden is waiting for (twelve of 3200 x
   // 8640, sixteen tokens 163 us with, 145 without; two 31.2 / 31.8).
   bp.rows_early = best.slots == 0 && n <= 2;
@@ -1144,17 +1160,10 @@ static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st)
   bp.off_h = (int)off; off += h_bytes;
   bp.off_red = (int)off; off += (size_t)2 * best.red_units * bp.red_tokens * 16 * 4;
   bp.off_rows = (int)off; off += best.slots * slot_bytes;
-  const size_t smem_main = off;
+  const size_t smem_main = apart ? kDecodeMainSmemLimit : off;
 
   // ---- k_decode_prep
   bp.early = bp.hidden_groups > 0;
-  // One CTA per SM; with rows of A_e beyond 4 KB, whose contraction is worth more than room for k_decode_main's CTAs beside it, up to
-  // three.  Per call, one CTA per cluster against two where two are more than the SMs hold: M = 11, 1056 x 7552 18.6 / 21.7 us, M = 4,
-  // INT8, 3200 x 8640 16.9 / 18.3; M = 13, 2816 x 4960 22.1 / 20.7, M = 16, 3200 x 8640 37.2 / 31.4.
-  // Up to four tokens and rows of one length, where pairs would be a few more than the SMs and a CTA of k_decode_main has room beside one
-  // of these, one: two linears of 3200 x 8640 (8640 x 3200), four tokens 21.2 (25.9) us, with pairs 24.8 (30.8).
-  const bool few_over = max_m <= 4 && 4 * bp.hidden_groups <= 2 * sms + sms / 2 && best.bytes <= kDecodeMainSmemBeside && min_c == max_c;
-  bp.hidden_cluster = 4 * bp.hidden_groups <= sms ? 4 : 2 * bp.hidden_groups <= (row_bytes > 4096 && !few_over ? 3 * sms : sms) ? 2 : 1;
   if (smem_prep > kDecodePrepSmemLimit) return PQ_ERR_UNSUPPORTED;
 
   using Kern = void (*)(DecodeBatch<CAP>);
