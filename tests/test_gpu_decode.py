@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 @pytest.fixture(autouse=True, params=["stream", "stream_dp4a", "stream_mma", "pair"])
 def decode_kernels(request):
     """Every test runs on the streaming kernel (weights in its own layout; bit product as the library picks it, on dp4a
-    only, on the tensor cores only) and on the two-kernel path."""
+    only, on the tensor cores only) and on the small-group kernels."""
     stream = request.param != "pair"
     PQLinear.stream_decode = stream
     pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 2 if stream else 0)   # 2: also for one small linear
@@ -325,7 +325,7 @@ def test_decode_on_two_streams_at_once():
 
 def test_decode_batch_mixing_items_with_and_without_the_streaming_layout(decode_kernels):
     # a batch whose items only partly carry the streaming kernel's weight layout is cut into runs: the runs that carry it
-    # go to the streaming kernel, the others to the two-kernel path; every item gets what a call of its own gives
+    # go to the streaming kernel, the others to the small-group kernels; every item gets what a call of its own gives
     if decode_kernels == "pair":
         pytest.skip("needs the streaming layout")
     shapes = [dict(T=2, K=512, N=640, r=32, E=4), dict(T=1, K=1024, N=256, r=64, E=2), dict(T=7, K=256, N=1152, r=16, E=8)]
