@@ -28,8 +28,8 @@ EXPORTS = ("pq_status_string", "pq_workspace_bytes", "pq_saved_bytes", "pq_saved
            "pq_device_status", "pq_kernel_launches", "pq_profile_events", "pq_set_option")
 
 KERNEL_IDS = dict(pack_sums=0, binarize_pack=1, router=2, route_scan=3, act_quant=4, hp_up=5, fwd=6, scatter_rows=7,
-                  scaled_sign=8, scaled_b=9, hp_dh=10, bwd_dx=11, bwd_dw=12, hp_db=13, hp_da=14, router_wgrad=15,
-                  sum_partials=16, sum_scalar=17, debug=18, decode_prep=19, decode_main=20, reduce_db=21, reduce_da=22, decode_pack=23, decode_stream=24)
+                  scaled_sign=8, bwd_dw=12, sum_partials=16, sum_scalar=17, debug=18, decode_prep=19, decode_main=20,
+                  decode_pack=23, decode_stream=24)
 
 
 class PqError(RuntimeError):

@@ -13,11 +13,11 @@ constexpr int kPackPartials = 1024;        // fp64 partial sums of the weight re
 constexpr float kActQmax = 128.0f;         // 2^7 of Eq. 9
 constexpr float kActAmaxFloor = 1e-5f;     // all-zero row guard
 
-// Kernel ids for launch counting and optional event timing (pq_profile_events).
+// Kernel ids for launch counting and optional event timing (pq_profile_events); callers know them by number.
 enum KernelId : int {
   KID_PACK_SUMS = 0, KID_BINARIZE_PACK, KID_ROUTER, KID_ROUTE_SCAN, KID_ACT_QUANT, KID_HP_UP, KID_FWD, KID_SCATTER_ROWS,
-  KID_SCALED_SIGN, KID_SCALED_B, KID_HP_DH, KID_BWD_DX, KID_BWD_DW, KID_HP_DB, KID_HP_DA, KID_ROUTER_WGRAD, KID_SUM_PARTIALS,
-  KID_SUM_SCALAR, KID_DEBUG, KID_DECODE_PREP, KID_DECODE_MAIN, KID_REDUCE_DB, KID_REDUCE_DA, KID_DECODE_PACK, KID_DECODE_STREAM, KID_COUNT
+  KID_SCALED_SIGN, KID_BWD_DW = 12, KID_SUM_PARTIALS = 16, KID_SUM_SCALAR, KID_DEBUG, KID_DECODE_PREP, KID_DECODE_MAIN,
+  KID_DECODE_PACK = 23, KID_DECODE_STREAM, KID_COUNT
 };
 struct ProfileSlot { cudaEvent_t start, stop; };
 extern ProfileSlot g_profile[KID_COUNT];
