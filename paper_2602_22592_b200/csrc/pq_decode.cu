@@ -1024,19 +1024,12 @@ void decode_set_pdl(int on) { g_decode_pdl = on ? 1 : 0; }
 static int g_decode_poll = 0;
 void decode_set_poll(int on) { g_decode_poll = on ? 1 : 0; }
 
-static int decode_sm_count() {
-  int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 148;
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
-  return n;
-}
-
 constexpr size_t kDecodeMainSmemLimit = 220 * 1024;   // dynamic shared memory of k_decode_main (it has a few KB of its own)
 constexpr size_t kDecodeMainSmemBeside = 185 * 1024;  // ... that leaves room for one CTA of k_decode_hidden on the SM
 
 template <int CAP>
 static int decode_launch_as(const DecodeItemArgs* items, int n, cudaStream_t st) {
-  static int sms = decode_sm_count();
+  const int sms = sm_count();
   DecodeBatch<CAP> bp;
   bp.n = n;
   bp.poll = g_decode_poll;
@@ -1226,7 +1219,7 @@ int decode_stream_max_batch();   // pq_decode_stream.cu
 struct StreamRun { int n; bool pays; };
 static StreamRun stream_run(const DecodeItemArgs* items, int most) {
   StreamRun run{0, false};
-  static const int sms = decode_sm_count();
+  const int sms = sm_count();
   int max_m = 1;
   long long units = 0;
   bool experts = false, routed = false;

@@ -1020,11 +1020,7 @@ static int stream_bar_slot(cudaStream_t st) {
 constexpr size_t kStreamSmemLimit = 200 * 1024;
 
 int decode_stream_launch(const DecodeItemArgs* items, int n, cudaStream_t st) {
-  static int sms = [] {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) return 148;
-    return v;
-  }();
+  const int sms = sm_count();
   if (n < 1 || n > kStreamMaxBatch) return PQ_ERR_UNSUPPORTED;
   StreamBatch bp{};
   bp.n = n;

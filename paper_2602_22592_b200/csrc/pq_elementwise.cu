@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(512) k_route_scan(int T, int E, int nblocks, c
 }
 
 // ---------------------------------------------------------------------------
-// K1: activation quantisation (Eq. 7-9), one warp per token.  gamma_t = 128 /
+// K1: activation quantisation (Eq. 7-9), one to eight warps per token.  gamma_t = 128 /
 // max(amax, 1e-5) (IEEE division), q = clamp(rint(x * gamma_t), -128, 127).
 // Rows are written at their sorted position p (tokens ordered by expert,
 // stable): q (int8), xt = q / gamma (bf16, the backward's operand) and, with
@@ -886,8 +886,8 @@ cudaError_t launch_route_and_quant(const uint16_t* X, const uint16_t* Wr, int T,
     else if (E <= 8) { kern = k_router<8>; smem = router_smem<8>(); }
     // One CTA per SM (two) where the grid needs no more: its CTAs become resident while the kernel before ends, and the SMs that
     // end first would otherwise take all they can hold.  2048 tokens x 3200: 17 us without this, 10 with it.
-    if (nblocks <= 148) smem = kRouterSmemLimit;
-    else if (nblocks <= 2 * 148) smem = 76 * 1024;
+    if (nblocks <= sm_count()) smem = kRouterSmemLimit;
+    else if (nblocks <= 2 * sm_count()) smem = 76 * 1024;
     if (const cudaError_t e = router_limits()) return e;
     const cudaError_t e = launch_pdl(kern, nblocks, 32 * kRouterWarps, smem, st, reinterpret_cast<const uint4*>(X), reinterpret_cast<const uint4*>(Wr), T, K,
                                      E, sv.expert, sc.gate_tok, sc.probs_tok, sc.block_counts, nw, sc.rms);

@@ -95,17 +95,6 @@ static bool map_mn(CUtensorMap* m, int* blk, const void* base, uint64_t mn_total
   return base_rank == 3 ? map3d(m, base, mn_total, k_total, batch, 64, 64) : map2d(m, false, base, mn_total, k_total, 64, 64);
 }
 
-static int g_sm_count = 0;
-static int sm_count() {
-  if (!g_sm_count) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev);
-    if (g_sm_count <= 0) g_sm_count = 148;
-  }
-  return g_sm_count;
-}
-
 // max_tiles: tiles of the launch, at most; one CTA (or CTA pair) each, as many as the SMs hold
 template <class P>
 static int launch_gemm(int kernel_id, void (*kernel)(typename P::Params), const typename P::Params& p, int max_tiles, cudaStream_t st) {

@@ -69,6 +69,15 @@ struct FwdScratch {
   float* rms;          // [T] per-token factor of a fused RMSNorm
 };
 
+// Multiprocessors of the device of the process's first call
+inline int sm_count() {
+  static const int n = [] {
+    int dev = 0, v = 0;
+    return cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0 ? v : 148;
+  }();
+  return n;
+}
+
 // Launch with programmatic stream serialisation: the kernel may be scheduled while its predecessor in the stream is
 // still draining, which hides its launch latency and set-up.  Every kernel launched this way starts with
 // griddepcontrol.launch_dependents and griddepcontrol.wait, i.e. touches no global memory before the predecessor
