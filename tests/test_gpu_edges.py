@@ -330,3 +330,28 @@ def test_decode_shapes_of_a_pass(M, K, N, r, E):
     finally:
         pqb.pq_set_option(pqb.PQ_OPT_DECODE_STREAM, 1)
     check_status()
+
+
+@pytest.mark.parametrize("hp8", [False, True])
+@pytest.mark.parametrize("T,K,N,r,E", [(1, 32, 32, 16, 1), (129, 1056, 96, 32, 4), (300, 512, 544, 128, 16), (300, 2080, 64, 0, 0)])
+def test_forward_that_keeps_nothing_for_a_backward(T, K, N, r, E, hp8):
+    # without a saved buffer the operands of the backward are not written: the same output
+    if hp8 and r == 0:
+        pytest.skip("needs experts")
+    c = I.make_linear_case(T, K, N, r, E, seed=T + K, with_grad=False)
+    L = PQLinear(T, K, N, r, E).load_case(c)
+    L.pack()
+    if hp8:
+        L.pack_experts()
+        L.forward_hp8()
+    else:
+        L.forward()
+    Y = torch.zeros_like(L.Y)
+    ws = torch.full((pqb.pq_workspace_bytes(L.desc, pqb.PQ_PHASE_FWD) + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+    if hp8:
+        pqb.pq_linear_forward_hp8(L.desc, L.X, L.w_s8, L.w_scales, L.A8, L.B8, L.hp_scales, L.Wr, L.alpha, L.beta, Y, None, ws[:-4096])
+    else:
+        pqb.pq_linear_forward(L.desc, L.X, L.w_bits, L.w_s8, L.w_scales, L.A, L.B, L.Wr, L.alpha, L.beta, Y, None, ws[:-4096])
+    torch.cuda.synchronize()
+    check_status()
+    assert torch.equal(Y, L.Y) and bool((ws[-4096:] == 0xA5).all())
