@@ -138,7 +138,8 @@ static inline bool misaligned(const void* p) { return (reinterpret_cast<uintptr_
 // ---------------------------------------------------------------------------
 // Helper stream: kernels of one call that do not depend on one another run side
 // by side (forward of a dense layer with an HP branch: the activation quantisation
-// next to the HP up-projection).
+// next to the HP up-projection; FFN form: the INT8 FFN's projections next to the
+// quantisation of the 1-bit FFN's hidden activation).
 // Every caller stream gets one non-blocking helper stream and two events, created
 // on first use and kept; work forked to the helper is always joined back before the
 // call's last kernel, so the caller sees plain stream order.  Event record and wait
@@ -393,7 +394,11 @@ static int check_decode_item(const pq_desc* d, const uint16_t* X, const uint32_t
 // hp_scales != nullptr: INT8 HP branch, A and B are int8 codes (training path only)
 // What the FFN form asks of a forward beyond a linear's: a second 1-bit matrix on the same codes, or an input that is still the
 // gate projection X and the up projection `up` (the product of the two is left in `mid`)
-struct FfnParts { SecondWeight second; const uint16_t* up = nullptr; uint16_t* mid = nullptr; bool inner = false; };   // inner: a linear of the form
+// (inner: a linear of the form; before_main: what its fused tile waits for; rt: tables of as many tokens that are there already)
+struct FfnParts {
+  SecondWeight second; const uint16_t* up = nullptr; uint16_t* mid = nullptr; bool inner = false; cudaEvent_t before_main = nullptr;
+  const RoutingTables* rt = nullptr;
+};
 
 static int forward_impl(const pq_desc* d, const uint16_t* X, const uint32_t* w_bits, const int8_t* w_s8, const float* w_scales,
                         const uint16_t* A, const uint16_t* B, const float* hp_scales, const uint16_t* Wr, const float* alpha, const float* beta,
@@ -461,12 +466,13 @@ static int forward_impl(const pq_desc* d, const uint16_t* X, const uint32_t* w_b
   // (with a fused norm the up-projection reads the normalised copy the quantiser writes, so it follows it)
   SideCtx* side = (d->r > 0 && !routed(d) && !hp_scales && !norm_weight) ? side_for(st) : nullptr;
   if (side && !side_fork(side, st)) return PQ_ERR_CUDA;
+  if (ffn.rt) sv.rt = *ffn.rt;
   if (launch_route_and_quant(X, Wr, d->T, d->K, routed(d) ? E : 1, sv, sc, st, side ? side->side : st, norm_weight, norm_eps,
-                             ffn.up, ffn.mid) != cudaSuccess)
+                             ffn.up, ffn.mid, ffn.rt == nullptr) != cudaSuccess)
     return PQ_ERR_CUDA;
   if (side && cudaEventRecord(side->join, side->side) != cudaSuccess) return PQ_ERR_CUDA;
   const uint16_t* xs = (routed(d) || norm_weight) ? sv.xs : X;
-  return gemm_forward(a, w_s8, sv, xs, Y, st, side ? side->join : nullptr, ffn.second);
+  return gemm_forward(a, w_s8, sv, xs, Y, st, side ? side->join : ffn.before_main, ffn.second);
 }
 
 int pq_linear_forward(const pq_desc* d, const uint16_t* X, const uint32_t* w_bits, const int8_t* w_s8, const float* w_scales,
@@ -603,16 +609,25 @@ int pq_ffn_forward(const pq_ffn_desc* d, const uint16_t* X, const int8_t* g_s8, 
   carve_saved(&dx, c.saved_x, &sx);
   carve_saved(&dd, c.saved_d, &sd);
   LayerArgs a8{d->T, d->D, d->D, d->r, 1, 0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  rc = gemm_hp_up8(a8, sx, G8, c.g_int, st, U8, c.u_int);
-  if (rc) return rc;
+  // These two keep a few SMs busy and the memory hardly; they run on the helper stream beside the quantisation of the 1-bit FFN's hidden
+  // activation, up to the fused tile.  2048 tokens of 2048 and 5504, in a row / beside one another: 103.2 / 98.5 us.
+  SideCtx* side = side_for(st);
+  if (side && !side_fork(side, st)) return PQ_ERR_CUDA;
+  const cudaStream_t st8 = side ? side->side : st;
+  rc = gemm_hp_up8(a8, sx, G8, c.g_int, st8, U8, c.u_int);
   int8_t* qm = reinterpret_cast<int8_t*>(sd.h);
   float* gamma_m = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(sd.h) + align_up((size_t)sd.max_items * kTileRows * d->r));
-  if (launch_ffn8_act(c.g_int, c.u_int, sx.gamma, hp_scales, d->T, d->r, qm, gamma_m, st) != cudaSuccess) return PQ_ERR_CUDA;
+  if (launch_ffn8_act(c.g_int, c.u_int, sx.gamma, hp_scales, d->T, d->r, qm, gamma_m, st8) != cudaSuccess && !rc) rc = PQ_ERR_CUDA;
+  if (side && cudaEventRecord(side->join, side->side) != cudaSuccess) return PQ_ERR_CUDA;
   FfnParts down;
-  down.up = c.U1; down.mid = c.M1; down.inner = true;
+  down.up = c.U1; down.mid = c.M1; down.inner = true; down.rt = &sx.rt;
+  if (side) down.before_main = side->join;
   // down projections of both FFNs in one fused tile: beta (lam / gamma) (q(M1) . S_d) + alpha (D8 qm) / (gamma_D gamma_m)
-  return forward_impl(&dd, c.G1, nullptr, d_s8, d_scales, reinterpret_cast<const uint16_t*>(D8), reinterpret_cast<const uint16_t*>(D8),
+  if (!rc)
+    rc = forward_impl(&dd, c.G1, nullptr, d_s8, d_scales, reinterpret_cast<const uint16_t*>(D8), reinterpret_cast<const uint16_t*>(D8),
                       hp_scales + 1, nullptr, alpha, beta, Y, c.saved_d, c.saved_d_bytes, c.ws_fwd, c.ws_fwd_bytes, stream, true, nullptr, 0.f, down);
+  if (rc && side) cudaStreamWaitEvent(st, side->join, 0);      // a call that fails leaves nothing on the helper stream either
+  return rc;
 }
 
 int pq_decode_pack_bytes(const pq_desc* d, size_t* bits_il_bytes, size_t* b_il_bytes) {

@@ -869,7 +869,7 @@ static cudaError_t router_limits() {
 }
 
 cudaError_t launch_route_and_quant(const uint16_t* X, const uint16_t* Wr, int T, int K, int E, const SavedPtrs& sv, const FwdScratch& sc,
-                                   cudaStream_t st, cudaStream_t st_quant, const uint16_t* norm_weight, float norm_eps, const uint16_t* up, uint16_t* mid) {
+                                   cudaStream_t st, cudaStream_t st_quant, const uint16_t* norm_weight, float norm_eps, const uint16_t* up, uint16_t* mid, bool tables) {
   if (E > 1) st_quant = st;   // the sorted position of a token comes from the router and the scan
   const uint4* nw = reinterpret_cast<const uint4*>(norm_weight);
   if (nw) {
@@ -893,7 +893,7 @@ cudaError_t launch_route_and_quant(const uint16_t* X, const uint16_t* Wr, int T,
                                      E, sv.expert, sc.gate_tok, sc.probs_tok, sc.block_counts, nw, sc.rms);
     if (e != cudaSuccess) return e;   // the kernels behind this one store where its counts say
   }
-  {
+  if (tables) {
     LaunchScope ls(KID_ROUTE_SCAN, st);
     if (const cudaError_t e = launch_pdl(k_route_scan, 1, 512, 0, st, T, E, nblocks, sc.block_counts, sc.block_base, sv.offsets, sv.rt)) return e;
   }

@@ -100,7 +100,8 @@ cudaError_t launch_pack(const float* W, int N, int K, uint32_t* bits, int8_t* s8
 // xs of the tokens is then written even without routing (it is the only place the normalised activation exists)
 cudaError_t launch_route_and_quant(const uint16_t* X, const uint16_t* Wr, int T, int K, int E, const SavedPtrs& sv, const FwdScratch& sc,
                                    cudaStream_t st, cudaStream_t st_quant, const uint16_t* norm_weight = nullptr, float norm_eps = 0.f,
-                                   const uint16_t* up = nullptr, uint16_t* mid = nullptr);   // up: X is silu's side of a SwiGLU, left in mid
+                                   const uint16_t* up = nullptr, uint16_t* mid = nullptr,    // up: X is silu's side of a SwiGLU, left in mid
+                                   bool tables = true);   // false: sv.rt has been made for as many tokens before (E == 1)
 cudaError_t launch_finalize_scales(const float* dbeta_partial, int nslots, const float* dalpha_partial, int E, int N, const float* w_scales,
                                    int vec, float* dbeta, float* dalpha, double* blk_sums, unsigned* arrivals, cudaStream_t st);
 cudaError_t launch_ffn8_act(const int* g_int, const int* u_int, const float* gamma, const float* hp_scales, int T, int r, int8_t* qm,

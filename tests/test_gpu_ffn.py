@@ -100,3 +100,49 @@ def test_ffn_rejects_bad_shapes():
     assert pqb.pq_ffn_workspace_bytes(pqb.make_ffn_desc(128, 256, 480, 24)) == 0       # r not a multiple of 16
     assert pqb.pq_ffn_workspace_bytes(pqb.make_ffn_desc(128, 250, 480, 32)) == 0
     assert pqb.pq_ffn_workspace_bytes(pqb.make_ffn_desc(128, 256, 480, 32)) > 0
+
+
+@pytest.mark.parametrize("T,Dm,F1,r", [(1, 64, 96, 16), (129, 256, 1056, 128), (700, 512, 2080, 48)])
+def test_ffn_with_and_without_the_helper_stream(T, Dm, F1, r):
+    # The INT8 FFN's projections run on a helper stream beside the hidden activation of the 1-bit one: the same bits without it, and in
+    # a graph that is captured and replayed on other inputs.
+    X, Wg, Wu, Wd, G, U, D = _weights(T, Dm, F1, r, seed=T)
+    one = [_pack(W) for W in (Wg, Wu, Wd)]
+    G8, D8, sc_gd = _pack8(G, D)
+    U8, _, sc_ud = _pack8(U, D)
+    hp = torch.stack([sc_gd[0, 0], sc_ud[0, 0], sc_gd[0, 1]]).contiguous()
+    d = pqb.make_ffn_desc(T, Dm, F1, r)
+    ws = torch.empty(pqb.pq_ffn_workspace_bytes(d), dtype=torch.uint8, device="cuda")
+    first, second = torch.from_numpy(X).cuda().to(torch.bfloat16), torch.from_numpy(X[::-1].copy()).cuda().to(torch.bfloat16)
+    Xd, Y = first.clone(), torch.empty((T, Dm), dtype=torch.bfloat16, device="cuda")
+    al, be = torch.full((1,), 2.0, device="cuda"), torch.full((1,), 0.2, device="cuda")
+
+    def call():
+        pqb.pq_ffn_forward(d, Xd, *one[0], *one[1], *one[2], G8, U8, D8, hp, al, be, Y, ws)
+
+    def out(x):
+        Xd.copy_(x)
+        Y.zero_()
+        call()
+        torch.cuda.synchronize()
+        return Y.clone()
+    pqb.pq_set_option(pqb.PQ_OPT_SIDE_STREAM, 0)
+    try:
+        want = out(first), out(second)
+    finally:
+        pqb.pq_set_option(pqb.PQ_OPT_SIDE_STREAM, 1)
+    assert torch.equal(out(first), want[0]) and torch.equal(out(second), want[1])
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.stream(stream):
+        call()                                           # the helper stream of this stream is made outside the capture
+        with torch.cuda.graph(graph, stream=stream):
+            call()
+    for x, y in zip((first, second), want):
+        torch.cuda.synchronize()
+        Xd.copy_(x)
+        Y.zero_()
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(Y, y)
+    check_status()
