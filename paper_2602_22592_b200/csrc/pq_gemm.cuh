@@ -362,7 +362,8 @@ __device__ __forceinline__ void gemm_body(const typename P::Params& p) {
           // with this one, it would keep a tile from a free pair for as long as this one lasts.  1024 x 1024 over 4096 tokens, sixteen long
           // tiles and 64 short ones: backward 43.6 -> 35.6 us.
           for (int lo = 0, hi; ok && lo < sg.nkb; lo = hi) {
-            hi = kTickets && s + 1 == nseg && lo < sg.nkb - kStages ? sg.nkb - kStages : sg.nkb;
+            const int late = sg.nkb - min(kStages, max(2, sg.nkb >> 2));   // (of a short contraction, its last two steps)
+            hi = kTickets && s + 1 == nseg && lo < late ? late : sg.nkb;
             if (s + 1 == nseg && hi == sg.nkb) draw();
             if (sg.mode <= MODE_BF_KK) produce(std::integral_constant<int, 0>{}, lo, hi);
             else if (sg.mode == MODE_BF_KM && sg.b_blk > 0) produce(std::integral_constant<int, 1>{}, lo, hi);

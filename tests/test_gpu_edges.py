@@ -355,3 +355,15 @@ def test_forward_that_keeps_nothing_for_a_backward(T, K, N, r, E, hp8):
     torch.cuda.synchronize()
     check_status()
     assert torch.equal(Y, L.Y) and bool((ws[-4096:] == 0xA5).all())
+
+
+@pytest.mark.parametrize("T,K,N,r,E,vector", [
+    (100, 1056, 288, 72, 16, False),      # experts without tokens, and several to a tile
+    (129, 96, 64, 16, 3, True), (4100, 64, 96, 24, 2, False), (16640, 64, 96, 24, 1, False),   # a tile more than one; many tiles of an expert
+])
+def test_gradients_of_experts_over_their_items(T, K, N, r, E, vector):
+    # dB and dA contract over an expert's items in one run: from its first tile on, in the tokens and in the hidden planes
+    c = I.make_linear_case(T, K, N, r, E, seed=T + E, scale_vector=vector, alpha=1.5, beta=0.5)
+    f = O.linear_forward(c["X"], c["W"], c["A"], c["B"], c["Wr"], c["alpha"], c["beta"])
+    g = O.linear_backward(c["dY"], c["X"], f, c["A"], c["B"], c["Wr"], c["alpha"], c["beta"])
+    check_backward(c, run_fwd_bwd(c, vector), f, g, vector)
