@@ -20,14 +20,16 @@
  *     small file-scope device variables (a status word, the spin limit, the
  *     64 KiB array of pq_pack_weights_static), and -- unless PQ_OPT_SIDE_STREAM
  *     is 0 -- one helper stream and two events per (device, caller stream)
- *     that has called pq_linear_forward, created on first
- *     use and kept until the process exits;
+ *     that has called pq_linear_forward for a dense layer with an HP branch or
+ *     pq_ffn_forward, created on first use and kept until the process exits.
+ *     cudaStreamPerThread is another stream in every host thread and has a
+ *     helper in each; those of a thread that has ended go to the next one;
  *   - work is only enqueued on `stream` (a cudaStream_t passed as void*) and on
  *     that helper stream, which is joined back into `stream` inside the same
  *     call; no call synchronises the device except pq_device_status and
  *     pq_set_option(PQ_OPT_SPIN_CYCLES);
- *   - threads: calls on different streams may come from different host threads;
- *     the helper-stream table is locked.  pq_set_option, pq_profile_events and the
+ *   - threads: calls on different streams (cudaStreamPerThread included) may come
+ *     from different host threads; the helper-stream table is locked.  pq_set_option, pq_profile_events and the
  *     launch counter behind pq_kernel_launches are plain process-wide state without
  *     locks: set options and register events while no other thread is inside the
  *     library, and read the counter as an approximate figure under concurrency;
@@ -382,7 +384,8 @@ int pq_device_status(void* stream, int* code, int* where);
  *   serialisation, so that a kernel's prologue (barrier set-up, the copy of the sign bits)
  *   overlaps the tail of the kernel before it in the stream.  0 = plain stream order.
  *   PQ_OPT_SIDE_STREAM (default 1): pq_linear_forward (dense layer with an HP branch) runs the
- *   activation quantisation beside the HP up-projection, on a helper stream the library keeps per
+ *   activation quantisation beside the HP up-projection, pq_ffn_forward the INT8 FFN's projections
+ *   beside the quantisation of the 1-bit FFN's hidden activation, on a helper stream the library keeps per
  *   caller stream (created on first use, never during a stream capture); the helper's work is joined
  *   back inside the same call, so the caller's stream order is unchanged and a stream capture records
  *   one graph with a fork and a join.  0 = every kernel on the caller's stream.

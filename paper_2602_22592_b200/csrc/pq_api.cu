@@ -3,12 +3,10 @@
 // synchronisation (except pq_device_status, which says so).
 #include <algorithm>
 #include <cstring>
-#include <map>
-#include <mutex>
 #include <new>
-#include <utility>
 
 #include "pq_kernels.cuh"
+#include "pq_side.cuh"
 
 namespace pq {
 
@@ -134,55 +132,6 @@ static size_t carve_bwd_scratch(const pq_desc* d, void* base, BwdScratch* out) {
 }
 
 static inline bool misaligned(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) != 0; }
-
-// ---------------------------------------------------------------------------
-// Helper stream: kernels of one call that do not depend on one another run side
-// by side (forward of a dense layer with an HP branch: the activation quantisation
-// next to the HP up-projection; FFN form: the INT8 FFN's projections next to the
-// quantisation of the 1-bit FFN's hidden activation).
-// Every caller stream gets one non-blocking helper stream and two events, created
-// on first use and kept; work forked to the helper is always joined back before the
-// call's last kernel, so the caller sees plain stream order.  Event record and wait
-// are legal under stream capture and become edges of the captured graph.
-// ---------------------------------------------------------------------------
-static int g_side_streams = 1;
-
-struct SideCtx {
-  cudaStream_t side = nullptr;
-  cudaEvent_t fork = nullptr, join = nullptr;
-};
-
-static SideCtx* side_for(cudaStream_t st) {
-  if (!g_side_streams) return nullptr;
-  static std::mutex mu;
-  static std::map<std::pair<int, cudaStream_t>, SideCtx> ctxs;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
-  std::lock_guard<std::mutex> lock(mu);
-  SideCtx& c = ctxs[std::make_pair(dev, st)];
-  if (!c.side) {
-    // nothing is created while the caller's stream is being captured: such a call keeps plain stream order
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-      cudaGetLastError();
-      return nullptr;
-    }
-    SideCtx n;
-    if (cudaStreamCreateWithFlags(&n.side, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&n.fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&n.join, cudaEventDisableTiming) != cudaSuccess) {
-      cudaGetLastError();
-      return nullptr;   // the caller falls back to plain stream order
-    }
-    c = n;
-  }
-  return &c;
-}
-
-// helper stream ordered after everything already in st
-static bool side_fork(SideCtx* c, cudaStream_t st) {
-  return cudaEventRecord(c->fork, st) == cudaSuccess && cudaStreamWaitEvent(c->side, c->fork, 0) == cudaSuccess;
-}
 
 // ---------------------------------------------------------------------------
 // Allocation-free weight pack: the fp64 partial sums live in a fixed device array
