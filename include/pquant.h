@@ -26,8 +26,9 @@
  *     helper in each; those of a thread that has ended go to the next one;
  *   - work is only enqueued on `stream` (a cudaStream_t passed as void*) and on
  *     that helper stream, which is joined back into `stream` inside the same
- *     call; no call synchronises the device except pq_device_status and
- *     pq_set_option(PQ_OPT_SPIN_CYCLES);
+ *     call, one that fails included; no call synchronises the device except
+ *     pq_device_status and pq_set_option(PQ_OPT_SPIN_CYCLES) (a call that fails
+ *     and cannot join the helper waits for the helper's work);
  *   - threads: calls on different streams (cudaStreamPerThread included) may come
  *     from different host threads; the helper-stream table is locked.  pq_set_option, pq_profile_events and the
  *     launch counter behind pq_kernel_launches are plain process-wide state without

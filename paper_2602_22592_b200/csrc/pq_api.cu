@@ -413,15 +413,17 @@ static int forward_impl(const pq_desc* d, const uint16_t* X, const uint32_t* w_b
   // dense layer with a bf16 HP branch: the quantisation runs on the helper stream next to scan -> up-projection
   // (the INT8 branch multiplies the codes themselves, so its up-projection follows the quantisation)
   // (with a fused norm the up-projection reads the normalised copy the quantiser writes, so it follows it)
-  SideCtx* side = (d->r > 0 && !routed(d) && !hp_scales && !norm_weight) ? side_for(st) : nullptr;
-  if (side && !side_fork(side, st)) return PQ_ERR_CUDA;
+  SideWork side(d->r > 0 && !routed(d) && !hp_scales && !norm_weight ? side_for(st) : nullptr, st);
+  if (!side.fork()) return PQ_ERR_CUDA;
   if (ffn.rt) sv.rt = *ffn.rt;
-  if (launch_route_and_quant(X, Wr, d->T, d->K, routed(d) ? E : 1, sv, sc, st, side ? side->side : st, norm_weight, norm_eps,
+  if (launch_route_and_quant(X, Wr, d->T, d->K, routed(d) ? E : 1, sv, sc, st, side.stream(), norm_weight, norm_eps,
                              ffn.up, ffn.mid, ffn.rt == nullptr) != cudaSuccess)
     return PQ_ERR_CUDA;
-  if (side && cudaEventRecord(side->join, side->side) != cudaSuccess) return PQ_ERR_CUDA;
+  if (!side.finish()) return PQ_ERR_CUDA;
   const uint16_t* xs = (routed(d) || norm_weight) ? sv.xs : X;
-  return gemm_forward(a, w_s8, sv, xs, Y, st, side ? side->join : ffn.before_main, ffn.second);
+  rc = gemm_forward(a, w_s8, sv, xs, Y, st, side.on() ? side.end() : ffn.before_main, ffn.second);
+  if (rc == PQ_OK) side.joined();
+  return rc;
 }
 
 int pq_linear_forward(const pq_desc* d, const uint16_t* X, const uint32_t* w_bits, const int8_t* w_s8, const float* w_scales,
@@ -560,22 +562,20 @@ int pq_ffn_forward(const pq_ffn_desc* d, const uint16_t* X, const int8_t* g_s8, 
   LayerArgs a8{d->T, d->D, d->D, d->r, 1, 0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   // These two keep a few SMs busy and the memory hardly; they run on the helper stream beside the quantisation of the 1-bit FFN's hidden
   // activation, up to the fused tile.  2048 tokens of 2048 and 5504, in a row / beside one another: 103.2 / 98.5 us.
-  SideCtx* side = side_for(st);
-  if (side && !side_fork(side, st)) return PQ_ERR_CUDA;
-  const cudaStream_t st8 = side ? side->side : st;
-  rc = gemm_hp_up8(a8, sx, G8, c.g_int, st8, U8, c.u_int);
+  SideWork side(side_for(st), st);
+  if (!side.fork()) return PQ_ERR_CUDA;
+  rc = gemm_hp_up8(a8, sx, G8, c.g_int, side.stream(), U8, c.u_int);
+  if (rc) return rc;
   int8_t* qm = reinterpret_cast<int8_t*>(sd.h);
   float* gamma_m = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(sd.h) + align_up((size_t)sd.max_items * kTileRows * d->r));
-  if (launch_ffn8_act(c.g_int, c.u_int, sx.gamma, hp_scales, d->T, d->r, qm, gamma_m, st8) != cudaSuccess && !rc) rc = PQ_ERR_CUDA;
-  if (side && cudaEventRecord(side->join, side->side) != cudaSuccess) return PQ_ERR_CUDA;
+  if (launch_ffn8_act(c.g_int, c.u_int, sx.gamma, hp_scales, d->T, d->r, qm, gamma_m, side.stream()) != cudaSuccess) return PQ_ERR_CUDA;
+  if (!side.finish()) return PQ_ERR_CUDA;
   FfnParts down;
-  down.up = c.U1; down.mid = c.M1; down.inner = true; down.rt = &sx.rt;
-  if (side) down.before_main = side->join;
+  down.up = c.U1; down.mid = c.M1; down.inner = true; down.rt = &sx.rt; down.before_main = side.end();
   // down projections of both FFNs in one fused tile: beta (lam / gamma) (q(M1) . S_d) + alpha (D8 qm) / (gamma_D gamma_m)
-  if (!rc)
-    rc = forward_impl(&dd, c.G1, nullptr, d_s8, d_scales, reinterpret_cast<const uint16_t*>(D8), reinterpret_cast<const uint16_t*>(D8),
-                      hp_scales + 1, nullptr, alpha, beta, Y, c.saved_d, c.saved_d_bytes, c.ws_fwd, c.ws_fwd_bytes, stream, true, nullptr, 0.f, down);
-  if (rc && side) cudaStreamWaitEvent(st, side->join, 0);      // a call that fails leaves nothing on the helper stream either
+  rc = forward_impl(&dd, c.G1, nullptr, d_s8, d_scales, reinterpret_cast<const uint16_t*>(D8), reinterpret_cast<const uint16_t*>(D8),
+                    hp_scales + 1, nullptr, alpha, beta, Y, c.saved_d, c.saved_d_bytes, c.ws_fwd, c.ws_fwd_bytes, stream, true, nullptr, 0.f, down);
+  if (rc == PQ_OK) side.joined();
   return rc;
 }
 

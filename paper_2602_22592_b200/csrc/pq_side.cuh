@@ -104,9 +104,35 @@ static SideCtx* side_for(cudaStream_t st) {
   }
 }
 
-// helper stream ordered after everything already in st
-static bool side_fork(SideCtx* c, cudaStream_t st) {
-  return cudaEventRecord(c->fork, st) == cudaSuccess && cudaStreamWaitEvent(c->side, c->fork, 0) == cudaSuccess;
-}
+// What one call runs on its helper: fork, launches on stream(), finish, a wait for end() in the caller's stream, joined.  A call that fails on
+// the way leaves the rest to the destructor: what the helper has then goes before whatever the caller's stream gets next or, where
+// not even that can be enqueued, has ended.
+class SideWork {
+ public:
+  SideWork(SideCtx* c, cudaStream_t st) : c_(c), st_(st) {}
+  SideWork(const SideWork&) = delete;
+  SideWork& operator=(const SideWork&) = delete;
+  ~SideWork() {
+    if (open_ && (cudaEventRecord(c_->join, c_->side) != cudaSuccess || cudaStreamWaitEvent(st_, c_->join, 0) != cudaSuccess))
+      cudaStreamSynchronize(c_->side);
+  }
+  bool on() const { return c_ != nullptr; }
+  cudaStream_t stream() const { return c_ ? c_->side : st_; }
+  // helper stream ordered after everything already in st
+  bool fork() {
+    if (!c_) return true;
+    if (cudaEventRecord(c_->fork, st_) != cudaSuccess || cudaStreamWaitEvent(c_->side, c_->fork, 0) != cudaSuccess) return false;
+    open_ = true;
+    return true;
+  }
+  bool finish() { return !c_ || cudaEventRecord(c_->join, c_->side) == cudaSuccess; }
+  cudaEvent_t end() const { return c_ ? c_->join : nullptr; }
+  void joined() { open_ = false; }
+
+ private:
+  SideCtx* c_;
+  cudaStream_t st_;
+  bool open_ = false;
+};
 
 }  // namespace pq

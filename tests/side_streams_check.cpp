@@ -21,7 +21,9 @@ std::mutex g_mu;
 std::condition_variable g_cv;
 int g_live = 0;                    // streams and events that exist
 int g_capturing = 0;
-int g_fail_event_create = 0;       // how many more event creations succeed, counted down; 0: all
+int g_fail_event_create = 0;       // the event creation that fails, counted down; 0: none
+int g_fail_record = 0, g_fail_wait = 0;   // the same of records and waits
+int g_synchronised = 0;
 // threads that meet between a record and the wait that follows it, so that all of them have recorded before any waits
 int g_meet = 0, g_met = 0, g_round = 0;
 
@@ -55,6 +57,7 @@ cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) {
 cudaError_t cudaEventDestroy(cudaEvent_t e) { std::lock_guard<std::mutex> l(g_mu); --g_live; delete e; return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t st) {
   std::unique_lock<std::mutex> l(g_mu);
+  if (g_fail_record && --g_fail_record == 0) return cudaErrorUnknown;
   e->at = name_of(st);
   if (g_meet) {
     const int round = g_round;
@@ -65,9 +68,11 @@ cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t st) {
 }
 cudaError_t cudaStreamWaitEvent(cudaStream_t st, cudaEvent_t e, unsigned) {
   std::lock_guard<std::mutex> l(g_mu);
+  if (g_fail_wait && --g_fail_wait == 0) return cudaErrorUnknown;
   if (st != cudaStreamPerThread) st->log.push_back(e->at);
   return cudaSuccess;
 }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { ++g_synchronised; return cudaSuccess; }
 }
 
 // Each of several threads forks from `st`: its helper has to wait for the thread's own stream, whatever the others record meanwhile
@@ -77,7 +82,8 @@ static void fork_from_every_thread(cudaStream_t st, int n, std::set<pq::SideCtx*
   for (int i = 0; i < n; ++i)
     threads.emplace_back([&] {
       pq::SideCtx* c = pq::side_for(st);
-      CHECK(c && pq::side_fork(c, st));
+      pq::SideWork work(c, st);
+      CHECK(c && work.fork());
       std::lock_guard<std::mutex> l(g_mu);
       CHECK(!c->side->log.empty() && c->side->log.back() == name_of(st));
       seen->insert(c);
@@ -117,6 +123,50 @@ int main(int argc, char** argv) {
     pq::SideCtx* c = pq::side_for(&a);
     g_capturing = 1;
     CHECK(c && pq::side_for(&a) == c);
+  } else if (what == "failed_calls") {
+    pq::SideCtx* c = pq::side_for(&a);
+    const std::string helper = name_of(c->side);
+    {   // a whole call: the caller's stream waits where the call says, nothing more
+      pq::SideWork work(c, &a);
+      CHECK(work.fork() && work.stream() == c->side && work.finish() && work.end() == c->join);
+      CHECK(cudaStreamWaitEvent(&a, work.end(), 0) == cudaSuccess);
+      work.joined();
+    }
+    CHECK(a.log.size() == 1 && a.log.back() == helper && g_synchronised == 0);
+    {   // left after its fork, or after the mark of its end: the caller's stream waits all the same
+      pq::SideWork work(c, &a);
+      CHECK(work.fork());
+    }
+    CHECK(a.log.size() == 2 && a.log.back() == helper && g_synchronised == 0);
+    {
+      pq::SideWork work(c, &a);
+      CHECK(work.fork());
+      g_fail_record = 1;                              // the mark fails, once
+      CHECK(!work.finish());
+    }
+    CHECK(a.log.size() == 3 && a.log.back() == helper && g_synchronised == 0);
+    {
+      pq::SideWork work(c, &a);
+      CHECK(work.fork());
+      g_fail_record = 1;                              // nothing can be marked: the helper's work has ended
+    }
+    CHECK(a.log.size() == 3 && g_synchronised == 1);
+    {
+      pq::SideWork work(c, &a);
+      CHECK(work.fork() && work.finish());
+      g_fail_wait = 1;
+    }
+    CHECK(a.log.size() == 3 && g_synchronised == 2);
+    for (int wait = 0; wait < 2; ++wait) {            // a fork that fails leaves nothing to wait for
+      (wait ? g_fail_wait : g_fail_record) = 1;
+      pq::SideWork work(c, &a);
+      CHECK(!work.fork());
+    }
+    {   // plain stream order
+      pq::SideWork work(nullptr, &a);
+      CHECK(work.fork() && work.stream() == &a && work.finish() && !work.end() && !work.on());
+    }
+    CHECK(a.log.size() == 3 && g_synchronised == 2);
   } else {
     std::fprintf(stderr, "which check?\n");
     return 2;
