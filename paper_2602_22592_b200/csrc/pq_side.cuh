@@ -63,6 +63,14 @@ struct ThreadSides {
   }
 };
 
+// the call is being recorded (and not refused, as the null stream's is beside another thread's capture)
+static bool stream_captured(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap == cudaStreamCaptureStatusActive;
+  cudaGetLastError();
+  return false;
+}
+
 // the helper of `st` on the current device, or null: the call then keeps plain stream order
 static SideCtx* side_for(cudaStream_t st) {
   if (!g_side_streams) return nullptr;
@@ -103,6 +111,13 @@ static SideCtx* side_for(cudaStream_t st) {
     return nullptr;
   }
 }
+
+// Whether an FFN form of so many 128-row tiles is worth a fork in a call that is not being captured: fork and join cost 3-6 us of host time,
+// about what a small call takes altogether.  The line, in a row / beside one another, us per call (called and waited for): one
+// token, 64 and 96 23.1 / 29.1 (33.4 / 38.5), 128 tokens, 256 and 256 26.9 / 29.9 (39.5 / 42.7), 512 and 512 29.8 / 30.8 (41.8 / 43.2);
+// 512 tokens, 512 and 512 30.8 / 30.8 (42.6 / 43.3), 128, 1024 and 1024 36.1 / 35.1 (47.2 / 45.9), 256, 1024 and 2816 41.2 / 39.2
+// (52.1 / 51.4).  Replayed from a graph the smallest of these takes 20.5 / 18.5, so that a call under capture always forks.
+static inline bool ffn_beside(int tiles, int D, int F1) { return 128LL * tiles * D * F1 >= 1LL << 27; }
 
 // What one call runs on its helper: fork, launches on stream(), finish, a wait for end() in the caller's stream, joined.  A call that fails on
 // the way leaves the rest to the destructor: what the helper has then goes before whatever the caller's stream gets next or, where

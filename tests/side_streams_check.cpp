@@ -20,7 +20,7 @@ namespace {
 std::mutex g_mu;
 std::condition_variable g_cv;
 int g_live = 0;                    // streams and events that exist
-int g_capturing = 0;
+int g_capturing = 0, g_refused = 0;
 int g_fail_event_create = 0;       // the event creation that fails, counted down; 0: none
 int g_fail_record = 0, g_fail_wait = 0;   // the same of records and waits
 int g_synchronised = 0;
@@ -42,6 +42,7 @@ extern "C" {
 cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s) {
+  if (g_refused) return cudaErrorStreamCaptureImplicit;
   *s = g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
   return cudaSuccess;
 }
@@ -121,8 +122,15 @@ int main(int argc, char** argv) {
     CHECK(!pq::side_for(&a));
     pq::g_side_streams = 1;
     pq::SideCtx* c = pq::side_for(&a);
+    CHECK(!pq::stream_captured(&a));
     g_capturing = 1;
-    CHECK(c && pq::side_for(&a) == c);
+    CHECK(c && pq::side_for(&a) == c && pq::stream_captured(&a));
+    g_refused = 1;
+    CHECK(!pq::stream_captured(&a));
+  } else if (what == "small_calls") {
+    // by tiles of 128 tokens and the two widths, without an overflow at the largest
+    CHECK(!pq::ffn_beside(1, 64, 96) && !pq::ffn_beside(1, 512, 1024) && !pq::ffn_beside(4, 512, 480));
+    CHECK(pq::ffn_beside(1, 1024, 1024) && pq::ffn_beside(4, 512, 512) && pq::ffn_beside(1, 2048, 5504) && pq::ffn_beside(1 << 16, 1 << 16, 1 << 16));
   } else if (what == "failed_calls") {
     pq::SideCtx* c = pq::side_for(&a);
     const std::string helper = name_of(c->side);

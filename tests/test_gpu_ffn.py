@@ -2,6 +2,9 @@
 ABI against the CPU oracle.  Every integer stage bit for bit (codes of x, exact sums and hidden codes of the INT8 FFN,
 and -- replayed on the hidden activation the GPU itself produced -- the codes feeding the 1-bit down projection); the
 bf16 tensors within the tolerance."""
+import ctypes
+from collections import Counter
+
 import numpy as np
 import pytest
 import torch
@@ -9,6 +12,7 @@ import torch
 from oracle import pquant_oracle as O
 from paper_2602_22592_b200 import binding as pqb
 from paper_2602_22592_b200 import inputs as I
+from paper_2602_22592_b200.layer import PQLinear
 from test_gpu_forward import TOL_BF16, TOL_RMS, check_status, f32, rel_err, rms_err
 
 pytestmark = pytest.mark.gpu
@@ -145,4 +149,41 @@ def test_ffn_with_and_without_the_helper_stream(T, Dm, F1, r):
         graph.replay()
         torch.cuda.synchronize()
         assert torch.equal(Y, y)
+    check_status()
+
+
+@pytest.mark.parametrize("T,Dm,F1,r", [(1, 64, 96, 16), (512, 512, 512, 32)])     # on either side of the line for calls outside a capture
+def test_ffn_forks_under_capture(T, Dm, F1, r):
+    # A captured call goes two ways behind the gate / up tile and meets again in front of the fused one, whatever its size; without
+    # the helper stream it is one chain.
+    X, Wg, Wu, Wd, G, U, D = _weights(T, Dm, F1, r, seed=T)
+    one = [_pack(W) for W in (Wg, Wu, Wd)]
+    G8, D8, sc_gd = _pack8(G, D)
+    U8, _, sc_ud = _pack8(U, D)
+    hp = torch.stack([sc_gd[0, 0], sc_ud[0, 0], sc_gd[0, 1]]).contiguous()
+    d = pqb.make_ffn_desc(T, Dm, F1, r)
+    ws = torch.empty(pqb.pq_ffn_workspace_bytes(d), dtype=torch.uint8, device="cuda")
+    Xd, Y = torch.from_numpy(X).cuda().to(torch.bfloat16), torch.empty((T, Dm), dtype=torch.bfloat16, device="cuda")
+    al, be = torch.full((1,), 2.0, device="cuda"), torch.full((1,), 0.2, device="cuda")
+
+    def branches(helper):
+        stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph(keep_graph=True)
+        pqb.pq_set_option(pqb.PQ_OPT_SIDE_STREAM, helper)
+        try:
+            with torch.cuda.stream(stream):
+                # a dense forward with an HP branch makes the stream's helper, at any size
+                L = PQLinear(64, 64, 64, 16, 1).load_case(I.make_linear_case(64, 64, 64, 16, 1, seed=3, with_grad=False))
+                L.pack()
+                L.forward()
+                torch.cuda.synchronize()
+                with torch.cuda.graph(graph, stream=stream):
+                    pqb.pq_ffn_forward(d, Xd, *one[0], *one[1], *one[2], G8, U8, D8, hp, al, be, Y, ws)
+        finally:
+            pqb.pq_set_option(pqb.PQ_OPT_SIDE_STREAM, 1)
+        # the edges of the graph, with their kind (8 bytes each): those of programmatic launches are not handed out without it
+        cuda, handle, n = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t(64)
+        ends, kinds = [(ctypes.c_void_p * 64)() for _ in range(2)], (ctypes.c_uint64 * 64)()
+        assert cuda.cuGraphGetEdges_v2(handle, ends[0], ends[1], kinds, ctypes.byref(n)) == 0 and 0 < n.value < 64
+        return tuple(max(Counter(e[:n.value]).values()) for e in ends)
+    assert branches(1) == (2, 2) and branches(0) == (1, 1)
     check_status()

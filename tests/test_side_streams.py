@@ -23,6 +23,6 @@ def check(tmp_path_factory):
     return run
 
 
-@pytest.mark.parametrize("what", ["per_thread", "ended_threads", "handles", "plain_order", "failed_calls"])
+@pytest.mark.parametrize("what", ["per_thread", "ended_threads", "handles", "plain_order", "small_calls", "failed_calls"])
 def test_helper_streams(check, what):
     check(what)
