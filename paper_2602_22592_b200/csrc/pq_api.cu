@@ -562,7 +562,8 @@ int pq_ffn_forward(const pq_ffn_desc* d, const uint16_t* X, const int8_t* g_s8, 
   LayerArgs a8{d->T, d->D, d->D, d->r, 1, 0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   // These two keep a few SMs busy and the memory hardly; they run on the helper stream beside the quantisation of the 1-bit FFN's hidden
   // activation, up to the fused tile.  2048 tokens of 2048 and 5504, in a row / beside one another: 103.2 / 98.5 us.
-  SideWork side(ffn_beside(mtiles_of(&dx), d->D, d->F1) || stream_captured(st) ? side_for(st) : nullptr, st);
+  SideCtx* const helper = side_for(st);     // made here by a small call too, for a later one under capture
+  SideWork side(ffn_beside(mtiles_of(&dx), d->D, d->F1) || stream_captured(st) ? helper : nullptr, st);
   if (!side.fork()) return PQ_ERR_CUDA;
   rc = gemm_hp_up8(a8, sx, G8, c.g_int, side.stream(), U8, c.u_int);
   if (rc) return rc;

@@ -12,7 +12,6 @@ import torch
 from oracle import pquant_oracle as O
 from paper_2602_22592_b200 import binding as pqb
 from paper_2602_22592_b200 import inputs as I
-from paper_2602_22592_b200.layer import PQLinear
 from test_gpu_forward import TOL_BF16, TOL_RMS, check_status, f32, rel_err, rms_err
 
 pytestmark = pytest.mark.gpu
@@ -166,18 +165,18 @@ def test_ffn_forks_under_capture(T, Dm, F1, r):
     Xd, Y = torch.from_numpy(X).cuda().to(torch.bfloat16), torch.empty((T, Dm), dtype=torch.bfloat16, device="cuda")
     al, be = torch.full((1,), 2.0, device="cuda"), torch.full((1,), 0.2, device="cuda")
 
+    def call():
+        pqb.pq_ffn_forward(d, Xd, *one[0], *one[1], *one[2], G8, U8, D8, hp, al, be, Y, ws)
+
     def branches(helper):
         stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph(keep_graph=True)
         pqb.pq_set_option(pqb.PQ_OPT_SIDE_STREAM, helper)
         try:
             with torch.cuda.stream(stream):
-                # a dense forward with an HP branch makes the stream's helper, at any size
-                L = PQLinear(64, 64, 64, 16, 1).load_case(I.make_linear_case(64, 64, 64, 16, 1, seed=3, with_grad=False))
-                L.pack()
-                L.forward()
+                call()                                   # makes the stream's helper, at any size
                 torch.cuda.synchronize()
                 with torch.cuda.graph(graph, stream=stream):
-                    pqb.pq_ffn_forward(d, Xd, *one[0], *one[1], *one[2], G8, U8, D8, hp, al, be, Y, ws)
+                    call()
         finally:
             pqb.pq_set_option(pqb.PQ_OPT_SIDE_STREAM, 1)
         # the edges of the graph, with their kind (8 bytes each): those of programmatic launches are not handed out without it
