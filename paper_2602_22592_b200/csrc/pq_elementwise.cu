@@ -850,9 +850,10 @@ cudaError_t launch_pack(const float* W, int N, int K, uint32_t* bits, int8_t* s8
 
 // The router's opt-in limit is set once per device, to the largest request: it belongs to the kernel, not to a launch, so that a
 // call which set a smaller one would take it from under a call of another thread, or from under a launch recorded in a CUDA graph.
+// The quantiser of long SwiGLU rows asks for shared memory that it does not use, under the same limit.
 constexpr int kRouterSmemLimit = 116 * 1024;
 static_assert(router_smem<kMaxExperts>() <= kRouterSmemLimit, "the bare ring fits too");
-static cudaError_t router_limits() {
+static cudaError_t smem_limits() {
   constexpr int kMaxDevices = 64;
   static std::once_flag done[kMaxDevices];
   static cudaError_t result[kMaxDevices] = {};
@@ -864,8 +865,17 @@ static cudaError_t router_limits() {
     result[dev] = set(k_router<4>);
     if (result[dev] == cudaSuccess) result[dev] = set(k_router<8>);
     if (result[dev] == cudaSuccess) result[dev] = set(k_router<kMaxExperts>);
+    if (result[dev] == cudaSuccess) result[dev] = set(k_act_quant<0, 1, true>);
   });
   return result[dev];
+}
+// Shared memory to ask for so that an SM holds no more blocks of this grid than an even spread puts there (`most` at most, else what is
+// needed): they become resident while the kernel before ends, and the SMs that end first would otherwise take all they can hold.
+// One more block of each size, with the KB that every block takes beside it, is more than the 228 KB of an SM.
+static int smem_for_spread(int grid, int most, int needed) {
+  constexpr int kKB[] = {kRouterSmemLimit / 1024, 76, 57, 45, 38};
+  const int per_sm = (grid + sm_count() - 1) / sm_count();
+  return per_sm <= most ? kKB[per_sm - 1] * 1024 : needed;
 }
 
 cudaError_t launch_route_and_quant(const uint16_t* X, const uint16_t* Wr, int T, int K, int E, const SavedPtrs& sv, const FwdScratch& sc,
@@ -884,11 +894,8 @@ cudaError_t launch_route_and_quant(const uint16_t* X, const uint16_t* Wr, int T,
     int smem = router_smem<kMaxExperts>();
     if (E <= 4) { kern = k_router<4>; smem = router_smem<4>(); }
     else if (E <= 8) { kern = k_router<8>; smem = router_smem<8>(); }
-    // One CTA per SM (two) where the grid needs no more: its CTAs become resident while the kernel before ends, and the SMs that
-    // end first would otherwise take all they can hold.  2048 tokens x 3200: 17 us without this, 10 with it.
-    if (nblocks <= sm_count()) smem = kRouterSmemLimit;
-    else if (nblocks <= 2 * sm_count()) smem = 76 * 1024;
-    if (const cudaError_t e = router_limits()) return e;
+    smem = smem_for_spread(nblocks, 2, smem);     // 2048 tokens x 3200: 17 us without this, 10 with it
+    if (const cudaError_t e = smem_limits()) return e;
     const cudaError_t e = launch_pdl(kern, nblocks, 32 * kRouterWarps, smem, st, reinterpret_cast<const uint4*>(X), reinterpret_cast<const uint4*>(Wr), T, K,
                                      E, sv.expert, sc.gate_tok, sc.probs_tok, sc.block_counts, nw, sc.rms);
     if (e != cudaSuccess) return e;   // the kernels behind this one store where its counts say
@@ -905,8 +912,18 @@ cudaError_t launch_route_and_quant(const uint16_t* X, const uint16_t* Wr, int T,
   else if (per_lane <= 8) { kern = up ? k_act_quant<4, 2, true> : k_act_quant<4, 2>; wpr = 2; }
   else if (per_lane <= 16) { kern = up ? k_act_quant<4, 4, true> : k_act_quant<4, 4>; wpr = 4; }
   else if (per_lane <= 32) { kern = up ? k_act_quant<4, 8, true> : k_act_quant<4, 8>; wpr = 8; }
-  const int rows_per_block = 8 / wpr;
-  launch_pdl(kern, (T + rows_per_block - 1) / rows_per_block, 256, 0, st_quant, reinterpret_cast<const uint4*>(X), T, K, E, sv.expert, sc.block_base, sv.offsets, sc.gate_tok,
+  const int rows_per_block = 8 / wpr, grid = (T + rows_per_block - 1) / rows_per_block;
+  // A warp with a SwiGLU row that no registers hold is bound by the instructions of two passes, and directly behind the gate / up tile the
+  // blocks of a short batch would share the first few SMs that are free.  Whole FFN form, behind two other kernels / there / there
+  // and spread, replayed from a graph: 1024 tokens of 512 and 8640 127 / 183 / 108 us, 512 of 3200 and 8640 169-198 / 173 / 117, 256 of 512 and
+  // 8640 123 / 131 / 94, 2048 of 3200 and 8640 302 / 275 / 226.  Rows in registers are bound by memory and do not differ (1024 of 2048
+  // and 5504 64.5 / 64.6).
+  size_t smem = 0;
+  if (up && per_lane > 32) {
+    if (const cudaError_t e = smem_limits()) return e;
+    smem = smem_for_spread(grid, 5, 0);
+  }
+  launch_pdl(kern, grid, 256, smem, st_quant, reinterpret_cast<const uint4*>(X), T, K, E, sv.expert, sc.block_base, sv.offsets, sc.gate_tok,
                                     sc.probs_tok, reinterpret_cast<uint2*>(sv.q), reinterpret_cast<uint4*>(sv.xt),
                                     reinterpret_cast<uint4*>(sv.xs), sv.gamma, sv.gate, sv.probs, sv.perm, sv.pos, nw, sc.rms,
                                     reinterpret_cast<const uint4*>(up), reinterpret_cast<uint4*>(mid));

@@ -186,3 +186,25 @@ def test_ffn_forks_under_capture(T, Dm, F1, r):
         return tuple(max(Counter(e[:n.value]).values()) for e in ends)
     assert branches(1) == (2, 2) and branches(0) == (1, 1)
     check_status()
+
+
+@pytest.mark.parametrize("T", [1, 1184, 1185, 2369])    # rows held by no registers: one, two and three blocks of the quantiser on an SM
+def test_ffn_of_rows_beyond_8192(T):
+    Dm, F1, r = 64, 8224, 16
+    X, Wg, Wu, Wd, G, U, D = _weights(T, Dm, F1, r, seed=T)
+    f = O.ffn_decoupled_forward(X, Wg, Wu, Wd, G, U, D, 2.0, 0.2)
+    one = [_pack(W) for W in (Wg, Wu, Wd)]
+    G8, D8, sc_gd = _pack8(G, D)
+    U8, _, sc_ud = _pack8(U, D)
+    hp = torch.stack([sc_gd[0, 0], sc_ud[0, 0], sc_gd[0, 1]]).contiguous()
+    d = pqb.make_ffn_desc(T, Dm, F1, r)
+    ws = torch.empty(pqb.pq_ffn_workspace_bytes(d), dtype=torch.uint8, device="cuda")
+    Xd, Y = torch.from_numpy(X).cuda().to(torch.bfloat16), torch.empty((T, Dm), dtype=torch.bfloat16, device="cuda")
+    al, be = torch.full((1,), 2.0, device="cuda"), torch.full((1,), 0.2, device="cuda")
+    pqb.pq_ffn_forward(d, Xd, *one[0], *one[1], *one[2], G8, U8, D8, hp, al, be, Y, ws)
+    torch.cuda.synchronize()
+    check_status()
+    v = pqb.pq_ffn_view_init(d, ws)
+    q_m1, g_m1 = O.act_quant(f32(v["M1"]))
+    assert np.array_equal(v["q_m1"].cpu().numpy(), q_m1) and np.array_equal(v["gamma_m1"].cpu().numpy(), g_m1)
+    assert rel_err(f32(v["M1"]), f["m1"]) <= TOL_BF16 and rel_err(f32(Y), f["Y"]) <= TOL_BF16 and rms_err(f32(Y), f["Y"]) <= TOL_RMS
