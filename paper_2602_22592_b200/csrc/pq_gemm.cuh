@@ -360,10 +360,11 @@ __device__ __forceinline__ void gemm_body(const typename P::Params& p) {
           };
           // The next ticket is drawn as late as its trip to memory allows, a ring's worth of steps before the end of the tile: drawn
           // with this one, it would keep a tile from a free pair for as long as this one lasts.  1024 x 1024 over 4096 tokens, sixteen long
-          // tiles and 64 short ones: backward 43.6 -> 35.6 us.
+          // tiles and 64 short ones: backward 43.6 -> 35.6 us.  What the ring holds whole draws with its first step: drawn in the last quarter, two steps
+          // at least, training steps of 200 and 300 tokens, 4096 -> 4096, took 193.8 and 149.7 us instead of 190.9 and 148.2, others from
+          // 1.7 % less (448, 2048 -> 2048, eight experts) to 0.8 % more (640, 2048 -> 2048, four).
           for (int lo = 0, hi; ok && lo < sg.nkb; lo = hi) {
-            const int late = sg.nkb - min(kStages, max(2, sg.nkb >> 2));   // (of a short contraction, its last two steps)
-            hi = kTickets && s + 1 == nseg && lo < late ? late : sg.nkb;
+            hi = kTickets && s + 1 == nseg && lo < sg.nkb - kStages ? sg.nkb - kStages : sg.nkb;
             if (s + 1 == nseg && hi == sg.nkb) draw();
             if (sg.mode <= MODE_BF_KK) produce(std::integral_constant<int, 0>{}, lo, hi);
             else if (sg.mode == MODE_BF_KM && sg.b_blk > 0) produce(std::integral_constant<int, 1>{}, lo, hi);
