@@ -358,7 +358,7 @@ def test_forward_that_keeps_nothing_for_a_backward(T, K, N, r, E, hp8):
 
 
 @pytest.mark.parametrize("T,K,N,r,E,vector", [
-    (100, 1056, 288, 72, 16, False),      # experts without tokens, and several to a tile
+    (100, 1056, 288, 72, 16, False),      # sixteen experts to a tile
     (129, 96, 64, 16, 3, True), (4100, 64, 96, 24, 2, False), (16640, 64, 96, 24, 1, False),   # a tile more than one; many tiles of an expert
 ])
 def test_gradients_of_experts_over_their_items(T, K, N, r, E, vector):
@@ -367,3 +367,51 @@ def test_gradients_of_experts_over_their_items(T, K, N, r, E, vector):
     f = O.linear_forward(c["X"], c["W"], c["A"], c["B"], c["Wr"], c["alpha"], c["beta"])
     g = O.linear_backward(c["dY"], c["X"], f, c["A"], c["B"], c["Wr"], c["alpha"], c["beta"])
     check_backward(c, run_fwd_bwd(c, vector), f, g, vector)
+
+
+@pytest.mark.parametrize("T", [128, 256, 300])        # whole tiles: the experts behind the last token then start a tile beyond it
+def test_gradients_beside_experts_without_tokens(T):
+    c = I.make_linear_case(T, 96, 160, 24, 8, seed=T)
+    planted = np.array([1, 2, 5])[np.arange(T) % 7 % 3]    # none for the first, the last two and two in the middle
+    c["X"] = I.bf16_values(np.random.default_rng(T).standard_normal((T, 96)).astype(np.float32) + 8 * c["Wr"][planted])
+    f = O.linear_forward(c["X"], c["W"], c["A"], c["B"], c["Wr"], c["alpha"], c["beta"])
+    g = O.linear_backward(c["dY"], c["X"], f, c["A"], c["B"], c["Wr"], c["alpha"], c["beta"])
+    tokens = np.bincount(f["idx"], minlength=8)
+    assert np.array_equal(np.flatnonzero(tokens == 0), [0, 3, 4, 6, 7])
+    L = run_fwd_bwd(c, False)
+    check_backward(c, L, f, g, False)
+    for e in (0, 3, 4, 6, 7):
+        assert not bool(L.dA[e].any()) and not bool(L.dB[e].any())
+
+
+@pytest.mark.parametrize("T,K,N,r,E", [(129, 96, 64, 16, 1), (300, 1056, 96, 32, 4), (200, 8704, 64, 0, 0)])
+def test_normalised_forward_that_keeps_nothing(T, K, N, r, E):
+    # the up-projection reads the normalised rows, which the quantiser leaves in the workspace then
+    c = I.make_linear_case(T, K, N, r, E, seed=T, with_grad=False)
+    L = PQLinear(T, K, N, r, E, fused_rmsnorm=True).load_case(c)
+    L.norm_weight, L.norm_eps = (1 + 0.1 * torch.randn(K, device="cuda")).to(torch.bfloat16), 1e-5
+    L.pack()
+    L.forward()
+    Y = torch.zeros_like(L.Y)
+    ws = torch.full((pqb.pq_workspace_bytes(L.desc, pqb.PQ_PHASE_FWD) + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+    pqb.pq_linear_forward_rms(L.desc, L.X, L.norm_weight, L.norm_eps, L.w_s8, L.w_scales, L.A, L.B, L.Wr, L.alpha, L.beta, Y, None, ws[:-4096])
+    torch.cuda.synchronize()
+    check_status()
+    assert torch.equal(Y, L.Y) and bool((ws[-4096:] == 0xA5).all())
+
+
+def test_all_experts_forward_that_keeps_nothing():
+    T, K, N, r, E = 129, 256, 320, 16, 8
+    c = I.make_linear_case(T, K, N, r, E, seed=5, with_grad=False)
+    L = PQLinear(T, K, N, r, E).load_case(c)
+    L.pack()
+    d = pqb.make_desc(T, K, N, r, E, top_k=E, unit_gates=True)
+    saved = torch.empty(pqb.pq_saved_bytes(d), dtype=torch.uint8, device="cuda")
+    ws = torch.full((pqb.pq_workspace_bytes(d, pqb.PQ_PHASE_FWD) + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+    out = []
+    for keep in (saved, None):
+        out.append(torch.zeros_like(L.Y))
+        pqb.pq_linear_forward(d, L.X, L.w_bits, L.w_s8, L.w_scales, L.A, L.B, None, L.alpha, L.beta, out[-1], keep, ws[:-4096])
+        torch.cuda.synchronize()
+    check_status()
+    assert torch.equal(*out) and bool(out[0].any()) and bool((ws[-4096:] == 0xA5).all())
