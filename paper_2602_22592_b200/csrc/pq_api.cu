@@ -397,8 +397,10 @@ static int forward_impl(const pq_desc* d, const uint16_t* X, const uint32_t* w_b
     used += carve_saved(d, static_cast<uint8_t*>(ws) + used, &sv);
   }
   if (ws_bytes < used) return PQ_ERR_WORKSPACE;
-  // Without a backward to come nobody reads q / gamma, nor, where the experts multiply the codes, the sorted copy of X: half and more of what the
-  // quantiser writes.  Whole call, 2048 tokens, with and without them: INT8 experts, 3200 -> 8640 84.1 / 80.9 us, FFN form of 2048 and 5504 106.7 / 103.2.
+  // Without a backward to come nobody reads q / gamma, nor, where the experts multiply the codes, the sorted copy of X.  Of the bytes that the quantiser
+  // writes per value that leaves one of three without routing, one of five with INT8 experts, three of five with bf16 experts (they read
+  // the copy), three of five in front of the FFN form's down projection.  Whole call, 2048 tokens, with and without them: INT8
+  // experts, 3200 -> 8640 84.1 / 80.9 us (repeated passes; the first one on new inputs gains less than 1 %), FFN form of 2048 and 5504 106.7 / 103.2.
   if (!saved || ffn.inner) {
     sv.xt = nullptr;
     if (hp_scales && !norm_weight) sv.xs = nullptr;

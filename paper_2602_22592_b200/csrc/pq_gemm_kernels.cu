@@ -689,15 +689,15 @@ __device__ __forceinline__ float dx_scale(const float* w_scales, const float* be
 // dWr and dA have K as the rows of the tile, 256 of them for the pair, and the short dimension (E or r) as columns: the
 // other way round half of a pair's rows would be empty.
 //
-// Bound by the tensor pipe and, equally, by what an SM takes in from L2 (32 KB per CTA and 512 MMA cycles); the tiles'
+// Bound by the tensor pipe, at the rate that a library's product reaches too: it is active 77 and 65 % of the time (2048 -> 5632 dense,
+// 5632 -> 2048 with eight experts; 32 KB per CTA and 512 MMA cycles from L2, and tiles that take a quarter less gained nothing).  The tiles'
 // contractions run over T, N, the tokens of an expert or a few hundred values, so what was left on the table was the last
 // waves: as three launches (dH, dX, the rest, on two streams) with tiles handed out in turn, pairs with an extra dW tile also
 // got the experts' tiles, and dH kept 64 SMs busy.  Here the longest tiles come first and whoever is free takes the next
 // one.  dH has the first tickets and its readers (dWr, dX, dB, dA) wait for a counter of finished dH tiles: a ticket is
 // drawn by a running pair only, a dH tile waits for nothing, so the counter gets there.  dW needs none of it and fills the
 // time.  Measured, whole training step, three GEMM launches on two streams -> this: 256 tokens, 512 -> 512 54.6 -> 51.8 us;
-// 8192 tokens, eight experts, 2048 -> 2048 329 -> 301 us, 5632 -> 2048 663 -> 671 us (all of it at the 11 TB/s that the SMs
-// together take in from L2).
+// 8192 tokens, eight experts, 2048 -> 2048 329 -> 301 us, 5632 -> 2048 663 -> 671 us.
 // ---------------------------------------------------------------------------
 struct BwdProblem {
   static constexpr int CG = 2, kEpiWarps = 8;
@@ -856,8 +856,8 @@ struct BwdProblem {
       case KIND_DB:
         // The 128 tokens of every item's tile (rows outside the item are zero in g H).  An expert's items lie behind one another, in tiles
         // behind one another, so that its contraction is one run on both sides.  As a segment per item, looked up each time, a step of
-        // these tiles took 1170 cycles, 310 or 512 of them the tensor pipe's.  Training step, eight experts / dense, 8192 tokens: 5632 -> 2048
-        // 654 -> 646 us, 2048 -> 2048 288 -> 284 us, dense 2048 -> 5632 518 -> 504 us.
+        // these tiles took 1170 cycles, 310 or 512 of them the tensor pipe's.  Training step, dense: 8192 tokens, 2048 -> 5632 518 -> 504 us, 4096,
+        // 2048 -> 1024 121 -> 110; with eight experts 1 % (8192 tokens, 5632 -> 2048 649 -> 642, 2048 -> 2048 285 -> 282), what runs differ by.
         s.nkb = 2 * (t.ie - t.ib);
         s.ta = &p.tdyT; s.a_y = t.lo * 128; s.a_blk = p.dy_blk;
         s.tb = &p.tgh; s.b_x = 0; s.b_y = t.rank * p.item_rows + t.ib * 128; s.b_blk = p.gh_blk; s.b_bytes = p.r64 * 128;
